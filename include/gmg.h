@@ -360,9 +360,9 @@ gmg_status gmg_profile_read(gmg_handle h, double *out /* 4 */);
 /* Per-level sums over the same timed cycles since the last call (then reset):
  * out[4l + 0] = ms in level l's Gauss-Seidel sweeps, out[4l + 1] = its colour
  * launches, out[4l + 2] = ms in its residual, restriction and prolongation,
- * out[4l + 3] = ms of the whole level including the coarser ones.  A level
- * run inside the FP32 cycle's cluster tail, or as the coarsest solve, has
- * only out[4l + 3] (the levels below it report 0).  out: 4 * nlev doubles. */
+ * out[4l + 3] = ms of the whole level including the coarser ones.  A cycle's
+ * cluster launch, or its coarsest solve, has only out[4l + 3] of its first level
+ * (the levels below report 0).  out: 4 * nlev doubles. */
 gmg_status gmg_profile_levels(gmg_handle h, double *out);
 
 /* ---- introspection (host outputs) ---- */
@@ -379,14 +379,15 @@ gmg_status gmg_num_levels(gmg_handle h, int *nlev);
 /* rows, stored entries (diagonal included) and colours of level l. */
 gmg_status gmg_level_info(gmg_handle h, int l, int64_t *n, int64_t *nnz, int *ncolors);
 
-/* How the FP32 V-cycle runs level l (the FP64 cycle always uses one launch per
- * colour): 0 = one kernel launch per Gauss-Seidel colour, residual,
- * restriction and prolongation; 1 = a cluster level: its sweeps, residual and
- * restriction in one thread-block-cluster launch and its prolongation and
- * sweeps in another, rows split over the cluster's CTAs with halo copies in
- * distributed shared memory (the same arithmetic per row as path 0 with
- * one warp per row); 2 = inside the cluster tail (this level and all coarser ones in
- * one launch); 3 = the coarsest level (direct solve).  Errors: INVALID_ARG. */
+/* How the FP32 V-cycle runs level l: 0 = one kernel launch per Gauss-Seidel
+ * colour, residual, restriction and prolongation; 1 and 2 = inside the one
+ * thread-block-cluster launch that runs this level and all coarser ones, rows
+ * split over the cluster's CTAs with halo copies in distributed shared memory,
+ * 1 with one thread per row (the same arithmetic per row as path 0 with one
+ * warp per row), 2 with each row's sum split over up to eight lanes; 3 = the
+ * coarsest level (direct solve).  The FP64 cycle runs its coarse levels the
+ * same way on handles whose options ask for FP64 cycles, and with one launch
+ * per colour on the others.  Errors: INVALID_ARG. */
 gmg_status gmg_level_path(gmg_handle h, int l, int *path);
 /* Copies level l's Galerkin operator A_l (CSR, caller numbering, rowptr n+1,
  * col/val nnz) and its colouring (n) into host buffers; any may be NULL. */
@@ -438,7 +439,7 @@ gmg_status gmg_pivot_reciprocal(int64_t n, const double *d, double *out, void *s
 gmg_status gmg_convert(int64_t n, int dir, const void *in, void *out, void *stream);
 
 /* Self-test of the bounded device-side wait (no counterpart in the paper).
- * The cluster-level kernels wait for their streamed matrix entries on an
+ * The cluster kernel waits for its streamed matrix entries on an
  * mbarrier with a limit of polls, after which they set an error word that
  * gmg_solve reports as GMG_ERR_TIMEOUT, instead of hanging.  This runs that
  * wait, in one warp, on an mbarrier that nothing arrives on: *timed_out

@@ -78,13 +78,6 @@ static gmg_status fetch_scalars(gmg_ctx* c, cudaStream_t s) {
         acc[1] += c->lev_gs[l];
         acc[2] += t0 + t1;
       }
-      if (c->lev_kind[l] == 3) {  // cluster level: its two launches hold the sweeps and the transfers
-        float p0 = 0, p1 = 0;
-        GMG_CK(cudaEventElapsedTime(&p0, E[0], E[1]));
-        GMG_CK(cudaEventElapsedTime(&p1, E[3], E[5]));
-        acc[0] += p0 + p1;
-        acc[1] += c->lev_gs[l];
-      }
       if (c->lev_kind[l] != 0) {
         GMG_CK(cudaEventElapsedTime(&t, E[0], E[5]));
         acc[3] += t;
@@ -429,7 +422,7 @@ gmg_status gmg_solve(gmg_handle h, const double* b, double* x, double tol, int m
     info->rel_res = rel;
   }
   GMG_TRY(inverse_status(c, s));  // the pivot check of an inverse this solve joined
-  GMG_TRY(cluster_level_status(c, s));
+  GMG_TRY(cluster_status(c, s));
   return st;
 }
 
@@ -617,10 +610,8 @@ gmg_status gmg_level_path(gmg_handle h, int l, int* path) {
   if (!h || !path || l < 0 || l >= h->nlev) return GMG_ERR_INVALID_ARG;
   if (l == h->nlev - 1)
     *path = 3;
-  else if (h->tail_l0 > 0 && l >= h->tail_l0)
-    *path = 2;
-  else if (h->clev.l > 0 && l == h->clev.l)
-    *path = 1;
+  else if (h->cl32.l0 >= 0 && l >= h->cl32.l0)
+    *path = h->cl32.wide[l - h->cl32.l0] ? 1 : 2;
   else
     *path = 0;
   return GMG_OK;

@@ -501,243 +501,6 @@ __global__ void k_copy(int64_t n, const double* a, double* b) {
   GRID_LOOP(i, n) b[i] = a[i];
 }
 
-// ------------------------------------------------------------------ tail of the FP32 cycle
-// The smoothed levels l0 .. lambda-1 whose vectors fit in shared memory and
-// the coarsest level run in one launch on one thread-block cluster of ncta
-// CTAs.  Every CTA keeps full copies of x, r, b, 1/a_ii and a_ii of each tail
-// level (and x, b of the coarsest level) in its shared memory, plus the
-// sliced-ELL entries of the slices it owns: a slice belongs to the CTA of
-// its first row's range of the caller's numbering (ncta contiguous ranges),
-// so that most neighbours of a row share its CTA.  A phase (one Gauss-Seidel
-// colour, the residual, the restriction, the coarsest GEMV, the
-// prolongation) updates the rows the CTA owns and stores every new value
-// through distributed shared memory into the copies that read it: x of a row
-// into the CTAs owning its neighbours or the finer tail level's rows
-// prolongated from it (a per-row mask), the residual, the restricted
-// right-hand side and the coarsest solution into every CTA; a cluster
-// barrier (release / acquire) ends the phase.  So a phase costs a hardware barrier
-// rather than a kernel boundary, and reads global memory only for the
-// restriction and prolongation weights and the coarsest inverse.  Rows of one
-// colour are never adjacent, so a colour phase reads only values that no CTA
-// writes during it.  All CTAs run the same sequence of barriers.
-
-__device__ __forceinline__ void tail_sync() {
-  __syncwarp();
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ unsigned cluster_rank() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// Stores v at the same shared-memory location in every CTA of the cluster.
-__device__ __forceinline__ void tail_bcast(float* p, float v, int ncta) {
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-  for (int r = 0; r < ncta; ++r) {
-    uint32_t ra;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(r));
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ra), "f"(v) : "memory");
-  }
-}
-
-// Stores v at p in this CTA and at the same location in every CTA whose bit
-// is set in `mask` (the CTAs that read it).
-__device__ __forceinline__ void tail_push(float* p, float v, unsigned mask) {
-  *p = v;
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-  while (mask) {
-    const int r = __ffs(mask) - 1;
-    mask &= mask - 1;
-    uint32_t ra;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(r));
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ra), "f"(v) : "memory");
-  }
-}
-
-template <class U>
-__device__ __forceinline__ U* sm_at(char* sm, int off) {
-  return reinterpret_cast<U*>(sm + off);
-}
-
-// acc = sum over the slice row's entries of a_ij x_j (shared-memory copies),
-// in entry order, loads issued eight entries ahead of the adds.
-__device__ __forceinline__ float tail_row_dot(const float* val, const int* col, const float* x, int off, int w) {
-  float acc = 0.f;
-  int q = 0;
-  for (; q + 8 <= w; q += 8) {
-    int c[8];
-    float v[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      c[j] = col[off + (q + j) * 32];
-      v[j] = val[off + (q + j) * 32];
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc += v[j] * x[c[j]];
-  }
-  for (; q < w; ++q) acc += val[off + q * 32] * x[col[off + q * 32]];
-  return acc;
-}
-
-// One Gauss-Seidel colour k over the owned slices of that colour; each new
-// value goes to this CTA's copy and to the copies of the CTAs that read it.
-__device__ void tail_colour(const TailLevel& L, char* sm, int k) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int* own = sm_at<int>(sm, L.o_own);
-  const int* ocs = sm_at<int>(sm, L.o_ocs);
-  const uint16_t* mask = sm_at<uint16_t>(sm, L.o_mask);
-  float* x = sm_at<float>(sm, L.o_x);
-  for (int j = ocs[k] + warp; j < ocs[k + 1]; j += nw) {
-    const int s = own[j];
-    const float acc = tail_row_dot(sm_at<float>(sm, L.o_val), sm_at<int>(sm, L.o_col), x,
-                                   sm_at<int>(sm, L.o_soff)[s] + lane, sm_at<int>(sm, L.o_width)[s]);
-    if (lane < sm_at<int>(sm, L.o_nrow)[s]) {
-      const int row = sm_at<int>(sm, L.o_row0)[s] + lane;
-      tail_push(x + row, (sm_at<float>(sm, L.o_b)[row] - acc) * sm_at<float>(sm, L.o_dinv)[row], mask[row]);
-    }
-  }
-}
-
-// Over all owned slices (every colour): the residual (mode 1), the
-// prolongation from the next level's x in xn (mode 2), or the copy of the
-// owned rows of x back to global memory (mode 3).
-__device__ void tail_owned(const TailLevel& L, char* sm, int mode, const float* xn, int ncta) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int* own = sm_at<int>(sm, L.o_own);
-  float* x = sm_at<float>(sm, L.o_x);
-  for (int j = warp; j < L.maxown; j += nw) {
-    const int s = own[j];
-    if (s < 0) continue;
-    const bool active = lane < sm_at<int>(sm, L.o_nrow)[s];
-    const int row = sm_at<int>(sm, L.o_row0)[s] + lane;
-    if (mode == 1) {
-      const float acc = tail_row_dot(sm_at<float>(sm, L.o_val), sm_at<int>(sm, L.o_col), x,
-                                     sm_at<int>(sm, L.o_soff)[s] + lane, sm_at<int>(sm, L.o_width)[s]);
-      if (active)
-        tail_bcast(sm_at<float>(sm, L.o_r) + row,
-                   sm_at<float>(sm, L.o_b)[row] - (acc + sm_at<float>(sm, L.o_diag)[row] * x[row]), ncta);
-    } else if (mode == 2) {
-      if (active) {
-        const int q = 3 * row;
-        const float v = x[row] + (L.p_w32[q] * xn[L.p_idx[q]] + L.p_w32[q + 1] * xn[L.p_idx[q + 1]] +
-                                  L.p_w32[q + 2] * xn[L.p_idx[q + 2]]);
-        tail_push(x + row, v, sm_at<uint16_t>(sm, L.o_mask)[row]);
-      }
-    } else if (active) {
-      L.x32[row] = x[row];
-    }
-  }
-}
-
-__global__ void __launch_bounds__(1024, 1) k_tail_cycle(const __grid_constant__ TailDesc D) {
-  extern __shared__ __align__(16) char sm[];
-  const int cta = (int)cluster_rank(), ncta = D.ncta;
-  const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
-  // load everything of the tail that is read during the phases
-  for (int t = 0; t < D.ntail; ++t) {
-    const TailLevel& L = D.lv[t];
-    for (int i = tid; i < L.n; i += nt) {
-      sm_at<float>(sm, L.o_dinv)[i] = L.dinv32[i];
-      sm_at<float>(sm, L.o_diag)[i] = L.diag32[i];
-    }
-    for (int s = tid; s < L.nslice; s += nt) {
-      sm_at<int>(sm, L.o_row0)[s] = L.a_row0[s];
-      sm_at<int>(sm, L.o_nrow)[s] = L.a_nrow[s];
-      sm_at<int>(sm, L.o_width)[s] = (int)((L.a_ptr[s + 1] - L.a_ptr[s]) >> 5);
-      sm_at<int>(sm, L.o_soff)[s] = L.soff[s];
-    }
-    for (int k = tid; k <= L.ncolor; k += nt) sm_at<int>(sm, L.o_cso)[k] = L.cso[k];
-    const int32_t* own = L.own + (int64_t)cta * L.maxown;
-    for (int j = tid; j < L.maxown; j += nt) sm_at<int>(sm, L.o_own)[j] = own[j];
-    for (int k = tid; k <= L.ncolor; k += nt) sm_at<int>(sm, L.o_ocs)[k] = L.ocs[(int64_t)cta * (L.ncolor + 1) + k];
-    for (int i = tid; i < L.n; i += nt) sm_at<uint16_t>(sm, L.o_mask)[i] = L.mask[i];
-    // owned slices' entries, one warp per slice
-    for (int j = warp; j < L.maxown; j += nw) {
-      const int s = own[j];
-      if (s < 0) continue;
-      const int64_t e0 = L.a_ptr[s], ne = L.a_ptr[s + 1] - e0;
-      const int o = L.soff[s];
-      for (int64_t e = lane; e < ne; e += 32) {
-        sm_at<float>(sm, L.o_val)[o + e] = L.a_v32[e0 + e];
-        sm_at<int>(sm, L.o_col)[o + e] = L.a_col[e0 + e];
-      }
-    }
-  }
-  pdl_wait();  // the vectors below are written by the previous kernel
-  pdl_trigger();
-  {
-    const TailLevel& L = D.lv[0];
-    for (int i = tid; i < L.n; i += nt) {
-      sm_at<float>(sm, L.o_x)[i] = L.x32[i];
-      sm_at<float>(sm, L.o_b)[i] = L.b32[i];
-    }
-  }
-  __syncthreads();
-  tail_sync();
-  // down: smoothing (colour 0 of the first sweep was applied from x = 0 by the
-  // restriction that produced b when c0_first), residual, restriction
-  for (int t = 0; t < D.ntail; ++t) {
-    const TailLevel& L = D.lv[t];
-    for (int it = 0; it < D.nu_pre; ++it)
-      for (int k = (it == 0 && D.c0_first) ? 1 : 0; k < L.ncolor; ++k) {
-        tail_colour(L, sm, k);
-        tail_sync();
-      }
-    tail_owned(L, sm, 1, nullptr, ncta);
-    tail_sync();
-    // restriction: b_next = P^T r over the owned slices of the transpose; the
-    // next iterate starts from zero (each CTA clears its own copy), except
-    // that a smoothed next level gets its colour-0 rows' first Gauss-Seidel
-    // update (b - 0) / a_ii right away, stored by their owner into every copy
-    const bool last = t + 1 == D.ntail;
-    float* bn = last ? sm_at<float>(sm, D.o_bc) : sm_at<float>(sm, D.lv[t + 1].o_b);
-    float* xn = last ? sm_at<float>(sm, D.o_xc) : sm_at<float>(sm, D.lv[t + 1].o_x);
-    const float* dn = last ? nullptr : sm_at<float>(sm, D.lv[t + 1].o_dinv);
-    const int nn = last ? D.nc : D.lv[t + 1].n;
-    const int n0 = (last || !D.c0_first) ? 0 : D.lv[t + 1].nc0;
-    for (int i = n0 + tid; i < nn; i += nt) xn[i] = 0.f;
-    const float* r = sm_at<float>(sm, L.o_r);
-    for (int s = cta + warp * ncta; s < L.r_nslice; s += nw * ncta) {
-      if (lane >= L.r_nrow[s]) continue;
-      const int64_t e0 = L.r_ptr[s] + lane;
-      const int wd = (int)((L.r_ptr[s + 1] - L.r_ptr[s]) >> 5);
-      float acc = 0.f;
-      for (int q = 0; q < wd; ++q) acc += L.r_v32[e0 + (int64_t)q * 32] * r[L.r_col[e0 + (int64_t)q * 32]];
-      const int row = L.r_row0[s] + lane;
-      tail_bcast(bn + row, acc, ncta);
-      if (row < n0) tail_bcast(xn + row, (acc - 0.f) * dn[row], ncta);
-    }
-    tail_sync();
-  }
-  // coarsest: x_c = A^-1 b_c, one warp per row
-  {
-    const float* bc = sm_at<float>(sm, D.o_bc);
-    float* xc = sm_at<float>(sm, D.o_xc);
-    for (int J = cta + warp * ncta; J < D.nc; J += nw * ncta) {
-      const float* a = D.ainv32 + (int64_t)J * D.nc;
-      float acc = 0.f;
-      for (int K = lane; K < D.nc; K += 32) acc += a[K] * bc[K];
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0) tail_bcast(xc + J, acc, ncta);
-    }
-    tail_sync();
-  }
-  // up: prolongation and post-smoothing
-  for (int t = D.ntail - 1; t >= 0; --t) {
-    const TailLevel& L = D.lv[t];
-    const float* xn = t + 1 == D.ntail ? sm_at<float>(sm, D.o_xc) : sm_at<float>(sm, D.lv[t + 1].o_x);
-    tail_owned(L, sm, 2, xn, ncta);
-    tail_sync();
-    for (int it = 0; it < D.nu_post; ++it)
-      for (int q = 0; q < L.ncolor; ++q) {
-        tail_colour(L, sm, D.post_forward ? q : L.ncolor - 1 - q);
-        tail_sync();
-      }
-  }
-  // the owned rows of the first tail level back to global memory
-  tail_owned(D.lv[0], sm, 3, nullptr, ncta);
-}
-
 // ------------------------------------------------------------------ launchers
 
 // Timing events: inside a stream capture they become external event nodes
@@ -808,56 +571,10 @@ gmg_status launch_coarse(gmg_ctx* c, const T* b, T* x, cudaStream_t s) {
   return launch(k_coarse<T>, (n * 32 + 255) / 256, 256, s, n, (const double*)c->Ainv, b, x);
 }
 
-// The tail of an FP32 cycle (levels tail_l0 .. lambda) as one cluster launch.
-static gmg_status launch_tail(gmg_ctx* c, cudaStream_t s) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(c->tail.ncta);
-  cfg.blockDim = dim3(c->tail_threads);
-  cfg.dynamicSmemBytes = (size_t)c->tail_smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = c->tail.ncta;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = use_pdl() ? 2 : 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_tail_cycle, c->tail);
-  ++g_launches;
-  if (e != cudaSuccess) {
-    set_error(std::string("tail cluster launch: ") + cudaGetErrorString(e));
-    return GMG_ERR_CUDA;
-  }
-  return GMG_OK;
-}
-
-gmg_status tail_configure(gmg_ctx* c, int ncta, int threads, int smem, bool* ok) {
-  *ok = false;
-  if (cudaFuncSetAttribute(k_tail_cycle, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-      cudaFuncSetAttribute(k_tail_cycle, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmemLimit) != cudaSuccess) {
-    cudaGetLastError();
-    return GMG_OK;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ncta);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = ncta;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  int nclusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&nclusters, k_tail_cycle, &cfg) != cudaSuccess) {
-    cudaGetLastError();
-    return GMG_OK;
-  }
-  *ok = nclusters >= 1;
-  return GMG_OK;
+// First level of the cluster form of the cycle in this precision (-1: none).
+template <class T>
+static int cluster_l0(const gmg_ctx* c) {
+  return sizeof(T) == 4 ? c->cl32.l0 : c->cl64.l0;
 }
 
 // MGI(x_l, b_l, l) of Alg. 2 on the level's own vectors.  x_l holds the
@@ -872,9 +589,7 @@ gmg_status vcycle(gmg_ctx* c, int l, cudaStream_t s, bool c0_done, T* x_in, cons
   const T* b = b_in ? b_in : Vec<T>::b(L);
   const bool lp = c->prof && (int)c->lev_ev.size() >= 6 * c->nlev;  // per-level events
   cudaEvent_t* E = lp ? &c->lev_ev[6 * l] : nullptr;
-  bool whole = l == c->nlev - 1;
-  if constexpr (std::is_same<T, float>::value) whole = whole || (c->tail_l0 > 0 && l == c->tail_l0);
-  if (whole) {  // the coarsest solve, or the cluster tail from this level down
+  if (l == c->nlev - 1 || l == cluster_l0<T>(c)) {  // the coarsest solve, or the cluster from this level down
     if (c->inv_pending) {  // a refresh's coarsest inverse may still be running: wait for it here
       cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
       GMG_CK(cudaStreamIsCapturing(s, &cs));
@@ -889,8 +604,14 @@ gmg_status vcycle(gmg_ctx* c, int l, cudaStream_t s, bool c0_done, T* x_in, cons
       c->lev_kind[l] = 2;
       c->lev_gs[l] = 0;
     }
+    if (c->prof && l == 0)  // no finest smoothing blocks of their own: an empty interval before and after
+      for (int q : {0, 1}) GMG_CK(record_timing_event(c->ev[q], s));
     if (l == c->nlev - 1) GMG_TRY(launch_coarse<T>(c, b, x, s));
-    else GMG_TRY(launch_tail(c, s));
+    else GMG_TRY(launch_cluster<T>(c, x, b, c0_done, s));
+    if (c->prof && l == 0) {
+      for (int q : {2, 3}) GMG_CK(record_timing_event(c->ev[q], s));
+      c->prof_gs = 0;
+    }
     if (lp) {
       GMG_CK(record_timing_event(E[5], s));
       for (int k = l + 1; k < c->nlev; ++k) c->lev_kind[k] = 0;
@@ -898,22 +619,6 @@ gmg_status vcycle(gmg_ctx* c, int l, cudaStream_t s, bool c0_done, T* x_in, cons
     return GMG_OK;
   }
   Level& C = c->L[l + 1];
-  if constexpr (std::is_same<T, float>::value) {
-    if (c->clev.l == l && l > 0 && c0_done && !x_in && !b_in) {  // this level on a thread-block cluster
-      if (lp) GMG_CK(record_timing_event(E[0], s));
-      GMG_TRY(launch_cluster_level(c, 0, s));
-      if (lp) GMG_CK(record_timing_event(E[1], s));
-      GMG_TRY(vcycle<T>(c, l + 1, s, true));
-      if (lp) GMG_CK(record_timing_event(E[3], s));
-      GMG_TRY(launch_cluster_level(c, 1, s));
-      if (lp) {
-        GMG_CK(record_timing_event(E[5], s));
-        c->lev_kind[l] = 3;
-        c->lev_gs[l] = c->opt.nu_pre * L.ncolor - 1 + c->opt.nu_post * L.ncolor;
-      }
-      return GMG_OK;
-    }
-  }
   const bool prof = c->prof && l == 0;
   if (prof) GMG_CK(record_timing_event(c->ev[0], s));
   if (lp) GMG_CK(record_timing_event(E[0], s));

@@ -169,6 +169,7 @@ struct Level {
   std::vector<int64_t> color_slice_off;  // host: first slice of each colour (+ end)
   std::vector<int32_t> h_color;          // host: colour of every row (caller numbering)
   std::vector<int32_t> h_key;            // host: locality rank of every row (caller numbering)
+  std::vector<int64_t> h_ptr;            // host: entry offsets of the slices of A (set-up only)
   // numbering: perm[new] = old, iperm[old] = new
   int32_t* perm = nullptr;
   int32_t* iperm = nullptr;
@@ -218,92 +219,50 @@ struct Level {
   float *X32 = nullptr, *B32 = nullptr, *R32 = nullptr;  // [n x kMaxRhs]
 };
 
-// The tail of an FP32 V-cycle (the smoothed levels l0 .. lambda-1 and the
-// coarsest level) runs as one launch on one thread-block cluster; these are
-// its descriptors (passed by value).  Offsets are bytes into the dynamic
-// shared memory of every CTA (the same layout in each).
-constexpr int kMaxTail = 4;            // smoothed levels in the tail
-constexpr int kTailSmemLimit = 227 * 1024;  // the largest dynamic shared memory of a CTA (no static shared memory)
-struct TailLevel {
-  int n, ncolor, nslice, r_nslice;
-  int nc0;  // rows of colour 0 (the first rows in the colour-major numbering)
-  // shared-memory copies: x, r, b, 1/a_ii, a_ii (all rows); per slice: first
-  // row, rows, width, offset of its entries in the owner's arrays; colour
-  // slice offsets; the owned slices' values and columns
-  int o_x, o_r, o_b, o_dinv, o_diag, o_row0, o_nrow, o_width, o_soff, o_cso, o_own, o_val, o_col, o_ocs, o_mask;
-  int maxown;             // owned slices per CTA (list padded with -1)
-  const int32_t* own;     // ncta x maxown: each CTA's slices, colour by colour
-  const int32_t* ocs;     // ncta x (ncolor + 1): where each colour starts in a CTA's list
-  const uint16_t* mask;   // per row: the other CTAs that read its x (bit per CTA)
-  const int64_t* a_ptr;
-  const int32_t *a_row0, *a_nrow, *a_col;
-  const float *a_v32, *dinv32, *diag32;
-  const int32_t* soff;  // offset of each slice's entries in its owner CTA's arrays
-  const int32_t* cso;   // first slice of every colour (+ end)
-  // restriction into the next level (sliced ELL over its rows) and
-  // prolongation from it (three slots per row of this level)
-  const int64_t* r_ptr;
-  const int32_t *r_row0, *r_nrow, *r_col;
-  const float* r_v32;
-  const int32_t* p_idx;
-  const float* p_w32;
-  float *x32, *b32;  // global vectors of this level (the first tail level reads x, b and writes x)
-};
-struct TailDesc {
-  int ntail, nc, ncta;
-  int nu_pre, nu_post, post_forward;
-  int c0_first;          // colour 0 of the first pre-smoothing sweep is done by the restriction
-  int o_xc, o_bc;        // shared-memory copies of the coarsest x and b
-  const float* ainv32;   // coarsest inverse, FP32, nc x nc
-  TailLevel lv[kMaxTail];
-};
-
-// A smoothed level whose FP32 sweeps, residual, restriction (one launch) and
-// prolongation, sweeps (another) run on one thread-block cluster: the rows
-// are split into ncta contiguous ranges of the caller's numbering (one per
-// CTA, every colour balanced), each CTA keeps x of its rows and of their
-// neighbours owned by other CTAs (the halo) in shared memory, an updated row
-// is stored into the halo copies of the CTAs that read it, and the entries of
-// the next phases' rows stream from L2 into shared memory while the current
-// phase computes.  Per-CTA arrays are concatenated; *_off[cta] is a CTA's
-// start in them.
-constexpr int kClusterStagesMax = 4;  // entry buffers (the current phase and up to three ahead)
+// The coarse part of a V-cycle on one thread-block cluster (gmg_cluster.cu):
+// the smoothed levels l0 .. lambda-1 and the coarsest, rows split over the
+// CTAs.  Offsets are bytes into the dynamic shared memory of every CTA (the
+// same layout in each); images are per CTA in global memory, copied whole.
+constexpr int kClMaxLevels = 6;         // smoothed levels in the cluster
+constexpr int kClStages = 4;            // entry buffers (the current phase and up to three ahead)
+constexpr int kSmemLimit = 227 * 1024;  // the largest dynamic shared memory of a CTA (no static shared memory)
+template <class T>
 struct ClusterLevel {
-  int l = 0, ncta = 0, threads = 0, ncolor = 0;
-  int nu_pre = 0, nu_post = 0, post_forward = 0, c0_first = 0;
-  int n_loc_max = 0, n_own_max = 0, nsl_max = 0, blk_max = 0;
-  int nstage = 0, push_max = 0;
-  // shared memory: x (own and halo rows), b (own rows), then the set-up image
-  // [o_st, o_st + st_bytes) holding 1/a_ii, a_ii, the slice and colour
-  // tables, the local-to-global rows and the halo stores (copied whole from
-  // img + cta * st_bytes), then the barriers of the copies and the entry stages
-  int o_x = 0, o_b = 0, o_st = 0, st_bytes = 0, o_dinv = 0, o_diag = 0, o_sl = 0, o_csl = 0, o_l2g = 0, o_pp = 0,
-      o_pd = 0, o_mbar = 0, o_buf = 0, smem = 0;
-  const char* img = nullptr;
+  int ncolor, tpr, lg_tpr, r_tpr, lg_r_tpr;  // lanes per row of the sweeps and of the restriction from this level
+  bool streamed;                             // entries stream from L2 instead of staying in shared memory
+  int n_own_max, n_loc_max, rsl_max;
+  // shared memory: the image (header: own rows, own and halo rows, slices,
+  // restriction slices, own rows of colour 0; then slices, colours, halo
+  // stores of x and of the residual, resident columns), the values (1/a_ii,
+  // then resident entries), x (own and halo rows), b (own rows)
+  int o_img, o_val, o_x, o_b;
+  int img_bytes, val_bytes;
+  int i_sl, i_csl, i_xp, i_xd, i_rp, i_rd, i_col, v_val;
+  const char *img, *vimg;
+  const T* diag;          // per CTA n_own_max
+  const uint16_t* p_idx;  // per CTA 3 x n_own_max: the prolongation into this level
+  const T* p_w;
+  const int4* r_sl;       // per CTA rsl_max slices of the restriction from this level
+  const uint16_t* r_col;
+  const T* r_w;
+  const int32_t *vsrc, *dsrc;  // where the values and the diagonal come from (refresh)
+  int64_t nvsrc, ndsrc, n_stream;
+};
+template <class T>
+struct ClusterDesc {
+  int l0 = -1;  // first level (-1: no cluster)
+  int ncta = 0, nlev = 0, nc = 0;
+  int nu_pre = 0, nu_post = 0, post_forward = 0;
+  int nstage = 0, nsteps = 0, stage_bytes = 0, stage_col = 0;
+  int o_mbar = 0, o_r = 0, o_bc = 0, o_buf = 0, i_steps = 0, smem = 0;
   int* err = nullptr;  // set when a bounded wait for an entry block gave up
-  const int32_t *n_own = nullptr, *n_loc = nullptr, *loc_off = nullptr, *loc2glob = nullptr;
-  // slices of each CTA, colour by colour: first local row, rows, width, first
-  // entry (relative to the CTA's entries); csl: first slice of every colour
-  // (+ end), relative to the CTA's slices
-  const int32_t *sl_off = nullptr, *sl_row0 = nullptr, *sl_nrow = nullptr, *sl_w = nullptr, *sl_eoff = nullptr;
-  const int32_t* csl = nullptr;  // ncta x (ncolor + 1)
-  const int64_t* ent_off = nullptr;
-  const float* ent_val = nullptr;  // [k][lane] per slice; refreshed with the level's values
-  const int32_t* ent_col = nullptr;  // local column
-  // halo stores: for each own row, the (CTA << 16 | local index) copies to update
-  const int32_t *push_off = nullptr, *push_ptr = nullptr, *push_dst = nullptr;
-  // the level's global vectors and transfers
-  float *x32 = nullptr, *b32 = nullptr, *r32 = nullptr;
-  const float *dinv32 = nullptr, *diag32 = nullptr;
-  const int32_t* p_idx = nullptr;
-  const float* p_w32 = nullptr;
-  const int64_t* r_ptr = nullptr;
-  const int32_t *r_row0 = nullptr, *r_nrow = nullptr, *r_col = nullptr;
-  const float* r_v32 = nullptr;
-  int64_t r_nslice = 0;
-  float *xc32 = nullptr, *bc32 = nullptr;  // next level's x and b
-  const float* dinvc32 = nullptr;
-  int64_t nc0 = 0;  // next level's colour-0 rows (their first update done by the restriction)
+  const T* ainv = nullptr;
+  const int32_t* l2g = nullptr;  // level l0: global rows of each CTA's own and halo rows
+  const T* s_val = nullptr;      // streamed entries
+  const uint16_t* s_col = nullptr;
+  const int32_t* s_src = nullptr;
+  ClusterLevel<T> lv[kClMaxLevels + 1] = {};
+  bool wide[kClMaxLevels] = {};  // one thread per row (the per-colour kernels' sums)
 };
 
 }  // namespace gmg
@@ -328,16 +287,10 @@ struct gmg_ctx {
   double* ml_L = nullptr;
   int64_t* ml_dpos = nullptr;
   double ml_t = 0.0;
-  // FP32 cycles run levels >= tail_l0 as one cluster launch (0 = off)
-  int tail_l0 = 0;
-  int tail_smem = 0;
-  int tail_threads = 1024;
-  gmg::TailDesc tail{};
-  // FP32 cycles run level clev.l (0 = none) as two cluster launches
-  gmg::ClusterLevel clev{};
-  int64_t* clev_src = nullptr;  // ELL slot of every cluster-level entry (-1: padding)
-  int64_t clev_nent = 0;
-  float* Ainv32 = nullptr;  // coarsest inverse in FP32 for the tail launch
+  // cycles run levels >= cl32.l0 (FP32) or cl64.l0 (FP64) as one cluster launch
+  gmg::ClusterDesc<float> cl32{};
+  gmg::ClusterDesc<double> cl64{};
+  float* Ainv32 = nullptr;  // coarsest inverse in FP32 for the cluster launch
   int* dstatus = nullptr;   // device status words
   // outer iteration (finest level, permuted numbering, FP64)
   double *xs = nullptr, *bs = nullptr, *rs = nullptr, *zs = nullptr, *ps = nullptr, *qs = nullptr, *ros = nullptr;
@@ -381,7 +334,7 @@ struct gmg_ctx {
   // per-level timing of the same cycles: six events per level (before and
   // after pre-smoothing, after the restriction, after the coarser levels,
   // after the prolongation, after post-smoothing); levels run inside the
-  // cluster tail or as the coarsest solve record only the first and last
+  // cluster launch or as the coarsest solve record only the first and last
   std::vector<cudaEvent_t> lev_ev;
   std::vector<int> lev_kind;    // per level: 0 not recorded, 1 all six events, 2 first and last only
   std::vector<int> lev_gs;      // GS launches of the level in the last timed cycle
@@ -394,16 +347,14 @@ namespace gmg {
 gmg_status join_inverse(gmg_ctx* c, cudaStream_t s, bool check);
 // Reads the pivot check of a joined inverse once (GMG_ERR_CHOLESKY on failure).
 gmg_status inverse_status(gmg_ctx* c, cudaStream_t s);
-// Whether a tail cluster of ncta CTAs with `smem` bytes of shared memory each
-// can be scheduled on the device (sets the kernel's attributes).
-gmg_status tail_configure(gmg_ctx* c, int ncta, int threads, int smem, bool* ok);
-// Cluster form of one smoothed level of the FP32 cycle (gmg_clevel.cu): the
-// tables from the level's pattern and numberings (host), the entry values
-// after a numeric set-up, and the two launches (mode 0: pre-smoothing,
-// residual, restriction; mode 1: prolongation, post-smoothing).
-gmg_status build_cluster_level(gmg_ctx* c, int l, const int64_t* rp, const int32_t* ci,
-                               const std::vector<int32_t>& perm, const std::vector<int32_t>& iperm);
+// The cluster form of the coarse levels (gmg_cluster.cu): tables from the
+// levels' patterns and numberings (host), values after a numeric set-up, the
+// launch x <- MGI(x, b, l0), and the state of its bounded waits.
+gmg_status build_cluster(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
+                         const std::vector<std::vector<int32_t>>& hcol, const std::vector<std::vector<int32_t>>& perm,
+                         const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P);
 gmg_status refresh_cluster_values(gmg_ctx* c, cudaStream_t s);
-gmg_status launch_cluster_level(gmg_ctx* c, int mode, cudaStream_t s);
-gmg_status cluster_level_status(gmg_ctx* c, cudaStream_t s);
+template <class T>
+gmg_status launch_cluster(gmg_ctx* c, T* x, const T* b, bool c0_first, cudaStream_t s);
+gmg_status cluster_status(gmg_ctx* c, cudaStream_t s);
 }  // namespace gmg
