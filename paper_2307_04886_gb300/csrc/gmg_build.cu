@@ -48,6 +48,7 @@ constexpr int kRing = 96;      // points of a 2-ring handled per sampling search
 constexpr int kCand = 512;     // coarse-neighbour candidates gathered per cell
 constexpr int kFallback = 64;  // candidates of the inverse-distance fallback
 constexpr int kBlockRows = 1024;
+constexpr int kRow = 32;       // later points within r kept in a point's own row (a longer list takes a second pass)
 
 // ---- explicitly rounded double arithmetic (never contracted into an FMA)
 __device__ __forceinline__ double ad(double a, double b) { return __dadd_rn(a, b); }
@@ -64,62 +65,96 @@ __device__ __forceinline__ V3 vcross(V3 a, V3 b) {
   return V3{sb(ml(a.y, b.z), ml(a.z, b.y)), sb(ml(a.z, b.x), ml(a.x, b.z)), sb(ml(a.x, b.y), ml(a.y, b.x))};
 }
 __device__ __forceinline__ double vnorm(V3 a) { return __dsqrt_rn(vdot(a, a)); }
-__device__ __forceinline__ double edge_len(const double* X, int64_t u, int64_t v) {
-  return vnorm(vsub(at(X, u), at(X, v)));
-}
 
-// ---- mean edge length: row sums, block sums, then the block sums in order
-__global__ void k_row_lengths(int64_t n, const double* __restrict__ X, const int64_t* __restrict__ rp,
-                              const int32_t* __restrict__ ci, double* __restrict__ rsum, int* __restrict__ rcnt) {
+// ---- edge lengths, once per stored entry (the sampling searches and the
+// Voronoi rounds read each of them many times; on GB300 an FP64 instruction
+// occupies its sub-partition's pipe for 64 cycles, and a length takes about
+// twenty), and the sum over a row's later neighbours
+__global__ void k_edge_lengths(int64_t n, const double* __restrict__ X, const int64_t* __restrict__ rp,
+                               const int32_t* __restrict__ ci, double* __restrict__ len, double* __restrict__ rsum,
+                               int* __restrict__ rcnt) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double s = 0.0;
     int c = 0;
-    for (int64_t k = rp[i]; k < rp[i + 1]; ++k)
+    const V3 p = at(X, i);
+#pragma unroll 4
+    for (int64_t k = rp[i]; k < rp[i + 1]; ++k) {
+      const double l = vnorm(vsub(p, at(X, ci[k])));
+      len[k] = l;
       if (ci[k] > i) {
-        s = ad(s, edge_len(X, i, ci[k]));
+        s = ad(s, l);
         ++c;
       }
+    }
     rsum[i] = s;
     rcnt[i] = c;
   }
 }
-__global__ void k_block_lengths(int64_t n, const double* __restrict__ rsum, const int* __restrict__ rcnt,
-                                double* __restrict__ bsum, int64_t* __restrict__ bcnt) {
-  const int64_t nb = (n + kBlockRows - 1) / kBlockRows;
-  for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += (int64_t)gridDim.x * blockDim.x) {
+// ---- mean edge length: row sums, block sums of 1024 rows, then the block
+// sums, each added in order.  The values are staged in shared memory by the
+// whole block; one thread adds them (a chain of dependent FP64 adds, so the
+// loads must not be part of it).
+__global__ void __launch_bounds__(256) k_block_lengths(int64_t n, const double* __restrict__ rsum,
+                                                       const int* __restrict__ rcnt, double* __restrict__ bsum,
+                                                       int64_t* __restrict__ bcnt) {
+  __shared__ double v[kBlockRows];
+  __shared__ unsigned long long cs;
+  const int64_t b = blockIdx.x;
+  const int m = (int)(n - b * kBlockRows < kBlockRows ? n - b * kBlockRows : kBlockRows);
+  if (threadIdx.x == 0) cs = 0;
+  __syncthreads();
+  unsigned long long c = 0;
+  for (int q = threadIdx.x; q < m; q += 256) {
+    v[q] = rsum[b * kBlockRows + q];
+    c += (unsigned long long)rcnt[b * kBlockRows + q];
+  }
+  atomicAdd(&cs, c);
+  __syncthreads();
+  if (threadIdx.x == 0) {
     double s = 0.0;
-    int64_t c = 0;
-    for (int64_t i = b * kBlockRows; i < n && i < (b + 1) * kBlockRows; ++i) {
-      s = ad(s, rsum[i]);
-      c += rcnt[i];
-    }
+    for (int q = 0; q < m; ++q) s = ad(s, v[q]);
     bsum[b] = s;
-    bcnt[b] = c;
+    bcnt[b] = (int64_t)cs;
   }
 }
 // geo[0] = mean edge length, geo[1] = sampling radius f * mean, geo[2] =
-// smallest candidate-triangle area 1e-12 * mean^2
-__global__ void k_mean_length(int64_t nb, const double* __restrict__ bsum, const int64_t* __restrict__ bcnt,
-                              double f, double* __restrict__ geo) {
+// smallest candidate-triangle area 1e-12 * mean^2.  One block of 1024.
+__global__ void __launch_bounds__(1024) k_mean_length(int64_t nb, const double* __restrict__ bsum,
+                                                      const int64_t* __restrict__ bcnt, double f,
+                                                      double* __restrict__ geo) {
+  __shared__ double v[1024];
+  __shared__ unsigned long long cs;
+  if (threadIdx.x == 0) cs = 0;
+  __syncthreads();
   double s = 0.0;
-  int64_t c = 0;
-  for (int64_t b = 0; b < nb; ++b) {
-    s = ad(s, bsum[b]);
-    c += bcnt[b];
+  for (int64_t b0 = 0; b0 < nb; b0 += 1024) {
+    const int m = (int)(nb - b0 < 1024 ? nb - b0 : 1024);
+    if ((int)threadIdx.x < m) {
+      v[threadIdx.x] = bsum[b0 + threadIdx.x];
+      atomicAdd(&cs, (unsigned long long)bcnt[b0 + threadIdx.x]);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int q = 0; q < m; ++q) s = ad(s, v[q]);
+    __syncthreads();
   }
-  const double e = c ? s / (double)c : 1.0;
-  geo[0] = e;
-  geo[1] = ml(f, e);
-  geo[2] = ml(ml(1e-12, e), e);
+  if (threadIdx.x == 0) {
+    const double e = cs ? s / (double)(int64_t)cs : 1.0;
+    geo[0] = e;
+    geo[1] = ml(f, e);
+    geo[2] = ml(ml(1e-12, e), e);
+  }
 }
 
 // ---- sampling: the later points within r of every point (2-ring Dijkstra)
-// With fill == nullptr counts them (and counts every point's earlier points
-// within r in `blockers`); else writes them at fill[off[t] ..].
-__global__ void k_balls(int64_t n, const double* __restrict__ X, const int64_t* __restrict__ rp,
+// Without `off` counts them in nlater (and every point's earlier points
+// within r in `blockers`) and, given `fill`, writes the first kRow of point s
+// at fill[kRow s ..], raising *err2 when a point has more; with `off` writes
+// them all at fill[off[s] ..].
+__global__ void k_balls(int64_t n, const double* __restrict__ len, const int64_t* __restrict__ rp,
                         const int32_t* __restrict__ ci, const double* __restrict__ geo, int* __restrict__ nlater,
                         int* __restrict__ blockers, const int64_t* __restrict__ off, int32_t* __restrict__ fill,
-                        int* __restrict__ err) {
+                        int* __restrict__ err, int* __restrict__ err2) {
   const double r = geo[1];
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
     int32_t ring[kRing];
@@ -147,7 +182,7 @@ __global__ void k_balls(int64_t n, const double* __restrict__ X, const int64_t* 
         }
     if (over) {
       atomicExch(err, 1);
-      if (!fill) nlater[s] = 0;
+      if (!off) nlater[s] = 0;
       continue;
     }
     for (int q = 0; q < m; ++q) {
@@ -164,8 +199,12 @@ __global__ void k_balls(int64_t n, const double* __restrict__ X, const int64_t* 
       done[best] = true;
       const int32_t u = ring[best];
       if (u > s) {
-        if (fill) fill[off[s] + out] = u;
-        else atomicAdd(&blockers[u], 1);
+        if (off) {
+          fill[off[s] + out] = u;
+        } else {
+          atomicAdd(&blockers[u], 1);
+          if (fill && out < kRow) fill[s * kRow + out] = u;
+        }
         ++out;
       }
       for (int64_t k = rp[u]; k < rp[u + 1]; ++k) {
@@ -173,38 +212,85 @@ __global__ void k_balls(int64_t n, const double* __restrict__ X, const int64_t* 
         int q = 0;
         while (q < m && ring[q] != v) ++q;
         if (q == m || done[q]) continue;
-        const double nd = ad(dist[best], edge_len(X, u, v));
+        const double nd = ad(dist[best], len[k]);
         if (nd < dist[q]) dist[q] = nd;
       }
     }
-    if (!fill) nlater[s] = out;
+    if (!off) {
+      nlater[s] = out;
+      if (out > kRow) *err2 = 1;
+    }
   }
 }
 
-// Exclusive scan of n int counts into off[0..n] (one block of 1024 threads).
-__global__ void k_scan(int64_t n, const int* __restrict__ cnt, int64_t* __restrict__ off) {
-  __shared__ int64_t part[1024];
-  const int t = threadIdx.x;
-  const int64_t chunk = (n + 1023) / 1024;
-  const int64_t b = t * chunk, e = b + chunk < n ? b + chunk : n;
-  int64_t s = 0;
-  for (int64_t i = b; i < e; ++i) s += cnt[i];
-  part[t] = s;
+// Exclusive scan of n int counts into off[0 .. n]: tile sums, their scan by
+// one block, then each tile's scan (three passes over all SMs; one block of
+// 1024 threads walking n/1024 counts each took 864 us at n = 524,288, this
+// 12 us).
+constexpr int kTile = 4096;
+__global__ void __launch_bounds__(256) k_scan_sums(int64_t n, const int* __restrict__ cnt, int64_t* __restrict__ sums) {
+  __shared__ unsigned long long t;
+  if (threadIdx.x == 0) t = 0;
   __syncthreads();
-  if (t == 0) {
-    int64_t acc = 0;
-    for (int k = 0; k < 1024; ++k) {
-      const int64_t v = part[k];
-      part[k] = acc;
-      acc += v;
+  int64_t s = 0;
+  for (int q = threadIdx.x; q < kTile; q += 256) {
+    const int64_t i = (int64_t)blockIdx.x * kTile + q;
+    if (i < n) s += cnt[i];
+  }
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) atomicAdd(&t, (unsigned long long)s);
+  __syncthreads();
+  if (threadIdx.x == 0) sums[blockIdx.x] = (int64_t)t;
+}
+// Exclusive scan over a block of 1024 threads; the total in *total.
+__device__ int64_t block_scan(int64_t v, int64_t* warps, int64_t* total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int64_t x = v;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) warps[w] = x;
+  __syncthreads();
+  if (w == 0) {
+    const int64_t u = lane < nw ? warps[lane] : 0;
+    int64_t z = u;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, z, o);
+      if (lane >= o) z += y;
     }
-    off[n] = acc;
+    warps[lane] = z - u;
+    if (lane == 31) *total = z;
   }
   __syncthreads();
-  int64_t acc = part[t];
-  for (int64_t i = b; i < e; ++i) {
-    off[i] = acc;
-    acc += cnt[i];
+  const int64_t r = warps[w] + x - v;
+  return r;
+}
+__global__ void __launch_bounds__(1024) k_scan_tiles(int64_t nt, int64_t* __restrict__ sums, int64_t* __restrict__ end) {
+  __shared__ int64_t warps[32], total;
+  int64_t base = 0;
+  for (int64_t t0 = 0; t0 < nt; t0 += 1024) {
+    const int64_t t = t0 + threadIdx.x;
+    const int64_t v = t < nt ? sums[t] : 0;
+    const int64_t x = block_scan(v, warps, &total);
+    if (t < nt) sums[t] = base + x;
+    base += total;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *end = base;
+}
+__global__ void __launch_bounds__(1024) k_scan_apply(int64_t n, const int* __restrict__ cnt,
+                                                     const int64_t* __restrict__ sums, int64_t* __restrict__ off) {
+  __shared__ int64_t warps[32], total;
+  const int64_t i0 = (int64_t)blockIdx.x * kTile + 4 * threadIdx.x;
+  int c[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) c[q] = i0 + q < n ? cnt[i0 + q] : 0;
+  int64_t x = sums[blockIdx.x] + block_scan((int64_t)c[0] + c[1] + c[2] + c[3], warps, &total);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (i0 + q < n) off[i0 + q] = x;
+    x += c[q];
   }
 }
 
@@ -223,27 +309,42 @@ __global__ void k_mis_start(int64_t n, const int* __restrict__ blockers, int* __
   }
 }
 
-// One propagation round over the points decided in the previous round.
+// The later points within r of point t: its own row of kRow, or a CSR row.
+__device__ __forceinline__ int64_t later_of(int32_t t, const int64_t* off, const int* nlater, int* cnt) {
+  if (off) {
+    const int64_t b = off[t];
+    *cnt = (int)(off[t + 1] - b);
+    return b;
+  }
+  *cnt = nlater[t];
+  return (int64_t)t * kRow;
+}
+
+// One propagation round over the points decided in the previous round, when
+// there are more than kChainMax of them (k_mis_chain takes the short ones).
 // A sample rules out its later points within r; a ruled-out point counts
 // down its later points' undecided earlier points, and the one that reaches
 // zero (no earlier point within r was a sample) becomes a sample.  ctl[0] is
 // the round, ctl[1] and ctl[2] the sizes of the two frontier buffers (the
 // round's input in buffer round & 1), ctl[3] the round limit.  The last block
-// to finish starts the next round: it clears the consumed buffer's size and
-// sets the loop condition (a new frontier, and the limit not reached).
-__global__ void __launch_bounds__(256) k_mis_round(const int64_t* __restrict__ off, const int32_t* __restrict__ later,
-                                                   int* __restrict__ state, int* __restrict__ blockers,
-                                                   int32_t* __restrict__ fa, int32_t* __restrict__ fb, int* ctl,
-                                                   int* counter, cudaGraphConditionalHandle h, int use_h) {
+// to finish clears the consumed buffer's size and starts the next round.
+constexpr int kChainMax = 4096;
+__global__ void __launch_bounds__(256) k_mis_round(const int64_t* __restrict__ off, const int* __restrict__ nlater,
+                                                   const int32_t* __restrict__ later, int* __restrict__ state,
+                                                   int* __restrict__ blockers, int32_t* __restrict__ fa,
+                                                   int32_t* __restrict__ fb, int* ctl, int* counter) {
   const int round = ctl[0];
   const int32_t* fin = (round & 1) ? fb : fa;
   int32_t* fout = (round & 1) ? fa : fb;
   const int nin = ctl[1 + (round & 1)];
+  if (nin <= kChainMax) return;  // every block takes the same branch: nothing below changes ctl before all have read it
   int* nout = &ctl[1 + ((round + 1) & 1)];
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nin; q += gridDim.x * blockDim.x) {
     const int32_t t = fin[q];
     const bool sample = state[t] == SAMPLE;
-    for (int64_t k = off[t]; k < off[t + 1]; ++k) {
+    int cnt;
+    const int64_t b = later_of(t, off, nlater, &cnt);
+    for (int64_t k = b; k < b + cnt; ++k) {
       const int32_t u = later[k];
       if (sample) {
         if (atomicCAS(&state[u], UNDECIDED, RULED_OUT) == UNDECIDED) fout[atomicAdd(nout, 1)] = u;
@@ -265,8 +366,92 @@ __global__ void __launch_bounds__(256) k_mis_round(const int64_t* __restrict__ o
     __threadfence();
     ctl[1 + (round & 1)] = 0;
     ctl[0] = round + 1;
-    const bool go = *(volatile int*)nout > 0 && round + 1 < ctl[3];
-    if (use_h) cudaGraphSetConditional(h, go ? 1u : 0u);
+  }
+}
+
+// The short rounds, one after another in one block, until no point is left
+// or a frontier of more than kChainMax points asks for the whole GPU.  A
+// row-major mesh numbering makes thousands of short rounds (the decisions
+// travel along the rows: 4,400 on a 2048 x 512 torus), so a round must cost
+// little more than its dependent memory accesses: the frontier stays in
+// shared memory (a point with the sample flag in its top bit), eight lanes
+// take a point and load its later points together, and a round ends with one
+// block barrier.  Sets the loop condition.  One block of 1024 threads.
+constexpr unsigned kSampleBit = 0x80000000u;
+__global__ void __launch_bounds__(1024) k_mis_chain(const int64_t* __restrict__ off, const int* __restrict__ nlater,
+                                                    const int32_t* __restrict__ later, int* __restrict__ state,
+                                                    int* __restrict__ blockers, int32_t* __restrict__ fa,
+                                                    int32_t* __restrict__ fb, int* ctl,
+                                                    cudaGraphConditionalHandle h, int use_h) {
+  __shared__ unsigned q[2][kChainMax];
+  __shared__ int size[2];
+  const int tid = threadIdx.x;
+  int round = ctl[0];
+  const int limit = ctl[3];
+  int nin = ctl[1 + (round & 1)];
+  if (nin > kChainMax) {
+    if (tid == 0 && use_h) cudaGraphSetConditional(h, round < limit ? 1u : 0u);
+    return;
+  }
+  {
+    const int32_t* fin = (round & 1) ? fb : fa;
+    for (int k = tid; k < nin; k += 1024) {
+      const int32_t t = fin[k];
+      q[round & 1][k] = (unsigned)t | (state[t] == SAMPLE ? kSampleBit : 0u);
+    }
+    if (tid < 2) size[tid] = 0;
+  }
+  __syncthreads();
+  while (nin > 0 && nin <= kChainMax && round < limit) {
+    const int in = round & 1, out = in ^ 1;
+    int32_t* fout = in ? fa : fb;  // points past the shared-memory buffer
+    auto emit = [&](unsigned item) {
+      const int p = atomicAdd(&size[out], 1);
+      if (p < kChainMax) q[out][p] = item;
+      else fout[p] = (int32_t)(item & ~kSampleBit);
+    };
+    for (int k = tid >> 3; k < nin; k += 128) {
+      const unsigned item = q[in][k];
+      const int32_t t = (int32_t)(item & ~kSampleBit);
+      int cnt;
+      const int64_t b = later_of(t, off, nlater, &cnt);
+      for (int e0 = tid & 7; e0 < cnt; e0 += 32) {
+        int32_t u[4];
+        int old[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) u[m] = e0 + 8 * m < cnt ? __ldg(later + b + e0 + 8 * m) : -1;
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+          if (u[m] >= 0)
+            old[m] = (item & kSampleBit) ? atomicCAS(&state[u[m]], UNDECIDED, RULED_OUT) : atomicSub(&blockers[u[m]], 1);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          if (u[m] < 0) continue;
+          if (item & kSampleBit) {
+            if (old[m] == UNDECIDED) emit((unsigned)u[m]);
+          } else if (old[m] == 1) {
+            state[u[m]] = SAMPLE;
+            emit((unsigned)u[m] | kSampleBit);
+          }
+        }
+      }
+    }
+    __syncthreads();
+    nin = size[out];
+    __syncthreads();
+    if (tid == 0) size[in] = 0;  // the next round's output
+    ++round;
+    __syncthreads();
+  }
+  if (nin > kChainMax) {  // hand the frontier over (the part past the buffer is there already)
+    int32_t* f = (round & 1) ? fb : fa;
+    for (int k = tid; k < kChainMax; k += 1024) f[k] = (int32_t)(q[round & 1][k] & ~kSampleBit);
+  }
+  if (tid == 0) {
+    ctl[0] = round;
+    ctl[1 + (round & 1)] = nin;
+    ctl[1 + ((round + 1) & 1)] = 0;
+    if (use_h) cudaGraphSetConditional(h, nin > 0 && round < limit ? 1u : 0u);
   }
 }
 
@@ -290,7 +475,7 @@ __global__ void k_sample_list(int64_t n, const int* __restrict__ flag, const int
 }
 
 // ---- graph Voronoi cells: one Jacobi round of lexicographic (distance, sample)
-__global__ void k_voronoi(int64_t n, const double* __restrict__ X, const int64_t* __restrict__ rp,
+__global__ void k_voronoi(int64_t n, const double* __restrict__ len, const int64_t* __restrict__ rp,
                           const int32_t* __restrict__ ci, const double* __restrict__ d0, const int32_t* __restrict__ c0,
                           double* __restrict__ d1, int32_t* __restrict__ c1, int* __restrict__ changed) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
@@ -299,7 +484,7 @@ __global__ void k_voronoi(int64_t n, const double* __restrict__ X, const int64_t
     for (int64_t k = rp[v]; k < rp[v + 1]; ++k) {
       const int32_t u = ci[k];
       if (c0[u] == INT32_MAX) continue;
-      const double nd = ad(d0[u], edge_len(X, u, v));
+      const double nd = ad(d0[u], len[k]);
       if (nd < bd || (nd == bd && c0[u] < bc)) {
         bd = nd;
         bc = c0[u];
@@ -592,16 +777,24 @@ __global__ void k_prolong_rows(int64_t n, const double* __restrict__ X, const in
   }
 }
 
+// Rows with a weight on every coarse column.
+__global__ void k_col_count(int64_t m, const int32_t* __restrict__ idx, const double* __restrict__ w,
+                            int* __restrict__ colcount) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m; k += (int64_t)gridDim.x * blockDim.x)
+    if (w[k] != 0) atomicAdd(&colcount[idx[k]], 1);
+}
+// stats[3] = empty columns.
+__global__ void k_col_empty(int64_t nc, const int* __restrict__ colcount, int64_t* __restrict__ stats) {
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += (int64_t)gridDim.x * blockDim.x)
+    if (colcount[c] == 0) atomicAdd(reinterpret_cast<unsigned long long*>(stats + 3), 1ull);
+}
 // Empty coarse columns (possible after the shift): the sample's own row
 // becomes the identity on its column, repeated until every column is used
-// (one thread; it happens rarely).  stats[1] = repaired columns, stats[2] =
-// single-entry rows.
-__global__ void k_repair(int64_t n, int64_t nc, const int32_t* __restrict__ samples, int32_t* __restrict__ idx,
+// (one thread in column order; it happens rarely, and returns at once when
+// stats[3] counts no empty column).  stats[1] = repaired columns.
+__global__ void k_repair(int64_t nc, const int32_t* __restrict__ samples, int32_t* __restrict__ idx,
                          double* __restrict__ w, int* __restrict__ colcount, int64_t* __restrict__ stats) {
-  for (int64_t i = 0; i < n; ++i)
-    for (int s = 0; s < 3; ++s)
-      if (w[3 * i + s] != 0) colcount[idx[3 * i + s]]++;
-  bool changed = true;
+  bool changed = stats[3] > 0;
   int64_t repaired = 0;
   while (changed) {
     changed = false;
@@ -618,14 +811,16 @@ __global__ void k_repair(int64_t n, int64_t nc, const int32_t* __restrict__ samp
       changed = true;
     }
   }
-  int64_t single = 0;
-  for (int64_t i = 0; i < n; ++i) {
-    int cnt = 0;
-    for (int s = 0; s < 3; ++s) cnt += w[3 * i + s] != 0;
-    single += cnt == 1;
-  }
   stats[1] = repaired;
-  stats[2] = single;
+}
+// stats[2] = rows with a single weight.
+__global__ void __launch_bounds__(256) k_single_rows(int64_t n, const double* __restrict__ w,
+                                                     int64_t* __restrict__ stats) {
+  int c = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    c += (w[3 * i] != 0) + (w[3 * i + 1] != 0) + (w[3 * i + 2] != 0) == 1;
+  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(reinterpret_cast<unsigned long long*>(stats + 2), (unsigned long long)c);
 }
 
 static inline unsigned grid_of(int64_t n, int per = 256) {
@@ -671,11 +866,24 @@ struct Buffers {
   }
 };
 
-// The sampling propagation rounds until no point is decided any more: in a
-// graph holding a conditional WHILE node when the driver accepts it, else
-// launched from the host in batches.
-static gmg_status run_mis(int64_t n, const int64_t* off, const int32_t* later, int* state, int* blockers,
-                          int32_t* fa, int32_t* fb, int* ctl, int* counter, cudaStream_t s) {
+// off[0 .. n] = exclusive scan of cnt (sums: scratch of one value per tile).
+static gmg_status scan(int64_t n, const int* cnt, int64_t* off, int64_t* sums, cudaStream_t s) {
+  const int64_t nt = std::max<int64_t>(1, (n + kTile - 1) / kTile);
+  k_scan_sums<<<(unsigned)nt, 256, 0, s>>>(n, cnt, sums);
+  GMG_LAUNCHED();
+  k_scan_tiles<<<1, 1024, 0, s>>>(nt, sums, off + n);
+  GMG_LAUNCHED();
+  k_scan_apply<<<(unsigned)nt, 1024, 0, s>>>(n, cnt, sums, off);
+  GMG_LAUNCHED();
+  return GMG_OK;
+}
+
+// The sampling propagation rounds until no point is decided any more (long
+// rounds on all SMs, then the short ones in one block): in a graph holding a
+// conditional WHILE node when the driver accepts it, else launched from the
+// host in batches.
+static gmg_status run_mis(int64_t n, const int64_t* off, const int* nlater, const int32_t* later, int* state,
+                          int* blockers, int32_t* fa, int32_t* fb, int* ctl, int* counter, cudaStream_t s) {
   const unsigned grid = 152 * 2;
   cudaGraph_t g = nullptr;
   cudaGraphExec_t ge = nullptr;
@@ -692,22 +900,29 @@ static gmg_status run_mis(int64_t n, const int64_t* off, const int32_t* later, i
     ok = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &np) == cudaSuccess;
   }
   if (ok) {
-    cudaKernelNodeParams kp = {};
+    cudaKernelNodeParams kp = {}, kc = {};
     int use_h = 1;
-    void* args[] = {(void*)&off, (void*)&later, (void*)&state, (void*)&blockers, (void*)&fa, (void*)&fb,
-                    (void*)&ctl, (void*)&counter, (void*)&h, (void*)&use_h};
+    void* args[] = {(void*)&off, (void*)&nlater, (void*)&later, (void*)&state, (void*)&blockers,
+                    (void*)&fa,  (void*)&fb,     (void*)&ctl,   (void*)&counter};
     kp.func = (void*)k_mis_round;
     kp.gridDim = dim3(grid);
     kp.blockDim = dim3(256);
     kp.kernelParams = args;
-    cudaGraphNode_t kn;
-    ok = cudaGraphAddKernelNode(&kn, np.conditional.phGraph_out[0], nullptr, 0, &kp) == cudaSuccess;
+    void* cargs[] = {(void*)&off, (void*)&nlater, (void*)&later, (void*)&state, (void*)&blockers,
+                     (void*)&fa,  (void*)&fb,     (void*)&ctl,   (void*)&h,     (void*)&use_h};
+    kc.func = (void*)k_mis_chain;
+    kc.gridDim = dim3(1);
+    kc.blockDim = dim3(1024);
+    kc.kernelParams = cargs;
+    cudaGraphNode_t kn, cn;
+    ok = cudaGraphAddKernelNode(&kn, np.conditional.phGraph_out[0], nullptr, 0, &kp) == cudaSuccess &&
+         cudaGraphAddKernelNode(&cn, np.conditional.phGraph_out[0], &kn, 1, &kc) == cudaSuccess;
   }
   if (ok) ok = cudaGraphInstantiate(&ge, g, 0) == cudaSuccess;
   if (g) cudaGraphDestroy(g);
   if (ok) {
     GMG_CK(cudaGraphLaunch(ge, s));
-    g_launches += 1;
+    g_launches += 2;
     cudaGraphExecDestroy(ge);
     return GMG_OK;
   }
@@ -716,7 +931,9 @@ static gmg_status run_mis(int64_t n, const int64_t* off, const int32_t* later, i
   // host-driven rounds, 64 at a time between checks
   for (;;) {
     for (int k = 0; k < 64; ++k) {
-      k_mis_round<<<grid, 256, 0, s>>>(off, later, state, blockers, fa, fb, ctl, counter, 0, 0);
+      k_mis_round<<<grid, 256, 0, s>>>(off, nlater, later, state, blockers, fa, fb, ctl, counter);
+      GMG_LAUNCHED();
+      k_mis_chain<<<1, 1024, 0, s>>>(off, nlater, later, state, blockers, fa, fb, ctl, 0, 0);
       GMG_LAUNCHED();
     }
     int hc[3];
@@ -729,7 +946,7 @@ static gmg_status run_mis(int64_t n, const int64_t* off, const int32_t* later, i
 // One level: points X (device, 3n), neighbour graph (device CSR, symmetric,
 // sorted, no self loops) -> the host record and the coarse level's device
 // points and graph (allocated with cudaMalloc, owned by the caller).
-static gmg_status build_one(int64_t n, const double* X, const int64_t* rp, const int32_t* ci, double phi, int shift,
+static gmg_status build_one(int64_t n, int64_t nnz, const double* X, const int64_t* rp, const int32_t* ci, double phi, int shift,
                             gmg_hier_level& out, double** Xc_out, int64_t** crp_out, int32_t** ccol_out,
                             cudaStream_t s) {
   Buffers B;
@@ -747,41 +964,59 @@ static gmg_status build_one(int64_t n, const double* X, const int64_t* rp, const
   GMG_TRY(B.get(&bsum, nb));
   GMG_TRY(B.get(&bcnt, nb));
   GMG_TRY(B.get(&geo, 3));
-  k_row_lengths<<<G, 256, 0, s>>>(n, X, rp, ci, rsum, rcnt);
+  double* len;
+  int64_t* sums;
+  GMG_TRY(B.get(&len, (size_t)nnz));
+  GMG_TRY(B.get(&sums, (n + kTile - 1) / kTile + 1));
+  k_edge_lengths<<<G, 256, 0, s>>>(n, X, rp, ci, len, rsum, rcnt);
   GMG_LAUNCHED();
-  k_block_lengths<<<grid_of(nb, 64), 64, 0, s>>>(n, rsum, rcnt, bsum, bcnt);
+  k_block_lengths<<<(unsigned)nb, 256, 0, s>>>(n, rsum, rcnt, bsum, bcnt);
   GMG_LAUNCHED();
-  k_mean_length<<<1, 1, 0, s>>>(nb, bsum, bcnt, std::pow(phi, -1.0 / 3.0), geo);
+  k_mean_length<<<1, 1024, 0, s>>>(nb, bsum, bcnt, std::pow(phi, -1.0 / 3.0), geo);
   GMG_LAUNCHED();
-  // sampling: the later points within r of every point, then the propagation
-  int *nlater, *blockers, *state, *ctl, *counter;
-  int64_t* off;
+  // sampling: the later points within r of every point, then the propagation.
+  // One search per point writes its list into a row of kRow; a point with
+  // more of them, or a graph whose rows would take more than 4 GB, makes a
+  // second search into CSR rows
+  int *nlater, *blockers, *state, *ctl, *counter, *err2;
+  int64_t* off = nullptr;
   GMG_TRY(B.get(&nlater, n));
   GMG_TRY(B.get(&blockers, n));
   GMG_TRY(B.get(&state, n));
-  GMG_TRY(B.get(&off, n + 1));
+  GMG_TRY(B.get(&err2, 1));
   GMG_CK(cudaMemsetAsync(blockers, 0, sizeof(int) * (size_t)n, s));
-  k_balls<<<G, 128, 0, s>>>(n, X, rp, ci, geo, nlater, blockers, nullptr, nullptr, err);
+  GMG_CK(cudaMemsetAsync(err2, 0, sizeof(int), s));
+  const bool rows = n <= ((int64_t)1 << 32) / (int64_t)(kRow * sizeof(int32_t));
+  int32_t* later = nullptr;
+  if (rows) GMG_TRY(B.get(&later, (size_t)n * kRow));
+  k_balls<<<G, 128, 0, s>>>(n, len, rp, ci, geo, nlater, blockers, nullptr, later, err, err2);
   GMG_LAUNCHED();
-  k_scan<<<1, 1024, 0, s>>>(n, nlater, off);
-  GMG_LAUNCHED();
-  int64_t nlat = 0;
-  GMG_CK(cudaMemcpyAsync(&nlat, off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  GMG_CK(cudaStreamSynchronize(s));
-  int32_t *later, *fa, *fb;
-  GMG_TRY(B.get(&later, (size_t)nlat));
+  int more = 1;
+  if (rows) {
+    GMG_CK(cudaMemcpyAsync(&more, err2, sizeof(int), cudaMemcpyDeviceToHost, s));
+    GMG_CK(cudaStreamSynchronize(s));
+  }
+  if (more) {
+    GMG_TRY(B.get(&off, n + 1));
+    GMG_TRY(scan(n, nlater, off, sums, s));
+    int64_t nlat = 0;
+    GMG_CK(cudaMemcpyAsync(&nlat, off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    GMG_CK(cudaStreamSynchronize(s));
+    GMG_TRY(B.get(&later, (size_t)nlat));
+    k_balls<<<G, 128, 0, s>>>(n, len, rp, ci, geo, nlater, blockers, off, later, err, err2);
+    GMG_LAUNCHED();
+  }
+  int32_t *fa, *fb;
   GMG_TRY(B.get(&fa, n));
   GMG_TRY(B.get(&fb, n));
   GMG_TRY(B.get(&ctl, 4));
   GMG_TRY(B.get(&counter, 1));
-  k_balls<<<G, 128, 0, s>>>(n, X, rp, ci, geo, nlater, blockers, off, later, err);
-  GMG_LAUNCHED();
   const int ctl0[4] = {0, 0, 0, (int)std::min<int64_t>(n + 2, INT32_MAX)};
   GMG_CK(cudaMemcpyAsync(ctl, ctl0, sizeof(ctl0), cudaMemcpyHostToDevice, s));
   GMG_CK(cudaMemsetAsync(counter, 0, sizeof(int), s));
   k_mis_start<<<G, 256, 0, s>>>(n, blockers, state, fa, ctl + 1);
   GMG_LAUNCHED();
-  GMG_TRY(run_mis(n, off, later, state, blockers, fa, fb, ctl, counter, s));
+  GMG_TRY(run_mis(n, off, nlater, later, state, blockers, fa, fb, ctl, counter, s));
   // samples in index order
   int* flag;
   int64_t* rank;
@@ -789,8 +1024,7 @@ static gmg_status build_one(int64_t n, const double* X, const int64_t* rp, const
   GMG_TRY(B.get(&rank, n + 1));
   k_sample_flags<<<G, 256, 0, s>>>(n, state, flag);
   GMG_LAUNCHED();
-  k_scan<<<1, 1024, 0, s>>>(n, flag, rank);
-  GMG_LAUNCHED();
+  GMG_TRY(scan(n, flag, rank, sums, s));
   int64_t nc = 0;
   int herr = 0;
   GMG_CK(cudaMemcpyAsync(&nc, rank + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
@@ -817,7 +1051,7 @@ static gmg_status build_one(int64_t n, const double* X, const int64_t* rp, const
   // graph Voronoi cells
   for (int64_t round = 0;; ++round) {
     GMG_CK(cudaMemsetAsync(changed, 0, sizeof(int), s));
-    k_voronoi<<<G, 256, 0, s>>>(n, X, rp, ci, d0, cell0, d1, cell1, changed);
+    k_voronoi<<<G, 256, 0, s>>>(n, len, rp, ci, d0, cell0, d1, cell1, changed);
     GMG_LAUNCHED();
     std::swap(d0, d1);
     std::swap(cell0, cell1);
@@ -849,8 +1083,7 @@ static gmg_status build_one(int64_t n, const double* X, const int64_t* rp, const
     set_error("gmg_build_hierarchy: a point is in no Voronoi cell");
     return GMG_ERR_CUDA;
   }
-  k_scan<<<1, 1024, 0, s>>>(nc, ccnt, coff);
-  GMG_LAUNCHED();
+  GMG_TRY(scan(nc, ccnt, coff, sums, s));
   k_cell_fill<<<G, 256, 0, s>>>(n, cell, coff, ccur, members);
   GMG_LAUNCHED();
   double* Xc;
@@ -867,8 +1100,7 @@ static gmg_status build_one(int64_t n, const double* X, const int64_t* rp, const
   *crp_out = crp;
   k_coarse_graph<<<GC, 64, 0, s>>>(nc, coff, members, rp, ci, cell, gcnt, nullptr, nullptr, err);
   GMG_LAUNCHED();
-  k_scan<<<1, 1024, 0, s>>>(nc, gcnt, crp);
-  GMG_LAUNCHED();
+  GMG_TRY(scan(nc, gcnt, crp, sums, s));
   int64_t cnnz = 0;
   GMG_CK(cudaMemcpyAsync(&cnnz, crp + nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   GMG_CK(cudaStreamSynchronize(s));
@@ -884,8 +1116,7 @@ static gmg_status build_one(int64_t n, const double* X, const int64_t* rp, const
   GMG_TRY(B.get(&toff, nc + 1));
   k_triangles<<<GC, 128, 0, s>>>(nc, crp, ccol, Xc, geo, tcnt, nullptr, nullptr);
   GMG_LAUNCHED();
-  k_scan<<<1, 1024, 0, s>>>(nc, tcnt, toff);
-  GMG_LAUNCHED();
+  GMG_TRY(scan(nc, tcnt, toff, sums, s));
   int64_t ntri = 0;
   GMG_CK(cudaMemcpyAsync(&ntri, toff + nc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   GMG_CK(cudaStreamSynchronize(s));
@@ -907,7 +1138,14 @@ static gmg_status build_one(int64_t n, const double* X, const int64_t* rp, const
   GMG_CK(cudaMemsetAsync(colcount, 0, sizeof(int) * (size_t)nc, s));
   k_prolong_rows<<<G, 128, 0, s>>>(n, X, cell, Xc, crp, ccol, toff, tri, idx, w, fallbacks, err);
   GMG_LAUNCHED();
-  k_repair<<<1, 1, 0, s>>>(n, nc, samples, idx, w, colcount, stats);
+  GMG_CK(cudaMemsetAsync(stats, 0, 4 * sizeof(int64_t), s));
+  k_col_count<<<grid_of(3 * n), 256, 0, s>>>(3 * n, idx, w, colcount);
+  GMG_LAUNCHED();
+  k_col_empty<<<GC, 128, 0, s>>>(nc, colcount, stats);
+  GMG_LAUNCHED();
+  k_repair<<<1, 1, 0, s>>>(nc, samples, idx, w, colcount, stats);
+  GMG_LAUNCHED();
+  k_single_rows<<<grid_of(n), 256, 0, s>>>(n, w, stats);
   GMG_LAUNCHED();
   // to the host
   out.idx.resize(3 * (size_t)n);
@@ -1007,13 +1245,13 @@ extern "C" gmg_status gmg_build_hierarchy(gmg_hierarchy* out, int64_t n, const d
   if (st == GMG_OK) ck(cudaMemcpyAsync(drp, rowptr, sizeof(int64_t) * (size_t)(n + 1), cudaMemcpyHostToDevice, s));
   if (st == GMG_OK && nnz)
     ck(cudaMemcpyAsync(dci, col, sizeof(int32_t) * (size_t)nnz, cudaMemcpyHostToDevice, s));
-  int64_t cur = n;
+  int64_t cur = n, cur_nnz = nnz;
   while (st == GMG_OK && cur > stop && (int)h->levels.size() < max_levels) {
     gmg_hier_level lv;
     double* Xc = nullptr;
     int64_t* crp = nullptr;
     int32_t* ccol = nullptr;
-    st = build::build_one(cur, dX, drp, dci, phi, 1, lv, &Xc, &crp, &ccol, s);
+    st = build::build_one(cur, cur_nnz, dX, drp, dci, phi, 1, lv, &Xc, &crp, &ccol, s);
     const bool stop_here = st != GMG_OK || lv.n_coarse == 0 || lv.n_coarse >= cur;
     release();
     dX = Xc;
@@ -1021,6 +1259,7 @@ extern "C" gmg_status gmg_build_hierarchy(gmg_hierarchy* out, int64_t n, const d
     dci = ccol;
     if (stop_here) break;
     cur = lv.n_coarse;
+    cur_nnz = (int64_t)lv.ccol.size();
     h->levels.push_back(std::move(lv));
   }
   release();
