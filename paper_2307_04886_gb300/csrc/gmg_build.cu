@@ -373,18 +373,20 @@ __global__ void __launch_bounds__(256) k_mis_round(const int64_t* __restrict__ o
 // or a frontier of more than kChainMax points asks for the whole GPU.  A
 // row-major mesh numbering makes thousands of short rounds (the decisions
 // travel along the rows: 4,400 on a 2048 x 512 torus), so a round must cost
-// little more than its dependent memory accesses: the frontier stays in
+// little more than one atomic's round trip to L2: the frontier stays in
 // shared memory (a point with the sample flag in its top bit), eight lanes
-// take a point and load its later points together, and a round ends with one
-// block barrier.  Sets the loop condition.  One block of 1024 threads.
+// take a point and load its later points together, the lists of those points
+// are prefetched into L1 while their atomics are in flight, the lists end in
+// -1 instead of a separate count, and a round ends with one block barrier.
+// Sets the loop condition.  One block of 1024 threads.
 constexpr unsigned kSampleBit = 0x80000000u;
-__global__ void __launch_bounds__(1024) k_mis_chain(const int64_t* __restrict__ off, const int* __restrict__ nlater,
+__global__ void __launch_bounds__(1024) k_mis_chain(const int64_t* __restrict__ off,
                                                     const int32_t* __restrict__ later, int* __restrict__ state,
                                                     int* __restrict__ blockers, int32_t* __restrict__ fa,
                                                     int32_t* __restrict__ fb, int* ctl,
                                                     cudaGraphConditionalHandle h, int use_h) {
   __shared__ unsigned q[2][kChainMax];
-  __shared__ int size[2];
+  __shared__ int size[3];  // frontier sizes of the rounds round, round + 1, round + 2 (mod 3)
   const int tid = threadIdx.x;
   int round = ctl[0];
   const int limit = ctl[3];
@@ -399,22 +401,25 @@ __global__ void __launch_bounds__(1024) k_mis_chain(const int64_t* __restrict__ 
       const int32_t t = fin[k];
       q[round & 1][k] = (unsigned)t | (state[t] == SAMPLE ? kSampleBit : 0u);
     }
-    if (tid < 2) size[tid] = 0;
+    if (tid < 3) size[tid] = 0;
   }
   __syncthreads();
+  int slot = 0;  // size[slot]: this round's input (known in nin), size[slot + 1]: its output
   while (nin > 0 && nin <= kChainMax && round < limit) {
     const int in = round & 1, out = in ^ 1;
+    const int so = slot == 2 ? 0 : slot + 1, sn = so == 2 ? 0 : so + 1;
+    if (tid == 0) size[sn] = 0;     // the next round's output, read and written by nobody in this round
     int32_t* fout = in ? fa : fb;  // points past the shared-memory buffer
     auto emit = [&](unsigned item) {
-      const int p = atomicAdd(&size[out], 1);
+      const int p = atomicAdd(&size[so], 1);
       if (p < kChainMax) q[out][p] = item;
       else fout[p] = (int32_t)(item & ~kSampleBit);
     };
     for (int k = tid >> 3; k < nin; k += 128) {
       const unsigned item = q[in][k];
       const int32_t t = (int32_t)(item & ~kSampleBit);
-      int cnt;
-      const int64_t b = later_of(t, off, nlater, &cnt);
+      const int64_t b = off ? off[t] : (int64_t)t * kRow;
+      const int cnt = off ? (int)(off[t + 1] - b) : kRow;
       for (int e0 = tid & 7; e0 < cnt; e0 += 32) {
         int32_t u[4];
         int old[4];
@@ -422,8 +427,11 @@ __global__ void __launch_bounds__(1024) k_mis_chain(const int64_t* __restrict__ 
         for (int m = 0; m < 4; ++m) u[m] = e0 + 8 * m < cnt ? __ldg(later + b + e0 + 8 * m) : -1;
 #pragma unroll
         for (int m = 0; m < 4; ++m)
-          if (u[m] >= 0)
+          if (u[m] >= 0) {
             old[m] = (item & kSampleBit) ? atomicCAS(&state[u[m]], UNDECIDED, RULED_OUT) : atomicSub(&blockers[u[m]], 1);
+            const int32_t* row = off ? later + off[u[m]] : later + (int64_t)u[m] * kRow;
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(row));
+          }
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
           if (u[m] < 0) continue;
@@ -437,11 +445,9 @@ __global__ void __launch_bounds__(1024) k_mis_chain(const int64_t* __restrict__ 
       }
     }
     __syncthreads();
-    nin = size[out];
-    __syncthreads();
-    if (tid == 0) size[in] = 0;  // the next round's output
+    nin = size[so];
+    slot = so;
     ++round;
-    __syncthreads();
   }
   if (nin > kChainMax) {  // hand the frontier over (the part past the buffer is there already)
     int32_t* f = (round & 1) ? fb : fa;
@@ -908,8 +914,8 @@ static gmg_status run_mis(int64_t n, const int64_t* off, const int* nlater, cons
     kp.gridDim = dim3(grid);
     kp.blockDim = dim3(256);
     kp.kernelParams = args;
-    void* cargs[] = {(void*)&off, (void*)&nlater, (void*)&later, (void*)&state, (void*)&blockers,
-                     (void*)&fa,  (void*)&fb,     (void*)&ctl,   (void*)&h,     (void*)&use_h};
+    void* cargs[] = {(void*)&off, (void*)&later, (void*)&state, (void*)&blockers, (void*)&fa,
+                     (void*)&fb,  (void*)&ctl,   (void*)&h,     (void*)&use_h};
     kc.func = (void*)k_mis_chain;
     kc.gridDim = dim3(1);
     kc.blockDim = dim3(1024);
@@ -933,7 +939,7 @@ static gmg_status run_mis(int64_t n, const int64_t* off, const int* nlater, cons
     for (int k = 0; k < 64; ++k) {
       k_mis_round<<<grid, 256, 0, s>>>(off, nlater, later, state, blockers, fa, fb, ctl, counter);
       GMG_LAUNCHED();
-      k_mis_chain<<<1, 1024, 0, s>>>(off, nlater, later, state, blockers, fa, fb, ctl, 0, 0);
+      k_mis_chain<<<1, 1024, 0, s>>>(off, later, state, blockers, fa, fb, ctl, 0, 0);
       GMG_LAUNCHED();
     }
     int hc[3];
@@ -988,7 +994,10 @@ static gmg_status build_one(int64_t n, int64_t nnz, const double* X, const int64
   GMG_CK(cudaMemsetAsync(err2, 0, sizeof(int), s));
   const bool rows = n <= ((int64_t)1 << 32) / (int64_t)(kRow * sizeof(int32_t));
   int32_t* later = nullptr;
-  if (rows) GMG_TRY(B.get(&later, (size_t)n * kRow));
+  if (rows) {  // a row ends in -1
+    GMG_TRY(B.get(&later, (size_t)n * kRow));
+    GMG_CK(cudaMemsetAsync(later, 0xFF, sizeof(int32_t) * (size_t)n * kRow, s));
+  }
   k_balls<<<G, 128, 0, s>>>(n, len, rp, ci, geo, nlater, blockers, nullptr, later, err, err2);
   GMG_LAUNCHED();
   int more = 1;
