@@ -270,6 +270,8 @@ gmg_status gmg_destroy(gmg_handle h) {
   if (!h) return GMG_OK;
   cudaSetDevice(h->device);
   drop_graphs(h);
+  for (auto& g : h->mloops)
+    if (g) cudaGraphExecDestroy(g);
   if (h->g_stream) cudaStreamDestroy(h->g_stream);
   for (auto& e : h->ev)
     if (e) cudaEventDestroy(e);

@@ -16,89 +16,115 @@
 
 namespace gmg {
 
+// Columns of a block are split over Q lanes of V columns each (NR = 1, 2: one
+// lane; 4, 8, 16: one, two, four lanes of a float4), so that the lanes of a
+// row read and write its NR values as one contiguous piece and 32 / Q rows
+// share a warp.
 template <int NR>
-struct alignas(16) Row {
-  float v[NR];
+struct MCols {
+  static constexpr int V = NR < 4 ? NR : 4;
+  static constexpr int Q = NR / V;
 };
+constexpr int kMPre = 8;            // entries of a row part whose gathers are in flight together
+constexpr int kMRestrictParts = 4;  // warps per coarse row in the restriction (18-40 terms per row)
 
-template <int NR>
-__device__ __forceinline__ void load_row(const float* __restrict__ p, float (&o)[NR]) {
-  if constexpr (NR % 4 == 0) {
-#pragma unroll
-    for (int c = 0; c < NR; c += 4) {
-      const float4 q = __ldg(reinterpret_cast<const float4*>(p + c));
-      o[c] = q.x;
-      o[c + 1] = q.y;
-      o[c + 2] = q.z;
-      o[c + 3] = q.w;
-    }
+template <int V>
+__device__ __forceinline__ void load_cols(const float* p, float (&o)[V]) {
+  if constexpr (V == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    o[0] = q.x;
+    o[1] = q.y;
+    o[2] = q.z;
+    o[3] = q.w;
+  } else if constexpr (V == 2) {
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    o[0] = q.x;
+    o[1] = q.y;
   } else {
-#pragma unroll
-    for (int c = 0; c < NR; ++c) o[c] = __ldg(p + c);
+    o[0] = *p;
   }
 }
-
-template <int NR>
-__device__ __forceinline__ void store_row(float* __restrict__ p, const float (&o)[NR]) {
-  if constexpr (NR % 4 == 0) {
-#pragma unroll
-    for (int c = 0; c < NR; c += 4) *reinterpret_cast<float4*>(p + c) = make_float4(o[c], o[c + 1], o[c + 2], o[c + 3]);
-  } else {
-#pragma unroll
-    for (int c = 0; c < NR; ++c) p[c] = o[c];
-  }
+template <int V>
+__device__ __forceinline__ void store_cols(float* p, const float (&o)[V]) {
+  if constexpr (V == 4) *reinterpret_cast<float4*>(p) = make_float4(o[0], o[1], o[2], o[3]);
+  else if constexpr (V == 2) *reinterpret_cast<float2*>(p) = make_float2(o[0], o[1]);
+  else *p = o[0];
 }
 
-// One warp's share of a slice row for a launch that splits every row over G
-// warps (warp `part` takes entries k = part, part + G, ...); 8 / G slices per
-// block of 256 threads.
+// One lane's share of a row: row group `group` (32 / Q rows of one slice),
+// warp `part` of the G that split its entries.  The first kMPre values and
+// columns are loaded here, before the dependency wait.
+template <int NR, int G>
 struct MRow {
   bool active;
-  int nk;
+  int nk, c;    // entries of this part, first column of this lane
   int64_t e, r;
-};
-template <int G>
-__device__ __forceinline__ MRow m_row(int64_t s, int64_t s_end, const int64_t* __restrict__ ptr,
-                                      const int32_t* __restrict__ row0, const int32_t* __restrict__ nrow, int part,
-                                      int lane) {
-  MRow m{false, 0, 0, 0};
-  if (s < s_end) {
-    m.active = lane < nrow[s];
-    const int64_t e0 = ptr[s];
-    const int w = (int)((ptr[s + 1] - e0) >> 5);
-    m.nk = (m.active && part < w) ? (w - part + G - 1) / G : 0;
-    m.e = e0 + (int64_t)part * 32 + lane;
-    m.r = row0[s] + lane;
-  }
-  return m;
-}
-
-// acc[c] += sum over this warp's entries of a_rk X[k][c], entries in order.
-template <int NR, int G>
-__device__ __forceinline__ void m_dot(const MRow& m, const int32_t* __restrict__ col, const float* __restrict__ val,
-                                      const float* X, float (&acc)[NR]) {
-  int64_t e = m.e;
-  for (int q = 0; q < m.nk; ++q, e += (int64_t)G * 32) {
-    const float a = val[e];
-    float xv[NR];
-    load_row<NR>(X + (int64_t)col[e] * NR, xv);
+  float v[kMPre];
+  int32_t j[kMPre];
+  __device__ __forceinline__ MRow(int64_t s0, int64_t s1, int64_t group, const int64_t* __restrict__ ptr,
+                                  const int32_t* __restrict__ row0, const int32_t* __restrict__ nrow,
+                                  const int32_t* __restrict__ col, const float* __restrict__ val, int part, int lane) {
+    constexpr int Q = MCols<NR>::Q;
+    const int64_t s = s0 + group / Q;
+    const int ri = (int)(group % Q) * (32 / Q) + lane / Q;
+    active = false;
+    nk = 0;
+    c = (lane % Q) * MCols<NR>::V;
+    e = r = 0;
+    if (s < s1) {
+      active = ri < nrow[s];
+      const int64_t e0 = ptr[s];
+      const int w = (int)((ptr[s + 1] - e0) >> 5);
+      nk = active && part < w ? (w - part + G - 1) / G : 0;
+      e = e0 + (int64_t)part * 32 + ri;
+      r = row0[s] + ri;
+    }
 #pragma unroll
-    for (int c = 0; c < NR; ++c) acc[c] += a * xv[c];
+    for (int q = 0; q < kMPre; ++q) {
+      v[q] = q < nk ? val[e + (int64_t)q * G * 32] : 0.f;
+      j[q] = q < nk ? col[e + (int64_t)q * G * 32] : 0;
+    }
   }
-}
+  // acc[c] += sum over this part's entries of a_rk X[k][c], entries in order;
+  // the gathers of kMPre entries are issued together (one after another, as
+  // a loop over the entries, a coarse colour took 10.5 us)
+  __device__ __forceinline__ void dot(const int32_t* __restrict__ col, const float* __restrict__ val, const float* X,
+                                      float (&acc)[MCols<NR>::V]) {
+    constexpr int V = MCols<NR>::V;
+    for (int q0 = 0; q0 < nk; q0 += kMPre) {
+      float xv[kMPre][V];
+#pragma unroll
+      for (int q = 0; q < kMPre; ++q)
+        if (q0 + q < nk) load_cols<V>(X + (int64_t)j[q] * NR + c, xv[q]);
+#pragma unroll
+      for (int q = 0; q < kMPre; ++q)
+        if (q0 + q < nk)
+#pragma unroll
+          for (int k = 0; k < V; ++k) acc[k] += v[q] * xv[q][k];
+      if (q0 + kMPre < nk)
+#pragma unroll
+        for (int q = 0; q < kMPre; ++q) {
+          const bool in = q0 + kMPre + q < nk;
+          v[q] = in ? val[e + (int64_t)(q0 + kMPre + q) * G * 32] : 0.f;
+          j[q] = in ? col[e + (int64_t)(q0 + kMPre + q) * G * 32] : 0;
+        }
+    }
+  }
+};
 
 // Adds the other G - 1 warps' partial sums to row part 0's, in warp order.
-template <int NR, int G>
-__device__ __forceinline__ void m_combine(float (&acc)[NR], int warp, int lane) {
+template <int V, int G>
+__device__ __forceinline__ void m_combine(float (&acc)[V], int warp, int lane) {
   if constexpr (G > 1) {
-    __shared__ float red[8][NR][32];
+    __shared__ float red[8][V][32];
 #pragma unroll
-    for (int c = 0; c < NR; ++c) red[warp][c][lane] = acc[c];
+    for (int c = 0; c < V; ++c) red[warp][c][lane] = acc[c];
     __syncthreads();
     if (warp % G == 0)
+#pragma unroll
       for (int g = 1; g < G; ++g)
 #pragma unroll
-        for (int c = 0; c < NR; ++c) acc[c] += red[warp + g][c][lane];
+        for (int c = 0; c < V; ++c) acc[c] += red[warp + g][c][lane];
   }
 }
 
@@ -107,24 +133,24 @@ template <int NR, int G>
 __global__ void __launch_bounds__(256) k_gs_m(int64_t s0, int64_t s1, const int64_t* __restrict__ ptr,
                                               const int32_t* __restrict__ row0, const int32_t* __restrict__ nrow,
                                               const int32_t* __restrict__ col, const float* __restrict__ val,
-                                              const float* __restrict__ dinv, const float* __restrict__ B, float* X) {
+                                              const float* __restrict__ dinv, const float* B, float* X) {
+  constexpr int V = MCols<NR>::V;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, part = warp % G;
-  const int64_t s = s0 + (int64_t)blockIdx.x * (8 / G) + warp / G;
-  const MRow m = m_row<G>(s, s1, ptr, row0, nrow, part, lane);
-  float acc[NR], bv[NR];
+  MRow<NR, G> m(s0, s1, (int64_t)blockIdx.x * (8 / G) + warp / G, ptr, row0, nrow, col, val, part, lane);
+  const bool own = part == 0 && m.active;
+  const float d = own ? dinv[m.r] : 0.f;
+  pdl_wait();
+  pdl_trigger();
+  float acc[V], bv[V];
 #pragma unroll
-  for (int c = 0; c < NR; ++c) acc[c] = bv[c] = 0.f;
-  float d = 0.f;
-  if (part == 0 && m.active) {  // issued with the gathers, not after the combining barrier
-    load_row<NR>(B + m.r * NR, bv);
-    d = dinv[m.r];
-  }
-  m_dot<NR, G>(m, col, val, X, acc);  // other colours: not written by this launch
-  m_combine<NR, G>(acc, warp, lane);
-  if (part == 0 && m.active) {
+  for (int c = 0; c < V; ++c) acc[c] = bv[c] = 0.f;
+  if (own) load_cols<V>(B + m.r * NR + m.c, bv);  // issued with the gathers, not after the combining barrier
+  m.dot(col, val, X, acc);                        // other colours: not written by this launch
+  m_combine<V, G>(acc, warp, lane);
+  if (own) {
 #pragma unroll
-    for (int c = 0; c < NR; ++c) acc[c] = (bv[c] - acc[c]) * d;
-    store_row<NR>(X + m.r * NR, acc);
+    for (int c = 0; c < V; ++c) acc[c] = (bv[c] - acc[c]) * d;
+    store_cols<V>(X + m.r * NR + m.c, acc);
   }
 }
 
@@ -133,161 +159,225 @@ template <int NR, int G>
 __global__ void __launch_bounds__(256) k_residual_m(int64_t nslice, const int64_t* __restrict__ ptr,
                                                     const int32_t* __restrict__ row0, const int32_t* __restrict__ nrow,
                                                     const int32_t* __restrict__ col, const float* __restrict__ val,
-                                                    const float* __restrict__ diag, const float* __restrict__ X,
-                                                    const float* __restrict__ B, float* __restrict__ R) {
+                                                    const float* __restrict__ diag, const float* X, const float* B,
+                                                    float* R) {
+  constexpr int V = MCols<NR>::V;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, part = warp % G;
-  const int64_t s = (int64_t)blockIdx.x * (8 / G) + warp / G;
-  const MRow m = m_row<G>(s, nslice, ptr, row0, nrow, part, lane);
-  float acc[NR], bv[NR];
+  MRow<NR, G> m(0, nslice, (int64_t)blockIdx.x * (8 / G) + warp / G, ptr, row0, nrow, col, val, part, lane);
+  const bool own = part == 0 && m.active;
+  const float d = own ? diag[m.r] : 0.f;
+  pdl_wait();
+  pdl_trigger();
+  float acc[V], bv[V];
 #pragma unroll
-  for (int c = 0; c < NR; ++c) acc[c] = bv[c] = 0.f;
-  if (part == 0 && m.active) {
-    float xv[NR];
-    load_row<NR>(X + m.r * NR, xv);
-    load_row<NR>(B + m.r * NR, bv);  // issued with the gathers, not after the combining barrier
-    const float d = diag[m.r];
+  for (int c = 0; c < V; ++c) acc[c] = bv[c] = 0.f;
+  if (own) {
+    load_cols<V>(X + m.r * NR + m.c, acc);
+    load_cols<V>(B + m.r * NR + m.c, bv);
 #pragma unroll
-    for (int c = 0; c < NR; ++c) acc[c] = d * xv[c];
+    for (int c = 0; c < V; ++c) acc[c] *= d;
   }
-  m_dot<NR, G>(m, col, val, X, acc);
-  m_combine<NR, G>(acc, warp, lane);
-  if (part == 0 && m.active) {
+  m.dot(col, val, X, acc);
+  m_combine<V, G>(acc, warp, lane);
+  if (own) {
 #pragma unroll
-    for (int c = 0; c < NR; ++c) acc[c] = bv[c] - acc[c];
-    store_row<NR>(R + m.r * NR, acc);
+    for (int c = 0; c < V; ++c) acc[c] = bv[c] - acc[c];
+    store_cols<V>(R + m.r * NR + m.c, acc);
   }
 }
 
+// Bc = P^T R; the coarse iterate Xc starts from zero, but its rows of colour 0
+// (the first nc0) take their first Gauss-Seidel update (b - 0) / a_ii.
 template <int NR>
 __global__ void __launch_bounds__(256) k_restrict_m(int64_t nslice, const int64_t* __restrict__ ptr,
                                                     const int32_t* __restrict__ row0, const int32_t* __restrict__ nrow,
                                                     const int32_t* __restrict__ col, const float* __restrict__ w,
-                                                    const float* __restrict__ R, float* __restrict__ Bc) {
-  const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (s >= nslice || lane >= nrow[s]) return;
-  const int64_t e0 = ptr[s];
-  const int wd = (int)((ptr[s + 1] - e0) >> 5);
-  float acc[NR], rv[NR];
+                                                    const float* R, float* Bc, float* Xc,
+                                                    const float* __restrict__ dinvc, int64_t nc0) {
+  constexpr int V = MCols<NR>::V, G = kMRestrictParts;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, part = warp % G;
+  MRow<NR, G> m(0, nslice, (int64_t)blockIdx.x * (8 / G) + warp / G, ptr, row0, nrow, col, w, part, lane);
+  const bool own = part == 0 && m.active;
+  const float d = own && m.r < nc0 ? dinvc[m.r] : 0.f;
+  pdl_wait();
+  pdl_trigger();
+  float acc[V];
 #pragma unroll
-  for (int c = 0; c < NR; ++c) acc[c] = 0.f;
-  int64_t e = e0 + lane;
-  for (int k = 0; k < wd; ++k, e += 32) {
-    const float a = w[e];
-    load_row<NR>(R + (int64_t)col[e] * NR, rv);
+  for (int c = 0; c < V; ++c) acc[c] = 0.f;
+  m.dot(col, w, R, acc);
+  m_combine<V, G>(acc, warp, lane);
+  if (own) {
+    store_cols<V>(Bc + m.r * NR + m.c, acc);
 #pragma unroll
-    for (int c = 0; c < NR; ++c) acc[c] += a * rv[c];
+    for (int c = 0; c < V; ++c) acc[c] = m.r < nc0 ? (acc[c] - 0.f) * d : 0.f;
+    store_cols<V>(Xc + m.r * NR + m.c, acc);
   }
-  store_row<NR>(Bc + (int64_t)(row0[s] + lane) * NR, acc);
 }
 
+// X += P U, one thread per row and column group.
 template <int NR>
 __global__ void __launch_bounds__(256) k_prolong_m(int64_t n, const int32_t* __restrict__ idx,
-                                                   const float* __restrict__ w, const float* __restrict__ U,
-                                                   float* __restrict__ X) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    float xv[NR], u[NR];
-    load_row<NR>(X + i * NR, xv);
+                                                   const float* __restrict__ w, const float* U, float* X) {
+  constexpr int V = MCols<NR>::V, Q = MCols<NR>::Q;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i = t / Q;
+  const int c0 = (int)(t % Q) * V;
+  int32_t id[3] = {0, 0, 0};
+  float a[3] = {0.f, 0.f, 0.f};
+  if (i < n)
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-      const float a = w[3 * i + m];
-      load_row<NR>(U + (int64_t)idx[3 * i + m] * NR, u);
-#pragma unroll
-      for (int c = 0; c < NR; ++c) xv[c] += a * u[c];
+      id[m] = idx[3 * i + m];
+      a[m] = w[3 * i + m];
     }
-    store_row<NR>(X + i * NR, xv);
-  }
+  pdl_wait();
+  pdl_trigger();
+  if (i >= n) return;
+  float xv[V], u[3][V];
+  load_cols<V>(X + i * NR + c0, xv);
+#pragma unroll
+  for (int m = 0; m < 3; ++m) load_cols<V>(U + (int64_t)id[m] * NR + c0, u[m]);
+#pragma unroll
+  for (int m = 0; m < 3; ++m)
+#pragma unroll
+    for (int c = 0; c < V; ++c) xv[c] += a[m] * u[m][c];
+  store_cols<V>(X + i * NR + c0, xv);
 }
 
-// X = Ainv B on the coarsest level (FP64 accumulation), one warp per row.
+// X = Ainv B on the coarsest level (FP64 accumulation), one warp per row and
+// pair of columns: the FP64 pipes bound it (a warp instruction occupies a
+// sub-partition's pipe for 64 cycles), so the work is spread over all of them.
 template <int NR>
-__global__ void __launch_bounds__(256) k_coarse_m(int n, const double* __restrict__ Ainv, const float* __restrict__ B,
-                                                  float* __restrict__ X) {
-  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(256) k_coarse_m(int n, const double* __restrict__ Ainv, const float* B, float* X) {
+  constexpr int W = NR < 2 ? 1 : 2;
+  const int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  const int row = t / (NR / W), c0 = (t % (NR / W)) * W;
+  pdl_wait();
+  pdl_trigger();
   if (row >= n) return;
-  double s[NR];
+  double s[W];
 #pragma unroll
-  for (int c = 0; c < NR; ++c) s[c] = 0.0;
+  for (int c = 0; c < W; ++c) s[c] = 0.0;
   const double* a = Ainv + (int64_t)row * n;
+#pragma unroll 4
   for (int j = lane; j < n; j += 32) {
     const double aj = a[j];
+    float bv[W];
+    load_cols<W>(B + (int64_t)j * NR + c0, bv);
 #pragma unroll
-    for (int c = 0; c < NR; ++c) s[c] += aj * f64_of(B[(int64_t)j * NR + c]);
+    for (int c = 0; c < W; ++c) s[c] += aj * f64_of(bv[c]);
   }
 #pragma unroll
-  for (int c = 0; c < NR; ++c)
+  for (int c = 0; c < W; ++c)
     for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
-  if (lane == 0)
+  if (lane == 0) {
+    float xv[W];
 #pragma unroll
-    for (int c = 0; c < NR; ++c) X[(int64_t)row * NR + c] = f32_rn(s[c]);
+    for (int c = 0; c < W; ++c) xv[c] = f32_rn(s[c]);
+    store_cols<W>(X + (int64_t)row * NR + c0, xv);
+  }
 }
 
-// FP64 outer residual R = B - A X with per-block, per-column partial sums of
-// R^2 (fixed-shape reduction), and the correction cast R32 = (float) R.
+// FP64 outer residual R = B - A X, one lane per row and pair of columns
+// (32 / Q rows per warp), a fixed grid walking the row groups: the correction
+// cycle's right-hand side R32 = (float) R and initial iterate X32 (zero, the
+// rows of colour 0, the first n0, at their first Gauss-Seidel update), and the
+// columns' sums of R^2 into out[0 .. NR) (block partials, finished in a fixed
+// order by the last block).
 template <int NR>
 __global__ void __launch_bounds__(256) k_outer_residual_m(int64_t nslice, const int64_t* __restrict__ ptr,
                                                           const int32_t* __restrict__ row0,
                                                           const int32_t* __restrict__ nrow,
                                                           const int32_t* __restrict__ col,
                                                           const double* __restrict__ val,
-                                                          const double* __restrict__ diag,
-                                                          const double* __restrict__ X, const double* __restrict__ B,
-                                                          float* __restrict__ R32, double* __restrict__ partial) {
-  const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  double sq[NR];
+                                                          const double* __restrict__ diag, const double* X,
+                                                          const double* B, float* R32, float* X32,
+                                                          const float* __restrict__ dinv32, int64_t n0,
+                                                          double* partial, int* counter, double* out) {
+  constexpr int V = NR < 2 ? 1 : 2, Q = NR / V, RW = 32 / Q, U = 4;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int c0 = (lane % Q) * V;
+  pdl_wait();
+  pdl_trigger();
+  double sq[V];
 #pragma unroll
-  for (int c = 0; c < NR; ++c) sq[c] = 0.0;
-  if (s < nslice && lane < nrow[s]) {
-    const int64_t r = row0[s] + lane;
-    const int64_t e0 = ptr[s];
-    const int w = (int)((ptr[s + 1] - e0) >> 5);
-    double acc[NR];
+  for (int c = 0; c < V; ++c) sq[c] = 0.0;
+  for (int64_t g = (int64_t)blockIdx.x * 8 + warp; g < nslice * Q; g += (int64_t)gridDim.x * 8) {
+    const int64_t s = g / Q;
+    const int ri = (int)(g % Q) * RW + lane / Q;
+    if (ri >= nrow[s]) continue;
+    const int64_t r = row0[s] + ri, e = ptr[s] + ri;
+    const int w = (int)((ptr[s + 1] - ptr[s]) >> 5);
+    double acc[V], bv[V];
     const double d = diag[r];
 #pragma unroll
-    for (int c = 0; c < NR; ++c) acc[c] = d * X[r * NR + c];
-    int64_t e = e0 + lane;
-    for (int k = 0; k < w; ++k, e += 32) {
-      const double a = val[e];
-      const double* xj = X + (int64_t)col[e] * NR;
-#pragma unroll
-      for (int c = 0; c < NR; ++c) acc[c] += a * xj[c];
+    for (int c = 0; c < V; ++c) {
+      acc[c] = d * X[r * NR + c0 + c];
+      bv[c] = B[r * NR + c0 + c];
     }
+    for (int k0 = 0; k0 < w; k0 += U) {
+      double a[U], xv[U][V];
+      int32_t j[U];
 #pragma unroll
-    for (int c = 0; c < NR; ++c) {
-      const double rv = B[r * NR + c] - acc[c];
-      R32[r * NR + c] = f32_rn(rv);
-      sq[c] = rv * rv;
+      for (int q = 0; q < U; ++q) {
+        a[q] = k0 + q < w ? val[e + (int64_t)(k0 + q) * 32] : 0.0;
+        j[q] = k0 + q < w ? col[e + (int64_t)(k0 + q) * 32] : (int32_t)r;
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+        if constexpr (V == 2) {
+          const double2 t = *reinterpret_cast<const double2*>(X + (int64_t)j[q] * NR + c0);
+          xv[q][0] = t.x;
+          xv[q][1] = t.y;
+        } else {
+          xv[q][0] = X[(int64_t)j[q] * NR + c0];
+        }
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+        if (k0 + q < w)
+#pragma unroll
+          for (int c = 0; c < V; ++c) acc[c] += a[q] * xv[q][c];
     }
+    const float di = r < n0 ? dinv32[r] : 0.f;
+    float rv32[V], xv32[V];
+#pragma unroll
+    for (int c = 0; c < V; ++c) {
+      const double rv = bv[c] - acc[c];
+      sq[c] += rv * rv;
+      rv32[c] = f32_rn(rv);
+      xv32[c] = r < n0 ? (rv32[c] - 0.f) * di : 0.f;
+    }
+    store_cols<V>(R32 + r * NR + c0, rv32);
+    store_cols<V>(X32 + r * NR + c0, xv32);
   }
-  __shared__ double red[NR][256];
+  // sums over the block's rows: lanes of a column group, then the warps in order
+  __shared__ double red[8][NR];
 #pragma unroll
-  for (int c = 0; c < NR; ++c) red[c][threadIdx.x] = sq[c];
+  for (int c = 0; c < V; ++c)
+    for (int o = 16; o >= Q; o >>= 1) sq[c] += __shfl_xor_sync(0xffffffffu, sq[c], o);
+  if (lane < Q)
+#pragma unroll
+    for (int c = 0; c < V; ++c) red[warp][c0 + c] = sq[c];
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o)
-#pragma unroll
-      for (int c = 0; c < NR; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + o];
-    __syncthreads();
+  if (threadIdx.x < NR) {
+    double t = 0.0;
+    for (int q = 0; q < 8; ++q) t += red[q][threadIdx.x];
+    partial[(int64_t)blockIdx.x * NR + threadIdx.x] = t;
   }
-  if (threadIdx.x < NR) partial[(int64_t)blockIdx.x * NR + threadIdx.x] = red[threadIdx.x][0];
-}
-
-// out[c] = sum over blocks of partial[b * NR + c] (fixed order).
-__global__ void k_reduce_cols(int nblocks, int nr, const double* __restrict__ partial, double* __restrict__ out) {
-  __shared__ double red[256];
-  for (int c = 0; c < nr; ++c) {
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += 256) s += partial[(int64_t)b * nr + c];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-      if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[c] = red[0];
-    __syncthreads();
+  __shared__ int is_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    is_last = atomicAdd(counter, 1) == (int)gridDim.x - 1;
+    if (is_last) *counter = 0;
+  }
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  for (int c = warp; c < NR; c += 8) {  // a warp per column
+    double t = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(partial + (int64_t)b * NR + c);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) out[c] = t;
   }
 }
 
@@ -313,12 +403,48 @@ __global__ void k_zero_cols(int64_t n, int NR, int mask, double* __restrict__ X)
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * NR; t += (int64_t)gridDim.x * blockDim.x)
     if ((mask >> (int)(t % NR)) & 1) X[t] = 0.0;
 }
-__global__ void k_add_f2d_m(int64_t m, const float* __restrict__ e, double* __restrict__ x) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
-    x[i] += f64_of(e[i]);
+// x += (double) e, four consecutive values per thread.
+__global__ void __launch_bounds__(256) k_add_f2d_m(int64_t m, const float* e, double* x) {
+  pdl_wait();
+  pdl_trigger();
+  for (int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); i < m; i += 4 * (int64_t)gridDim.x * blockDim.x) {
+    if (i + 4 <= m) {
+      const float4 q = *reinterpret_cast<const float4*>(e + i);
+      double2* p = reinterpret_cast<double2*>(x + i);
+      double2 a = p[0], b = p[1];
+      a.x += f64_of(q.x);
+      a.y += f64_of(q.y);
+      b.x += f64_of(q.z);
+      b.y += f64_of(q.w);
+      p[0] = a;
+      p[1] = b;
+    } else {
+      for (int64_t k = i; k < m; ++k) x[k] += f64_of(e[k]);
+    }
+  }
+}
+// After an iteration of the batched solve (one warp): the worst column's
+// relative residual into hist[k] (a non-finite column's value as it is), and
+// whether the loop goes on.  it: iterations done, limit, columns; nb: column
+// norms of B (0: a zero column).
+__global__ void k_batched_check(int* it, double* hist, const double* rr, const double* nb, const double* tol,
+                                cudaGraphConditionalHandle h) {
+  pdl_wait();
+  pdl_trigger();
+  const int lane = threadIdx.x;
+  const double b = lane < it[2] ? nb[lane] : 0.0;
+  const double r = b > 0.0 ? sqrt(rr[lane]) / b : 0.0;
+  const unsigned bad = __ballot_sync(0xffffffffu, !isfinite(r));
+  double w = r;
+  for (int o = 16; o > 0; o >>= 1) w = fmax(w, __shfl_xor_sync(0xffffffffu, w, o));
+  if (bad) w = __shfl_sync(0xffffffffu, r, __ffs(bad) - 1);
+  if (lane == 0) {
+    const int k = ++it[0];
+    hist[k] = w;
+    cudaGraphSetConditional(h, !bad && !(w <= *tol) && k < it[1] ? 1u : 0u);
+  }
 }
 
-static inline int nblk(int64_t threads) { return (int)std::max<int64_t>(1, (threads + 255) / 256); }
 static inline int gblk(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 64)); }
 
 #define LCK() GMG_LAUNCHED()
@@ -339,81 +465,79 @@ static gmg_status sweep_m(Level& L, int k, cudaStream_t s, int G = 0) {
   const int64_t s0 = L.color_slice_off[k], s1 = L.color_slice_off[k + 1];
   if (s1 <= s0) return GMG_OK;
   if (G == 0) G = m_lanes<NR>(L);
-  const int64_t grid = (s1 - s0 + 8 / G - 1) / (8 / G);
+  const int64_t grid = ((s1 - s0) * MCols<NR>::Q + 8 / G - 1) / (8 / G);
   const Ell& A = L.A;
+  const float *v = A.v32, *d = L.dinv32, *b = L.B32;
   switch (G) {
-    case 1: k_gs_m<NR, 1><<<(unsigned)grid, 256, 0, s>>>(s0, s1, A.ptr, A.row0, A.nrow, A.col, A.v32, L.dinv32, L.B32, L.X32); break;
-    case 2: k_gs_m<NR, 2><<<(unsigned)grid, 256, 0, s>>>(s0, s1, A.ptr, A.row0, A.nrow, A.col, A.v32, L.dinv32, L.B32, L.X32); break;
-    case 4: k_gs_m<NR, 4><<<(unsigned)grid, 256, 0, s>>>(s0, s1, A.ptr, A.row0, A.nrow, A.col, A.v32, L.dinv32, L.B32, L.X32); break;
-    default: k_gs_m<NR, 8><<<(unsigned)grid, 256, 0, s>>>(s0, s1, A.ptr, A.row0, A.nrow, A.col, A.v32, L.dinv32, L.B32, L.X32);
+    case 1: return launch(k_gs_m<NR, 1>, grid, 256, s, s0, s1, A.ptr, A.row0, A.nrow, A.col, v, d, b, L.X32);
+    case 2: return launch(k_gs_m<NR, 2>, grid, 256, s, s0, s1, A.ptr, A.row0, A.nrow, A.col, v, d, b, L.X32);
+    case 4: return launch(k_gs_m<NR, 4>, grid, 256, s, s0, s1, A.ptr, A.row0, A.nrow, A.col, v, d, b, L.X32);
+    default: return launch(k_gs_m<NR, 8>, grid, 256, s, s0, s1, A.ptr, A.row0, A.nrow, A.col, v, d, b, L.X32);
   }
-  LCK();
-  return GMG_OK;
 }
 
 template <int NR>
 static gmg_status residual_m(Level& L, cudaStream_t s, int G = 0) {
   if (G == 0) G = m_lanes<NR>(L);
   const Ell& A = L.A;
-  const int64_t grid = std::max<int64_t>(1, (A.nslice + 8 / G - 1) / (8 / G));
+  const int64_t grid = (A.nslice * MCols<NR>::Q + 8 / G - 1) / (8 / G);
+  const float *v = A.v32, *d = L.diag32, *x = L.X32, *b = L.B32;
   switch (G) {
-    case 1: k_residual_m<NR, 1><<<(unsigned)grid, 256, 0, s>>>(A.nslice, A.ptr, A.row0, A.nrow, A.col, A.v32, L.diag32, L.X32, L.B32, L.R32); break;
-    case 2: k_residual_m<NR, 2><<<(unsigned)grid, 256, 0, s>>>(A.nslice, A.ptr, A.row0, A.nrow, A.col, A.v32, L.diag32, L.X32, L.B32, L.R32); break;
-    case 4: k_residual_m<NR, 4><<<(unsigned)grid, 256, 0, s>>>(A.nslice, A.ptr, A.row0, A.nrow, A.col, A.v32, L.diag32, L.X32, L.B32, L.R32); break;
-    default: k_residual_m<NR, 8><<<(unsigned)grid, 256, 0, s>>>(A.nslice, A.ptr, A.row0, A.nrow, A.col, A.v32, L.diag32, L.X32, L.B32, L.R32);
+    case 1: return launch(k_residual_m<NR, 1>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, v, d, x, b, L.R32);
+    case 2: return launch(k_residual_m<NR, 2>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, v, d, x, b, L.R32);
+    case 4: return launch(k_residual_m<NR, 4>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, v, d, x, b, L.R32);
+    default: return launch(k_residual_m<NR, 8>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, v, d, x, b, L.R32);
   }
-  LCK();
-  return GMG_OK;
 }
 
-// MGI(X_l, B_l, l) on [n_l x NR] blocks.  Every level starts from X_l = 0
-// (the recursive calls of Alg. 2, and the correction cycle of the outer
-// refinement on the finest level) unless keep_x, which keeps the caller's
-// initial iterate in the finest level's X32.
+// MGI(X_l, B_l, l) on [n_l x NR] blocks from the iterate in X_l.  With c0_done
+// the kernel that set B_l has set X_l to zero and applied the first
+// Gauss-Seidel colour (the outer residual on the finest level, the
+// restriction on the others).
 template <int NR>
-static gmg_status vcycle_m(gmg_ctx* c, int l, cudaStream_t s, bool keep_x = false) {
+static gmg_status vcycle_m(gmg_ctx* c, int l, cudaStream_t s, bool c0_done) {
   Level& L = c->L[l];
   if (l == c->nlev - 1) {
-    k_coarse_m<NR><<<(int)((L.n * 32 + 255) / 256), 256, 0, s>>>((int)L.n, c->Ainv, L.B32, L.X32);
-    LCK();
-    return GMG_OK;
+    constexpr int W = NR < 2 ? 1 : 2;
+    return launch(k_coarse_m<NR>, (L.n * (NR / W) * 32 + 255) / 256, 256, s, (int)L.n, (const double*)c->Ainv,
+                  (const float*)L.B32, L.X32);
   }
   Level& C = c->L[l + 1];
-  if (!keep_x) GMG_CK(cudaMemsetAsync(L.X32, 0, sizeof(float) * (size_t)(L.n * NR), s));
   for (int it = 0; it < c->opt.nu_pre; ++it)
-    for (int k = 0; k < L.ncolor; ++k) GMG_TRY(sweep_m<NR>(L, k, s));
+    for (int k = it == 0 && c0_done ? 1 : 0; k < L.ncolor; ++k) GMG_TRY(sweep_m<NR>(L, k, s));
   GMG_TRY(residual_m<NR>(L, s));
-  k_restrict_m<NR><<<nblk(L.R.nslice * 32), 256, 0, s>>>(L.R.nslice, L.R.ptr, L.R.row0, L.R.nrow, L.R.col, L.R.v32,
-                                                        L.R32, C.B32);
-  LCK();
-  GMG_TRY(vcycle_m<NR>(c, l + 1, s));
-  k_prolong_m<NR><<<gblk(L.n), 256, 0, s>>>(L.n, L.p_idx, L.p_w32, C.X32, L.X32);
-  LCK();
+  const bool next_c0 = c->opt.nu_pre > 0 && l + 1 < c->nlev - 1;
+  const int64_t rgrid = (L.R.nslice * MCols<NR>::Q + 8 / kMRestrictParts - 1) / (8 / kMRestrictParts);
+  GMG_TRY(launch(k_restrict_m<NR>, rgrid, 256, s, L.R.nslice, L.R.ptr, L.R.row0, L.R.nrow, L.R.col, L.R.v32,
+                 (const float*)L.R32, C.B32, C.X32, (const float*)C.dinv32, next_c0 ? C.color_off[1] : (int64_t)0));
+  GMG_TRY(vcycle_m<NR>(c, l + 1, s, next_c0));
+  GMG_TRY(launch(k_prolong_m<NR>, (L.n * MCols<NR>::Q + 255) / 256, 256, s, L.n, L.p_idx, L.p_w32,
+                 (const float*)C.X32, L.X32));
   for (int it = 0; it < c->opt.nu_post; ++it)
     for (int q = 0; q < L.ncolor; ++q) GMG_TRY(sweep_m<NR>(L, c->opt.post_forward ? q : L.ncolor - 1 - q, s));
   return GMG_OK;
 }
 
-// R = B - A X (FP64) -> level-0 B32 and per-column ||R||^2 into scal[8 + c].
+// Rows of the finest level whose first update the outer residual applies.
+static int64_t first_rows(const gmg_ctx* c) { return c->opt.nu_pre > 0 && c->nlev > 1 ? c->L[0].color_off[1] : 0; }
+
+// R = B - A X (FP64) -> level-0 B32, X32 and per-column ||R||^2 into scal[8 + c].
 template <int NR>
-static gmg_status outer_m(gmg_ctx* c, cudaStream_t s) {
+static gmg_status outer_m(gmg_ctx* c, const double* X, cudaStream_t s) {
   Level& L = c->L[0];
-  const int nb = nblk(L.A.nslice * 32);
-  k_outer_residual_m<NR><<<nb, 256, 0, s>>>(L.A.nslice, L.A.ptr, L.A.row0, L.A.nrow, L.A.col, L.A.v64, L.diag64,
-                                           c->XS, c->BS, L.B32, c->red);
-  LCK();
-  k_reduce_cols<<<1, 256, 0, s>>>(nb, NR, c->red, c->scal + 8);
-  LCK();
-  return GMG_OK;
+  constexpr int Q = NR < 2 ? 1 : NR / 2;
+  const int64_t nb = std::min<int64_t>(kRedBlocks, (L.A.nslice * Q + 7) / 8);
+  return launch(k_outer_residual_m<NR>, nb, 256, s, L.A.nslice, L.A.ptr, L.A.row0, L.A.nrow, L.A.col, L.A.v64,
+                L.diag64, X, (const double*)c->BS, L.B32, L.X32, (const float*)L.dinv32, first_rows(c), c->red,
+                c->red_cnt + 3, c->scal + 8);
 }
 
 template <int NR>
 static gmg_status iteration_m(gmg_ctx* c, cudaStream_t s) {
   Level& L = c->L[0];
-  GMG_TRY(vcycle_m<NR>(c, 0, s));
-  k_add_f2d_m<<<gblk(L.n * NR), 256, 0, s>>>(L.n * NR, L.X32, c->XS);
-  LCK();
-  return outer_m<NR>(c, s);
+  GMG_TRY(vcycle_m<NR>(c, 0, s, first_rows(c) > 0));
+  GMG_TRY(launch(k_add_f2d_m, gblk((L.n * NR + 3) / 4), 256, s, L.n * NR, (const float*)L.X32, c->XS));
+  return outer_m<NR>(c, c->XS, s);
 }
 
 static gmg_status ensure_batched(gmg_ctx* c) {
@@ -429,12 +553,81 @@ static gmg_status ensure_batched(gmg_ctx* c) {
   GMG_TRY(c->arena.alloc(&c->RS, (size_t)n * kMaxRhs));
   // per-column partials of the batched residual, and never smaller than the
   // single-vector partials the buffer already serves
-  const int64_t need = std::max<int64_t>((int64_t)nblk(c->L[0].A.nslice * 32) * kMaxRhs + 64, c->red_cap);
+  const int64_t need = std::max<int64_t>((int64_t)kRedBlocks * kMaxRhs, c->red_cap);
   double* red2;
   GMG_TRY(c->arena.alloc(&red2, (size_t)need));
   c->red = red2;
   c->red_cap = need;
   return GMG_OK;
+}
+
+// The device-side loop of the batched solve for blocks of NR columns: a graph
+// whose conditional WHILE node repeats one iteration and its convergence test
+// (programmatic launch edges kept where the CUDA driver instantiates them,
+// else plain stream order).  Leaves mloops[slot] null when refused.
+template <int NR>
+static gmg_status build_mloop(gmg_ctx* c) {
+  const int slot = nr_index(NR);
+  if (!c->g_stream) GMG_CK(cudaStreamCreateWithFlags(&c->g_stream, cudaStreamNonBlocking));
+  for (int attempt = 0; attempt < 2 && !c->mloops[slot]; ++attempt) {
+    cudaGraph_t g = nullptr;
+    GMG_CK(cudaGraphCreate(&g, 0));
+    cudaGraphConditionalHandle h = 0;
+    cudaGraphNodeParams np = {};
+    cudaError_t e = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault);
+    if (e == cudaSuccess) {
+      np.type = cudaGraphNodeTypeConditional;
+      np.conditional.handle = h;
+      np.conditional.type = cudaGraphCondTypeWhile;
+      np.conditional.size = 1;
+      cudaGraphNode_t node;
+      e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &np);
+    }
+    gmg_status st = GMG_OK;
+    if (e == cudaSuccess) {
+      const uint64_t before = g_launches;
+      g_pdl_suspended = attempt == 1;
+      e = cudaStreamBeginCaptureToGraph(c->g_stream, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                        cudaStreamCaptureModeThreadLocal);
+      if (e == cudaSuccess) {
+        st = iteration_m<NR>(c, c->g_stream);
+        if (st == GMG_OK)
+          st = launch(k_batched_check, 1, 32, c->g_stream, c->dloop, c->dhist, (const double*)(c->scal + 8),
+                      (const double*)(c->scal + 24), (const double*)(c->scal + 40), h);
+        cudaGraph_t body = nullptr;
+        e = cudaStreamEndCapture(c->g_stream, &body);
+      }
+      g_pdl_suspended = false;
+      c->mloop_kernels[slot] = g_launches - before;
+      g_launches = before;
+      if (st == GMG_OK && e == cudaSuccess) e = cudaGraphInstantiate(&c->mloops[slot], g, 0);
+    }
+    cudaGraphDestroy(g);
+    if (st != GMG_OK) return st;
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      c->mloops[slot] = nullptr;
+    }
+  }
+  if (!c->mloops[slot]) c->mloop_refused[slot] = true;
+  return GMG_OK;
+}
+
+// Forgets the batched loops (their launch shapes are stale).
+static void drop_mloops(gmg_ctx* c) {
+  for (int q = 0; q < 5; ++q) {
+    if (c->mloops[q]) cudaGraphExecDestroy(c->mloops[q]);
+    c->mloops[q] = nullptr;
+    c->mloop_refused[q] = false;
+  }
+}
+
+static bool device_loop_off() {
+  static const bool off = [] {
+    const char* v = std::getenv("GMG_NO_DEVICE_LOOP");
+    return v && v[0] == '1';
+  }();
+  return off;
 }
 
 template <int NR>
@@ -462,11 +655,8 @@ static gmg_status solve_m(gmg_ctx* c, int nrhs, const double* B, double* X, doub
   double nb[kMaxRhs];
   bool all_zero = true;
   {
-    double* keep = c->XS;
-    c->XS = c->RS;
     GMG_CK(cudaMemsetAsync(c->RS, 0, sizeof(double) * (size_t)(n * NR), s));
-    GMG_TRY(outer_m<NR>(c, s));
-    c->XS = keep;
+    GMG_TRY(outer_m<NR>(c, c->RS, s));
     GMG_CK(cudaMemcpyAsync(c->h_scal + 8, c->scal + 8, NR * sizeof(double), cudaMemcpyDeviceToHost, s));
     GMG_CK(cudaStreamSynchronize(s));
     int zmask = 0;
@@ -489,7 +679,7 @@ static gmg_status solve_m(gmg_ctx* c, int nrhs, const double* B, double* X, doub
     }
     return w;
   };
-  GMG_TRY(outer_m<NR>(c, s));
+  GMG_TRY(outer_m<NR>(c, c->XS, s));
   GMG_CK(cudaMemcpyAsync(c->h_scal + 8, c->scal + 8, NR * sizeof(double), cudaMemcpyDeviceToHost, s));
   GMG_CK(cudaStreamSynchronize(s));
   double rel = worst();
@@ -501,6 +691,35 @@ static gmg_status solve_m(gmg_ctx* c, int nrhs, const double* B, double* X, doub
   } else if (all_zero) {
     st = GMG_OK;
   } else {
+    const int slot = nr_index(NR);
+    const bool loop = c->opt.use_graphs && !device_loop_off();
+    if (loop && c->opt.max_iter > 0 && !(rel <= tol) && !c->mloops[slot] && !c->mloop_refused[slot])
+      GMG_TRY(build_mloop<NR>(c));
+    if (loop && c->opt.max_iter > 0 && c->mloops[slot]) {
+      // at least one iteration is made, as in the host-driven loop
+      const int it[3] = {0, c->opt.max_iter, nrhs};
+      double par[17];
+      for (int q = 0; q < 16; ++q) par[q] = q < nrhs ? nb[q] : 0.0;
+      par[16] = tol;
+      GMG_CK(cudaMemcpyAsync(c->scal + 24, par, sizeof(par), cudaMemcpyHostToDevice, s));
+      GMG_CK(cudaMemcpyAsync(c->dloop, it, sizeof(it), cudaMemcpyHostToDevice, s));
+      GMG_CK(cudaGraphLaunch(c->mloops[slot], s));
+      int* hk = reinterpret_cast<int*>(c->h_scal + 40);
+      GMG_CK(cudaMemcpyAsync(hk, c->dloop, sizeof(int), cudaMemcpyDeviceToHost, s));
+      GMG_CK(cudaMemcpyAsync(c->h_scal + 8, c->scal + 8, NR * sizeof(double), cudaMemcpyDeviceToHost, s));
+      GMG_CK(cudaStreamSynchronize(s));
+      k = *hk;
+      if (k < 1 || k > c->opt.max_iter) {
+        set_error("gmg_solve_batched: iteration counter out of range");
+        return GMG_ERR_CUDA;
+      }
+      g_launches += (uint64_t)k * c->mloop_kernels[slot];
+      if (info && info->history && info->history_cap > 1)
+        GMG_CK(cudaMemcpy(info->history + 1, c->dhist + 1,
+                          sizeof(double) * (size_t)std::min(k, info->history_cap - 1), cudaMemcpyDeviceToHost));
+      rel = worst();
+      st = !std::isfinite(rel) ? GMG_ERR_NONFINITE : rel <= tol ? GMG_OK : GMG_ERR_NOT_CONVERGED;
+    } else
     while (k < c->opt.max_iter) {
       GMG_TRY(iteration_m<NR>(c, s));
       GMG_CK(cudaMemcpyAsync(c->h_scal + 8, c->scal + 8, NR * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -570,7 +789,7 @@ static gmg_status vcycle_step_m(gmg_ctx* c, int nrhs, const double* B, double* X
   LCK();
   GMG_TRY(launch_d2f(n * NR, c->BS, L0.B32, s));
   GMG_TRY(launch_d2f(n * NR, c->XS, L0.X32, s));
-  GMG_TRY(vcycle_m<NR>(c, 0, s, true));
+  GMG_TRY(vcycle_m<NR>(c, 0, s, false));
   GMG_TRY(launch_f2d(n * NR, L0.X32, c->XS, s));
   k_scatter_m<<<gblk(n * nrhs), 256, 0, s>>>(n, nrhs, NR, L0.perm, c->XS, X);
   LCK();
@@ -654,6 +873,7 @@ static gmg_status autotune_m(gmg_ctx* c, int* lanes_out, cudaStream_t stream) {
   cudaStreamSynchronize(cs);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  drop_mloops(c);
   return st;
 }
 
@@ -693,6 +913,8 @@ extern "C" gmg_status gmg_set_lanes_batched(gmg_handle h, int nrhs, const int* l
     }
   const int slot = nr_index(block_width(nrhs));
   for (int l = 0; l + 1 < h->nlev; ++l) h->L[l].mlanes[slot] = lanes[l];
+  GMG_CK(cudaSetDevice(h->device));
+  drop_mloops(h);
   return GMG_OK;
 }
 
@@ -910,12 +1132,8 @@ static gmg_status many_solve(gmg_many_ctx* m, int nrhs, const double* const* B, 
     k_gather_m<<<gblk(n * NR), 256, 0, s>>>(n, nrhs, NR, L0.perm, xsrc, c->XS);
     LCK();
     // ||B_c||: the outer residual of a zero iterate
-    double* keep = c->XS;
-    c->XS = c->RS;
     GMG_CK(cudaMemsetAsync(c->RS, 0, sizeof(double) * (size_t)(n * NR), s));
-    gmg_status st = outer_m<NR>(c, s);
-    c->XS = keep;
-    GMG_TRY(st);
+    GMG_TRY(outer_m<NR>(c, c->RS, s));
     GMG_CK(cudaMemcpyAsync(c->h_scal + 8, c->scal + 8, NR * sizeof(double), cudaMemcpyDeviceToHost, s));
     GMG_CK(cudaStreamSynchronize(s));
     int zmask = 0;
@@ -927,7 +1145,7 @@ static gmg_status many_solve(gmg_many_ctx* m, int nrhs, const double* const* B, 
       k_zero_cols<<<gblk(n * NR), 256, 0, s>>>(n, NR, zmask, c->XS);
       LCK();
     }
-    GMG_TRY(outer_m<NR>(c, s));
+    GMG_TRY(outer_m<NR>(c, c->XS, s));
   }
   // host-side residuals of every mesh not yet done (a done mesh keeps the
   // residual it converged with)
@@ -963,12 +1181,15 @@ static gmg_status many_solve(gmg_many_ctx* m, int nrhs, const double* const* B, 
   }
   if (bad) st = GMG_ERR_NONFINITE;
   else if (!open) st = GMG_OK;
-  static const bool no_loop = [] {
-    const char* v = std::getenv("GMG_NO_DEVICE_LOOP");
-    return v && v[0] == '1';
-  }();
+  const bool no_loop = device_loop_off();
   if (st == GMG_ERR_NOT_CONVERGED && max_iter > 0 && !no_loop && !m->loop_refused[slot] && !m->loop[slot])
-    GMG_TRY(many_loop<NR>(m, slot, nrhs));
+    for (int attempt = 0; attempt < 2 && !m->loop[slot]; ++attempt) {
+      g_pdl_suspended = attempt == 1;  // plain stream order if the driver refuses programmatic edges here
+      m->loop_refused[slot] = false;
+      const gmg_status sl = many_loop<NR>(m, slot, nrhs);
+      g_pdl_suspended = false;
+      GMG_TRY(sl);
+    }
   if (st == GMG_ERR_NOT_CONVERGED && max_iter > 0 && m->loop[slot]) {
     // device-side loop: state, norms and the IF handles of this loop, one launch
     std::vector<int> hs(3 + 2 * K, 0);

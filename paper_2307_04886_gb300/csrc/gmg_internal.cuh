@@ -313,7 +313,11 @@ struct gmg_ctx {
   uint64_t loop_kernels[4] = {};  // kernel nodes of one loop iteration
   bool loop_refused[4] = {};      // instantiation failed: the host loop serves the mode
   bool loop_pdl[4] = {};          // the loop body kept its programmatic launch edges
-  int* dloop = nullptr;           // device iteration counter, iteration limit
+  // the same for the batched solve, by block width NR = 1, 2, 4, 8, 16
+  cudaGraphExec_t mloops[5] = {};
+  uint64_t mloop_kernels[5] = {};
+  bool mloop_refused[5] = {};
+  int* dloop = nullptr;           // device iteration counter, iteration limit, columns
   double* dhist = nullptr;        // relative residual per iteration (max_iter + 1)
   cudaStream_t g_stream = nullptr;
   bool values_ready = false;

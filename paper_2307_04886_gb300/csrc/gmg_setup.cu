@@ -1918,7 +1918,7 @@ gmg_status setup_impl(gmg_ctx* c, const gmg_csr* A, int nP, const gmg_prolong* P
   c->red_cap = std::max<int64_t>(4 * kRedBlocks, L0.A.nslice + 64);
   GMG_TRY(a.alloc(&c->red, (size_t)c->red_cap));
   GMG_TRY(a.alloc(&c->scal, 64));
-  GMG_TRY(a.alloc(&c->dloop, 2));
+  GMG_TRY(a.alloc(&c->dloop, 4));
   GMG_TRY(a.alloc(&c->red_cnt, 4));
   GMG_CK(cudaMemset(c->red_cnt, 0, 4 * sizeof(int)));
   GMG_TRY(a.alloc(&c->dhist, (size_t)c->opt.max_iter + 2));
