@@ -15,14 +15,33 @@
 // CTAs read is stored into their halo copies through distributed shared
 // memory as it is updated.
 //
-// What bounds a phase is its chain of dependent shared-memory accesses and
-// the barrier (16 CTAs of 512 threads: 660 cycles with remote stores,
-// measured alone), not bandwidth.  So everything that does not depend on the
-// phase before (slice descriptor, first eight entries per lane, b, 1/a_ii,
-// list of halo stores) is loaded into registers between the barrier's arrive
-// and its wait; after the wait only the gathers of x, the adds, and the
-// stores remain.  Levels with few rows per phase split each row over 2, 4 or
-// 8 lanes.
+// What bounds a phase is its chain of dependent steps, not bandwidth, so the
+// chain is kept short:
+//  * a phase ends with a message, not a barrier: a halo store is an
+//    asynchronous remote store that completes on the receiving CTA's
+//    mbarrier, each CTA knows how many bytes a phase brings it, and its warps
+//    arrive on the same mbarrier, so one wait covers both (375 cycles per
+//    phase measured alone, against 660 for remote stores and a cluster
+//    barrier, whose release has to wait for the stores);
+//  * what does not depend on the phase before (slice descriptor, entries,
+//    b, 1/a_ii, list of halo stores) is loaded into registers before the wait;
+//  * an entry holds the shared-memory address of its x beside its value, two
+//    FP32 entries (one FP64) to a 16-byte load;
+//  * levels with few rows per phase split each row over 2, 4 or 8 lanes.
+// A cycle's levels then take 0.5-0.6 us per phase against 1.1-1.2 us with a
+// cluster barrier per phase and 2.0-2.9 us as grid launches.
+//
+// Messages and skew.  Every phase a CTA also sends a token to each CTA it
+// exchanges halo values with, once it has waited for the previous phase.  A
+// CTA can therefore be at most one phase ahead of a partner, so that two
+// mbarriers, used in turn, tell the phases apart.  A halo value is only
+// overwritten after its reader has used it: the phase that overwrites row s
+// of a partner's halo waits for the values of all the partner's rows
+// adjacent to s that were updated in earlier phases, each sent after it had
+// read s (the pattern is symmetric); and between a residual, restriction,
+// prolongation and the sweeps around them no array is read in the phase
+// before the one that writes it.  Prolongated values of the colour that the
+// post-smoothing updates first are not sent: nobody reads them.
 //
 // Entries stay in shared memory where they fit; the entries of the largest
 // levels stream from L2 by TMA bulk copies, one phase's block per stage,
@@ -45,9 +64,9 @@ namespace gmg {
 
 namespace {
 
-constexpr int kClThreads = 512;
+constexpr int kClThreads = 256;
 constexpr int kClWarps = kClThreads / 32;
-constexpr int kClPre = 8;    // entries per lane loaded before the phase's wait
+constexpr int kClSlack = 2048;  // shared memory past the last entry unit
 constexpr int kClWide = 64;  // rows per phase and CTA from which a level keeps one thread per row
 // Entries per phase and CTA up to which a level runs here: above, a phase is
 // bound by the shared-memory gathers of 16 SMs and a grid launch over all SMs
@@ -68,316 +87,640 @@ __device__ __forceinline__ void cl_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-// v into the same shared-memory location of CTA `rank` of the cluster.
-__device__ __forceinline__ void cl_store(float* p, unsigned rank, float v) {
+__device__ __forceinline__ uint32_t cl_map(uint32_t a, unsigned rank) {
   uint32_t ra;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(smem_addr(p)), "r"(rank));
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ra), "f"(v) : "memory");
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+  return ra;
 }
-__device__ __forceinline__ void cl_store(double* p, unsigned rank, double v) {
-  uint32_t ra;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(smem_addr(p)), "r"(rank));
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
+// v to the (cluster) address a, its bytes completing on the mbarrier at m of the same CTA.
+__device__ __forceinline__ void cl_send(uint32_t a, uint32_t m, float v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(a),
+               "r"(__float_as_uint(v)), "r"(m)
+               : "memory");
 }
-__device__ __forceinline__ void mbar_init(uint64_t* m, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(m)), "r"(count) : "memory");
+__device__ __forceinline__ void cl_send(uint32_t a, uint32_t m, double v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(a),
+               "l"(__double_as_longlong(v)), "r"(m)
+               : "memory");
 }
-// One arrival that also expects `bytes` of bulk copies to complete on m.
-__device__ __forceinline__ void mbar_expect(uint64_t* m, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(m)), "r"(bytes) : "memory");
+__device__ __forceinline__ void mbar_init(uint32_t m, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(m), "r"(count) : "memory");
+}
+// One arrival that also expects `bytes` of copies or messages to complete on m.
+__device__ __forceinline__ void mbar_expect(uint32_t m, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(m), "r"(bytes) : "memory");
 }
 // Bulk copy (TMA engine) of `bytes` (a multiple of 16, both addresses 16-byte
 // aligned) from global to this CTA's shared memory, completing on m.
-__device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned bytes, uint64_t* m) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_addr(dst)),
-               "l"(src), "r"(bytes), "r"(smem_addr(m))
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, unsigned bytes, uint32_t m) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(m)
                : "memory");
 }
+__device__ __forceinline__ bool mbar_try(uint32_t m, unsigned parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(done)
+      : "r"(m), "r"(parity)
+      : "memory");
+  return done != 0;
+}
 // Waits for the phase of m with the given parity to complete; gives up after
-// `polls` polls (sets *err) so that a lost copy cannot hang the GPU.  A
-// failing poll suspends the warp for about 3.8 us on GB300 (measured with
-// gmg_wait_selftest), so the limit gives up after about one second; a poll
-// does not advance while the context is switched out.
+// `polls` polls (sets *err, and polls to 1 for the waits that follow) so that
+// a lost copy or message cannot hang the GPU.  A failing poll suspends the
+// warp for about 3.8 us on GB300 (measured with gmg_wait_selftest), so the
+// limit gives up after about one second; a poll does not advance while the
+// context is switched out.
 constexpr int kWaitPolls = 1 << 18;
-__device__ __forceinline__ void mbar_wait(uint64_t* m, unsigned parity, int* err, int polls = kWaitPolls) {
-  for (int it = 0; it < polls; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(smem_addr(m)), "r"(parity)
-        : "memory");
-    if (done) return;
-  }
+__device__ __forceinline__ void mbar_wait(uint32_t m, unsigned parity, int* err, int& polls) {
+#pragma unroll 1
+  for (int it = 0; it < polls; ++it)
+    if (mbar_try(m, parity)) return;
   atomicOr(err, 1);
+  polls = 1;
 }
 
-// A list of halo stores packed in one word: first entry of the CTA's store
-// list << 4 | number of stores (at most 15 other CTAs).
-template <class T>
-__device__ __forceinline__ void push(T* base, unsigned list, const uint32_t* dst, T v) {
-  const uint32_t* d = dst + (list >> 4);
-  for (unsigned q = 0; q < (list & 15u); ++q) cl_store(base + (d[q] & 0xFFFFu), d[q] >> 16, v);
+// Shared-memory accesses by 32-bit address, kept in program order with the
+// waits (the sweeps are written with them: a phase is some eighty dependent
+// instructions per warp, and address arithmetic on generic pointers doubled
+// that).
+__device__ __forceinline__ uint4 lds4(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void lds_pair(uint32_t a, float& x, float& y) {
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(x), "=f"(y) : "r"(a));
+}
+__device__ __forceinline__ void lds_pair(uint32_t a, double& x, double& y) {
+  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(x), "=d"(y) : "r"(a));
+}
+__device__ __forceinline__ void lds1(uint32_t a, float& x) { asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(a)); }
+__device__ __forceinline__ void lds1(uint32_t a, double& x) { asm volatile("ld.shared.f64 %0, [%1];" : "=d"(x) : "r"(a)); }
+__device__ __forceinline__ void lds1(uint32_t a, int& x) { asm volatile("ld.shared.s32 %0, [%1];" : "=r"(x) : "r"(a)); }
+__device__ __forceinline__ void sts(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+__device__ __forceinline__ void sts(uint32_t a, double v) { asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory"); }
+
+// The same under a predicate (no branch).
+__device__ __forceinline__ void sts_if(bool p, uint32_t a, float v) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.f32 [%0], %1;\n\t}" ::"r"(a), "f"(v),
+               "r"((unsigned)p)
+               : "memory");
+}
+__device__ __forceinline__ void sts_if(bool p, uint32_t a, double v) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.f64 [%0], %1;\n\t}" ::"r"(a), "d"(v),
+               "r"((unsigned)p)
+               : "memory");
+}
+__device__ __forceinline__ void cl_send_if(bool p, uint32_t a, uint32_t m, float v) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t"
+      "@p st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];\n\t}" ::"r"(a),
+      "r"(__float_as_uint(v)), "r"(m), "r"((unsigned)p)
+      : "memory");
+}
+__device__ __forceinline__ void cl_send_if(bool p, uint32_t a, uint32_t m, double v) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t"
+      "@p st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];\n\t}" ::"r"(a),
+      "l"(__double_as_longlong(v)), "r"(m), "r"((unsigned)p)
+      : "memory");
 }
 
-// What a lane needs of its row before the values of the previous phase.
-template <class T>
-struct RowPre {
-  int row, w, e;  // local row, entries of this lane, first entry
-  bool lead;      // this lane writes the row
-  T v[kClPre], d;
-  int c[kClPre];
-  unsigned list;
-};
+// A halo store in one word: CTA << 28 | local index there << 14 | local index
+// here (16,384 local rows of 16 or more bytes would not fit a CTA).
+constexpr int kClMaxLocal = 1 << 14;
+__device__ __forceinline__ unsigned store_cta(int d) { return (unsigned)d >> 28; }
+__device__ __forceinline__ uint32_t store_there(int d) { return ((uint32_t)d >> 14) & 16383u; }
+__device__ __forceinline__ uint32_t store_row(int d) { return (uint32_t)d & 16383u; }
 
-// The row of `lane` in slice `s` (descriptors in `sl`), its first entries, 1/a_ii and halo stores.
+// Halo stores e = e0 + k * step of a list, e < e1, of the array at `base` (the
+// same address in every CTA), messages to m.
 template <class T>
-__device__ __forceinline__ void load_row_pre(RowPre<T>& p, const int4* sl, int s, int lane, int tpr, int lg,
-                                             const T* val, const uint16_t* col, const T* dinv, const uint32_t* xp) {
-  const int4 d = sl[s];
-  const int ri = lane >> lg;
-  const bool in = ri < (d.x >> 16);
-  p.row = (d.x & 0xFFFF) + (in ? ri : 0);
-  p.w = in ? d.y : 0;
-  p.e = d.z + lane;
-  p.lead = in && (lane & (tpr - 1)) == 0;
-#pragma unroll
-  for (int q = 0; q < kClPre; ++q) {
-    p.v[q] = q < p.w ? val[p.e + q * 32] : T(0);
-    p.c[q] = q < p.w ? col[p.e + q * 32] : 0;
+__device__ __forceinline__ void push_list(uint32_t list, int e0, int e1, int step, uint32_t base, uint32_t m) {
+#pragma unroll 1
+  for (int e = e0; e < e1; e += step) {
+    int d;
+    lds1(list + 4u * (uint32_t)e, d);
+    const uint32_t a = base + store_there(d) * (uint32_t)sizeof(T), to = cl_map(a, store_cta(d));
+    T v;
+    lds1(base + store_row(d) * (uint32_t)sizeof(T), v);
+    cl_send(to, to + (m - a), v);  // the barrier lies in the same CTA's window
   }
-  p.d = p.lead && dinv ? dinv[p.row] : T(0);
-  p.list = p.lead ? xp[p.row] : 0u;
 }
 
-// sum of the row's a_ij x_j, terms in entry order per lane, the lanes of a
-// split row added pairwise (every lane of the row gets the sum).
+// acc += the terms of one entry unit: two FP32 entries (value, byte offset of
+// x) or one FP64 entry (value, offset, unused).
+__device__ __forceinline__ void unit_gather(const uint4& u, uint32_t sm0, float (&x)[2]) {
+  lds1(sm0 + u.y, x[0]);
+  lds1(sm0 + u.w, x[1]);
+}
+__device__ __forceinline__ void unit_add(const uint4& u, const float (&x)[2], float& acc) {
+  acc += __uint_as_float(u.x) * x[0];
+  acc += __uint_as_float(u.z) * x[1];
+}
+__device__ __forceinline__ void unit_gather(const uint4& u, uint32_t sm0, double (&x)[1]) { lds1(sm0 + u.z, x[0]); }
+__device__ __forceinline__ void unit_add(const uint4& u, const double (&x)[1], double& acc) {
+  acc += __hiloint2double((int)u.y, (int)u.x) * x[0];
+}
 template <class T>
-__device__ __forceinline__ T row_sum(const RowPre<T>& p, const T* val, const uint16_t* col, const T* x, int tpr) {
+constexpr int kPerUnit = sizeof(T) == 4 ? 2 : 1;
+
+// The sum of a row: its w2 pairs of units in order, the first two pairs in u,
+// the rest from address ea on (a lane's units lie 512 bytes apart); then the
+// lanes of a split row are added pairwise (every lane of the row gets the
+// sum).  w2 is the same for the warp.  The next pair is loaded while the
+// current one is added, without a test (up to two units past the row's, which
+// the layout keeps inside the shared memory).
+__device__ __forceinline__ void load_units(uint4 (&u)[4], uint32_t ea) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) u[q] = lds4(ea + 512u * q);
+}
+template <class T>
+__device__ __forceinline__ T row_sum(uint4 (&u)[4], uint32_t ea, int w2, uint32_t sm0, int tpr) {
   T acc = 0;
-  T xv[kClPre];
-#pragma unroll
-  for (int q = 0; q < kClPre; ++q) xv[q] = x[p.c[q]];
-#pragma unroll
-  for (int q = 0; q < kClPre; ++q)
-    if (q < p.w) acc += p.v[q] * xv[q];
-  for (int q0 = kClPre; q0 < p.w; q0 += kClPre) {
-    T v[kClPre];
-    int c[kClPre];
-#pragma unroll
-    for (int q = 0; q < kClPre; ++q) {
-      v[q] = q0 + q < p.w ? val[p.e + (q0 + q) * 32] : T(0);
-      c[q] = q0 + q < p.w ? col[p.e + (q0 + q) * 32] : 0;
-    }
-#pragma unroll
-    for (int q = 0; q < kClPre; ++q) xv[q] = x[c[q]];
-#pragma unroll
-    for (int q = 0; q < kClPre; ++q)
-      if (q0 + q < p.w) acc += v[q] * xv[q];
+#pragma unroll 1
+  for (;;) {
+    T xa[kPerUnit<T>], xb[kPerUnit<T>];
+    unit_gather(u[0], sm0, xa);
+    unit_gather(u[1], sm0, xb);
+    unit_add(u[0], xa, acc);
+    unit_add(u[1], xb, acc);
+    if (--w2 <= 0) break;
+    u[0] = u[2];
+    u[1] = u[3];
+    ea += 1024u;
+    u[2] = lds4(ea + 1024u);
+    u[3] = lds4(ea + 1536u);
   }
-  for (int o = 1; o < tpr; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (tpr > 1) {
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    if (tpr > 2) {
+      acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+      if (tpr > 4) acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+    }
+  }
   return acc;
+}
+
+// Asks L2 for `bytes` from p (a kernel's later reads of set-up data, which the
+// finest level's sweeps may have pushed out).
+__device__ __forceinline__ void l2_prefetch(const void* p, int64_t bytes, int tid, int nt = kClThreads) {
+  const char* c = reinterpret_cast<const char*>(p);
+#pragma unroll 1
+  for (int64_t o = (int64_t)tid * 128; o < bytes; o += (int64_t)nt * 128)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(c + o));
 }
 
 }  // namespace
 
 // x <- MGI(x, b, l0) of Alg. 2 for the levels of D.  With c0_first the rows
 // of colour 0 of level l0 have already had their first update from x = 0.
-// All CTAs run the same sequence of cluster barriers.
+// All CTAs run the same sequence of phases.
 template <class T>
 __global__ void __launch_bounds__(kClThreads, 1)
     k_cluster_cycle(const __grid_constant__ ClusterDesc<T> D, T* xg, const T* bg, int c0_first) {
-  extern __shared__ __align__(16) char sm[];
+  extern __shared__ __align__(16) char smem[];
+  // the base of the shared memory in a register that the compiler keeps: in a
+  // cluster launch it forms the address from special registers wherever the
+  // array is named, some ten times a phase
+  uint32_t sm0;
+  asm volatile("mov.u32 %0, %1;" : "=r"(sm0) : "r"(smem_addr(smem)));
+  char* sm;
+  asm volatile("cvta.shared.u64 %0, %1;" : "=l"(sm) : "l"((uint64_t)sm0));
   const int cta = (int)cl_rank();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  uint64_t* mimg = reinterpret_cast<uint64_t*>(sm + D.o_mbar);
-  uint64_t* mst = mimg + kClMaxLevels + 1;
+  const uint32_t mimg = sm0 + (uint32_t)D.o_mbar, mst = mimg + 8u * (kClMaxLevels + 1);
+  const uint32_t mph = mst + 8u * kClStages, mbc = mph + 16u;  // two phase barriers, the coarsest right-hand side's
   const int NL = D.nlev;  // smoothed levels; lv[NL] is the coarsest
+  // after a wait that gave up, in this launch or an earlier one, nothing is worth waiting for
+  int polls = *reinterpret_cast<volatile int*>(D.err) ? 1 : kWaitPolls;
   if (tid == 0) {
-    for (int q = 0; q <= NL; ++q) mbar_init(mimg + q, 1);
-    for (int q = 0; q < kClStages; ++q) mbar_init(mst + q, 1);
+#pragma unroll 1
+    for (int q = 0; q <= NL; ++q) mbar_init(mimg + 8u * q, 1);
+#pragma unroll 1
+    for (int q = 0; q < kClStages; ++q) mbar_init(mst + 8u * q, 1);
+#pragma unroll 1
+    for (int q = 0; q < 2; ++q) mbar_init(mph + 8u * q, 1);
+    mbar_init(mbc, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   // every level's set-up tables and resident values, before the wait for the previous kernel
   if (tid == 0)
+#pragma unroll 1
     for (int t = 0; t <= NL; ++t) {
       const ClusterLevel<T>& L = D.lv[t];
-      mbar_expect(mimg + t, (unsigned)(L.img_bytes + L.val_bytes));
-      bulk_copy(sm + L.o_img, L.img + (int64_t)cta * L.img_bytes, (unsigned)L.img_bytes, mimg + t);
+      mbar_expect(mimg + 8u * t, (unsigned)(L.img_bytes + L.val_bytes));
+      bulk_copy(sm0 + (uint32_t)L.o_img, L.img + (int64_t)cta * L.img_bytes, (unsigned)L.img_bytes, mimg + 8u * t);
       if (L.val_bytes)
-        bulk_copy(sm + L.o_val, L.vimg + (int64_t)cta * L.val_bytes, (unsigned)L.val_bytes, mimg + t);
+        bulk_copy(sm0 + (uint32_t)L.o_val, L.vimg + (int64_t)cta * L.val_bytes, (unsigned)L.val_bytes,
+                  mimg + 8u * t);
     }
+  // the transfers' weights are read once, late: into L2 now
+#pragma unroll 1
+  for (int t = 0; t < NL; ++t) {
+    const ClusterLevel<T>& L = D.lv[t];
+    l2_prefetch(L.p_idx + (int64_t)cta * 3 * L.n_own_max, 6 * (int64_t)L.n_own_max, tid);
+    l2_prefetch(L.p_w + (int64_t)cta * 3 * L.n_own_max, 3 * (int64_t)sizeof(T) * L.n_own_max, tid);
+    l2_prefetch(L.r_col + (int64_t)cta * L.r_max, 2 * (int64_t)L.r_max, tid);
+    l2_prefetch(L.r_w + (int64_t)cta * L.r_max, (int64_t)sizeof(T) * L.r_max, tid);
+  }
   // the coarse iterates start from zero, halo copies included
+#pragma unroll 1
   for (int t = 1; t <= NL; ++t) {
     T* x = reinterpret_cast<T*>(sm + D.lv[t].o_x);
+#pragma unroll 1
     for (int i = tid; i < D.lv[t].n_loc_max; i += kClThreads) x[i] = T(0);
   }
-  mbar_wait(mimg, 0u, D.err);
-  // stream step j's entry block (values, then columns) into stage j % nstage
-  // (level l0's table starts with the phase of colour 0, skipped with c0_first)
+  mbar_wait(mimg, 0u, D.err, polls);
+  // stream step j's entry block into stage j % nstage (level l0's table
+  // starts with the phase of colour 0, skipped with c0_first)
   const int skip = c0_first && D.lv[0].streamed ? 1 : 0;
   const uint2* steps = reinterpret_cast<const uint2*>(sm + D.lv[0].o_img + D.i_steps) + skip;
   const int NS = D.nstage, S = D.nsteps - skip;
-  auto issue = [&](int j) {
-    if (tid != kClThreads - 32 || j >= S) return;
-    const uint2 st = steps[j];
-    char* buf = sm + D.o_buf + (j % NS) * D.stage_bytes;
-    uint64_t* m = mst + j % NS;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the stage's earlier reads come first
-    mbar_expect(m, st.y * (unsigned)(sizeof(T) + 2));
-    if (st.y) {
-      bulk_copy(buf, D.s_val + st.x, st.y * (unsigned)sizeof(T), m);
-      bulk_copy(buf + D.stage_col, D.s_col + st.x, st.y * 2u, m);
+  int j = 0, jst = 0;     // next stream step to use, its stage
+  unsigned jpar = 0;      // and that stage's parity
+  int ji = 0, jist = 0;   // next step to issue, its stage
+  auto issue = [&]() {
+    if (ji < S && tid == kClThreads - 32) {
+      const uint2 st = steps[ji];
+      const uint32_t m = mst + 8u * (uint32_t)jist;
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the stage's earlier reads come first
+      mbar_expect(m, st.y * 16u);
+      if (st.y) bulk_copy(sm0 + (uint32_t)(D.o_buf + jist * D.stage_bytes), D.s_ent + st.x, st.y * 16u, m);
+    }
+    ++ji;
+    if (++jist == NS) jist = 0;
+  };
+  auto stage_used = [&]() {
+    ++j;
+    if (++jst == NS) {
+      jst = 0;
+      jpar ^= 1u;
     }
   };
-  int j = 0;  // next stream step
-  if (NS > 0)
-    for (int q = 0; q < NS - 1; ++q) issue(q);
+#pragma unroll 1
+  for (int q = 0; q + 1 < NS; ++q) issue();
+  const int* partners = reinterpret_cast<const int*>(sm + D.lv[0].o_img + D.i_partners);
+  const int npart = reinterpret_cast<const int*>(sm + D.lv[0].o_img)[7];
+  // global rows of the CTA's rows of level l0 (first ones), before the wait
+  const int n0own = reinterpret_cast<const int*>(sm + D.lv[0].o_img)[0];
+  const int n0loc = reinterpret_cast<const int*>(sm + D.lv[0].o_img)[1];
+  const int32_t* l2g = D.l2g + (int64_t)cta * D.lv[0].n_loc_max;
+  constexpr int kX = 8;
+  int g[kX];
+#pragma unroll
+  for (int k = 0; k < kX; ++k) g[k] = tid + k * kClThreads < n0loc ? l2g[tid + k * kClThreads] : 0;
+  mbar_wait(mimg + 8u * NL, 0u, D.err, polls);
+#pragma unroll 1
+  for (int i = warp; i < reinterpret_cast<const int*>(sm + D.lv[NL].o_img)[0]; i += kClWarps)
+    l2_prefetch(D.ainv + (int64_t)reinterpret_cast<const int*>(sm + D.lv[NL].o_img + D.lv[NL].i_cr)[i] * D.nc,
+                (int64_t)sizeof(T) * D.nc, lane, 32);
   pdl_wait();  // x and b were written by the previous kernels
   pdl_trigger();
   {
     const ClusterLevel<T>& L = D.lv[0];
-    const int* hd = reinterpret_cast<const int*>(sm + L.o_img);
-    const int nown = hd[0], nloc = hd[1];
-    T* x = reinterpret_cast<T*>(sm + L.o_x);
-    T* b = reinterpret_cast<T*>(sm + L.o_b);
-    const int32_t* l2g = D.l2g + (int64_t)cta * L.n_loc_max;
-    for (int i0 = tid; i0 < nloc; i0 += 4 * kClThreads) {
-      int g[4];
-      T v[4], w[4];
+    const uint32_t a_x = sm0 + (uint32_t)L.o_x, a_bd = sm0 + (uint32_t)L.o_val;
+#pragma unroll 1
+    for (int i0 = tid; i0 < n0loc; i0 += kX * kClThreads) {
+      if (i0 != tid)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) g[k] = i0 + k * kClThreads < nloc ? l2g[i0 + k * kClThreads] : 0;
+        for (int k = 0; k < kX; ++k) g[k] = i0 + k * kClThreads < n0loc ? l2g[i0 + k * kClThreads] : 0;
+      T v[kX], w[kX];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < kX; ++k) {
         v[k] = xg[g[k]];
-        w[k] = i0 + k * kClThreads < nown ? bg[g[k]] : T(0);
+        w[k] = i0 + k * kClThreads < n0own ? bg[g[k]] : T(0);
       }
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (i0 + k * kClThreads < nloc) x[i0 + k * kClThreads] = v[k];
-        if (i0 + k * kClThreads < nown) b[i0 + k * kClThreads] = w[k];
+      for (int k = 0; k < kX; ++k) {
+        const uint32_t o = (uint32_t)sizeof(T) * (uint32_t)(i0 + k * kClThreads);
+        if (i0 + k * kClThreads < n0loc) sts(a_x + o, v[k]);
+        if (i0 + k * kClThreads < n0own) sts(a_bd + 2u * o, w[k]);
       }
     }
   }
-  cl_arrive();
-  bool pending = true;  // a cluster barrier has been arrived at and not waited for
+  if (tid == 0)  // what the other CTAs send of the coarsest right-hand side
+    mbar_expect(mbc, (unsigned)((D.nc - reinterpret_cast<const int*>(sm + D.lv[0].o_img)[8]) * (int)sizeof(T)));
+  cl_arrive();  // every CTA's barriers and copies are set before any message
+  cl_wait();
+
+  // Phase p: begin() waits for phase p - 1 (this CTA's threads, then the
+  // messages to it; before phase 0 the wait is for the phase before a fresh
+  // barrier's first, which counts as complete) and sends this phase's tokens;
+  // end(bytes), called by every thread when its messages are on their way,
+  // sets the halo bytes that the phase brings.
+  int ph = 0;
+    const bool sends_token = warp == kClWarps - 1 && lane < npart;
+  uint32_t tok_a = 0, tok_m = 0;
+  if (sends_token) {
+    tok_a = cl_map(sm0 + (uint32_t)D.o_tok + 4u * (uint32_t)cta, (unsigned)partners[lane]);
+    tok_m = cl_map(mph, (unsigned)partners[lane]);
+  }
+  auto mcur = [&]() { return mph + 8u * (uint32_t)(ph & 1); };
+  auto begin = [&]() {
+    __syncthreads();
+    mbar_wait(mph + 8u * (uint32_t)((ph - 1) & 1), (unsigned)((ph - 1) >> 1) & 1u, D.err, polls);
+    cl_send_if(sends_token, tok_a, tok_m + 8u * (uint32_t)(ph & 1), 0.f);
+  };
+  auto end = [&](int bytes) {
+    if (tid == 0) mbar_expect(mcur(), (unsigned)(bytes + 4 * npart));
+    ++ph;
+  };
 
   // Gauss-Seidel phases q0 .. nq-1 of level t, colour q mod C (descending:
-  // C-1-(q mod C)); b_ready: b of the level was set before the last barrier
-  // that this thread waited for.
+  // C-1-(q mod C)); b_ready: b of the level was set before the last phase
+  // that this thread waited for.  A warp takes slices warp, warp + kClWarps,
+  // ... of the colour, a lane a row or a part of it.  The colour's record
+  // (first slice, slices, halo bytes) and the first slice's descriptor are
+  // loaded a phase ahead, the slice's entries, b, 1/a_ii and halo stores
+  // before the wait.
   auto sweeps = [&](int t, int q0, int nq, bool descending, bool b_ready) {
     const ClusterLevel<T>& L = D.lv[t];
-    char* img = sm + L.o_img;
-    const int4* sl = reinterpret_cast<const int4*>(img + L.i_sl);
-    const int* csl = reinterpret_cast<const int*>(img + L.i_csl);
-    const uint32_t* xp = reinterpret_cast<const uint32_t*>(img + L.i_xp);
-    const uint32_t* xd = reinterpret_cast<const uint32_t*>(img + L.i_xd);
-    T* x = reinterpret_cast<T*>(sm + L.o_x);
-    const T* b = reinterpret_cast<const T*>(sm + L.o_b);
-    const T* dinv = reinterpret_cast<const T*>(sm + L.o_val);
-    const T* val = reinterpret_cast<const T*>(sm + L.o_val + L.v_val);
-    const uint16_t* col = reinterpret_cast<const uint16_t*>(img + L.i_col);
-    const int C = L.ncolor, tpr = L.tpr, lg = L.lg_tpr;
+    const int C = L.ncolor, tpr = L.tpr, lg = L.lg_tpr, ri = lane >> lg;
+    const bool first_part = (lane & (tpr - 1)) == 0, streamed = L.streamed;
+    const uint32_t a_img = sm0 + (uint32_t)L.o_img, a_x = sm0 + (uint32_t)L.o_x, a_bd = sm0 + (uint32_t)L.o_val;
+    const uint32_t a_cr = a_img + (uint32_t)L.i_cr, a_xd = a_img + (uint32_t)L.i_xd;
+    const uint32_t a_sl = a_img + (uint32_t)L.i_sl + 16u * (uint32_t)warp;
+    uint32_t a_ent = a_bd + (uint32_t)L.v_ent + 16u * (uint32_t)lane;
+    if (q0 >= nq) return;
     int k = q0 % C;
-    for (int q = q0; q < nq; ++q) {
-      const int kc = descending ? C - 1 - k : k;
-      if (++k == C) k = 0;
-      if (L.streamed) {
-        const char* buf = sm + D.o_buf + (j % NS) * D.stage_bytes;
-        val = reinterpret_cast<const T*>(buf);
-        col = reinterpret_cast<const uint16_t*>(buf + D.stage_col);
-        mbar_wait(mst + j % NS, (unsigned)(j / NS) & 1u, D.err);
+    uint4 cr = lds4(a_cr + 16u * (uint32_t)(descending ? C - 1 - k : k)), d = make_uint4(0, 0, 0, 0);
+    if (warp < (int)cr.y) d = lds4(a_sl + 16u * cr.x);
+#pragma unroll 1
+    for (int q = q0;;) {
+      if (streamed) {
+        a_ent = sm0 + (uint32_t)(D.o_buf + jst * D.stage_bytes) + 16u * (uint32_t)lane;
+        mbar_wait(mst + 8u * (uint32_t)jst, jpar, D.err, polls);
       }
-      const int s1 = csl[kc + 1];
-      int s = csl[kc] + warp;
-      RowPre<T> p;
-      const bool any = s < s1;
-      T bv = 0;
-      if (any) {
-        load_row_pre<T>(p, sl, s, lane, tpr, lg, val, col, dinv, xp);
-        if (b_ready && p.lead) bv = b[p.row];
-      }
-      if (pending) cl_wait();
-      if (L.streamed) {
-        issue(j + NS - 1);  // every warp has finished step j - 1
-        ++j;
-      }
-      if (any) {
-        if (!b_ready && p.lead) bv = b[p.row];
-        for (;;) {
-          const T acc = row_sum<T>(p, val, col, x, tpr);
-          if (p.lead) {
-            const T xn = (bv - acc) * p.d;
-            x[p.row] = xn;
-            push<T>(x, p.list, xd, xn);
-          }
-          s += kClWarps;
-          if (s >= s1) break;
-          load_row_pre<T>(p, sl, s, lane, tpr, lg, val, col, dinv, xp);
-          if (p.lead) bv = b[p.row];
+      uint4 ncr = cr, nd = d;
+      bool waited = false;
+#pragma unroll 1
+      for (int si = warp;;) {
+        const bool any = si < (int)cr.y;
+        const int row0 = (int)(d.x & 0xFFFFu), row = row0 + ri, np = (int)(d.w & 1023u);
+        const uint32_t ea = a_ent + 16u * d.z, a_row = a_bd + 2u * (uint32_t)sizeof(T) * (uint32_t)row;
+        uint4 u[4];
+        T bv, dv;
+        uint32_t pa = 0, pm = 0;  // this lane's first halo store: where to, which barrier, which lane has the value
+        int src = 0;
+        if (any) {
+          load_units(u, ea);
+          lds_pair(a_row, bv, dv);
+          int e;  // lanes past the list: not sent
+          lds1(a_xd + 4u * ((d.w >> 10) + (uint32_t)lane), e);
+          const uint32_t a = a_x + store_there(e) * (uint32_t)sizeof(T);
+          pa = cl_map(a, lane < np ? store_cta(e) : 0u);
+          pm = pa + (mcur() - a);  // the same CTA's window
+          src = (((int)store_row(e) - row0) << lg) & 31;
         }
+        if (!waited) {
+          waited = true;
+          if (++k == C) k = 0;
+          if (q + 1 < nq) {
+            ncr = lds4(a_cr + 16u * (uint32_t)(descending ? C - 1 - k : k));
+            if (warp < (int)ncr.y) nd = lds4(a_sl + 16u * ncr.x);
+          }
+          begin();
+          if (streamed) {
+            issue();  // every warp has finished the step before
+            stage_used();
+          }
+          if (!b_ready && any) lds_pair(a_row, bv, dv);
+          b_ready = true;
+        }
+        if (any) {
+          const T xn = (bv - row_sum<T>(u, ea, (int)d.y, sm0, tpr)) * dv;
+          sts_if(first_part && ri < (int)(d.x >> 16), a_x + (uint32_t)sizeof(T) * (uint32_t)row, xn);
+          if (np) {  // the slice's halo stores, one per lane
+            cl_send_if(lane < np, pa, pm, __shfl_sync(0xffffffffu, xn, src));
+            if (np > 32) {
+              __syncwarp();
+              push_list<T>(a_xd, (int)(d.w >> 10) + 32 + lane, (int)(d.w >> 10) + np, 32, a_x, mcur());
+            }
+          }
+        }
+        si += kClWarps;
+        if (si >= (int)cr.y) break;
+        d = lds4(a_sl + 16u * (cr.x + (uint32_t)(si - warp)));
       }
-      cl_arrive();
-      pending = true;
-      b_ready = true;
+      end((int)cr.z);
+      cr = ncr;
+      d = nd;
+      if (++q >= nq) break;
     }
   };
 
-  T* r = reinterpret_cast<T*>(sm + D.o_r);
-  T* bc = reinterpret_cast<T*>(sm + D.o_bc);
-  for (int t = 0; t < NL; ++t) {
+  const uint32_t a_bc = sm0 + (uint32_t)D.o_bc;
+  // down the levels, and up again: one loop, so that the code of the sweeps
+  // is there once
+#pragma unroll 1
+  for (int h = 0; h < 2 * NL; ++h) {
+    const bool down = h < NL;
+    const int t = down ? h : 2 * NL - 1 - h;
+    if (h == NL) {
+      // coarsest: x_c = A^-1 b_c, a warp per kC own rows at a time, the first
+      // rows' coefficients loaded before the wait (they come from L2, so many have
+      // to be in flight)
+      {
+        const ClusterLevel<T>& L = D.lv[NL];
+        char* img = sm + L.o_img;
+        const int nown = reinterpret_cast<const int*>(img)[0], nxd = reinterpret_cast<const int*>(img)[9];
+        const int* gid = reinterpret_cast<const int*>(img + L.i_cr);
+        const int bytes = *reinterpret_cast<const int*>(img + L.i_ex);
+        const uint32_t a_xd = sm0 + (uint32_t)(L.o_img + L.i_xd), a_x = sm0 + (uint32_t)L.o_x;
+        constexpr int kC = sizeof(T) == 4 ? 4 : 1, kA = 24;
+        const int n = D.nc;
+        T a[kC][kA];
+        auto coefs = [&](int i) {
+#pragma unroll
+          for (int c = 0; c < kC; ++c) {
+            const T* ar = D.ainv + (int64_t)gid[i + c < nown ? i + c : i] * n;
+#pragma unroll
+            for (int q = 0; q < kA; ++q) a[c][q] = lane + 32 * q < n ? ar[lane + 32 * q] : T(0);
+          }
+        };
+        int i = warp * kC;
+        if (i < nown) coefs(i);
+        begin();
+        mbar_wait(mbc, 0u, D.err, polls);
+#pragma unroll 1
+        while (i < nown) {
+          T acc[kC];
+#pragma unroll
+          for (int c = 0; c < kC; ++c) acc[c] = 0;
+#pragma unroll
+          for (int q = 0; q < kA; ++q) {
+            T bv = 0;
+            if (lane + 32 * q < n) lds1(a_bc + (uint32_t)sizeof(T) * (uint32_t)(lane + 32 * q), bv);
+#pragma unroll
+            for (int c = 0; c < kC; ++c) acc[c] += a[c][q] * bv;
+          }
+          if (n > 32 * kA)
+#pragma unroll 1
+            for (int c = 0; c < kC; ++c) {
+              const T* ar = D.ainv + (int64_t)gid[i + c < nown ? i + c : i] * n;
+              T t = 0;
+#pragma unroll 4
+              for (int q = lane + 32 * kA; q < n; q += 32) {
+                T bv;
+                lds1(a_bc + (uint32_t)sizeof(T) * (uint32_t)q, bv);
+                t += ar[q] * bv;
+              }
+              acc[c] += t;
+            }
+          const int cur = i;
+          i += kClWarps * kC;
+          if (i < nown) coefs(i);
+#pragma unroll
+          for (int c = 0; c < kC; ++c) {
+#pragma unroll 1
+            for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+            if (lane == c && cur + c < nown) sts(a_x + (uint32_t)sizeof(T) * (uint32_t)(cur + c), acc[c]);
+          }
+        }
+        __syncthreads();
+        push_list<T>(a_xd, tid, nxd, kClThreads, a_x, mcur());
+        end(bytes);
+      }
+    }
+    if (!down) {  // prolongation
+      const ClusterLevel<T>& L = D.lv[t];
+      char* img = sm + L.o_img;
+      const int* hd = reinterpret_cast<const int*>(img);
+      // halo stores [lo, hi) are of rows that the post-smoothing updates first
+      const int nown = hd[0], lo = hd[5], hi = hd[6], nxd = hd[9];
+      const int bytes = reinterpret_cast<const int*>(img + L.i_ex)[2];
+      const uint32_t a_xd = sm0 + (uint32_t)(L.o_img + L.i_xd), a_x = sm0 + (uint32_t)L.o_x;
+      const uint32_t a_u = sm0 + (uint32_t)D.lv[t + 1].o_x;
+      const int64_t p0 = (int64_t)cta * 3 * L.n_own_max;
+      constexpr int kP = 4;
+      int id[kP][3];
+      T w[kP][3];
+      auto weights = [&](int i0) {
+#pragma unroll
+        for (int k = 0; k < kP; ++k) {
+          const int i = i0 + k * kClThreads < nown ? i0 + k * kClThreads : 0;
+#pragma unroll
+          for (int m = 0; m < 3; ++m) {
+            id[k][m] = L.p_idx[p0 + m * L.n_own_max + i];
+            w[k][m] = L.p_w[p0 + m * L.n_own_max + i];
+          }
+        }
+      };
+      weights(tid);
+      begin();
+#pragma unroll 1
+      for (int i0 = tid; i0 < nown; i0 += kP * kClThreads) {
+        if (i0 != tid) weights(i0);
+#pragma unroll
+        for (int k = 0; k < kP; ++k) {
+          const int i = i0 + k * kClThreads;
+          if (i < nown) {
+            T v, u[3];
+            lds1(a_x + (uint32_t)sizeof(T) * (uint32_t)i, v);
+#pragma unroll
+            for (int m = 0; m < 3; ++m) lds1(a_u + (uint32_t)sizeof(T) * (uint32_t)id[k][m], u[m]);
+            v += w[k][0] * u[0] + w[k][1] * u[1] + w[k][2] * u[2];
+            sts(a_x + (uint32_t)sizeof(T) * (uint32_t)i, v);
+          }
+        }
+      }
+      __syncthreads();
+      push_list<T>(a_xd, tid, lo, kClThreads, a_x, mcur());
+      push_list<T>(a_xd, hi + tid, nxd, kClThreads, a_x, mcur());
+      end(bytes);
+    }
+    const bool first_done = down && (t == 0 ? c0_first != 0 : D.nu_pre > 0);
+    sweeps(t, first_done ? 1 : 0, (down ? D.nu_pre : D.nu_post) * D.lv[t].ncolor, !down && !D.post_forward,
+           t == 0 || !down);
+    if (!down) continue;
     const ClusterLevel<T>& L = D.lv[t];
     const ClusterLevel<T>& N = D.lv[t + 1];
     char* img = sm + L.o_img;
     const int* hd = reinterpret_cast<const int*>(img);
+    const int* ex = reinterpret_cast<const int*>(img + L.i_ex);  // residual, restriction, prolongation
     const int C = L.ncolor;
-    const bool first_done = t == 0 ? c0_first != 0 : D.nu_pre > 0;
-    sweeps(t, first_done ? 1 : 0, D.nu_pre * C, false, false);
-    // residual of the own rows, stored into the CTAs that restrict it
+    // the residual's buffer alternates between the levels: without
+    // pre-smoothing a level's residual follows the finer one's restriction
+    const uint32_t a_r = sm0 + (uint32_t)D.o_r[t & 1];
+    // residual of the own rows, sent to the CTAs that restrict it
     {
-      const int4* sl = reinterpret_cast<const int4*>(img + L.i_sl);
-      const int* csl = reinterpret_cast<const int*>(img + L.i_csl);
-      const uint32_t* rp = reinterpret_cast<const uint32_t*>(img + L.i_rp);
-      const uint32_t* rd = reinterpret_cast<const uint32_t*>(img + L.i_rd);
-      const T* x = reinterpret_cast<const T*>(sm + L.o_x);
-      const T* b = reinterpret_cast<const T*>(sm + L.o_b);
-      const T* val = reinterpret_cast<const T*>(sm + L.o_val + L.v_val);
-      const uint16_t* col = reinterpret_cast<const uint16_t*>(img + L.i_col);
-      const T* dg = L.diag + (int64_t)cta * L.n_own_max;
-      RowPre<T> p;
-      auto load = [&](int s) { load_row_pre<T>(p, sl, s, lane, L.tpr, L.lg_tpr, val, col, dg, rp); };
-      auto rows = [&](int s, int se) {  // slices s, s + kClWarps, ..., the first one loaded
-        while (s < se) {
-          const T acc = row_sum<T>(p, val, col, x, L.tpr);
-          if (p.lead) {
-            const T rv = b[p.row] - (acc + p.d * x[p.row]);
-            r[p.row] = rv;
-            push<T>(r, p.list, rd, rv);
-          }
-          s += kClWarps;
-          if (s < se) load(s);
-        }
+      const uint32_t a_sl = sm0 + (uint32_t)(L.o_img + L.i_sl);
+      const int4* cr = reinterpret_cast<const int4*>(img + L.i_cr);
+      const uint32_t a_x = sm0 + (uint32_t)L.o_x, a_bd = sm0 + (uint32_t)L.o_val, a_dg = a_bd + (uint32_t)L.v_diag;
+      const int tpr = L.tpr, ri = lane >> L.lg_tpr;
+      uint32_t a_ent = sm0 + (uint32_t)(L.o_val + L.v_ent) + 16u * (uint32_t)lane;
+      uint4 d = make_uint4(0, 0, 0, 0), u[4];
+      auto load = [&](uint4& dd, uint4 (&uu)[4], int s) {
+        dd = lds4(a_sl + 16u * (uint32_t)s);
+        load_units(uu, a_ent + 16u * dd.z);
       };
-      if (!L.streamed && warp < hd[2]) load(warp);
-      if (pending) cl_wait();
+      auto row = [&]() {
+        const T acc = row_sum<T>(u, a_ent + 16u * d.z, (int)d.y, sm0, tpr);
+        const uint32_t o = (uint32_t)sizeof(T) * (uint32_t)((int)(d.x & 0xFFFFu) + ri);
+        T bv, dg, xv;
+        lds1(a_bd + 2u * o, bv);
+        lds1(a_dg + o, dg);
+        lds1(a_x + o, xv);
+        sts_if((lane & (tpr - 1)) == 0 && ri < (int)(d.x >> 16), a_r + o, bv - (acc + dg * xv));
+      };
       if (!L.streamed) {
-        rows(warp, hd[2]);
+        int s = warp;
+        const int se = hd[2];
+        if (s < se) load(d, u, s);
+        begin();
+#pragma unroll 1
+        while (s < se) {
+          uint4 dn = d, un[4] = {u[0], u[1], u[2], u[3]};
+          s += kClWarps;
+          if (s < se) load(dn, un, s);
+          row();
+          d = dn;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) u[q] = un[q];
+        }
+        __syncthreads();
       } else {
-        for (int k = 0; k < C; ++k) {
-          const char* buf = sm + D.o_buf + (j % NS) * D.stage_bytes;
-          val = reinterpret_cast<const T*>(buf);
-          col = reinterpret_cast<const uint16_t*>(buf + D.stage_col);
-          issue(j + NS - 1);
-          mbar_wait(mst + j % NS, (unsigned)(j / NS) & 1u, D.err);
-          if (csl[k] + warp < csl[k + 1]) load(csl[k] + warp);
-          rows(csl[k] + warp, csl[k + 1]);
-          ++j;
+        // as many colours at a time as stages hold (the colours' slices follow one another)
+        begin();
+        issue();
+#pragma unroll 1
+        for (int k = 0; k < C;) {
+          const int nk = C - k < NS ? C - k : NS;
+#pragma unroll 1
+          for (int q = 0, st = jst, par = (int)jpar; q < nk; ++q) {
+            mbar_wait(mst + 8u * (uint32_t)st, (unsigned)par, D.err, polls);
+            if (++st == NS) {
+              st = 0;
+              par ^= 1;
+            }
+          }
+          const int se = cr[k + nk - 1].x + cr[k + nk - 1].y;
+#pragma unroll 1
+          for (int s = cr[k].x + warp, q = 0; s < se; s += kClWarps) {
+#pragma unroll 1
+            while (s >= cr[k + q].x + cr[k + q].y) ++q;
+            const int st = jst + q < NS ? jst + q : jst + q - NS;
+            a_ent = sm0 + (uint32_t)(D.o_buf + st * D.stage_bytes) + 16u * (uint32_t)lane;
+            load(d, u, s);
+            row();
+          }
           __syncthreads();
+          // the stages of this group may be filled again; one issue stays for
+          // the next user of the stream, which makes one when it begins
+#pragma unroll 1
+          for (int q = 0; q < nk; ++q) {
+            stage_used();
+            if (k + nk < C || q + 1 < nk) issue();
+          }
+          k += nk;
         }
       }
-      cl_arrive();
+      push_list<T>(sm0 + (uint32_t)(L.o_img + L.i_rd), tid, hd[11], kClThreads, a_r, mcur());
+      end(ex[0]);
     }
     // restriction b_{l+1} = P^T r over the own coarse rows; x_{l+1} is zero,
     // but the rows of colour 0 of a smoothed level take their first update
@@ -385,15 +728,8 @@ __global__ void __launch_bounds__(kClThreads, 1)
     {
       const int4* rs = L.r_sl + (int64_t)cta * L.rsl_max;
       const int nrs = hd[3], tpr = L.r_tpr, lg = L.lg_r_tpr;
-      mbar_wait(mimg + t + 1, 0u, D.err);
-      char* nimg = sm + N.o_img;
-      const int nc0 = D.nu_pre > 0 && t + 1 < NL ? reinterpret_cast<const int*>(nimg)[4] : 0;
-      const uint32_t* xp = reinterpret_cast<const uint32_t*>(nimg + N.i_xp);
-      const uint32_t* xd = reinterpret_cast<const uint32_t*>(nimg + N.i_xd);
-      const int* gid = reinterpret_cast<const int*>(nimg + N.i_csl);  // coarsest level: global rows of the own rows
-      T* xn = reinterpret_cast<T*>(sm + N.o_x);
-      T* bn = reinterpret_cast<T*>(sm + N.o_b);
-      const T* dn = reinterpret_cast<const T*>(sm + N.o_val);
+      const uint16_t* rcol = L.r_col + (int64_t)cta * L.r_max;
+      const T* rw = L.r_w + (int64_t)cta * L.r_max;
       constexpr int kR = 16;
       T wv[kR];
       int ci[kR];
@@ -402,8 +738,8 @@ __global__ void __launch_bounds__(kClThreads, 1)
       auto terms = [&](int q0) {
 #pragma unroll
         for (int q = 0; q < kR; ++q) {
-          wv[q] = q0 + q < w ? L.r_w[e + (q0 + q) * 32] : T(0);
-          ci[q] = q0 + q < w ? L.r_col[e + (q0 + q) * 32] : 0;
+          wv[q] = q0 + q < w ? rw[e + (q0 + q) * 32] : T(0);
+          ci[q] = q0 + q < w ? rcol[e + (q0 + q) * 32] : 0;
         }
       };
       auto start = [&](int s) {
@@ -418,141 +754,82 @@ __global__ void __launch_bounds__(kClThreads, 1)
       };
       int s = warp;
       if (s < nrs) start(s);
-      cl_wait();
+      mbar_wait(mimg + 8u * (t + 1), 0u, D.err, polls);
+      char* nimg = sm + N.o_img;
+      const bool first_upd = D.nu_pre > 0 && t + 1 < NL;
+      const int nc0 = first_upd ? reinterpret_cast<const int*>(nimg)[4] : 0;
+      const uint32_t a_gid = sm0 + (uint32_t)(N.o_img + N.i_cr);  // coarsest level: global rows of the own rows
+      const uint32_t a_xn = sm0 + (uint32_t)N.o_x, a_bdn = sm0 + (uint32_t)N.o_val;
+      begin();
+#pragma unroll 1
       for (; s < nrs;) {
         T acc = 0;
+#pragma unroll 1
         for (int q0 = 0; q0 < w; q0 += kR) {
           T rv[kR];
 #pragma unroll
-          for (int q = 0; q < kR; ++q) rv[q] = r[ci[q]];
+          for (int q = 0; q < kR; ++q) lds1(a_r + (uint32_t)sizeof(T) * (uint32_t)ci[q], rv[q]);
 #pragma unroll
           for (int q = 0; q < kR; ++q)
             if (q0 + q < w) acc += wv[q] * rv[q];
           if (q0 + kR < w) terms(q0 + kR);
         }
+#pragma unroll 1
         for (int o = 1; o < tpr; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lead) {
-          if (t + 1 < NL) {
-            bn[row] = acc;
+        if (t + 1 < NL) {
+          if (lead) {
+            const uint32_t o = (uint32_t)sizeof(T) * (uint32_t)row;
+            sts(a_bdn + 2u * o, acc);
             if (row < nc0) {
-              const T v = (acc - T(0)) * dn[row];
-              xn[row] = v;
-              push<T>(xn, xp[row], xd, v);
+              T dv;
+              lds1(a_bdn + 2u * o + (uint32_t)sizeof(T), dv);
+              sts(a_xn + o, (acc - T(0)) * dv);
             }
-          } else {
-            for (int c = 0; c < D.ncta; ++c) cl_store(bc + gid[row], (unsigned)c, acc);
+          }
+        } else if (lead) {  // the coarsest right-hand side goes to every CTA
+          int gr;
+          lds1(a_gid + 4u * (uint32_t)row, gr);
+          const uint32_t a = a_bc + (uint32_t)sizeof(T) * (uint32_t)gr;
+          sts(a, acc);
+#pragma unroll 1
+          for (int c = 1; c < D.ncta; ++c) {
+            const uint32_t to = cl_map(a, (unsigned)(cta + c >= D.ncta ? cta + c - D.ncta : cta + c));
+            cl_send(to, to + (mbc - a), acc);
           }
         }
         s += kClWarps;
         if (s < nrs) start(s);
       }
-      cl_arrive();
-      pending = true;
+      if (first_upd) {
+        __syncthreads();
+        push_list<T>(sm0 + (uint32_t)(N.o_img + N.i_xd), tid, reinterpret_cast<const int*>(nimg)[10], kClThreads, a_xn, mcur());
+      }
+      end(ex[1]);
     }
   }
-  // coarsest: x_c = A^-1 b_c, one warp per own row, the first row's
-  // coefficients loaded before the wait
+  __syncthreads();
+  if (ph > 0) mbar_wait(mph + 8u * (uint32_t)((ph - 1) & 1), (unsigned)((ph - 1) >> 1) & 1u, D.err, polls);
   {
-    const ClusterLevel<T>& L = D.lv[NL];
-    char* img = sm + L.o_img;
-    const int nown = reinterpret_cast<const int*>(img)[0];
-    const int* gid = reinterpret_cast<const int*>(img + L.i_csl);
-    const uint32_t* xp = reinterpret_cast<const uint32_t*>(img + L.i_xp);
-    const uint32_t* xd = reinterpret_cast<const uint32_t*>(img + L.i_xd);
-    T* x = reinterpret_cast<T*>(sm + L.o_x);
-    constexpr int kA = sizeof(T) == 4 ? 24 : 12;
-    const int n = D.nc;
-    T a[kA];
-    auto coefs = [&](int i) {
-      const T* ar = D.ainv + (int64_t)gid[i] * n;
-#pragma unroll
-      for (int q = 0; q < kA; ++q) a[q] = lane + 32 * q < n ? ar[lane + 32 * q] : T(0);
-    };
-    int i = warp;
-    if (i < nown) coefs(i);
-    cl_wait();
-    while (i < nown) {
-      T acc = 0;
-#pragma unroll
-      for (int q = 0; q < kA; ++q)
-        if (lane + 32 * q < n) acc += a[q] * bc[lane + 32 * q];
-      const T* ar = D.ainv + (int64_t)gid[i] * n;
-      for (int q = lane + 32 * kA; q < n; q += 32) acc += ar[q] * bc[q];
-      const int cur = i;
-      i += kClWarps;
-      if (i < nown) coefs(i);
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0) {
-        x[cur] = acc;
-        push<T>(x, xp[cur], xd, acc);
-      }
-    }
-    cl_arrive();
-    pending = true;
+    const T* x = reinterpret_cast<const T*>(sm + D.lv[0].o_x);
+#pragma unroll 1
+    for (int i = tid; i < n0own; i += kClThreads) xg[l2g[i]] = x[i];
   }
-  // up: prolongation and post-smoothing
-  for (int t = NL - 1; t >= 0; --t) {
-    const ClusterLevel<T>& L = D.lv[t];
-    char* img = sm + L.o_img;
-    const int nown = reinterpret_cast<const int*>(img)[0];
-    const uint32_t* xp = reinterpret_cast<const uint32_t*>(img + L.i_xp);
-    const uint32_t* xd = reinterpret_cast<const uint32_t*>(img + L.i_xd);
-    T* x = reinterpret_cast<T*>(sm + L.o_x);
-    const T* u = reinterpret_cast<const T*>(sm + D.lv[t + 1].o_x);
-    const int64_t p0 = (int64_t)cta * 3 * L.n_own_max;
-    constexpr int kP = 4;
-    int id[kP][3];
-    T w[kP][3];
-    auto weights = [&](int i0) {
-#pragma unroll
-      for (int k = 0; k < kP; ++k) {
-        const int i = i0 + k * kClThreads < nown ? i0 + k * kClThreads : 0;
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-          id[k][m] = L.p_idx[p0 + m * L.n_own_max + i];
-          w[k][m] = L.p_w[p0 + m * L.n_own_max + i];
-        }
-      }
-    };
-    weights(tid);
-    cl_wait();
-    for (int i0 = tid; i0 < nown; i0 += kP * kClThreads) {
-      if (i0 != tid) weights(i0);
-#pragma unroll
-      for (int k = 0; k < kP; ++k) {
-        const int i = i0 + k * kClThreads;
-        if (i < nown) {
-          T v = x[i];
-          v += w[k][0] * u[id[k][0]] + w[k][1] * u[id[k][1]] + w[k][2] * u[id[k][2]];
-          x[i] = v;
-          push<T>(x, xp[i], xd, v);
-        }
-      }
-    }
-    cl_arrive();
-    pending = true;
-    sweeps(t, 0, D.nu_post * L.ncolor, !D.post_forward, true);
-  }
-  if (pending) cl_wait();
-  {
-    const ClusterLevel<T>& L = D.lv[0];
-    const int nown = reinterpret_cast<const int*>(sm + L.o_img)[0];
-    const T* x = reinterpret_cast<const T*>(sm + L.o_x);
-    const int32_t* l2g = D.l2g + (int64_t)cta * L.n_loc_max;
-    for (int i = tid; i < nown; i += kClThreads) xg[l2g[i]] = x[i];
-  }
+  cl_arrive();  // no CTA's shared memory goes before every message has landed
+  cl_wait();
 }
 
-// out[e] of every job: the level's value in slot src[e] >= 0, 0 for -1, or
-// vector element -2 - src[e] (1/a_ii or a_ii) below.
+// Element e of a job is the level's value in slot src[e] >= 0, 0 for -1, or
+// vector element -2 - src[e] (1/a_ii or a_ii) below; it goes to byte
+// (e / per) * cta_bytes + (e % per) * step of out.
 template <class T>
 struct RefreshJobs {
   int njob = 0;
   struct Job {
-    int64_t n;
+    int64_t n, per, cta_bytes;
+    int step;
     const int32_t* src;
     const T *val, *vec;
-    T* out;
+    char* out;
   } job[3 * kClMaxLevels];
 };
 template <class T>
@@ -560,7 +837,8 @@ __global__ void k_cluster_values(const __grid_constant__ RefreshJobs<T> J) {
   const auto& q = J.job[blockIdx.y];
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < q.n; e += (int64_t)gridDim.x * blockDim.x) {
     const int32_t s = q.src[e];
-    q.out[e] = s >= 0 ? q.val[s] : s == -1 ? T(0) : q.vec[-2 - s];
+    const T v = s >= 0 ? q.val[s] : s == -1 ? T(0) : q.vec[-2 - s];
+    *reinterpret_cast<T*>(q.out + (e / q.per) * q.cta_bytes + (e % q.per) * q.step) = v;
   }
 }
 
@@ -614,13 +892,14 @@ struct Part {
   std::vector<int32_t> own, halo, rhalo;  // permuted rows
   std::vector<Slice> sl, rsl;
   std::vector<int32_t> csl, blk;  // per colour: first slice, first entry (+ end)
-  std::vector<uint16_t> ecol, rcol;
+  std::vector<uint16_t> ecol, rcol;  // per entry slot: unit u, lane q, slot v of the unit at (32 u + q) per + v
   std::vector<int32_t> esrc;
   std::vector<double> rw;
   std::vector<uint32_t> xp, xd, rp, rd;  // halo stores of x and of the residual
   std::vector<uint16_t> pidx;            // 3 x own
   std::vector<double> pw;
-  int own0 = 0;  // own rows of colour 0
+  std::vector<int> hcol, rows0;          // per colour: halo rows, first own row (+ end)
+  int own0 = 0;                          // own rows of colour 0
 };
 struct Tab {
   int64_t n = 0;
@@ -628,7 +907,8 @@ struct Tab {
   bool wide = false;
   std::vector<int32_t> owner, local;
   std::vector<Part> part;
-  int n_own = 0, n_loc = 0, n_r = 0, nsl = 0, nrsl = 0, nxd = 0, nrd = 0, blk = 0, ent = 0;  // largest over the CTAs
+  std::vector<std::vector<int32_t>> partners;  // level l0 only: the CTAs each CTA exchanges messages with
+  int n_own = 0, n_loc = 0, n_r = 0, nsl = 0, nrsl = 0, nxd = 0, nrd = 0, blk = 0, ent = 0, r_max = 0;  // largest over the CTAs (entries in units)
 };
 
 int lanes_per_row(double rows, double len) {
@@ -639,12 +919,13 @@ int lanes_per_row(double rows, double len) {
 
 // Slices of `rows` rows per slice from rows [0, n) of given lengths; emit(slice, first row, rows, width).
 template <class Len, class Emit>
-void cut_slices(int i0, int i1, int per, int tpr, Len len, Emit emit) {
+void cut_slices(int i0, int i1, int per, int tpr, int per_unit, bool pairs, Len len, Emit emit) {
   for (int a = i0; a < i1; a += per) {
     const int nr = std::min(per, i1 - a);
     int w = 0;
     for (int q = 0; q < nr; ++q) w = std::max(w, (len(a + q) + tpr - 1) / tpr);
-    emit(a, nr, w);
+    w = (w + per_unit - 1) / per_unit;
+    emit(a, nr, pairs ? std::max(2, (w + 1) & ~1) : w);
   }
 }
 
@@ -678,8 +959,8 @@ void push_lists(const std::vector<int32_t>& owner, const std::vector<int32_t>& l
   }
 }
 
-// The tables of levels l0 .. lambda over ncta CTAs (host); false when a local index does not fit 16 bits.
-bool build_tables(gmg_ctx* c, int l0, int ncta, const std::vector<std::vector<int64_t>>& hrp,
+// The tables of levels l0 .. lambda over ncta CTAs (host); false when a CTA would hold too many rows.
+bool build_tables(gmg_ctx* c, int l0, int ncta, int per_unit, const std::vector<std::vector<int64_t>>& hrp,
                   const std::vector<std::vector<int32_t>>& hcol, const std::vector<std::vector<int32_t>>& perm,
                   const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P, std::vector<Tab>& tab) {
   const int lam = c->nlev - 1, nl = lam - l0;
@@ -729,7 +1010,7 @@ bool build_tables(gmg_ctx* c, int l0, int ncta, const std::vector<std::vector<in
             if (P[l - 1].w[3 * old + s] != 0.0) see(ip[P[l - 1].idx[3 * old + s]]);
         }
       std::sort(p.halo.begin(), p.halo.end());
-      if (p.own.size() + p.halo.size() > 65535) return false;
+      if ((int)(p.own.size() + p.halo.size()) >= kClMaxLocal) return false;
       for (size_t q = 0; q < p.halo.size(); ++q) loc[p.halo[q]] = (int32_t)(p.own.size() + q);
       auto at = [&](int32_t r) { return T.owner[r] == a ? T.local[r] : loc[r]; };
       if (t > 0) {  // prolongation slots of the finer level's own rows
@@ -753,36 +1034,49 @@ bool build_tables(gmg_ctx* c, int l0, int ncta, const std::vector<std::vector<in
         int i0 = 0;
         for (int k = 0; k < T.ncolor; ++k) {
           p.csl.push_back((int32_t)p.sl.size());
-          p.blk.push_back((int32_t)p.ecol.size());
+          p.blk.push_back((int32_t)(p.ecol.size() / per_unit));
+          p.rows0.push_back(i0);
           int i1 = i0;
           while (i1 < (int)p.own.size() && p.own[i1] < L.color_off[k + 1]) ++i1;
-          cut_slices(i0, i1, per, T.tpr, len, [&](int r0, int nr, int w) {
-            const size_t base = p.ecol.size();
-            p.sl.push_back({r0 | (nr << 16), w, (int32_t)base, 0});
-            p.ecol.resize(base + 32 * (size_t)w);
-            p.esrc.resize(base + 32 * (size_t)w, -1);
+          cut_slices(i0, i1, per, T.tpr, per_unit, true, len, [&](int r0, int nr, int w) {
+            const size_t base = p.ecol.size();  // entry slots before this slice
+            p.sl.push_back({r0 | (nr << 16), w, (int32_t)(base / per_unit), 0});
+            p.ecol.resize(base + 32 * (size_t)w * per_unit, 0);
+            p.esrc.resize(base + 32 * (size_t)w * per_unit, -1);
             for (int q = 0; q < nr; ++q) {
               const int32_t r = p.own[r0 + q];
               const int64_t old = pm[r];
               const int64_t slice = L.color_slice_off[k] + (r - L.color_off[k]) / kSlice;
-              const int64_t slot = L.h_ptr[slice] + (r - L.color_off[k]) % kSlice;
-              for (int m = 0; m < T.tpr * w; ++m)  // padding: the row itself, value 0
-                p.ecol[base + 32 * (size_t)(m / T.tpr) + q * T.tpr + m % T.tpr] = (uint16_t)(r0 + q);
+              int64_t slot = L.h_ptr[slice] + (r - L.color_off[k]) % kSlice;
+              // entry m of the row: lane part m mod tpr, unit (m / tpr) / per_unit, slot (m / tpr) % per_unit
+              auto at_slot = [&](int m) {
+                const int u = m / T.tpr;
+                return base + (32 * (size_t)(u / per_unit) + q * T.tpr + m % T.tpr) * per_unit + u % per_unit;
+              };
               int m = 0;
               for (int64_t e = rp[old]; e < rp[old + 1]; ++e) {
                 if (ci[e] == old) continue;
-                const size_t g = base + 32 * (size_t)(m / T.tpr) + q * T.tpr + m % T.tpr;
+                const size_t g = at_slot(m);
                 p.ecol[g] = (uint16_t)at(ip[ci[e]]);
-                p.esrc[g] = (int32_t)(slot + (int64_t)m * kSlice);
+                p.esrc[g] = (int32_t)slot;
+                slot += kSlice;
                 ++m;
               }
+              for (; m < T.tpr * w * per_unit; ++m) p.ecol[at_slot(m)] = (uint16_t)(r0 + q);  // padding: itself, value 0
             }
           });
           i0 = i1;
-          T.blk = std::max(T.blk, (int)p.ecol.size() - p.blk.back());
+          T.blk = std::max(T.blk, (int)(p.ecol.size() / per_unit) - p.blk.back());
         }
         p.csl.push_back((int32_t)p.sl.size());
-        p.blk.push_back((int32_t)p.ecol.size());
+        p.blk.push_back((int32_t)(p.ecol.size() / per_unit));
+        p.rows0.push_back(i0);
+        p.hcol.assign(T.ncolor, 0);
+        int k = 0;
+        for (int32_t r : p.halo) {  // ascending: colour by colour
+          while (r >= L.color_off[k + 1]) ++k;
+          p.hcol[k]++;
+        }
       }
     }
     push_lists(T.owner, T.local, T.part, false);
@@ -825,10 +1119,10 @@ bool build_tables(gmg_ctx* c, int l0, int ncta, const std::vector<std::vector<in
             f.rhalo.push_back(tcol[q]);
           }
       std::sort(f.rhalo.begin(), f.rhalo.end());
-      if (f.own.size() + f.rhalo.size() > 65535) return false;
+      if ((int)(f.own.size() + f.rhalo.size()) >= kClMaxLocal) return false;
       for (size_t q = 0; q < f.rhalo.size(); ++q) loc[f.rhalo[q]] = (int32_t)(f.own.size() + q);
       auto len = [&](int i) { return (int)(cnt[n.own[i] + 1] - cnt[n.own[i]]); };
-      cut_slices(0, (int)n.own.size(), 32 / F.r_tpr, F.r_tpr, len, [&](int r0, int nr, int w) {
+      cut_slices(0, (int)n.own.size(), 32 / F.r_tpr, F.r_tpr, 1, false, len, [&](int r0, int nr, int w) {
         const size_t base = f.rcol.size();
         f.rsl.push_back({r0 | (nr << 16), w, (int32_t)base, 0});
         f.rcol.resize(base + 32 * (size_t)w, 0);
@@ -845,6 +1139,16 @@ bool build_tables(gmg_ctx* c, int l0, int ncta, const std::vector<std::vector<in
     }
     push_lists(F.owner, F.local, F.part, true);
   }
+  // partners: the CTAs that send a CTA values on some level, or that it sends to
+  std::vector<char> ex((size_t)ncta * ncta, 0);
+  for (int t = 0; t <= nl; ++t)
+    for (int a = 0; a < ncta; ++a)
+      for (const auto* h : {&tab[t].part[a].halo, &tab[t].part[a].rhalo})
+        for (int32_t r : *h) ex[a * ncta + tab[t].owner[r]] = ex[tab[t].owner[r] * ncta + a] = 1;
+  tab[0].partners.assign(ncta, {});
+  for (int a = 0; a < ncta; ++a)
+    for (int b = 0; b < ncta; ++b)
+      if (a != b && ex[a * ncta + b]) tab[0].partners[a].push_back(b);
   for (Tab& T : tab)
     for (Part& p : T.part) {
       T.n_own = std::max(T.n_own, (int)p.own.size());
@@ -854,14 +1158,15 @@ bool build_tables(gmg_ctx* c, int l0, int ncta, const std::vector<std::vector<in
       T.nrsl = std::max(T.nrsl, (int)p.rsl.size());
       T.nxd = std::max(T.nxd, (int)p.xd.size());
       T.nrd = std::max(T.nrd, (int)p.rd.size());
-      T.ent = std::max(T.ent, (int)p.ecol.size());
+      T.ent = std::max(T.ent, (int)(p.ecol.size() / per_unit));
+      T.r_max = std::max(T.r_max, (int)p.rcol.size());
     }
   return true;
 }
 
 // Every index the kernel uses: columns and halo stores in range, each halo
 // copy written by its row's owner exactly once, slices covering the rows.
-bool check_tables(const std::vector<Tab>& tab) {
+bool check_tables(const std::vector<Tab>& tab, int per_unit) {
   const int nl = (int)tab.size() - 1;
   for (int t = 0; t <= nl; ++t) {
     const Tab& T = tab[t];
@@ -894,7 +1199,7 @@ bool check_tables(const std::vector<Tab>& tab) {
         int covered = 0;
         for (const Slice& s : p.sl) {
           if ((s.x & 0xFFFF) != covered || (s.x >> 16) < 1 || (s.x >> 16) * T.tpr > 32 || s.z < 0 ||
-              (size_t)s.z + 32 * (size_t)s.y > p.ecol.size())
+              ((size_t)s.z + 32 * (size_t)s.y) * per_unit > p.ecol.size())
             return false;
           covered += s.x >> 16;
         }
@@ -920,15 +1225,6 @@ bool check_tables(const std::vector<Tab>& tab) {
   return true;
 }
 
-template <class T>
-gmg_status upload_vec(Arena& a, const T** d, const std::vector<T>& h) {
-  T* p;
-  GMG_TRY(a.alloc(&p, std::max<size_t>(h.size(), 1)));
-  if (!h.empty()) GMG_CK(cudaMemcpy(p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
-  *d = p;
-  return GMG_OK;
-}
-
 int64_t al16(int64_t v) { return (v + 15) & ~(int64_t)15; }
 
 // Shared-memory layout: resident levels' entries in shared memory where
@@ -938,6 +1234,8 @@ template <class T>
 bool lay_out(const std::vector<Tab>& tab, int nu_pre, int nu_post, ClusterDesc<T>& D) {
   const int nl = (int)tab.size() - 1;
   std::vector<char> streamed(nl, 0);
+  int npart = 0;
+  for (const auto& p : tab[0].partners) npart = std::max(npart, (int)p.size());
   for (;;) {
     int64_t cur = 0, blk = 0;
     int nsteps = 0;
@@ -946,11 +1244,11 @@ bool lay_out(const std::vector<Tab>& tab, int nu_pre, int nu_post, ClusterDesc<T
         nsteps += (nu_pre + 1 + nu_post) * tab[t].ncolor;  // an upper bound: a skipped first phase has no step
         blk = std::max<int64_t>(blk, tab[t].blk);
       }
-    D.stage_col = (int)al16(blk * sizeof(T));
-    D.stage_bytes = (int)(D.stage_col + al16(2 * blk));
+    D.stage_bytes = (int)(16 * blk);
     D.o_mbar = 0;
-    cur = al16(8 * (kClMaxLevels + 1 + kClStages));
-    int64_t nr = 1;
+    D.o_tok = (int)al16(8 * (kClMaxLevels + 1 + kClStages + 3));
+    cur = D.o_tok + 64;
+    int64_t nr[2] = {1, 1};
     for (int t = 0; t <= nl; ++t) {
       const Tab& A = tab[t];
       ClusterLevel<T>& L = D.lv[t];
@@ -964,51 +1262,57 @@ bool lay_out(const std::vector<Tab>& tab, int nu_pre, int nu_post, ClusterDesc<T
       L.n_own_max = std::max(1, A.n_own);
       L.n_loc_max = std::max(1, A.n_loc);
       L.rsl_max = std::max(1, A.nrsl);
-      // image: header, slices, colours (the coarsest level: global rows), halo stores, resident columns, steps
-      int64_t o = 32;
+      L.r_max = std::max(32, A.r_max);
+      // image: header, slices, colour records (the coarsest level: global rows), halo stores, steps, partners
+      int64_t o = 64;
+      L.i_ex = (int)o;
+      o += 16;
       L.i_sl = (int)o;
       o += 16 * (int64_t)A.nsl;
-      L.i_csl = (int)o;
-      o = al16(o + 4 * (int64_t)(t < nl ? A.ncolor + 1 : L.n_own_max));
-      L.i_xp = (int)o;
-      o = al16(o + 4 * (int64_t)L.n_own_max);
+      L.i_cr = (int)o;
+      o = al16(o + (t < nl ? 16 * (int64_t)A.ncolor : 4 * (int64_t)L.n_own_max));
       L.i_xd = (int)o;
       o = al16(o + 4 * (int64_t)A.nxd);
-      L.i_rp = (int)o;
-      if (t < nl) o = al16(o + 4 * (int64_t)L.n_own_max);
       L.i_rd = (int)o;
       if (t < nl) o = al16(o + 4 * (int64_t)A.nrd);
-      L.i_col = (int)o;
-      if (res) o = al16(o + 2 * (int64_t)A.ent);
       if (t == 0) {
+        D.i_partners = (int)o;
+        o = al16(o + 4 * (int64_t)npart);
         D.i_steps = (int)o;
         o = al16(o + 8 * (int64_t)nsteps);
       }
       L.img_bytes = (int)o;
-      L.v_val = (int)al16((int64_t)sizeof(T) * L.n_own_max);
-      L.val_bytes = t < nl ? (int)(L.v_val + (res ? al16((int64_t)sizeof(T) * A.ent) : 0)) : 0;
+      // values: pairs (b, 1/a_ii), a_ii, resident entries
+      L.v_diag = (int)al16(2 * (int64_t)sizeof(T) * L.n_own_max);
+      L.v_ent = (int)(L.v_diag + al16((int64_t)sizeof(T) * L.n_own_max));
+      const int64_t vb = t < nl ? L.v_ent + (res ? 16 * (int64_t)A.ent : 0) : 0;
+      if (vb > kSmemLimit || o > kSmemLimit) {
+        cur = kSmemLimit + 1;
+        break;
+      }
+      L.val_bytes = (int)vb;
       L.o_img = (int)cur;
       cur += L.img_bytes;
       L.o_val = (int)cur;
       cur += L.val_bytes;
       L.o_x = (int)cur;
       cur = al16(cur + (int64_t)sizeof(T) * L.n_loc_max);
-      L.o_b = (int)cur;
-      if (t < nl) cur = al16(cur + (int64_t)sizeof(T) * L.n_own_max);
-      if (t < nl) nr = std::max<int64_t>(nr, A.n_r);
-      if (cur > 4 * (int64_t)kSmemLimit) return false;
+      if (t < nl) nr[t & 1] = std::max<int64_t>(nr[t & 1], A.n_r);
     }
-    D.o_r = (int)cur;
-    cur = al16(cur + (int64_t)sizeof(T) * nr);
-    D.o_bc = (int)cur;
+    for (int q = 0; q < 2; ++q) {
+      D.o_r[q] = (int)std::min<int64_t>(cur, INT32_MAX);
+      cur = al16(cur + (int64_t)sizeof(T) * nr[q]);
+    }
+    D.o_bc = (int)std::min<int64_t>(cur, INT32_MAX);
     cur = al16(cur + (int64_t)sizeof(T) * tab[nl].n);
-    D.o_buf = (int)cur;
+    D.o_buf = (int)std::min<int64_t>(cur, INT32_MAX);
     D.nsteps = nsteps;
     const bool all = std::all_of(streamed.begin(), streamed.end(), [](char v) { return v != 0; });
-    const int need = blk == 0 ? 0 : all ? 2 : 3;
-    if (cur + (int64_t)need * D.stage_bytes <= kSmemLimit) {
-      D.nstage = blk == 0 ? 0 : (int)std::min<int64_t>(kClStages, (kSmemLimit - cur) / D.stage_bytes);
-      D.smem = (int)(cur + (int64_t)D.nstage * D.stage_bytes);
+    // a lane loads up to two units (1 KB of a warp) past its row's
+    const int64_t need = (blk == 0 ? 0 : (all ? 2 : 3) * 16 * blk) + kClSlack;
+    if (cur + need <= kSmemLimit) {
+      D.nstage = blk == 0 ? 0 : (int)std::min<int64_t>(kClStages, (kSmemLimit - kClSlack - cur) / D.stage_bytes);
+      D.smem = (int)(cur + (int64_t)D.nstage * D.stage_bytes + kClSlack);
       return true;
     }
     int big = -1;  // stream the largest level that does not stream yet
@@ -1032,27 +1336,68 @@ struct Src<double> {
   static ClusterDesc<double>& desc(gmg_ctx* c) { return c->cl64; }
 };
 
-// Uploads the tables of `tab` in the layout of D.
+// Device arrays of one handle's tables, gathered in one host buffer so that
+// they take one allocation and one copy.
+struct Blob {
+  std::vector<char> h;
+  std::vector<std::pair<const void**, size_t>> ptrs;
+  template <class U>
+  char* add(const U** d, size_t n) {  // n elements, zeroed; returns where to write them (valid until the next add)
+    const size_t o = (h.size() + 255) & ~(size_t)255;
+    h.resize(o + std::max<size_t>(n, 1) * sizeof(U));
+    ptrs.push_back({reinterpret_cast<const void**>(d), o});
+    return h.data() + o;
+  }
+  gmg_status upload(Arena& a) {
+    char* p;
+    GMG_TRY(a.alloc(&p, h.size()));
+    GMG_CK(cudaMemcpy(p, h.data(), h.size(), cudaMemcpyHostToDevice));
+    for (auto& q : ptrs) *q.first = p + q.second;
+    return GMG_OK;
+  }
+};
+
+// Entry units of one part: the x addresses (byte offsets into shared memory); the values come with every refresh.
+template <class T>
+void fill_units(const Part& p, int o_x, char* out) {
+  for (size_t e = 0; e < p.ecol.size(); ++e) {
+    const uint32_t off = (uint32_t)o_x + (uint32_t)sizeof(T) * p.ecol[e];
+    std::memcpy(out + (sizeof(T) == 4 ? 8 * e + 4 : 16 * e + 8), &off, 4);
+  }
+}
+
+// The first halo store of the rows from local row i on.
+int32_t first_store(const Part& p, int i) {
+  return i < (int)p.xp.size() ? (int32_t)(p.xp[i] >> 4) : (int32_t)p.xd.size();
+}
+
+// Lays the tables of `tab` out as D says and uploads them.
 template <class T>
 gmg_status upload_tables(gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>& D) {
-  Arena& a = c->arena;
+  constexpr int pu = sizeof(T) == 4 ? 2 : 1;  // entries per unit
   const int nl = (int)tab.size() - 1, ncta = D.ncta;
+  Blob B;
   // streamed entries of all levels, CTA after CTA
-  std::vector<uint16_t> s_col;
-  std::vector<int32_t> s_src;
-  std::vector<std::vector<uint32_t>> s_off(nl);  // per level and CTA: first entry
+  std::vector<std::vector<uint32_t>> s_off(nl);  // per level and CTA: first unit
+  size_t units = 0;
   for (int t = 0; t < nl; ++t)
     if (D.lv[t].streamed)
       for (const Part& p : tab[t].part) {
-        s_off[t].push_back((uint32_t)s_col.size());
-        s_col.insert(s_col.end(), p.ecol.begin(), p.ecol.end());
-        s_src.insert(s_src.end(), p.esrc.begin(), p.esrc.end());
-        D.lv[t].n_stream += (int64_t)p.ecol.size();
+        s_off[t].push_back((uint32_t)units);
+        units += p.ecol.size() / pu;
       }
-  GMG_TRY(upload_vec(a, &D.s_col, s_col));
-  T* sv;
-  GMG_TRY(a.alloc(&sv, std::max<size_t>(s_col.size(), 1)));
-  D.s_val = sv;
+  {
+    char* u = B.add(&D.s_ent, units);
+    for (int t = 0; t < nl; ++t)
+      for (size_t q = 0; q < s_off[t].size(); ++q) fill_units<T>(tab[t].part[q], D.lv[t].o_x, u + 16 * (size_t)s_off[t][q]);
+    char* src = B.add(&D.s_src, units * pu);
+    for (int t = 0; t < nl; ++t)
+      for (size_t q = 0; q < s_off[t].size(); ++q) {
+        const Part& p = tab[t].part[q];
+        std::memcpy(src + 4 * pu * (size_t)s_off[t][q], p.esrc.data(), 4 * p.esrc.size());
+        D.lv[t].n_stream += (int64_t)p.esrc.size();
+      }
+  }
   // the stream steps in the kernel's order; the first phase of level l0 has
   // one (the kernel skips it when colour 0 is done), that of a coarser level,
   // done by the restriction, has none
@@ -1075,89 +1420,121 @@ gmg_status upload_tables(gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>
     const int C = tab[t].ncolor;
     for (int q = 0; q < D.nu_post * C; ++q) step(t, D.post_forward ? q % C : C - 1 - q % C);
   }
-  D.nsteps = ncta > 0 ? (int)(steps[0].size() / 2) : 0;
+  D.nsteps = (int)(steps[0].size() / 2);
   for (int t = 0; t <= nl; ++t) {
     const Tab& A = tab[t];
     ClusterLevel<T>& L = D.lv[t];
     const bool res = t < nl && !L.streamed;
-    std::vector<char> img((size_t)ncta * L.img_bytes, 0);
-    const size_t nval = (size_t)L.val_bytes / sizeof(T), v0 = (size_t)L.v_val / sizeof(T);
-    std::vector<int32_t> vsrc((size_t)ncta * nval, -1), dsrc((size_t)ncta * L.n_own_max, -1);
-    std::vector<Slice> rsl((size_t)ncta * L.rsl_max, Slice{0, 0, 0, 0});
-    std::vector<uint16_t> rcol, pidx((size_t)ncta * 3 * L.n_own_max, 0);
-    std::vector<T> rw, pw((size_t)ncta * 3 * L.n_own_max, T(0));
-    std::vector<int32_t> l2g(t == 0 ? (size_t)ncta * L.n_loc_max : 0, 0);
+    const size_t S = sizeof(T), no = (size_t)L.n_own_max;
+    char* img = B.add(&L.img, (size_t)ncta * L.img_bytes);
     for (int q = 0; q < ncta; ++q) {
       const Part& p = A.part[q];
       const size_t m = p.own.size();
-      char* base = img.data() + (size_t)q * L.img_bytes;
+      char* base = img + (size_t)q * L.img_bytes;
       auto put = [&](int off, const void* v, size_t bytes) {
         if (bytes) std::memcpy(base + off, v, bytes);
       };
-      const int32_t hd[8] = {(int32_t)m, (int32_t)(m + p.halo.size()), (int32_t)p.sl.size(), (int32_t)p.rsl.size(),
-                             p.own0,     0,                            0,                    0};
-      put(0, hd, sizeof(hd));
-      std::vector<Slice> sl = p.sl;
-      if (L.streamed)  // entry offsets within the colour's block
-        for (int k = 0; k < A.ncolor; ++k)
-          for (int s = p.csl[k]; s < p.csl[k + 1]; ++s) sl[s].z -= p.blk[k];
-      put(L.i_sl, sl.data(), sl.size() * sizeof(Slice));
-      if (t < nl) put(L.i_csl, p.csl.data(), p.csl.size() * 4);
-      else put(L.i_csl, p.own.data(), m * 4);
-      put(L.i_xp, p.xp.data(), p.xp.size() * 4);
-      put(L.i_xd, p.xd.data(), p.xd.size() * 4);
+      int32_t hd[16] = {(int32_t)m, (int32_t)(m + p.halo.size()), (int32_t)p.sl.size(), (int32_t)p.rsl.size(), p.own0};
+      hd[9] = (int32_t)p.xd.size();
+      int32_t ex[4] = {0, 0, 0, 0};  // halo bytes that the residual, restriction, prolongation brings (coarsest: the solve)
       if (t < nl) {
-        put(L.i_rp, p.rp.data(), p.rp.size() * 4);
-        put(L.i_rd, p.rd.data(), p.rd.size() * 4);
-        if (res) put(L.i_col, p.ecol.data(), p.ecol.size() * 2);
-        for (size_t i = 0; i < m; ++i) {
-          vsrc[(size_t)q * nval + i] = -2 - p.own[i];
-          dsrc[(size_t)q * L.n_own_max + i] = -2 - p.own[i];
-          for (int s = 0; s < 3; ++s) {
-            pidx[((size_t)q * 3 + s) * L.n_own_max + i] = p.pidx[s * m + i];
-            pw[((size_t)q * 3 + s) * L.n_own_max + i] = (T)p.pw[s * m + i];
-          }
+        const int kf = D.post_forward ? 0 : A.ncolor - 1;  // the colour that the post-smoothing updates first
+        hd[5] = first_store(p, D.nu_post > 0 ? p.rows0[kf] : 0);
+        hd[6] = first_store(p, D.nu_post > 0 ? p.rows0[kf + 1] : 0);
+        hd[10] = first_store(p, p.own0);
+        hd[11] = (int32_t)p.rd.size();
+        for (int k = 0; k < A.ncolor; ++k) {  // first slice, slices, halo bytes of the colour's phase
+          const int32_t rec[4] = {p.csl[k], p.csl[k + 1] - p.csl[k], (int32_t)(S * p.hcol[k]), 0};
+          put(L.i_cr + 16 * k, rec, 16);
         }
-        if (res)
-          for (size_t e = 0; e < p.esrc.size(); ++e) vsrc[(size_t)q * nval + v0 + e] = p.esrc[e];
-        for (size_t s = 0; s < p.rsl.size(); ++s) {
-          rsl[(size_t)q * L.rsl_max + s] = p.rsl[s];
-          rsl[(size_t)q * L.rsl_max + s].z += (int32_t)rcol.size();
-        }
-        rcol.insert(rcol.end(), p.rcol.begin(), p.rcol.end());
-        for (double w : p.rw) rw.push_back((T)w);
+        ex[0] = (int32_t)(S * p.rhalo.size());
+        if (D.nu_pre > 0 && t + 1 < nl) ex[1] = (int32_t)(S * tab[t + 1].part[q].hcol[0]);
+        ex[2] = (int32_t)(S * (p.halo.size() - (D.nu_post > 0 ? p.hcol[kf] : 0)));
+      } else {
+        ex[0] = (int32_t)(S * p.halo.size());
       }
       if (t == 0) {
-        put(D.i_steps, steps[q].data(), steps[q].size() * 4);
-        for (size_t i = 0; i < m; ++i) l2g[(size_t)q * L.n_loc_max + i] = p.own[i];
-        for (size_t i = 0; i < p.halo.size(); ++i) l2g[(size_t)q * L.n_loc_max + m + i] = p.halo[i];
+        hd[7] = (int32_t)A.partners[q].size();
+        hd[8] = (int32_t)tab[nl].part[q].own.size();
+        put(D.i_partners, A.partners[q].data(), 4 * A.partners[q].size());
+        put(D.i_steps, steps[q].data(), 4 * steps[q].size());
+      }
+      put(0, hd, sizeof(hd));
+      put(L.i_ex, ex, sizeof(ex));
+      put(L.i_sl, p.sl.data(), p.sl.size() * sizeof(Slice));
+      if (L.streamed)  // entry offsets within the colour's block
+        for (int k = 0; k < A.ncolor; ++k)
+          for (int s = p.csl[k]; s < p.csl[k + 1]; ++s) reinterpret_cast<Slice*>(base + L.i_sl)[s].z -= p.blk[k];
+      if (t == nl) put(L.i_cr, p.own.data(), m * 4);
+      // halo stores in row order
+      auto put_list = [&](int off, const std::vector<uint32_t>& lp, const std::vector<uint32_t>& ld) {
+        uint32_t* o = reinterpret_cast<uint32_t*>(base + off);
+        for (size_t i = 0; i < lp.size(); ++i)
+          for (uint32_t q = 0; q < (lp[i] & 15u); ++q) {
+            const uint32_t d = ld[(lp[i] >> 4) + q];  // CTA << 16 | local index there
+            *o++ = (d >> 16) << 28 | (d & 0xFFFFu) << 14 | (uint32_t)i;
+          }
+      };
+      put_list(L.i_xd, p.xp, p.xd);
+      if (t < nl) put_list(L.i_rd, p.rp, p.rd);
+      for (size_t s = 0; s < p.sl.size(); ++s) {  // the slices' halo stores
+        const int r0 = p.sl[s].x & 0xFFFF, r1 = r0 + (p.sl[s].x >> 16);
+        reinterpret_cast<Slice*>(base + L.i_sl)[s].w = (first_store(p, r0) << 10) | (first_store(p, r1) - first_store(p, r0));
+        reinterpret_cast<Slice*>(base + L.i_sl)[s].y /= 2;  // pairs of units
       }
     }
-    GMG_TRY(upload_vec(a, &L.img, img));
-    if (t == 0) GMG_TRY(upload_vec(a, &D.l2g, l2g));
-    if (t == nl) continue;
-    T *vi, *dg;
-    GMG_TRY(a.alloc(&vi, std::max<size_t>(vsrc.size(), 1)));
-    GMG_TRY(a.alloc(&dg, dsrc.size()));
-    L.vimg = reinterpret_cast<const char*>(vi);
-    L.diag = dg;
-    const int4* d_rsl;
-    {
-      std::vector<int4> h(rsl.size());
-      for (size_t s = 0; s < rsl.size(); ++s) h[s] = make_int4(rsl[s].x, rsl[s].y, rsl[s].z, rsl[s].w);
-      GMG_TRY(upload_vec(a, &d_rsl, h));
+    if (t == 0) {
+      int32_t* l2g = reinterpret_cast<int32_t*>(B.add(&D.l2g, (size_t)ncta * L.n_loc_max));
+      for (int q = 0; q < ncta; ++q) {
+        const Part& p = A.part[q];
+        std::copy(p.own.begin(), p.own.end(), l2g + (size_t)q * L.n_loc_max);
+        std::copy(p.halo.begin(), p.halo.end(), l2g + (size_t)q * L.n_loc_max + p.own.size());
+      }
     }
-    L.r_sl = d_rsl;
-    GMG_TRY(upload_vec(a, &L.r_col, rcol));
-    GMG_TRY(upload_vec(a, &L.r_w, rw));
-    GMG_TRY(upload_vec(a, &L.p_idx, pidx));
-    GMG_TRY(upload_vec(a, &L.p_w, pw));
-    GMG_TRY(upload_vec(a, &L.vsrc, vsrc));
-    GMG_TRY(upload_vec(a, &L.dsrc, dsrc));
-    L.nvsrc = (int64_t)vsrc.size();
-    L.ndsrc = (int64_t)dsrc.size();
+    if (t == nl) continue;
+    char* vi = B.add(&L.vimg, (size_t)ncta * L.val_bytes);
+    if (res)
+      for (int q = 0; q < ncta; ++q) {
+        char* u = vi + (size_t)q * L.val_bytes + L.v_ent;
+        const uint32_t pad = (uint32_t)L.o_x;  // units past a CTA's own are never read; give them a valid address
+        for (size_t e = 0; e < (size_t)A.ent * pu; ++e) std::memcpy(u + (pu == 2 ? 8 * e + 4 : 16 * e + 8), &pad, 4);
+        fill_units<T>(A.part[q], L.o_x, u);
+      }
+    int32_t* ds = reinterpret_cast<int32_t*>(B.add(&L.dsrc, (size_t)ncta * no));
+    std::fill(ds, ds + (size_t)ncta * no, -1);
+    for (int q = 0; q < ncta; ++q)
+      for (size_t i = 0; i < A.part[q].own.size(); ++i) ds[(size_t)q * no + i] = -2 - A.part[q].own[i];
+    L.nvsrc = res ? (int64_t)ncta * A.ent * pu : 0;
+    L.n_ent = res ? (int64_t)A.ent * pu : 0;
+    int32_t* vs = reinterpret_cast<int32_t*>(B.add(&L.vsrc, (size_t)L.nvsrc));
+    if (res) {
+      std::fill(vs, vs + L.nvsrc, -1);
+      for (int q = 0; q < ncta; ++q)
+        std::copy(A.part[q].esrc.begin(), A.part[q].esrc.end(), vs + (size_t)q * A.ent * pu);
+    }
+    Slice* rsl = reinterpret_cast<Slice*>(B.add(&L.r_sl, (size_t)ncta * L.rsl_max));
+    for (int q = 0; q < ncta; ++q)
+      std::copy(A.part[q].rsl.begin(), A.part[q].rsl.end(), rsl + (size_t)q * L.rsl_max);
+    uint16_t* rc = reinterpret_cast<uint16_t*>(B.add(&L.r_col, (size_t)ncta * L.r_max));
+    for (int q = 0; q < ncta; ++q)
+      std::copy(A.part[q].rcol.begin(), A.part[q].rcol.end(), rc + (size_t)q * L.r_max);
+    T* rw = reinterpret_cast<T*>(B.add(&L.r_w, (size_t)ncta * L.r_max));
+    for (int q = 0; q < ncta; ++q)
+      for (size_t e = 0; e < A.part[q].rw.size(); ++e) rw[(size_t)q * L.r_max + e] = (T)A.part[q].rw[e];
+    uint16_t* pi = reinterpret_cast<uint16_t*>(B.add(&L.p_idx, (size_t)ncta * 3 * no));
+    for (int q = 0; q < ncta; ++q)
+      for (int s = 0; s < 3; ++s) {
+        const size_t m = A.part[q].own.size();
+        std::copy(A.part[q].pidx.begin() + s * m, A.part[q].pidx.begin() + (s + 1) * m, pi + ((size_t)q * 3 + s) * no);
+      }
+    T* pw = reinterpret_cast<T*>(B.add(&L.p_w, (size_t)ncta * 3 * no));
+    for (int q = 0; q < ncta; ++q)
+      for (int s = 0; s < 3; ++s) {
+        const size_t m = A.part[q].own.size();
+        for (size_t i = 0; i < m; ++i) pw[((size_t)q * 3 + s) * no + i] = (T)A.part[q].pw[s * m + i];
+      }
   }
-  return upload_vec(a, &D.s_src, s_src);
+  return B.upload(c->arena);
 }
 
 template <class T>
@@ -1180,18 +1557,23 @@ gmg_status build_one(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
     if (ncta < 1 || ncta > 16) continue;
     for (int l0 = std::max(0, lam - kClMaxLevels); l0 < lam; ++l0) {
       // a quick lower bound of the shared memory before the tables are built
-      int64_t least = 4 * c->L[lam].n;
+      constexpr int pu = sizeof(T) == 4 ? 2 : 1;
+      int64_t least = (int64_t)sizeof(T) * c->L[lam].n, stage = 0, ent = 0;
       bool skip = false;
       for (int l = l0; l < lam; ++l) {
         const Level& L = c->L[l];
         const int64_t rows = L.n / (std::max(1, L.ncolor) * ncta);
         skip = skip || (L.nnz - L.n) / (std::max(1, L.ncolor) * (int64_t)ncta) > kClPhaseEntries ||
                (small_only && rows >= kClWide) || L.A.entries > INT32_MAX;
-        least += (L.n / ncta) * (int64_t)(3 * sizeof(T) + 8);
+        // x, b, 1/a_ii and a_ii of the rows; entries in shared memory, or two stages of a phase
+        least += (L.n / ncta) * (int64_t)(4 * sizeof(T)) + (l == l0 ? (int64_t)sizeof(T) * (L.n / ncta) : 0);
+        const int64_t e = (L.nnz - L.n) * (16 / pu) / ncta;
+        ent += e;
+        stage = std::max(stage, 2 * e / std::max(1, L.ncolor));
       }
-      if (skip || least > kSmemLimit) continue;
+      if (skip || least + std::min(ent, stage) > kSmemLimit) continue;
       std::vector<Tab> tab;
-      if (!build_tables(c, l0, ncta, hrp, hcol, perm, iperm, P, tab)) continue;
+      if (!build_tables(c, l0, ncta, pu, hrp, hcol, perm, iperm, P, tab)) continue;
       // where the ranks are not local (random order: 11-13 halo stores per
       // row on a kNN cloud) a phase would store nearly every row into every CTA
       bool local = true;
@@ -1210,7 +1592,7 @@ gmg_status build_one(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
       E.nu_post = c->opt.nu_post;
       E.post_forward = c->opt.post_forward;
       if (!lay_out(tab, E.nu_pre, E.nu_post, E)) continue;
-      if (!check_tables(tab)) {
+      if (!check_tables(tab, pu)) {
         set_error("internal: cluster tables failed their host check");
         return GMG_ERR_INVALID_ARG;
       }
@@ -1232,23 +1614,26 @@ gmg_status refresh_one(gmg_ctx* c, cudaStream_t s) {
   ClusterDesc<T>& D = Src<T>::desc(c);
   if (D.l0 < 0) return GMG_OK;
   RefreshJobs<T> J;
-  int64_t most = 1;
+  const int step = sizeof(T) == 4 ? 8 : 16;
+  int64_t most = 1, off = 0;
   for (int t = 0; t < D.nlev; ++t) {
     Level& L = c->L[D.l0 + t];
     const ClusterLevel<T>& C = D.lv[t];
     const T* v = Vec<T>::v(L.A);
-    J.job[J.njob++] = {C.nvsrc, C.vsrc, v, Vec<T>::dinv(L), reinterpret_cast<T*>(const_cast<char*>(C.vimg))};
-    J.job[J.njob++] = {C.ndsrc, C.dsrc, v, Vec<T>::diag(L), const_cast<T*>(C.diag)};
-    most = std::max(most, C.nvsrc);
-  }
-  int64_t off = 0;
-  for (int t = 0; t < D.nlev; ++t)
-    if (D.lv[t].streamed) {
-      const int64_t n = D.lv[t].n_stream;
-      J.job[J.njob++] = {n, D.s_src + off, Vec<T>::v(c->L[D.l0 + t].A), nullptr, const_cast<T*>(D.s_val) + off};
-      off += n;
-      most = std::max(most, n);
+    char* out = const_cast<char*>(C.vimg);
+    const int64_t nd = (int64_t)D.ncta * C.n_own_max;
+    J.job[J.njob++] = {nd, C.n_own_max, C.val_bytes, 2 * (int)sizeof(T), C.dsrc, v, Vec<T>::dinv(L), out + sizeof(T)};
+    J.job[J.njob++] = {nd, C.n_own_max, C.val_bytes, (int)sizeof(T), C.dsrc, v, Vec<T>::diag(L), out + C.v_diag};
+    if (C.streamed) {
+      char* ent = reinterpret_cast<char*>(const_cast<uint4*>(D.s_ent)) + off * step;
+      J.job[J.njob++] = {C.n_stream, std::max<int64_t>(1, C.n_stream), 0, step, D.s_src + off, v, nullptr, ent};
+      off += C.n_stream;
+      most = std::max(most, C.n_stream);
+    } else if (C.nvsrc > 0) {
+      J.job[J.njob++] = {C.nvsrc, C.n_ent, C.val_bytes, step, C.vsrc, v, nullptr, out + C.v_ent};
+      most = std::max(most, C.nvsrc);
     }
+  }
   k_cluster_values<T><<<dim3((unsigned)std::min<int64_t>((most + 255) / 256, 304), (unsigned)J.njob), 256, 0, s>>>(J);
   GMG_LAUNCHED();
   return GMG_OK;
@@ -1293,12 +1678,13 @@ template gmg_status launch_cluster<double>(gmg_ctx*, double*, const double*, boo
 // arrives on, so every poll fails and the wait gives up; elapsed device time
 // in *ns.
 __global__ void k_wait_selftest(int polls, int* err, unsigned long long* ns) {
-  __shared__ uint64_t m;
-  if (threadIdx.x == 0) mbar_init(&m, 1);
+  __shared__ uint64_t bar;
+  const uint32_t m = smem_addr(&bar);
+  if (threadIdx.x == 0) mbar_init(m, 1);
   __syncthreads();
   unsigned long long t0, t1;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-  mbar_wait(&m, 0u, err, polls);
+  mbar_wait(m, 0u, err, polls);
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
   if (threadIdx.x == 0) *ns = t1 - t0;
 }

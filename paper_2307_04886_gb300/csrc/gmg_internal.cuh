@@ -230,36 +230,38 @@ template <class T>
 struct ClusterLevel {
   int ncolor, tpr, lg_tpr, r_tpr, lg_r_tpr;  // lanes per row of the sweeps and of the restriction from this level
   bool streamed;                             // entries stream from L2 instead of staying in shared memory
-  int n_own_max, n_loc_max, rsl_max;
-  // shared memory: the image (header: own rows, own and halo rows, slices,
-  // restriction slices, own rows of colour 0; then slices, colours, halo
-  // stores of x and of the residual, resident columns), the values (1/a_ii,
-  // then resident entries), x (own and halo rows), b (own rows)
-  int o_img, o_val, o_x, o_b;
+  int n_own_max, n_loc_max, rsl_max, r_max;
+  // shared memory: the image (header, halo bytes of the transfers' phases,
+  // slices, colour records or the coarsest level's global rows, halo stores of
+  // x and of the residual; level l0: partners, stream steps), the values
+  // (pairs of b and 1/a_ii, a_ii, then resident entry units), x (own and halo
+  // rows).  Header: own rows, own and halo rows,
+  // slices, restriction slices, own rows of colour 0, halo stores [5], [6) of
+  // the rows that the post-smoothing updates first, partners, own rows of the
+  // coarsest level, halo stores of x, of its colour 0, of the residual
+  int o_img, o_val, o_x;
   int img_bytes, val_bytes;
-  int i_sl, i_csl, i_xp, i_xd, i_rp, i_rd, i_col, v_val;
+  int i_ex, i_sl, i_cr, i_xd, i_rd, v_diag, v_ent;
   const char *img, *vimg;
-  const T* diag;          // per CTA n_own_max
   const uint16_t* p_idx;  // per CTA 3 x n_own_max: the prolongation into this level
   const T* p_w;
-  const int4* r_sl;       // per CTA rsl_max slices of the restriction from this level
+  const int4* r_sl;       // per CTA rsl_max slices of the restriction from this level, r_max terms
   const uint16_t* r_col;
   const T* r_w;
-  const int32_t *vsrc, *dsrc;  // where the values and the diagonal come from (refresh)
-  int64_t nvsrc, ndsrc, n_stream;
+  const int32_t *vsrc, *dsrc;  // where the entries and the diagonal come from (refresh)
+  int64_t nvsrc, n_ent, n_stream;  // entries of all CTAs, of a CTA, streamed
 };
 template <class T>
 struct ClusterDesc {
   int l0 = -1;  // first level (-1: no cluster)
   int ncta = 0, nlev = 0, nc = 0;
   int nu_pre = 0, nu_post = 0, post_forward = 0;
-  int nstage = 0, nsteps = 0, stage_bytes = 0, stage_col = 0;
-  int o_mbar = 0, o_r = 0, o_bc = 0, o_buf = 0, i_steps = 0, smem = 0;
+  int nstage = 0, nsteps = 0, stage_bytes = 0;
+  int o_mbar = 0, o_tok = 0, o_r[2] = {0, 0}, o_bc = 0, o_buf = 0, i_steps = 0, i_partners = 0, smem = 0;
   int* err = nullptr;  // set when a bounded wait for an entry block gave up
   const T* ainv = nullptr;
   const int32_t* l2g = nullptr;  // level l0: global rows of each CTA's own and halo rows
-  const T* s_val = nullptr;      // streamed entries
-  const uint16_t* s_col = nullptr;
+  const uint4* s_ent = nullptr;  // streamed entry units
   const int32_t* s_src = nullptr;
   ClusterLevel<T> lv[kClMaxLevels + 1] = {};
   bool wide[kClMaxLevels] = {};  // one thread per row (the per-colour kernels' sums)
