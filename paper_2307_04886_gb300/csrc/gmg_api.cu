@@ -102,106 +102,127 @@ static void drop_graphs(gmg_ctx* c) {
       g = nullptr;
     }
   for (int m = 0; m < 4; ++m) {
-    if (c->loops[m]) cudaGraphExecDestroy(c->loops[m]);
-    c->loops[m] = nullptr;
+    for (auto& g : c->loops[m]) {
+      if (g) cudaGraphExecDestroy(g);
+      g = nullptr;
+    }
     c->loop_refused[m] = false;
   }
 }
 
-// Builds the device-side loop of `mode`: a graph holding one conditional
-// WHILE node (condition 1 at every launch) whose body is captured from
-// loop_body.  The body keeps its programmatic launch edges if the CUDA driver
-// instantiates them inside a conditional body, else it is captured again in
-// plain stream order; if neither instantiates, the mode keeps the host loop.
-static gmg_status build_loop(gmg_ctx* c, int mode) {
+// Captures what `body` launches on the handle's stream into `g` behind the
+// nodes `deps`, which it replaces by the nodes the captured work ends with.
+template <class F>
+static cudaError_t capture_into(gmg_ctx* c, cudaGraph_t g, std::vector<cudaGraphNode_t>* deps, gmg_status* st,
+                                F&& body) {
+  cudaError_t e = cudaStreamBeginCaptureToGraph(c->g_stream, g, deps->data(), nullptr, deps->size(),
+                                                cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return e;
+  *st = body();
+  cudaStreamCaptureStatus cs;
+  const cudaGraphNode_t* tail = nullptr;
+  size_t count = 0;
+  e = cudaStreamGetCaptureInfo(c->g_stream, &cs, nullptr, nullptr, &tail, nullptr, &count);
+  if (e == cudaSuccess && count) deps->assign(tail, tail + count);
+  cudaGraph_t done = nullptr;
+  const cudaError_t e2 = cudaStreamEndCapture(c->g_stream, &done);
+  return e != cudaSuccess ? e : e2;
+}
+
+// Builds a device-driven solve of `mode`: the start (with `whole`: the initial
+// residual and its test, for CG also the first cycle and direction), for CG the
+// first step, a conditional WHILE node (condition 1 at every launch) whose body
+// is captured from loop_body, and for CG the true residual at the end.  One
+// launch and one synchronisation then serve a solve.  The kernels keep their
+// programmatic launch edges if the CUDA driver instantiates them around and
+// inside a conditional body, else all is captured again in plain stream order;
+// if neither instantiates, the mode keeps the host loop.
+static gmg_status build_loop(gmg_ctx* c, int mode, bool whole) {
   if (!c->g_stream) GMG_CK(cudaStreamCreateWithFlags(&c->g_stream, cudaStreamNonBlocking));
-  for (int attempt = 0; attempt < 2 && !c->loops[mode]; ++attempt) {
+  cudaGraphExec_t& exec = c->loops[mode][whole];
+  const uint64_t before = g_launches;
+  bool pdl = false;
+  // a pending coarsest inverse is joined by whoever launches the graph
+  const bool pending = c->inv_pending;
+  c->inv_pending = false;
+  struct Restore {
+    gmg_ctx* c;
+    bool pending;
+    ~Restore() { c->inv_pending = pending; }
+  } restore{c, pending};
+  for (int attempt = 0; attempt < 2 && !exec; ++attempt) {
     cudaGraph_t g = nullptr;
     GMG_CK(cudaGraphCreate(&g, 0));
     cudaGraphConditionalHandle h = 0;
-    cudaGraphNodeParams np = {};
+    std::vector<cudaGraphNode_t> deps, none;
+    gmg_status st = GMG_OK;
+    uint64_t once = 0;
+    g_pdl_suspended = attempt == 1;
     cudaError_t e = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault);
-    if (e == cudaSuccess) {
+    if (e == cudaSuccess && (whole || is_pcg(mode)))
+      e = capture_into(c, g, &deps, &st, [&]() -> gmg_status {
+        if (whole) GMG_TRY(outer_residual_norm(c, true, c->g_stream));
+        if (!is_pcg(mode)) return GMG_OK;
+        if (whole) GMG_TRY(pcg_start(c, mode, c->g_stream));
+        return iteration_body(c, mode, 0, c->g_stream, h, true);
+      });
+    once = g_launches - before;
+    g_launches = before;
+    cudaGraphNodeParams np = {};
+    if (e == cudaSuccess && st == GMG_OK) {
       np.type = cudaGraphNodeTypeConditional;
       np.conditional.handle = h;
       np.conditional.type = cudaGraphCondTypeWhile;
       np.conditional.size = 1;
       cudaGraphNode_t node;
-      e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &np);
+      e = cudaGraphAddNode(&node, g, deps.data(), nullptr, deps.size(), &np);
+      deps.assign(1, node);
     }
-    if (e == cudaSuccess) {
-      const uint64_t before = g_launches;
-      g_pdl_suspended = attempt == 1;
-      e = cudaStreamBeginCaptureToGraph(c->g_stream, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
-                                        cudaStreamCaptureModeThreadLocal);
-      gmg_status st = GMG_OK;
-      if (e == cudaSuccess) {
-        st = loop_body(c, mode, h, c->g_stream);
-        cudaGraph_t body = nullptr;
-        e = cudaStreamEndCapture(c->g_stream, &body);
-      }
-      g_pdl_suspended = false;
-      c->loop_kernels[mode] = g_launches - before;
+    if (e == cudaSuccess && st == GMG_OK)
+      e = capture_into(c, np.conditional.phGraph_out[0], &none, &st,
+                       [&] { return loop_body(c, mode, h, c->g_stream); });
+    c->loop_kernels[mode] = g_launches - before;
+    g_launches = before;
+    if (e == cudaSuccess && st == GMG_OK && is_pcg(mode)) {
+      g_pdl_suspended = true;  // the loop node is no programmatic predecessor
+      e = capture_into(c, g, &deps, &st, [&] { return outer_residual_norm(c, false, c->g_stream); });
+      once += g_launches - before;
       g_launches = before;
-      if (st != GMG_OK) {
-        cudaGraphDestroy(g);
-        return st;
-      }
-      if (e == cudaSuccess) e = cudaGraphInstantiate(&c->loops[mode], g, 0);
-      if (e == cudaSuccess) c->loop_pdl[mode] = attempt == 0 && use_pdl();
     }
+    c->loop_once[mode][whole] = once;
+    g_pdl_suspended = false;
+    if (st == GMG_OK && e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
+    if (st == GMG_OK && e == cudaSuccess) pdl = attempt == 0 && use_pdl();
     cudaGraphDestroy(g);
+    if (st != GMG_OK) {
+      exec = nullptr;
+      return st;
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
-      c->loops[mode] = nullptr;
+      exec = nullptr;
     }
   }
-  if (!c->loops[mode]) c->loop_refused[mode] = true;
+  if (!exec) c->loop_refused[mode] = true;
   if (const char* e = std::getenv("GMG_VERBOSE"))
     if (e[0] == '1')
       std::fprintf(stderr, "gmg: device-side loop for mode %d: %s\n", mode,
-                   !c->loops[mode] ? "refused, host loop" : c->loop_pdl[mode] ? "programmatic launches" : "plain stream order");
+                   !exec ? "refused, host loop" : pdl ? "programmatic launches" : "plain stream order");
   return GMG_OK;
 }
 
-// Whether the iterations of `mode` run in the device-side loop: graphs on,
-// no per-cycle timing (event nodes are not allowed in a conditional body),
-// GMG_NO_DEVICE_LOOP unset, and the loop graph instantiated.
-static gmg_status device_loop_ready(gmg_ctx* c, int mode, bool* ok) {
+// Whether a solve in `mode` runs device-driven: graphs on, no per-cycle timing
+// (event nodes are not allowed in a conditional body), GMG_NO_DEVICE_LOOP
+// unset, an iteration to do, and the graph instantiated.
+static gmg_status device_loop_ready(gmg_ctx* c, int mode, bool whole, bool* ok) {
   static const bool off = [] {
     const char* e = std::getenv("GMG_NO_DEVICE_LOOP");
     return e && e[0] == '1';
   }();
   *ok = false;
-  if (off || !c->opt.use_graphs || c->prof || c->loop_refused[mode]) return GMG_OK;
-  if (!c->loops[mode]) GMG_TRY(build_loop(c, mode));
-  *ok = c->loops[mode] != nullptr;
-  return GMG_OK;
-}
-
-// Runs the device-side loop from iteration *k until k_iter_check stops it;
-// returns the new iteration count in *k, the scalars in h_scal and the
-// loop's residual history in info->history.
-static gmg_status run_loop(gmg_ctx* c, int mode, double tol, int* k, gmg_solve_info* info, cudaStream_t s) {
-  const int it[2] = {*k, c->opt.max_iter};
-  GMG_CK(cudaMemcpyAsync(c->scal + S_TOL, &tol, sizeof(double), cudaMemcpyHostToDevice, s));
-  GMG_CK(cudaMemcpyAsync(c->dloop, it, sizeof(it), cudaMemcpyHostToDevice, s));
-  GMG_CK(cudaGraphLaunch(c->loops[mode], s));
-  int* hk = reinterpret_cast<int*>(c->h_scal + 40);
-  GMG_CK(cudaMemcpyAsync(hk, c->dloop, sizeof(int), cudaMemcpyDeviceToHost, s));
-  GMG_TRY(fetch_scalars(c, s));
-  const int k1 = *hk;
-  if (k1 <= *k || k1 > c->opt.max_iter) {
-    set_error("device loop: iteration counter out of range");
-    return GMG_ERR_CUDA;
-  }
-  g_launches += (uint64_t)(k1 - *k) * c->loop_kernels[mode];
-  if (info && info->history && *k + 1 < info->history_cap) {
-    const int last = std::min(k1, info->history_cap - 1);
-    GMG_CK(cudaMemcpy(info->history + *k + 1, c->dhist + *k + 1, sizeof(double) * (size_t)(last - *k),
-                      cudaMemcpyDeviceToHost));
-  }
-  *k = k1;
+  if (off || !c->opt.use_graphs || c->prof || c->loop_refused[mode] || c->opt.max_iter <= 0) return GMG_OK;
+  if (!c->loops[mode][whole]) GMG_TRY(build_loop(c, mode, whole));
+  *ok = c->loops[mode][whole] != nullptr;
   return GMG_OK;
 }
 
@@ -228,6 +249,156 @@ static gmg_status store_vec(gmg_ctx* c, int l, const double* src, double* dst, i
   }
   return launch_scatter(L.n, L.perm, src, dst, s);
 }
+
+// The outer iteration of one gmg_solve, from the loaded system on.
+struct SolveRun {
+  gmg_ctx* c;
+  cudaStream_t s;
+  int mode;
+  double tol;
+  gmg_solve_info* info;
+  int k = 0;
+  double rel = 0.0;
+  gmg_status st = GMG_ERR_NOT_CONVERGED;
+  bool rewrite = false;      // on_device: xs changed after it was stored
+  bool wait_failed = false;  // on_device: a bounded wait ran out
+
+  void record(int kk, double v) {
+    if (info && info->history && kk < info->history_cap) info->history[kk] = v;
+  }
+
+  // The start's test from ||b||^2 and ||r||^2: false ends the solve.
+  gmg_status start(double nb, double rr, bool* go) {
+    *go = false;
+    if (!std::isfinite(nb)) {
+      set_error("gmg_solve: non-finite right-hand side");
+      st = GMG_ERR_NONFINITE;
+    } else if (nb == 0.0) {
+      GMG_CK(cudaMemsetAsync(c->xs, 0, sizeof(double) * (size_t)c->L[0].n, s));
+      rewrite = true;
+      record(0, 0.0);
+      st = GMG_OK;
+    } else {
+      rel = std::sqrt(rr) / nb;
+      record(0, rel);
+      if (!std::isfinite(rel)) {
+        set_error("gmg_solve: non-finite initial residual");
+        st = GMG_ERR_NONFINITE;
+      } else {
+        *go = true;
+      }
+    }
+    return GMG_OK;
+  }
+
+  // Graph launches only (build_loop): the solution goes out with the report of
+  // every launch, so a solve whose first report confirms the tolerance has
+  // synchronised once.
+  gmg_status on_device(double* x, double* x_dev, size_t bytes, bool whole) {
+    const double* R = c->h_scal;
+    if (!is_pcg(mode)) GMG_TRY(join_inverse(c, s, false));
+    if (!whole) {
+      GMG_TRY(outer_residual_norm(c, true, s));
+      GMG_TRY(pcg_start(c, mode, s));
+    }
+    for (;;) {
+      GMG_CK(cudaGraphLaunch(c->loops[mode][whole], s));
+      GMG_TRY(store_solution(c, x_dev, s));
+      if (x != x_dev) GMG_CK(cudaMemcpyAsync(x, x_dev, bytes, cudaMemcpyDeviceToHost, s));
+      GMG_CK(cudaStreamSynchronize(s));
+      wait_failed |= R[REP_WAIT] != 0.0;
+      if (R[REP_PIVOT] == 0.0) c->inv_check = false;  // else read, and reported, by inverse_status
+      const double nb = std::sqrt(R[REP_NB2]);
+      if (R[REP_OK] != 1.0) {  // the start failed its test: x has not been written
+        bool go = false;
+        return start(nb, R[REP_HIST] * nb, &go);  // infinite or NaN stays so
+      }
+      const int k1 = (int)R[REP_ITERS];
+      if (k1 <= k || k1 > c->opt.max_iter) {
+        set_error("device loop: iteration counter out of range");
+        return GMG_ERR_CUDA;
+      }
+      g_launches += c->loop_once[mode][whole] + (uint64_t)(k1 - k - (is_pcg(mode) ? 1 : 0)) * c->loop_kernels[mode];
+      const int from = k == 0 ? 0 : k + 1;
+      if (info && info->history && from < info->history_cap) {
+        const int last = std::min(k1, info->history_cap - 1);
+        if (last < REP_HIST_CAP)
+          std::copy(R + REP_HIST + from, R + REP_HIST + last + 1, info->history + from);
+        else
+          GMG_CK(cudaMemcpy(info->history + from, c->dhist + from, sizeof(double) * (size_t)(last - from + 1),
+                            cudaMemcpyDeviceToHost));
+      }
+      k = k1;
+      rel = R[REP_REL];
+      if (!std::isfinite(rel)) {
+        set_error("gmg_solve: iterate became non-finite");
+        st = GMG_ERR_NONFINITE;
+        return GMG_OK;
+      }
+      if (rel <= tol && is_pcg(mode)) {  // confirmed on the true residual
+        rel = std::sqrt(R[REP_RR]) / nb;
+        record(k, rel);
+      }
+      if (rel <= tol) {
+        st = GMG_OK;
+        return GMG_OK;
+      }
+      bool again = false;
+      if (is_pcg(mode) && k < c->opt.max_iter) GMG_TRY(device_loop_ready(c, mode, false, &again));
+      if (!again) break;
+      GMG_TRY(pcg_start(c, mode, s));  // restart from the current iterate
+      whole = false;
+    }
+    set_error("gmg_solve: max_iter reached");
+    return GMG_OK;
+  }
+
+  // One synchronisation per iteration.
+  gmg_status on_host() {
+    GMG_TRY(outer_residual_norm(c, false, s));
+    GMG_TRY(fetch_scalars(c, s));
+    const double nb = std::sqrt(c->h_scal[S_NB2]);
+    bool go = true;
+    GMG_TRY(start(nb, c->h_scal[S_RR], &go));
+    if (!go) return GMG_OK;
+    if (!is_pcg(mode)) GMG_TRY(join_inverse(c, s, false));
+    if (is_pcg(mode)) GMG_TRY(pcg_start(c, mode, s));
+    bool fresh = true;  // CG: no step since the (re)start
+    while (k < c->opt.max_iter) {
+      if (is_pcg(mode) && !fresh) GMG_TRY(run_cycle_body(c, mode, 1, s));
+      GMG_TRY(run_cycle_body(c, mode, 0, s));
+      GMG_TRY(fetch_scalars(c, s));
+      ++k;
+      fresh = false;
+      rel = std::sqrt(c->h_scal[S_RR]) / nb;
+      if (!std::isfinite(rel)) {
+        set_error("gmg_solve: iterate became non-finite");
+        st = GMG_ERR_NONFINITE;
+        return GMG_OK;
+      }
+      if (rel <= tol && is_pcg(mode)) {  // confirm on the true residual
+        GMG_TRY(outer_residual_norm(c, false, s));
+        GMG_TRY(fetch_scalars(c, s));
+        rel = std::sqrt(c->h_scal[S_RR]) / nb;
+        record(k, rel);
+        if (rel <= tol) {
+          st = GMG_OK;
+          return GMG_OK;
+        }
+        GMG_TRY(pcg_start(c, mode, s));  // restart from the current iterate
+        fresh = true;
+        continue;
+      }
+      record(k, rel);
+      if (rel <= tol) {
+        st = GMG_OK;
+        return GMG_OK;
+      }
+    }
+    set_error("gmg_solve: max_iter reached");
+    return GMG_OK;
+  }
+};
 
 }  // namespace gmg
 
@@ -343,89 +514,32 @@ gmg_status gmg_solve(gmg_handle h, const double* b, double* x, double tol, int m
   }
   gmg_ctx* c = h;
   cudaStream_t s = (cudaStream_t)stream;
-  Level& L0 = c->L[0];
-  const int64_t n = L0.n;
-  GMG_TRY(load_vec(c, 0, b, mem, c->bs, c->io, s));
-  GMG_TRY(load_vec(c, 0, x, mem, c->xs, c->io2, s));
-  GMG_TRY(norm_b(c, s));
-  GMG_TRY(outer_residual_norm(c, s));
-  GMG_TRY(fetch_scalars(c, s));
-  const double nb = std::sqrt(c->h_scal[S_NB2]);
-  int k = 0;
-  double rel = 0.0;
-  gmg_status st = GMG_ERR_NOT_CONVERGED;
-  auto record = [&](int kk, double v) {
-    if (info && info->history && kk < info->history_cap) info->history[kk] = v;
-  };
-  if (!std::isfinite(nb)) {
-    set_error("gmg_solve: non-finite right-hand side");
-    st = GMG_ERR_NONFINITE;
-  } else if (nb == 0.0) {
-    GMG_CK(cudaMemsetAsync(c->xs, 0, sizeof(double) * (size_t)n, s));
-    record(0, 0.0);
-    st = GMG_OK;
-  } else {
-    rel = std::sqrt(c->h_scal[S_RR]) / nb;
-    record(0, rel);
-    const int mode = c->nlev == 1 ? GMG_FP64 : c->opt.precision;
-    if (!std::isfinite(rel)) {
-      set_error("gmg_solve: non-finite initial residual");
-      st = GMG_ERR_NONFINITE;
-    } else {
-      // a CG start joins a pending coarsest inverse right before its first
-      // coarse solve (its down-leg overlaps the inverse); the other modes
-      // join before their first iteration
-      if (!is_pcg(mode)) GMG_TRY(join_inverse(c, s, false));
-      if (is_pcg(mode)) GMG_TRY(pcg_start(c, mode, s));
-      bool fresh = true;  // CG: no step since the (re)start
-      while (k < c->opt.max_iter) {
-        bool dev = false;
-        if (!(is_pcg(mode) && fresh)) GMG_TRY(device_loop_ready(c, mode, &dev));
-        if (dev) {
-          GMG_TRY(run_loop(c, mode, tol, &k, info, s));
-        } else {
-          if (is_pcg(mode) && !fresh) GMG_TRY(run_cycle_body(c, mode, 1, s));
-          GMG_TRY(run_cycle_body(c, mode, 0, s));
-          GMG_TRY(fetch_scalars(c, s));
-          ++k;
-        }
-        fresh = false;
-        rel = std::sqrt(c->h_scal[S_RR]) / nb;
-        if (!std::isfinite(rel)) {
-          set_error("gmg_solve: iterate became non-finite");
-          st = GMG_ERR_NONFINITE;
-          break;
-        }
-        if (rel <= tol && is_pcg(mode)) {  // confirm on the true residual
-          GMG_TRY(outer_residual_norm(c, s));
-          GMG_TRY(fetch_scalars(c, s));
-          rel = std::sqrt(c->h_scal[S_RR]) / nb;
-          record(k, rel);
-          if (rel <= tol) {
-            st = GMG_OK;
-            break;
-          }
-          GMG_TRY(pcg_start(c, mode, s));  // restart from the current iterate
-          fresh = true;
-          continue;
-        }
-        if (!dev) record(k, rel);  // the device loop wrote its own history
-        if (rel <= tol) {
-          st = GMG_OK;
-          break;
-        }
-      }
-      if (st == GMG_ERR_NOT_CONVERGED) set_error("gmg_solve: max_iter reached");
-    }
+  const int64_t n = c->L[0].n;
+  const size_t bytes = sizeof(double) * (size_t)n;
+  const int mode = c->nlev == 1 ? GMG_FP64 : c->opt.precision;
+  const bool host = mem == GMG_MEM_HOST;
+  if (host) {
+    GMG_CK(cudaMemcpyAsync(c->io, b, bytes, cudaMemcpyHostToDevice, s));
+    GMG_CK(cudaMemcpyAsync(c->io2, x, bytes, cudaMemcpyHostToDevice, s));
   }
-  GMG_TRY(store_vec(c, 0, c->xs, x, mem, c->io2, s));
+  GMG_TRY(load_system(c, host ? c->io : b, host ? c->io2 : x, tol, s));
+  SolveRun run{c, s, mode, tol, info};
+  // a CG start joins a pending coarsest inverse right before its first coarse
+  // solve (its down-leg overlaps the inverse), so it runs on the stream, not
+  // in a graph; the other modes join before their first iteration
+  bool dev = false;
+  const bool whole = !(is_pcg(mode) && c->inv_pending);
+  GMG_TRY(device_loop_ready(c, mode, whole, &dev));
+  if (dev) GMG_TRY(run.on_device(x, host ? c->io2 : x, bytes, whole));
+  else GMG_TRY(run.on_host());
+  if (!dev || run.rewrite) GMG_TRY(store_vec(c, 0, c->xs, x, mem, c->io2, s));
   if (info) {
-    info->iters = k;
-    info->rel_res = rel;
+    info->iters = run.k;
+    info->rel_res = run.rel;
   }
   GMG_TRY(inverse_status(c, s));  // the pivot check of an inverse this solve joined
-  GMG_TRY(cluster_status(c, s));
-  return st;
+  if (!dev || run.wait_failed) GMG_TRY(cluster_status(c, s));
+  return run.st;
 }
 
 gmg_status gmg_profile(gmg_handle h, int enable) {

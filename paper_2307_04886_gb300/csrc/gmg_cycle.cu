@@ -169,13 +169,64 @@ __global__ void __launch_bounds__(256, (G == 1 && sizeof(T) == 4) ? 8 : 1) k_gs(
   if (part == 0 && p.active) x[p.row] = (bv - acc) * di;
 }
 
-// r = b - A x over all slices; with `partial`, per-block sums of r^2.
-template <class T, int G>
+// Block sums in the fixed order of k_dot_partial (same grid, same per-thread
+// ranges, same tree), so the fused kernels below give the same bits as a
+// separate dot product.
+__device__ __forceinline__ void block_sum_store(double v, double* red, double* out) {
+  red[threadIdx.x] = v;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *out = red[0];
+}
+
+// The start of a device-driven solve (one thread): the initial relative
+// residual, and whether the right-hand side is nonzero and both are finite
+// (the iterations of a solve that must not run are discarded by k_store).
+__device__ void start_check(double* sc, double* hist) {
+  const double nb = sqrt(sc[S_NB2]), rel = sqrt(sc[S_RR]) / nb;
+  hist[0] = rel;
+  sc[S_OK] = isfinite(nb) && nb > 0.0 && isfinite(rel) ? 1.0 : 0.0;
+}
+
+// The convergence test of the device-side loop (one thread): advances the
+// iteration counter it[0], records rel = ||r|| / ||b|| (same arithmetic as the
+// host test) and keeps the loop going while rel is finite, above the
+// tolerance and the counter below it[1].
+__device__ void iter_check(const double* sc, int* it, double* hist, cudaGraphConditionalHandle h) {
+  const int k = ++it[0];
+  const double rel = sqrt(sc[S_RR]) / sqrt(sc[S_NB2]);
+  hist[k] = rel;
+  const bool go = isfinite(rel) && !(rel <= sc[S_TOL]) && k < it[1];
+  cudaGraphSetConditional(h, go ? 1u : 0u);
+}
+
+// What the last block of a residual with a norm does with ||r||^2 besides
+// storing it: nothing, the test of a solve's start (start_check), or the
+// convergence test of the device-side loop (iter_check).
+enum { kNormOnly = 0, kNormStart = 1, kNormIter = 2 };
+struct NormEnd {
+  double* partial;  // one sum of r^2 per block
+  int* counter;
+  double* sc;
+  int* it;
+  double* hist;
+  cudaGraphConditionalHandle h;
+  int what;
+};
+
+// r = b - A x over all slices.  With NORM also ||r||^2 into sc[S_RR]: fixed
+// block sums, added in block order by the last block, which then runs the
+// test named in `end` (a separate one-block sum and a one-thread test cost a
+// launch each: 5 us per iteration of the refinement modes).
+template <class T, int G, bool NORM>
 __global__ void __launch_bounds__(256) k_residual(int64_t nslice, const int64_t* __restrict__ ptr,
                                                   const int32_t* __restrict__ row0, const int32_t* __restrict__ nrow,
                                                   const int32_t* __restrict__ col, const T* __restrict__ val,
                                                   const T* __restrict__ diag, const T* x, const T* b, T* r,
-                                                  double* __restrict__ partial) {
+                                                  NormEnd end) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, part = warp % G;
   const int64_t s = (int64_t)blockIdx.x * (8 / G) + warp / G;
   const RowPart p = row_part<G>(s, nslice, ptr, row0, nrow, part, lane);
@@ -195,15 +246,17 @@ __global__ void __launch_bounds__(256) k_residual(int64_t nslice, const int64_t*
     r[p.row] = rv;
     sq = to_f64(rv) * to_f64(rv);
   }
-  if (partial) {  // fixed-shape block reduction of r^2
+  if constexpr (NORM) {
     __shared__ double red[256];
-    red[threadIdx.x] = sq;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-      if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-      __syncthreads();
+    block_sum_store(sq, red, end.partial + blockIdx.x);
+    if (last_block(end.counter)) {
+      const double v = block_final_sum(gridDim.x, end.partial, red);
+      if (threadIdx.x == 0) {
+        end.sc[S_RR] = v;
+        if (end.what == kNormStart) start_check(end.sc, end.hist);
+        if (end.what == kNormIter) iter_check(end.sc, end.it, end.hist, end.h);
+      }
     }
-    if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
   }
 }
 
@@ -346,59 +399,69 @@ __global__ void k_add_f2d(int64_t n, const float* e, double* x) {
   GRID_LOOP(i, n) x[i] += f64_of(e[i]);
 }
 
-// Deterministic dot product: fixed grid, fixed per-thread ranges, fixed tree.
-__global__ void __launch_bounds__(256) k_dot_partial(int64_t n, const double* a, const double* b, double* partial) {
+// The vectors of a solve in the level's numbering, bs = b[perm] and
+// xs = x[perm], ||b||^2 into sc[S_NB2], and the solve's tolerance, iteration
+// counter and limit: one launch instead of two gathers, two reduction kernels
+// and two copies from the host.  Sums: fixed grid (kRedBlocks x 256), fixed
+// per-thread ranges, fixed tree.
+__global__ void __launch_bounds__(256) k_load(int64_t n, const int32_t* __restrict__ perm,
+                                              const double* __restrict__ b, const double* __restrict__ x,
+                                              double* __restrict__ bs, double* __restrict__ xs,
+                                              double* __restrict__ partial, int* counter, double* sc, int* it,
+                                              double tol, int max_iter) {
   __shared__ double red[256];
   pdl_wait();
   pdl_trigger();
   double s = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) s += a[i] * b[i];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
+#pragma unroll 2
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+    const int32_t o = perm[i];
+    const double bi = b[o];
+    bs[i] = bi;
+    xs[i] = x[o];
+    s += bi * bi;
   }
-  if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
+  block_sum_store(s, red, partial + blockIdx.x);
+  if (last_block(counter)) {
+    const double v = block_final_sum(gridDim.x, partial, red);
+    if (threadIdx.x == 0) {
+      sc[S_NB2] = v;
+      sc[S_TOL] = tol;
+      it[0] = 0;
+      it[1] = max_iter;
+    }
+  }
 }
 
-// out = sum of `count` partials (one block of 256, fixed order).
-__global__ void k_reduce_final(int count, const double* partial, double* out) {
-  __shared__ double red[256];
+// The end of a device-driven solve: x[perm] = xs unless the start's test
+// failed, and the solve's report straight into pinned host memory (block 0):
+// the host reads it after the one synchronisation of the solve.
+__global__ void __launch_bounds__(256) k_store(int64_t n, const int32_t* __restrict__ perm,
+                                               const double* __restrict__ xs, double* __restrict__ x,
+                                               const double* sc, const int* it, const double* hist,
+                                               const int* status, double* rep) {
   pdl_wait();
   pdl_trigger();
-  const double v = block_final_sum(count, partial, red);
-  if (threadIdx.x == 0) *out = v;
+  if (blockIdx.x == 0) {
+    const int k = it[0];
+    if (threadIdx.x == 0) {
+      rep[REP_NB2] = sc[S_NB2];
+      rep[REP_RR] = sc[S_RR];
+      rep[REP_OK] = sc[S_OK];
+      rep[REP_ITERS] = k;
+      rep[REP_REL] = hist[k];
+      rep[REP_PIVOT] = status[1];
+      rep[REP_WAIT] = status[3];
+    }
+    for (int i = threadIdx.x; i <= k && i < REP_HIST_CAP; i += 256) rep[REP_HIST + i] = hist[i];
+  }
+  if (sc[S_OK] != 1.0) return;
+  GRID_LOOP(i, n) x[perm[i]] = xs[i];
 }
 
 // PCG scalars live on the device (slots S_*): r.z, p.Ap, the Polak-Ribiere
 // numerator z.(r - r_old), beta.
 //
-// Block sums in the fixed order of k_dot_partial (same grid, same per-thread
-// ranges, same tree), so the fused kernels below give the same bits as a
-// separate dot product.
-__device__ __forceinline__ void block_sum_store(double v, double* red, double* out) {
-  red[threadIdx.x] = v;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *out = red[0];
-}
-
-// The convergence test of the device-side loop (one thread): advances the
-// iteration counter it[0], records rel = ||r|| / ||b|| (same arithmetic as the
-// host test) and keeps the loop going while rel is finite, above the
-// tolerance and the counter below it[1].
-__device__ void iter_check(const double* sc, int* it, double* hist, cudaGraphConditionalHandle h) {
-  const int k = ++it[0];
-  const double rel = sqrt(sc[S_RR]) / sqrt(sc[S_NB2]);
-  hist[k] = rel;
-  const bool go = isfinite(rel) && !(rel <= sc[S_TOL]) && k < it[1];
-  cudaGraphSetConditional(h, go ? 1u : 0u);
-}
-
 // alpha = rz / pq; r_old = r; x += alpha p; r -= alpha q; rr = r.r into
 // sc[S_RR] (partials, finished by the last block); and the initial iterate of
 // the next preconditioning cycle MGI(0, r): with an FP32 cycle its right-hand
@@ -479,6 +542,29 @@ __global__ void __launch_bounds__(256) k_pcg_zdots(int64_t n, const Z* __restric
   }
 }
 
+// The start of CG, z = MGI(0, r) given: p = z and r.z into sc[S_RZ] (partials,
+// finished by the last block).  Grid: kRedBlocks x 256.
+template <class Z>
+__global__ void __launch_bounds__(256) k_pcg_first(int64_t n, const Z* __restrict__ z, const double* __restrict__ r,
+                                                   double* __restrict__ p, double* __restrict__ partial,
+                                                   int* counter, double* sc) {
+  __shared__ double red[256];
+  pdl_wait();
+  pdl_trigger();
+  double rz = 0.0;
+#pragma unroll 4
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+    const double zi = to_f64(z[i]);
+    p[i] = zi;
+    rz += r[i] * zi;
+  }
+  block_sum_store(rz, red, partial + blockIdx.x);
+  if (last_block(counter)) {
+    const double v = block_final_sum(gridDim.x, partial, red);
+    if (threadIdx.x == 0) sc[S_RZ] = v;
+  }
+}
+
 // p = z + beta p.
 template <class Z>
 __global__ void k_pcg_dir(int64_t n, const double* sc, const Z* __restrict__ z, double* __restrict__ p) {
@@ -494,11 +580,6 @@ __global__ void k_zero_c0(int64_t n, const double* r, double* z, const double* _
   pdl_wait();
   pdl_trigger();
   GRID_LOOP(i, n) z[i] = i < n0 ? (r[i] - 0.0) * dinv[i] : 0.0;
-}
-__global__ void k_copy(int64_t n, const double* a, double* b) {
-  pdl_wait();
-  pdl_trigger();
-  GRID_LOOP(i, n) b[i] = a[i];
 }
 
 // ------------------------------------------------------------------ launchers
@@ -533,24 +614,22 @@ gmg_status launch_gs_colour(Level& L, int colour, const T* b, T* x, cudaStream_t
   }
 }
 
-template <class T>
-static gmg_status launch_residual_p(Level& L, const T* x, const T* b, T* r, double* partial, cudaStream_t s,
-                                    int64_t* nblocks = nullptr) {
+template <class T, bool NORM>
+static gmg_status launch_residual_n(Level& L, const T* x, const T* b, T* r, const NormEnd& end, cudaStream_t s) {
   const int G = L.rlanes;
   const int64_t grid = (L.A.nslice + (8 / G) - 1) / (8 / G);
-  if (nblocks) *nblocks = grid;
   const Ell& A = L.A;
   switch (G) {
-    case 1: return launch(k_residual<T, 1>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, Vec<T>::v(A), Vec<T>::diag(L), x, b, r, partial);
-    case 2: return launch(k_residual<T, 2>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, Vec<T>::v(A), Vec<T>::diag(L), x, b, r, partial);
-    case 4: return launch(k_residual<T, 4>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, Vec<T>::v(A), Vec<T>::diag(L), x, b, r, partial);
-    default: return launch(k_residual<T, 8>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, Vec<T>::v(A), Vec<T>::diag(L), x, b, r, partial);
+    case 1: return launch(k_residual<T, 1, NORM>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, Vec<T>::v(A), Vec<T>::diag(L), x, b, r, end);
+    case 2: return launch(k_residual<T, 2, NORM>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, Vec<T>::v(A), Vec<T>::diag(L), x, b, r, end);
+    case 4: return launch(k_residual<T, 4, NORM>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, Vec<T>::v(A), Vec<T>::diag(L), x, b, r, end);
+    default: return launch(k_residual<T, 8, NORM>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, Vec<T>::v(A), Vec<T>::diag(L), x, b, r, end);
   }
 }
 
 template <class T>
 gmg_status launch_residual(Level& L, const T* x, const T* b, T* r, cudaStream_t s) {
-  return launch_residual_p<T>(L, x, b, r, nullptr, s);
+  return launch_residual_n<T, false>(L, x, b, r, NormEnd{}, s);
 }
 
 template <class T>
@@ -683,22 +762,17 @@ gmg_status launch_f2d(int64_t n, const float* a, double* b, cudaStream_t s) {
 
 // ------------------------------------------------------------------ outer iteration
 
-// rs = bs - A xs (FP64, finest level) and scal[slot] = ||rs||^2.
-static gmg_status outer_residual(gmg_ctx* c, int slot, cudaStream_t s) {
+// rs = bs - A xs (FP64, finest level) and sc[S_RR] = ||rs||^2, then `what`
+// (kNorm*) with the loop condition h.
+static gmg_status outer_residual(gmg_ctx* c, int what, cudaStream_t s, cudaGraphConditionalHandle h = 0) {
   Level& L = c->L[0];
   const int64_t blocks = (L.A.nslice + (8 / L.rlanes) - 1) / (8 / L.rlanes);
   if (blocks > c->red_cap) {
     set_error("outer residual: more blocks than reduction partials");
     return GMG_ERR_TOO_LARGE;
   }
-  int64_t nb = 0;
-  GMG_TRY(launch_residual_p<double>(L, c->xs, c->bs, c->rs, c->red, s, &nb));
-  return launch(k_reduce_final, 1, 256, s, (int)nb, (const double*)c->red, c->scal + slot);
-}
-
-static gmg_status dot(gmg_ctx* c, int64_t n, const double* a, const double* b, int slot, cudaStream_t s) {
-  GMG_TRY(launch(k_dot_partial, kRedBlocks, 256, s, n, a, b, c->red));
-  return launch(k_reduce_final, 1, 256, s, kRedBlocks, (const double*)c->red, c->scal + slot);
+  const NormEnd end{c->red, c->red_cnt + 4, c->scal, c->dloop, c->dhist, h, what};
+  return launch_residual_n<double, true>(L, c->xs, c->bs, c->rs, end, s);
 }
 
 // A finest-level V-cycle, bracketed by timing events when profiling is on;
@@ -713,20 +787,6 @@ static gmg_status timed_vcycle(gmg_ctx* c, cudaStream_t s, bool c0_done, T* x = 
 
 static bool pcg_mode(int mode) { return mode == GMG_FP32_PCG || mode == GMG_FP64_PCG; }
 
-// z = MGI(0, r) in the mode's cycle precision (FP64: z itself is the cycle's
-// iterate; FP32: widened from the finest level's x32).
-static gmg_status precond(gmg_ctx* c, int mode, const double* r, double* z, cudaStream_t s) {
-  Level& L = c->L[0];
-  const int64_t n0 = c->opt.nu_pre > 0 ? L.color_off[1] : 0;
-  if (mode == GMG_FP64_PCG) {
-    GMG_TRY(launch(k_zero_c0, blocks_for(L.n), 256, s, L.n, r, z, (const double*)L.dinv64, n0));
-    return timed_vcycle<double>(c, s, n0 > 0, z, r);
-  }
-  GMG_TRY(launch(k_d2f_zero, blocks_for(L.n), 256, s, L.n, r, L.b32, L.x32, (const float*)L.dinv32, n0));
-  GMG_TRY(timed_vcycle<float>(c, s, n0 > 0));
-  return launch_f2d(L.n, L.x32, z, s);
-}
-
 // One outer iteration (captured as a graph when enabled).
 //  FP64         : x <- MGI(x, b) (FP64 cycle on the iterate), r = b - A x, rr
 //  FP32_REFINE  : e = MGI32(0, r), x += e, r = b - A x, rr
@@ -739,14 +799,14 @@ gmg_status iteration_body(gmg_ctx* c, int mode, int seg, cudaStream_t s, cudaGra
   const int64_t n0 = c->opt.nu_pre > 0 ? L.color_off[1] : 0;
   if (mode == GMG_FP64) {
     GMG_TRY(timed_vcycle<double>(c, s, false));  // level-0 x64/b64 alias xs/bs
-    return outer_residual(c, S_RR, s);
+    return outer_residual(c, check ? kNormIter : kNormOnly, s, h);
   }
   if (mode == GMG_FP32_REFINE) {
     GMG_TRY(launch(k_d2f_zero, blocks_for(n), 256, s, n, (const double*)c->rs, L.b32, L.x32, (const float*)L.dinv32,
                    n0));
     GMG_TRY(timed_vcycle<float>(c, s, n0 > 0));
     GMG_TRY(launch(k_add_f2d, blocks_for(n), 256, s, n, (const float*)L.x32, c->xs));
-    return outer_residual(c, S_RR, s);
+    return outer_residual(c, check ? kNormIter : kNormOnly, s, h);
   }
   const bool f64 = mode == GMG_FP64_PCG;
   if (seg == 0) {
@@ -779,32 +839,44 @@ gmg_status iteration_body(gmg_ctx* c, int mode, int seg, cudaStream_t s, cudaGra
   return launch(k_pcg_dir<float>, blocks_for(n), 256, s, n, (const double*)c->scal, (const float*)L.x32, c->ps);
 }
 
-// PCG start: z = MGI(0, r), rz = r.z, p = z (r must be current).
+// PCG start: z = MGI(0, r) in the mode's cycle precision (FP64: zs is the
+// cycle's iterate, FP32: the finest level's x32), rz = r.z, p = z (r must be
+// current).
 gmg_status pcg_start(gmg_ctx* c, int mode, cudaStream_t s) {
-  const int64_t n = c->L[0].n;
-  GMG_TRY(precond(c, mode, c->rs, c->zs, s));
-  GMG_TRY(dot(c, n, c->rs, c->zs, S_RZ, s));
-  return launch(k_copy, blocks_for(n), 256, s, n, (const double*)c->zs, c->ps);
-}
-
-// Convergence test of the device-side loop as its own one-thread kernel (the
-// CG form runs it inside the last block of k_pcg_axpy instead).
-__global__ void k_iter_check(double* sc, int* it, double* hist, cudaGraphConditionalHandle h) {
-  pdl_wait();
-  pdl_trigger();
-  iter_check(sc, it, hist, h);
+  Level& L = c->L[0];
+  const int64_t n = L.n, n0 = c->opt.nu_pre > 0 ? L.color_off[1] : 0;
+  const double* r = c->rs;
+  if (mode == GMG_FP64_PCG) {
+    GMG_TRY(launch(k_zero_c0, blocks_for(n), 256, s, n, r, c->zs, (const double*)L.dinv64, n0));
+    GMG_TRY(timed_vcycle<double>(c, s, n0 > 0, c->zs, r));
+    return launch(k_pcg_first<double>, kRedBlocks, 256, s, n, (const double*)c->zs, r, c->ps, c->red, c->red_cnt + 2,
+                  c->scal);
+  }
+  GMG_TRY(launch(k_d2f_zero, blocks_for(n), 256, s, n, r, L.b32, L.x32, (const float*)L.dinv32, n0));
+  GMG_TRY(timed_vcycle<float>(c, s, n0 > 0));
+  return launch(k_pcg_first<float>, kRedBlocks, 256, s, n, (const float*)L.x32, r, c->ps, c->red, c->red_cnt + 2,
+                c->scal);
 }
 
 gmg_status loop_body(gmg_ctx* c, int mode, cudaGraphConditionalHandle h, cudaStream_t s) {
-  if (pcg_mode(mode)) {
-    GMG_TRY(iteration_body(c, mode, 1, s));
-    return iteration_body(c, mode, 0, s, h, true);
-  }
-  GMG_TRY(iteration_body(c, mode, 0, s));
-  return launch(k_iter_check, 1, 1, s, c->scal, c->dloop, c->dhist, h);
+  if (pcg_mode(mode)) GMG_TRY(iteration_body(c, mode, 1, s));
+  return iteration_body(c, mode, 0, s, h, true);
 }
 
-gmg_status outer_residual_norm(gmg_ctx* c, cudaStream_t s) { return outer_residual(c, S_RR, s); }
-gmg_status norm_b(gmg_ctx* c, cudaStream_t s) { return dot(c, c->L[0].n, c->bs, c->bs, S_NB2, s); }
+gmg_status outer_residual_norm(gmg_ctx* c, bool start, cudaStream_t s) {
+  return outer_residual(c, start ? kNormStart : kNormOnly, s);
+}
+
+gmg_status load_system(gmg_ctx* c, const double* b, const double* x, double tol, cudaStream_t s) {
+  Level& L = c->L[0];
+  return launch(k_load, kRedBlocks, 256, s, L.n, L.perm, b, x, c->bs, c->xs, c->red, c->red_cnt + 5, c->scal, c->dloop,
+                tol, c->opt.max_iter);
+}
+
+gmg_status store_solution(gmg_ctx* c, double* x, cudaStream_t s) {
+  Level& L = c->L[0];
+  return launch(k_store, blocks_for(L.n), 256, s, L.n, L.perm, (const double*)c->xs, x, (const double*)c->scal,
+                (const int*)c->dloop, (const double*)c->dhist, (const int*)c->dstatus, c->h_scal);
+}
 
 }  // namespace gmg

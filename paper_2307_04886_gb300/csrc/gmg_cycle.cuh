@@ -54,11 +54,24 @@ gmg_status launch_f2d(int64_t n, const float* a, double* b, cudaStream_t s);
 gmg_status iteration_body(gmg_ctx* c, int mode, int seg, cudaStream_t s, cudaGraphConditionalHandle h = 0,
                           bool check = false);
 gmg_status pcg_start(gmg_ctx* c, int mode, cudaStream_t s);
-gmg_status outer_residual_norm(gmg_ctx* c, cudaStream_t s);
-gmg_status norm_b(gmg_ctx* c, cudaStream_t s);
-enum { S_NB2 = 0, S_RR = 1, S_RZ = 2, S_PQ = 3, S_NUM = 4, S_RZN = 5, S_BETA = 6, S_TOL = 7 };
+// rs = b - A x and its squared norm into S_RR; with `start` also the test of a
+// solve's start (history entry 0 and S_OK).
+gmg_status outer_residual_norm(gmg_ctx* c, bool start, cudaStream_t s);
+// First launch of a solve: b and x (device, caller numbering) into the finest
+// level's bs and xs, ||b||^2, tolerance and iteration counters.
+gmg_status load_system(gmg_ctx* c, const double* b, const double* x, double tol, cudaStream_t s);
+// Last launch of a device-driven solve: xs into x (device, caller numbering)
+// if the start's test passed, and the report into h_scal (REP_* below).
+gmg_status store_solution(gmg_ctx* c, double* x, cudaStream_t s);
+// Device scalars (c->scal); slots 8 to 55 belong to the batched solve.
+enum { S_NB2 = 0, S_RR = 1, S_RZ = 2, S_PQ = 3, S_NUM = 4, S_RZN = 5, S_BETA = 6, S_TOL = 7, S_OK = 56 };
+// Report of a device-driven solve (pinned host memory): ||b||^2, the last true
+// ||r||^2, the start's test, iterations, relative residual of the last
+// iteration, status words of the coarsest inverse and of the bounded waits,
+// and the history's first entries.
+enum { REP_NB2 = 0, REP_RR = 1, REP_OK = 2, REP_ITERS = 3, REP_REL = 4, REP_PIVOT = 5, REP_WAIT = 6, REP_HIST = 64, REP_HIST_CAP = 64 };
 // One iteration of the device-side loop (PCG: segment 1 of the previous
-// iteration, then segment 0) followed by the convergence test that sets the
+// iteration, then segment 0), ending with the convergence test that sets the
 // loop's condition `h` (captured into the body of a WHILE node).
 gmg_status loop_body(gmg_ctx* c, int mode, cudaGraphConditionalHandle h, cudaStream_t s);
 gmg_status launch_gather(int64_t n, const int32_t* perm, const double* src, double* dst, cudaStream_t s);

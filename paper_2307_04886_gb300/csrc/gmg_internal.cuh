@@ -309,12 +309,14 @@ struct gmg_ctx {
   // captured iteration bodies, indexed by mode * 2 + segment
   cudaGraphExec_t graphs[8] = {};
   uint64_t graph_kernels[8] = {};  // kernel nodes of each captured graph
-  // device-side outer loop per mode: a graph whose conditional WHILE node
-  // repeats the iteration until the convergence test fails on the device
-  cudaGraphExec_t loops[4] = {};
-  uint64_t loop_kernels[4] = {};  // kernel nodes of one loop iteration
-  bool loop_refused[4] = {};      // instantiation failed: the host loop serves the mode
-  bool loop_pdl[4] = {};          // the loop body kept its programmatic launch edges
+  // device-driven solves per mode: graphs whose conditional WHILE node repeats
+  // the iteration until the convergence test fails on the device.  [mode][1]
+  // starts at the initial residual; [mode][0] (CG only) after the start's
+  // cycle, for a start that ran on the stream
+  cudaGraphExec_t loops[4][2] = {};
+  uint64_t loop_once[4][2] = {};     // kernel nodes outside the loop
+  uint64_t loop_kernels[4] = {};     // kernel nodes of one loop iteration
+  bool loop_refused[4] = {};         // instantiation failed: the host loop serves the mode
   // the same for the batched solve, by block width NR = 1, 2, 4, 8, 16
   cudaGraphExec_t mloops[5] = {};
   uint64_t mloop_kernels[5] = {};

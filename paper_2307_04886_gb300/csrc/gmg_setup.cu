@@ -1919,10 +1919,10 @@ gmg_status setup_impl(gmg_ctx* c, const gmg_csr* A, int nP, const gmg_prolong* P
   GMG_TRY(a.alloc(&c->red, (size_t)c->red_cap));
   GMG_TRY(a.alloc(&c->scal, 64));
   GMG_TRY(a.alloc(&c->dloop, 4));
-  GMG_TRY(a.alloc(&c->red_cnt, 4));
-  GMG_CK(cudaMemset(c->red_cnt, 0, 4 * sizeof(int)));
+  GMG_TRY(a.alloc(&c->red_cnt, 8));
+  GMG_CK(cudaMemset(c->red_cnt, 0, 8 * sizeof(int)));
   GMG_TRY(a.alloc(&c->dhist, (size_t)c->opt.max_iter + 2));
-  GMG_CK(cudaMallocHost((void**)&c->h_scal, 64 * sizeof(double)));
+  GMG_CK(cudaMallocHost((void**)&c->h_scal, 128 * sizeof(double)));
   lap(3, "gmg_setup: cluster tables");
   GMG_TRY(build_cluster(c, hrp, hcol, perm, iperm, P));
   for (Level& L : c->L) std::vector<int64_t>().swap(L.h_ptr);
