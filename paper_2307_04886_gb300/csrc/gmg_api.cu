@@ -404,6 +404,40 @@ struct SolveRun {
 
 using namespace gmg;
 
+namespace gmg {
+gmg_status new_handle(gmg_handle* h, const gmg_csr* A, int n_prolong, const gmg_prolong* P,
+                      const int32_t* const* coloring, const gmg_options* opt, bool single_rhs, void* stream) {
+  g_last_error.clear();
+  if (!h || n_prolong < 0 || (n_prolong > 0 && !P)) {
+    set_error("gmg_setup: null output handle or bad prolongation list");
+    return GMG_ERR_INVALID_ARG;
+  }
+  *h = nullptr;
+  gmg_ctx* c = new (std::nothrow) gmg_ctx();
+  if (!c) return GMG_ERR_OOM;
+  c->single_rhs = single_rhs;
+  if (opt) c->opt = *opt;
+  else gmg_default_options(&c->opt);
+  if (const char* e = std::getenv("GMG_NO_GRAPHS"))  // profilers list graph nodes slowly
+    if (e[0] == '1') c->opt.use_graphs = 0;
+  if (c->opt.nu_pre < 0 || c->opt.nu_post < 0 || c->opt.max_iter < 0 || c->opt.precision < GMG_FP64 ||
+      c->opt.precision > GMG_FP64_PCG) {
+    set_error("gmg_setup: invalid options");
+    delete c;
+    return GMG_ERR_INVALID_ARG;
+  }
+  gmg_status st = setup_impl(c, A, n_prolong, P, coloring, (cudaStream_t)stream);
+  if (st != GMG_OK) {
+    std::string keep = g_last_error;
+    gmg_destroy(c);
+    g_last_error = keep;
+    return st;
+  }
+  *h = c;
+  return GMG_OK;
+}
+}  // namespace gmg
+
 extern "C" {
 
 void gmg_default_options(gmg_options* opt) {
@@ -460,33 +494,7 @@ gmg_status gmg_destroy(gmg_handle h) {
 
 gmg_status gmg_setup(gmg_handle* h, const gmg_csr* A, int n_prolong, const gmg_prolong* P,
                      const int32_t* const* coloring, const gmg_options* opt, void* stream) {
-  g_last_error.clear();
-  if (!h || n_prolong < 0 || (n_prolong > 0 && !P)) {
-    set_error("gmg_setup: null output handle or bad prolongation list");
-    return GMG_ERR_INVALID_ARG;
-  }
-  *h = nullptr;
-  gmg_ctx* c = new (std::nothrow) gmg_ctx();
-  if (!c) return GMG_ERR_OOM;
-  if (opt) c->opt = *opt;
-  else gmg_default_options(&c->opt);
-  if (const char* e = std::getenv("GMG_NO_GRAPHS"))  // profilers list graph nodes slowly
-    if (e[0] == '1') c->opt.use_graphs = 0;
-  if (c->opt.nu_pre < 0 || c->opt.nu_post < 0 || c->opt.max_iter < 0 || c->opt.precision < GMG_FP64 ||
-      c->opt.precision > GMG_FP64_PCG) {
-    set_error("gmg_setup: invalid options");
-    delete c;
-    return GMG_ERR_INVALID_ARG;
-  }
-  gmg_status st = setup_impl(c, A, n_prolong, P, coloring, (cudaStream_t)stream);
-  if (st != GMG_OK) {
-    std::string keep = g_last_error;
-    gmg_destroy(c);
-    g_last_error = keep;
-    return st;
-  }
-  *h = c;
-  return GMG_OK;
+  return new_handle(h, A, n_prolong, P, coloring, opt, true, stream);
 }
 
 gmg_status gmg_set_values(gmg_handle h, const double* val, int mem, void* stream) {

@@ -1289,7 +1289,7 @@ extern "C" gmg_status gmg_setup_many(gmg_many* out, int nmesh, const gmg_csr* A,
   gmg_many_ctx* m = new gmg_many_ctx();
   for (int k = 0; k < nmesh; ++k) {
     gmg_handle h = nullptr;
-    gmg_status st = gmg_setup(&h, &A[k], n_prolong[k], P[k], nullptr, opt, stream);
+    gmg_status st = new_handle(&h, &A[k], n_prolong[k], P[k], nullptr, opt, false, stream);
     if (st == GMG_OK) st = ensure_batched(h);
     if (st != GMG_OK) {
       std::string keep = gmg_last_error();

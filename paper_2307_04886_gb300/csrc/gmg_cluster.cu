@@ -4,25 +4,25 @@
 // on a cluster of 16 CTAs.  Their colour phases are dependent and small (a
 // few hundred rows per CTA), so as grid launches each costs a kernel boundary
 // and a dependent L2 round trip (2.0-2.9 us measured) whatever its size; here
-// a phase is the row arithmetic from shared memory and a cluster barrier.
+// a phase is the row arithmetic from shared memory and a message to the CTAs
+// that read its rows.
 //
 // Rows of a level are split into contiguous ranges of its locality rank, one
 // per CTA, so that most neighbours of a row share its CTA and every range
 // holds about 1/16 of each colour.  A CTA keeps x of its own rows and of the
 // rows of other CTAs that it reads (its halo: neighbours, and the coarse
 // parents of its finer rows), b and 1/a_ii of its own rows, and the entries of
-// its rows as slices of 32 lanes with 16-bit local columns.  A row that other
-// CTAs read is stored into their halo copies through distributed shared
-// memory as it is updated.
+// its rows as slices of 32 lanes.  A row that other CTAs read is stored into
+// their halo copies through distributed shared memory as it is updated.
 //
 // What bounds a phase is its chain of dependent steps, not bandwidth, so the
 // chain is kept short:
 //  * a phase ends with a message, not a barrier: a halo store is an
 //    asynchronous remote store that completes on the receiving CTA's
-//    mbarrier, each CTA knows how many bytes a phase brings it, and its warps
-//    arrive on the same mbarrier, so one wait covers both (375 cycles per
-//    phase measured alone, against 660 for remote stores and a cluster
-//    barrier, whose release has to wait for the stores);
+//    mbarrier, each CTA knows how many bytes a phase brings it, and after its
+//    own block barrier it waits for those bytes (375 cycles per phase measured
+//    alone, against 660 for remote stores and a cluster barrier, whose release
+//    has to wait for the stores);
 //  * what does not depend on the phase before (slice descriptor, entries,
 //    b, 1/a_ii, list of halo stores) is loaded into registers before the wait;
 //  * an entry holds the shared-memory address of its x beside its value, two
@@ -53,9 +53,14 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
+#include <mutex>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "gmg_cycle.cuh"
@@ -959,44 +964,119 @@ void push_lists(const std::vector<int32_t>& owner, const std::vector<int32_t>& l
   }
 }
 
-// The tables of levels l0 .. lambda over ncta CTAs (host); false when a CTA would hold too many rows.
+// Runs f(0) .. f(n - 1) on as many threads as the work (in table entries) is
+// worth: a thread costs about 30 us to start, which some 20,000 entries take.
+// What a call throws is thrown again here, after every thread has ended.
+template <class F>
+void run_parts(int n, int64_t work, F f) {
+  const int hw = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+  const int m = (int)std::min<int64_t>({(int64_t)n, (int64_t)hw, 1 + work / 20000});
+  std::atomic<int> next{0};
+  std::exception_ptr err;
+  std::mutex lock;
+  auto work_on = [&] {
+    try {
+      for (int i = next++; i < n; i = next++) f(i);
+    } catch (...) {
+      std::lock_guard<std::mutex> g(lock);
+      err = std::current_exception();
+    }
+  };
+  std::vector<std::thread> th;
+  th.reserve(m);
+  for (int i = 1; i < m; ++i) {
+    try {
+      th.emplace_back(work_on);
+    } catch (const std::system_error&) {
+      break;  // no more threads: the others do the rest
+    }
+  }
+  work_on();
+  for (auto& x : th) x.join();
+  if (err) std::rethrow_exception(err);
+}
+
+// The tables of levels l0 .. lambda over ncta CTAs (host); false when a CTA
+// would hold too many rows.  The CTAs' parts are independent given the owners
+// and local indices of the rows, and so are the levels' halo lists: they are
+// built side by side.
 bool build_tables(gmg_ctx* c, int l0, int ncta, int per_unit, const std::vector<std::vector<int64_t>>& hrp,
                   const std::vector<std::vector<int32_t>>& hcol, const std::vector<std::vector<int32_t>>& perm,
                   const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P, std::vector<Tab>& tab) {
   const int lam = c->nlev - 1, nl = lam - l0;
   tab.assign(nl + 1, Tab());
-  for (int t = 0; t <= nl; ++t) {
-    const Level& L = c->L[l0 + t];
-    Tab& T = tab[t];
-    T.n = L.n;
-    T.ncolor = t < nl ? L.ncolor : 0;
-    T.part.assign(ncta, Part());
-    T.owner.resize(L.n);
-    T.local.resize(L.n);
-    for (int64_t r = 0; r < L.n; ++r) {
-      const int o = (int)((int64_t)L.h_key[perm[l0 + t][r]] * ncta / L.n);
-      T.owner[r] = o;
-      T.local[r] = (int32_t)T.part[o].own.size();
-      T.part[o].own.push_back((int32_t)r);  // ascending: colour by colour
-      if (L.color_off.size() > 1 && r < L.color_off[1]) T.part[o].own0++;
+  int64_t entries = 0, nmax = 0;
+  for (int t = 0; t < nl; ++t) entries += c->L[l0 + t].nnz;
+  // transposed prolongation from level t + 1's rows (fine rows ascending)
+  std::vector<std::vector<int64_t>> tptr(nl);
+  std::vector<std::vector<int32_t>> tcol(nl);
+  std::vector<std::vector<double>> tw(nl);
+  for (int t = 0; t <= nl; ++t) nmax = std::max(nmax, c->L[l0 + t].n);
+  run_parts(2 * nl + 1, entries, [&](int q) {
+    if (q <= nl) {
+      const int t = q;
+      const Level& L = c->L[l0 + t];
+      Tab& T = tab[t];
+      T.n = L.n;
+      T.ncolor = t < nl ? L.ncolor : 0;
+      T.part.assign(ncta, Part());
+      for (Part& p : T.part) p.own.reserve(L.n / ncta + 1);
+      T.owner.resize(L.n);
+      T.local.resize(L.n);
+      for (int64_t r = 0; r < L.n; ++r) {
+        const int o = (int)((int64_t)L.h_key[perm[l0 + t][r]] * ncta / L.n);
+        T.owner[r] = o;
+        T.local[r] = (int32_t)T.part[o].own.size();
+        T.part[o].own.push_back((int32_t)r);  // ascending: colour by colour
+        if (L.color_off.size() > 1 && r < L.color_off[1]) T.part[o].own0++;
+      }
+      const double rows = (double)L.n / (std::max(1, L.ncolor) * (double)ncta);
+      T.wide = rows >= kClWide;
+      T.tpr = T.wide ? 1 : lanes_per_row(rows, (double)(L.nnz - L.n) / (double)L.n);
+      return;
     }
-    const double rows = (double)L.n / (std::max(1, L.ncolor) * (double)ncta);
-    T.wide = rows >= kClWide;
-    T.tpr = T.wide ? 1 : lanes_per_row(rows, (double)(L.nnz - L.n) / (double)L.n);
-  }
-  std::vector<int32_t> loc, stamp;
-  for (int t = 0; t <= nl; ++t) {
-    Tab& T = tab[t];
-    const int l = l0 + t;
-    const int64_t *rp = hrp[l].data();
-    const int32_t *ci = hcol[l].data(), *pm = perm[l].data(), *ip = iperm[l].data();
-    loc.assign(T.n, 0);
-    stamp.assign(T.n, -1);
-    for (int a = 0; a < ncta; ++a) {
+    const int t = q - nl - 1, l = l0 + t;
+    const gmg_prolong& p = P[l];
+    const int64_t nf = c->L[l].n, nn = c->L[l + 1].n;
+    auto& cnt = tptr[t];
+    cnt.assign(nn + 1, 0);
+    for (int64_t r = 0; r < nf; ++r)
+      for (int s = 0; s < 3; ++s)
+        if (p.w[3 * r + s] != 0.0) cnt[iperm[l + 1][p.idx[3 * r + s]] + 1]++;
+    for (int64_t J = 0; J < nn; ++J) cnt[J + 1] += cnt[J];
+    tcol[t].resize(cnt[nn]);
+    tw[t].resize(cnt[nn]);
+    std::vector<int64_t> fill(cnt.begin(), cnt.end() - 1);
+    for (int64_t r = 0; r < nf; ++r) {
+      const int64_t old = perm[l][r];
+      for (int s = 0; s < 3; ++s)
+        if (p.w[3 * old + s] != 0.0) {
+          const int64_t at = fill[iperm[l + 1][p.idx[3 * old + s]]]++;
+          tcol[t][at] = (int32_t)r;
+          tw[t][at] = p.w[3 * old + s];
+        }
+    }
+  });
+  for (int t = 0; t < nl; ++t)
+    tab[t].r_tpr = tab[t].wide ? 1
+                               : lanes_per_row((double)tab[t + 1].n / ncta,
+                                               (double)tptr[t].back() / (double)tab[t + 1].n);
+  std::atomic<bool> fits{true};
+  run_parts(ncta, 2 * entries, [&](int a) {
+    std::vector<int32_t> loc, stamp;
+    loc.reserve(nmax);
+    stamp.reserve(nmax);
+    for (int t = 0; t <= nl; ++t) {
+      Tab& T = tab[t];
+      const int l = l0 + t;
+      const int64_t *rp = hrp[l].data();
+      const int32_t *ci = hcol[l].data(), *pm = perm[l].data(), *ip = iperm[l].data();
+      loc.resize(T.n);  // read only where written below
+      stamp.assign(T.n, 0);
       Part& p = T.part[a];
       auto see = [&](int32_t r) {
-        if (T.owner[r] != a && stamp[r] != a) {
-          stamp[r] = a;
+        if (T.owner[r] != a && !stamp[r]) {
+          stamp[r] = 1;
           p.halo.push_back(r);
         }
       };
@@ -1010,7 +1090,10 @@ bool build_tables(gmg_ctx* c, int l0, int ncta, int per_unit, const std::vector<
             if (P[l - 1].w[3 * old + s] != 0.0) see(ip[P[l - 1].idx[3 * old + s]]);
         }
       std::sort(p.halo.begin(), p.halo.end());
-      if ((int)(p.own.size() + p.halo.size()) >= kClMaxLocal) return false;
+      if ((int)(p.own.size() + p.halo.size()) >= kClMaxLocal) {
+        fits = false;
+        return;
+      }
       for (size_t q = 0; q < p.halo.size(); ++q) loc[p.halo[q]] = (int32_t)(p.own.size() + q);
       auto at = [&](int32_t r) { return T.owner[r] == a ? T.local[r] : loc[r]; };
       if (t > 0) {  // prolongation slots of the finer level's own rows
@@ -1027,118 +1110,98 @@ bool build_tables(gmg_ctx* c, int l0, int ncta, int per_unit, const std::vector<
             }
         }
       }
-      if (t < nl) {  // entries in the order of the level's sliced ELL, tpr lanes per row
-        const Level& L = c->L[l];
-        const int per = 32 / T.tpr;
-        auto len = [&](int i) { return (int)(rp[pm[p.own[i]] + 1] - rp[pm[p.own[i]]] - 1); };
-        int i0 = 0;
-        for (int k = 0; k < T.ncolor; ++k) {
-          p.csl.push_back((int32_t)p.sl.size());
-          p.blk.push_back((int32_t)(p.ecol.size() / per_unit));
-          p.rows0.push_back(i0);
-          int i1 = i0;
-          while (i1 < (int)p.own.size() && p.own[i1] < L.color_off[k + 1]) ++i1;
-          cut_slices(i0, i1, per, T.tpr, per_unit, true, len, [&](int r0, int nr, int w) {
-            const size_t base = p.ecol.size();  // entry slots before this slice
-            p.sl.push_back({r0 | (nr << 16), w, (int32_t)(base / per_unit), 0});
-            p.ecol.resize(base + 32 * (size_t)w * per_unit, 0);
-            p.esrc.resize(base + 32 * (size_t)w * per_unit, -1);
-            for (int q = 0; q < nr; ++q) {
-              const int32_t r = p.own[r0 + q];
-              const int64_t old = pm[r];
-              const int64_t slice = L.color_slice_off[k] + (r - L.color_off[k]) / kSlice;
-              int64_t slot = L.h_ptr[slice] + (r - L.color_off[k]) % kSlice;
-              // entry m of the row: lane part m mod tpr, unit (m / tpr) / per_unit, slot (m / tpr) % per_unit
-              auto at_slot = [&](int m) {
-                const int u = m / T.tpr;
-                return base + (32 * (size_t)(u / per_unit) + q * T.tpr + m % T.tpr) * per_unit + u % per_unit;
-              };
-              int m = 0;
-              for (int64_t e = rp[old]; e < rp[old + 1]; ++e) {
-                if (ci[e] == old) continue;
-                const size_t g = at_slot(m);
-                p.ecol[g] = (uint16_t)at(ip[ci[e]]);
-                p.esrc[g] = (int32_t)slot;
-                slot += kSlice;
-                ++m;
-              }
-              for (; m < T.tpr * w * per_unit; ++m) p.ecol[at_slot(m)] = (uint16_t)(r0 + q);  // padding: itself, value 0
-            }
-          });
-          i0 = i1;
-          T.blk = std::max(T.blk, (int)(p.ecol.size() / per_unit) - p.blk.back());
-        }
+      if (t == nl) continue;
+      // entries in the order of the level's sliced ELL, tpr lanes per row
+      const Level& L = c->L[l];
+      const int per = 32 / T.tpr;
+      auto len = [&](int i) { return (int)(rp[pm[p.own[i]] + 1] - rp[pm[p.own[i]]] - 1); };
+      const size_t guess = (size_t)(1.25 * (double)(L.nnz - L.n) / ncta);
+      p.ecol.reserve(guess);
+      p.esrc.reserve(guess);
+      int i0 = 0;
+      for (int k = 0; k < T.ncolor; ++k) {
         p.csl.push_back((int32_t)p.sl.size());
         p.blk.push_back((int32_t)(p.ecol.size() / per_unit));
         p.rows0.push_back(i0);
-        p.hcol.assign(T.ncolor, 0);
-        int k = 0;
-        for (int32_t r : p.halo) {  // ascending: colour by colour
-          while (r >= L.color_off[k + 1]) ++k;
-          p.hcol[k]++;
-        }
-      }
-    }
-    push_lists(T.owner, T.local, T.part, false);
-  }
-  // restriction: the own coarse rows gather the residual (fine rows ascending)
-  for (int t = 0; t < nl; ++t) {
-    Tab &F = tab[t], &N = tab[t + 1];
-    const int l = l0 + t;
-    const gmg_prolong& p = P[l];
-    std::vector<int64_t> cnt(N.n + 1, 0);
-    for (int64_t r = 0; r < F.n; ++r) {
-      const int64_t old = perm[l][r];
-      for (int s = 0; s < 3; ++s)
-        if (p.w[3 * old + s] != 0.0) cnt[iperm[l + 1][p.idx[3 * old + s]] + 1]++;
-    }
-    for (int64_t J = 0; J < N.n; ++J) cnt[J + 1] += cnt[J];
-    std::vector<int32_t> tcol(cnt[N.n]);
-    std::vector<double> tw(cnt[N.n]);
-    {
-      std::vector<int64_t> fill(cnt.begin(), cnt.end() - 1);
-      for (int64_t r = 0; r < F.n; ++r) {
-        const int64_t old = perm[l][r];
-        for (int s = 0; s < 3; ++s)
-          if (p.w[3 * old + s] != 0.0) {
-            const int64_t q = fill[iperm[l + 1][p.idx[3 * old + s]]]++;
-            tcol[q] = (int32_t)r;
-            tw[q] = p.w[3 * old + s];
+        int i1 = i0;
+        while (i1 < (int)p.own.size() && p.own[i1] < L.color_off[k + 1]) ++i1;
+        cut_slices(i0, i1, per, T.tpr, per_unit, true, len, [&](int r0, int nr, int w) {
+          const size_t base = p.ecol.size();  // entry slots before this slice
+          p.sl.push_back({r0 | (nr << 16), w, (int32_t)(base / per_unit), 0});
+          p.ecol.resize(base + 32 * (size_t)w * per_unit, 0);
+          p.esrc.resize(base + 32 * (size_t)w * per_unit, -1);
+          for (int q = 0; q < nr; ++q) {
+            const int32_t r = p.own[r0 + q];
+            const int64_t old = pm[r];
+            const int64_t slice = L.color_slice_off[k] + (r - L.color_off[k]) / kSlice;
+            int64_t slot = L.h_ptr[slice] + (r - L.color_off[k]) % kSlice;
+            // entry m of the row: lane part m mod tpr, unit (m / tpr) / per_unit, slot (m / tpr) % per_unit
+            auto at_slot = [&](int m) {
+              const int u = m / T.tpr;
+              return base + (32 * (size_t)(u / per_unit) + q * T.tpr + m % T.tpr) * per_unit + u % per_unit;
+            };
+            int m = 0;
+            for (int64_t e = rp[old]; e < rp[old + 1]; ++e) {
+              if (ci[e] == old) continue;
+              const size_t g = at_slot(m);
+              p.ecol[g] = (uint16_t)at(ip[ci[e]]);
+              p.esrc[g] = (int32_t)slot;
+              slot += kSlice;
+              ++m;
+            }
+            for (; m < T.tpr * w * per_unit; ++m) p.ecol[at_slot(m)] = (uint16_t)(r0 + q);  // padding: itself, value 0
           }
+        });
+        i0 = i1;
       }
-    }
-    F.r_tpr = F.wide ? 1 : lanes_per_row((double)N.n / ncta, (double)cnt[N.n] / (double)N.n);
-    loc.assign(F.n, 0);
-    stamp.assign(F.n, -1);
-    for (int a = 0; a < ncta; ++a) {
-      Part &f = F.part[a], &n = N.part[a];
-      for (int32_t J : n.own)
+      p.csl.push_back((int32_t)p.sl.size());
+      p.blk.push_back((int32_t)(p.ecol.size() / per_unit));
+      p.rows0.push_back(i0);
+      p.hcol.assign(T.ncolor, 0);
+      int k = 0;
+      for (int32_t r : p.halo) {  // ascending: colour by colour
+        while (r >= L.color_off[k + 1]) ++k;
+        p.hcol[k]++;
+      }
+      // restriction: the own coarse rows gather the residual (fine rows ascending)
+      const std::vector<int64_t>& cnt = tptr[t];
+      const std::vector<int32_t>& tc = tcol[t];
+      const std::vector<int32_t>& coarse = tab[t + 1].part[a].own;
+      stamp.assign(T.n, 0);
+      for (int32_t J : coarse)
         for (int64_t q = cnt[J]; q < cnt[J + 1]; ++q)
-          if (F.owner[tcol[q]] != a && stamp[tcol[q]] != a) {
-            stamp[tcol[q]] = a;
-            f.rhalo.push_back(tcol[q]);
+          if (T.owner[tc[q]] != a && !stamp[tc[q]]) {
+            stamp[tc[q]] = 1;
+            p.rhalo.push_back(tc[q]);
           }
-      std::sort(f.rhalo.begin(), f.rhalo.end());
-      if ((int)(f.own.size() + f.rhalo.size()) >= kClMaxLocal) return false;
-      for (size_t q = 0; q < f.rhalo.size(); ++q) loc[f.rhalo[q]] = (int32_t)(f.own.size() + q);
-      auto len = [&](int i) { return (int)(cnt[n.own[i] + 1] - cnt[n.own[i]]); };
-      cut_slices(0, (int)n.own.size(), 32 / F.r_tpr, F.r_tpr, 1, false, len, [&](int r0, int nr, int w) {
-        const size_t base = f.rcol.size();
-        f.rsl.push_back({r0 | (nr << 16), w, (int32_t)base, 0});
-        f.rcol.resize(base + 32 * (size_t)w, 0);
-        f.rw.resize(base + 32 * (size_t)w, 0.0);
+      std::sort(p.rhalo.begin(), p.rhalo.end());
+      if ((int)(p.own.size() + p.rhalo.size()) >= kClMaxLocal) {
+        fits = false;
+        return;
+      }
+      for (size_t q = 0; q < p.rhalo.size(); ++q) loc[p.rhalo[q]] = (int32_t)(p.own.size() + q);
+      auto rlen = [&](int i) { return (int)(cnt[coarse[i] + 1] - cnt[coarse[i]]); };
+      cut_slices(0, (int)coarse.size(), 32 / T.r_tpr, T.r_tpr, 1, false, rlen, [&](int r0, int nr, int w) {
+        const size_t base = p.rcol.size();
+        p.rsl.push_back({r0 | (nr << 16), w, (int32_t)base, 0});
+        p.rcol.resize(base + 32 * (size_t)w, 0);
+        p.rw.resize(base + 32 * (size_t)w, 0.0);
         for (int q = 0; q < nr; ++q) {
           int m = 0;
-          for (int64_t k = cnt[n.own[r0 + q]]; k < cnt[n.own[r0 + q] + 1]; ++k, ++m) {
-            const size_t g = base + 32 * (size_t)(m / F.r_tpr) + q * F.r_tpr + m % F.r_tpr;
-            f.rcol[g] = (uint16_t)(F.owner[tcol[k]] == a ? F.local[tcol[k]] : loc[tcol[k]]);
-            f.rw[g] = tw[k];
+          for (int64_t e = cnt[coarse[r0 + q]]; e < cnt[coarse[r0 + q] + 1]; ++e, ++m) {
+            const size_t g = base + 32 * (size_t)(m / T.r_tpr) + q * T.r_tpr + m % T.r_tpr;
+            p.rcol[g] = (uint16_t)(T.owner[tc[e]] == a ? T.local[tc[e]] : loc[tc[e]]);
+            p.rw[g] = tw[t][e];
           }
         }
       });
     }
-    push_lists(F.owner, F.local, F.part, true);
-  }
+  });
+  if (!fits) return false;
+  run_parts(2 * nl + 1, entries / 4, [&](int q) {
+    Tab& T = tab[q / 2];
+    push_lists(T.owner, T.local, T.part, q % 2 != 0);
+  });
   // partners: the CTAs that send a CTA values on some level, or that it sends to
   std::vector<char> ex((size_t)ncta * ncta, 0);
   for (int t = 0; t <= nl; ++t)
@@ -1160,15 +1223,16 @@ bool build_tables(gmg_ctx* c, int l0, int ncta, int per_unit, const std::vector<
       T.nrd = std::max(T.nrd, (int)p.rd.size());
       T.ent = std::max(T.ent, (int)(p.ecol.size() / per_unit));
       T.r_max = std::max(T.r_max, (int)p.rcol.size());
+      for (size_t k = 0; k + 1 < p.blk.size(); ++k) T.blk = std::max(T.blk, p.blk[k + 1] - p.blk[k]);
     }
   return true;
 }
 
 // Every index the kernel uses: columns and halo stores in range, each halo
 // copy written by its row's owner exactly once, slices covering the rows.
-bool check_tables(const std::vector<Tab>& tab, int per_unit) {
+bool check_level(const std::vector<Tab>& tab, int per_unit, int t) {
   const int nl = (int)tab.size() - 1;
-  for (int t = 0; t <= nl; ++t) {
+  {
     const Tab& T = tab[t];
     for (int kind = 0; kind < (t < nl ? 2 : 1); ++kind) {
       std::vector<std::vector<int>> written(T.part.size());
@@ -1223,6 +1287,17 @@ bool check_tables(const std::vector<Tab>& tab, int per_unit) {
     }
   }
   return true;
+}
+
+bool check_tables(const std::vector<Tab>& tab, int per_unit) {
+  int64_t entries = 0;
+  for (const Tab& T : tab)
+    for (const Part& p : T.part) entries += (int64_t)p.ecol.size();
+  std::atomic<bool> ok{true};
+  run_parts((int)tab.size(), entries / 4, [&](int t) {
+    if (!check_level(tab, per_unit, t)) ok = false;
+  });
+  return ok;
 }
 
 int64_t al16(int64_t v) { return (v + 15) & ~(int64_t)15; }
@@ -1337,16 +1412,22 @@ struct Src<double> {
 };
 
 // Device arrays of one handle's tables, gathered in one host buffer so that
-// they take one allocation and one copy.
+// they take one allocation and one copy: the arrays are declared with add(),
+// then at() gives their places in the buffer.
 struct Blob {
   std::vector<char> h;
+  size_t size = 0;
   std::vector<std::pair<const void**, size_t>> ptrs;
   template <class U>
-  char* add(const U** d, size_t n) {  // n elements, zeroed; returns where to write them (valid until the next add)
-    const size_t o = (h.size() + 255) & ~(size_t)255;
-    h.resize(o + std::max<size_t>(n, 1) * sizeof(U));
+  size_t add(const U** d, size_t n) {  // n elements, zeroed
+    const size_t o = (size + 255) & ~(size_t)255;
+    size = o + std::max<size_t>(n, 1) * sizeof(U);
     ptrs.push_back({reinterpret_cast<const void**>(d), o});
-    return h.data() + o;
+    return o;
+  }
+  template <class U>
+  U* at(size_t o) {
+    return reinterpret_cast<U*>(h.data() + o);
   }
   gmg_status upload(Arena& a) {
     char* p;
@@ -1374,7 +1455,7 @@ int32_t first_store(const Part& p, int i) {
 // Lays the tables of `tab` out as D says and uploads them.
 template <class T>
 gmg_status upload_tables(gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>& D) {
-  constexpr int pu = sizeof(T) == 4 ? 2 : 1;  // entries per unit
+  constexpr size_t pu = sizeof(T) == 4 ? 2 : 1;  // entries per unit
   const int nl = (int)tab.size() - 1, ncta = D.ncta;
   Blob B;
   // streamed entries of all levels, CTA after CTA
@@ -1386,18 +1467,9 @@ gmg_status upload_tables(gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>
         s_off[t].push_back((uint32_t)units);
         units += p.ecol.size() / pu;
       }
-  {
-    char* u = B.add(&D.s_ent, units);
-    for (int t = 0; t < nl; ++t)
-      for (size_t q = 0; q < s_off[t].size(); ++q) fill_units<T>(tab[t].part[q], D.lv[t].o_x, u + 16 * (size_t)s_off[t][q]);
-    char* src = B.add(&D.s_src, units * pu);
-    for (int t = 0; t < nl; ++t)
-      for (size_t q = 0; q < s_off[t].size(); ++q) {
-        const Part& p = tab[t].part[q];
-        std::memcpy(src + 4 * pu * (size_t)s_off[t][q], p.esrc.data(), 4 * p.esrc.size());
-        D.lv[t].n_stream += (int64_t)p.esrc.size();
-      }
-  }
+  for (int t = 0; t < nl; ++t)
+    if (D.lv[t].streamed)
+      for (const Part& p : tab[t].part) D.lv[t].n_stream += (int64_t)p.esrc.size();
   // the stream steps in the kernel's order; the first phase of level l0 has
   // one (the kernel skips it when colour 0 is done), that of a coarser level,
   // done by the restriction, has none
@@ -1421,18 +1493,43 @@ gmg_status upload_tables(gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>
     for (int q = 0; q < D.nu_post * C; ++q) step(t, D.post_forward ? q % C : C - 1 - q % C);
   }
   D.nsteps = (int)(steps[0].size() / 2);
+  const size_t o_ent = B.add(&D.s_ent, units), o_src = B.add(&D.s_src, units * pu);
+  struct Off {
+    size_t img, vi, ds, vs, rsl, rc, rw, pi, pw;
+  };
+  std::vector<Off> off(nl + 1);
+  size_t o_l2g = 0;
+  int64_t entries = 0;
   for (int t = 0; t <= nl; ++t) {
-    const Tab& A = tab[t];
     ClusterLevel<T>& L = D.lv[t];
-    const bool res = t < nl && !L.streamed;
-    const size_t S = sizeof(T), no = (size_t)L.n_own_max;
-    char* img = B.add(&L.img, (size_t)ncta * L.img_bytes);
-    for (int q = 0; q < ncta; ++q) {
+    const size_t no = (size_t)ncta * L.n_own_max;
+    off[t].img = B.add(&L.img, (size_t)ncta * L.img_bytes);
+    if (t == 0) o_l2g = B.add(&D.l2g, (size_t)ncta * L.n_loc_max);
+    if (t == nl) break;
+    const int64_t ent = L.streamed ? 0 : (int64_t)tab[t].ent * pu;
+    L.n_ent = ent;
+    L.nvsrc = ncta * ent;
+    entries += c->L[D.l0 + t].nnz;
+    off[t].vi = B.add(&L.vimg, (size_t)ncta * L.val_bytes);
+    off[t].ds = B.add(&L.dsrc, no);
+    off[t].vs = B.add(&L.vsrc, (size_t)L.nvsrc);
+    off[t].rsl = B.add(&L.r_sl, (size_t)ncta * L.rsl_max);
+    off[t].rc = B.add(&L.r_col, (size_t)ncta * L.r_max);
+    off[t].rw = B.add(&L.r_w, (size_t)ncta * L.r_max);
+    off[t].pi = B.add(&L.p_idx, 3 * no);
+    off[t].pw = B.add(&L.p_w, 3 * no);
+  }
+  B.h.resize(B.size);
+  // each CTA's part of every array
+  run_parts(ncta, entries, [&](int q) {
+    for (int t = 0; t <= nl; ++t) {
+      const Tab& A = tab[t];
+      const ClusterLevel<T>& L = D.lv[t];
       const Part& p = A.part[q];
-      const size_t m = p.own.size();
-      char* base = img + (size_t)q * L.img_bytes;
-      auto put = [&](int off, const void* v, size_t bytes) {
-        if (bytes) std::memcpy(base + off, v, bytes);
+      const size_t S = sizeof(T), no = (size_t)L.n_own_max, m = p.own.size();
+      char* base = B.at<char>(off[t].img) + (size_t)q * L.img_bytes;
+      auto put = [&](int at, const void* v, size_t bytes) {
+        if (bytes) std::memcpy(base + at, v, bytes);
       };
       int32_t hd[16] = {(int32_t)m, (int32_t)(m + p.halo.size()), (int32_t)p.sl.size(), (int32_t)p.rsl.size(), p.own0};
       hd[9] = (int32_t)p.xd.size();
@@ -1458,82 +1555,62 @@ gmg_status upload_tables(gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>
         hd[8] = (int32_t)tab[nl].part[q].own.size();
         put(D.i_partners, A.partners[q].data(), 4 * A.partners[q].size());
         put(D.i_steps, steps[q].data(), 4 * steps[q].size());
+        int32_t* l2g = B.at<int32_t>(o_l2g) + (size_t)q * L.n_loc_max;
+        std::copy(p.own.begin(), p.own.end(), l2g);
+        std::copy(p.halo.begin(), p.halo.end(), l2g + m);
       }
       put(0, hd, sizeof(hd));
       put(L.i_ex, ex, sizeof(ex));
       put(L.i_sl, p.sl.data(), p.sl.size() * sizeof(Slice));
-      if (L.streamed)  // entry offsets within the colour's block
-        for (int k = 0; k < A.ncolor; ++k)
-          for (int s = p.csl[k]; s < p.csl[k + 1]; ++s) reinterpret_cast<Slice*>(base + L.i_sl)[s].z -= p.blk[k];
       if (t == nl) put(L.i_cr, p.own.data(), m * 4);
       // halo stores in row order
-      auto put_list = [&](int off, const std::vector<uint32_t>& lp, const std::vector<uint32_t>& ld) {
-        uint32_t* o = reinterpret_cast<uint32_t*>(base + off);
+      auto put_list = [&](int at, const std::vector<uint32_t>& lp, const std::vector<uint32_t>& ld) {
+        uint32_t* o = reinterpret_cast<uint32_t*>(base + at);
         for (size_t i = 0; i < lp.size(); ++i)
-          for (uint32_t q = 0; q < (lp[i] & 15u); ++q) {
-            const uint32_t d = ld[(lp[i] >> 4) + q];  // CTA << 16 | local index there
+          for (uint32_t e = 0; e < (lp[i] & 15u); ++e) {
+            const uint32_t d = ld[(lp[i] >> 4) + e];  // CTA << 16 | local index there
             *o++ = (d >> 16) << 28 | (d & 0xFFFFu) << 14 | (uint32_t)i;
           }
       };
       put_list(L.i_xd, p.xp, p.xd);
       if (t < nl) put_list(L.i_rd, p.rp, p.rd);
+      Slice* sl = reinterpret_cast<Slice*>(base + L.i_sl);
+      if (L.streamed)  // entry offsets within the colour's block
+        for (int k = 0; k < A.ncolor; ++k)
+          for (int s = p.csl[k]; s < p.csl[k + 1]; ++s) sl[s].z -= p.blk[k];
       for (size_t s = 0; s < p.sl.size(); ++s) {  // the slices' halo stores
         const int r0 = p.sl[s].x & 0xFFFF, r1 = r0 + (p.sl[s].x >> 16);
-        reinterpret_cast<Slice*>(base + L.i_sl)[s].w = (first_store(p, r0) << 10) | (first_store(p, r1) - first_store(p, r0));
-        reinterpret_cast<Slice*>(base + L.i_sl)[s].y /= 2;  // pairs of units
+        sl[s].w = (first_store(p, r0) << 10) | (first_store(p, r1) - first_store(p, r0));
+        sl[s].y /= 2;  // pairs of units
       }
-    }
-    if (t == 0) {
-      int32_t* l2g = reinterpret_cast<int32_t*>(B.add(&D.l2g, (size_t)ncta * L.n_loc_max));
-      for (int q = 0; q < ncta; ++q) {
-        const Part& p = A.part[q];
-        std::copy(p.own.begin(), p.own.end(), l2g + (size_t)q * L.n_loc_max);
-        std::copy(p.halo.begin(), p.halo.end(), l2g + (size_t)q * L.n_loc_max + p.own.size());
-      }
-    }
-    if (t == nl) continue;
-    char* vi = B.add(&L.vimg, (size_t)ncta * L.val_bytes);
-    if (res)
-      for (int q = 0; q < ncta; ++q) {
-        char* u = vi + (size_t)q * L.val_bytes + L.v_ent;
+      if (t == nl) continue;
+      int32_t* ds = B.at<int32_t>(off[t].ds) + (size_t)q * no;
+      std::fill(ds, ds + no, -1);
+      for (size_t i = 0; i < m; ++i) ds[i] = -2 - p.own[i];
+      if (L.streamed) {
+        fill_units<T>(p, L.o_x, B.at<char>(o_ent) + 16 * (size_t)s_off[t][q]);
+        std::copy(p.esrc.begin(), p.esrc.end(), B.at<int32_t>(o_src) + pu * (size_t)s_off[t][q]);
+      } else {
+        char* u = B.at<char>(off[t].vi) + (size_t)q * L.val_bytes + L.v_ent;
         const uint32_t pad = (uint32_t)L.o_x;  // units past a CTA's own are never read; give them a valid address
-        for (size_t e = 0; e < (size_t)A.ent * pu; ++e) std::memcpy(u + (pu == 2 ? 8 * e + 4 : 16 * e + 8), &pad, 4);
-        fill_units<T>(A.part[q], L.o_x, u);
+        for (size_t e = p.ecol.size(); e < (size_t)A.ent * pu; ++e)
+          std::memcpy(u + (pu == 2 ? 8 * e + 4 : 16 * e + 8), &pad, 4);
+        fill_units<T>(p, L.o_x, u);
+        int32_t* vs = B.at<int32_t>(off[t].vs) + (size_t)q * L.n_ent;
+        std::fill(std::copy(p.esrc.begin(), p.esrc.end(), vs), vs + L.n_ent, -1);
       }
-    int32_t* ds = reinterpret_cast<int32_t*>(B.add(&L.dsrc, (size_t)ncta * no));
-    std::fill(ds, ds + (size_t)ncta * no, -1);
-    for (int q = 0; q < ncta; ++q)
-      for (size_t i = 0; i < A.part[q].own.size(); ++i) ds[(size_t)q * no + i] = -2 - A.part[q].own[i];
-    L.nvsrc = res ? (int64_t)ncta * A.ent * pu : 0;
-    L.n_ent = res ? (int64_t)A.ent * pu : 0;
-    int32_t* vs = reinterpret_cast<int32_t*>(B.add(&L.vsrc, (size_t)L.nvsrc));
-    if (res) {
-      std::fill(vs, vs + L.nvsrc, -1);
-      for (int q = 0; q < ncta; ++q)
-        std::copy(A.part[q].esrc.begin(), A.part[q].esrc.end(), vs + (size_t)q * A.ent * pu);
+      std::copy(p.rsl.begin(), p.rsl.end(), B.at<Slice>(off[t].rsl) + (size_t)q * L.rsl_max);
+      std::copy(p.rcol.begin(), p.rcol.end(), B.at<uint16_t>(off[t].rc) + (size_t)q * L.r_max);
+      T* rw = B.at<T>(off[t].rw) + (size_t)q * L.r_max;
+      for (size_t e = 0; e < p.rw.size(); ++e) rw[e] = (T)p.rw[e];
+      for (int s = 0; s < 3; ++s) {
+        std::copy(p.pidx.begin() + s * m, p.pidx.begin() + (s + 1) * m,
+                  B.at<uint16_t>(off[t].pi) + ((size_t)q * 3 + s) * no);
+        T* pw = B.at<T>(off[t].pw) + ((size_t)q * 3 + s) * no;
+        for (size_t i = 0; i < m; ++i) pw[i] = (T)p.pw[s * m + i];
+      }
     }
-    Slice* rsl = reinterpret_cast<Slice*>(B.add(&L.r_sl, (size_t)ncta * L.rsl_max));
-    for (int q = 0; q < ncta; ++q)
-      std::copy(A.part[q].rsl.begin(), A.part[q].rsl.end(), rsl + (size_t)q * L.rsl_max);
-    uint16_t* rc = reinterpret_cast<uint16_t*>(B.add(&L.r_col, (size_t)ncta * L.r_max));
-    for (int q = 0; q < ncta; ++q)
-      std::copy(A.part[q].rcol.begin(), A.part[q].rcol.end(), rc + (size_t)q * L.r_max);
-    T* rw = reinterpret_cast<T*>(B.add(&L.r_w, (size_t)ncta * L.r_max));
-    for (int q = 0; q < ncta; ++q)
-      for (size_t e = 0; e < A.part[q].rw.size(); ++e) rw[(size_t)q * L.r_max + e] = (T)A.part[q].rw[e];
-    uint16_t* pi = reinterpret_cast<uint16_t*>(B.add(&L.p_idx, (size_t)ncta * 3 * no));
-    for (int q = 0; q < ncta; ++q)
-      for (int s = 0; s < 3; ++s) {
-        const size_t m = A.part[q].own.size();
-        std::copy(A.part[q].pidx.begin() + s * m, A.part[q].pidx.begin() + (s + 1) * m, pi + ((size_t)q * 3 + s) * no);
-      }
-    T* pw = reinterpret_cast<T*>(B.add(&L.p_w, (size_t)ncta * 3 * no));
-    for (int q = 0; q < ncta; ++q)
-      for (int s = 0; s < 3; ++s) {
-        const size_t m = A.part[q].own.size();
-        for (size_t i = 0; i < m; ++i) pw[((size_t)q * 3 + s) * no + i] = (T)A.part[q].pw[s * m + i];
-      }
-  }
+  });
   return B.upload(c->arena);
 }
 
@@ -1644,9 +1721,10 @@ gmg_status refresh_one(gmg_ctx* c, cudaStream_t s) {
 gmg_status build_cluster(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
                          const std::vector<std::vector<int32_t>>& hcol, const std::vector<std::vector<int32_t>>& perm,
                          const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P) {
+  c->cl32.l0 = c->cl64.l0 = -1;
+  if (!c->single_rhs) return GMG_OK;
   GMG_TRY(build_one<float>(c, hrp, hcol, perm, iperm, P));
   // FP64 cycles in a solve: the modes that run them
-  c->cl64.l0 = -1;
   if (c->opt.precision == GMG_FP64 || c->opt.precision == GMG_FP64_PCG)
     GMG_TRY(build_one<double>(c, hrp, hcol, perm, iperm, P));
   return GMG_OK;

@@ -11,6 +11,10 @@ namespace gmg {
 gmg_status numeric_setup(gmg_ctx* c, cudaStream_t s, bool defer = false);
 gmg_status setup_impl(gmg_ctx* c, const gmg_csr* A, int nP, const gmg_prolong* P, const int32_t* const* coloring,
                       cudaStream_t s);
+// gmg_setup; single_rhs = false leaves out what only cycles with one
+// right-hand side use (the cluster form).
+gmg_status new_handle(gmg_handle* h, const gmg_csr* A, int n_prolong, const gmg_prolong* P,
+                      const int32_t* const* coloring, const gmg_options* opt, bool single_rhs, void* stream);
 
 // level-vector selection by precision
 template <class T> struct Vec;

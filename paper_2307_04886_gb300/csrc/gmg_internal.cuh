@@ -290,6 +290,7 @@ struct gmg_ctx {
   int64_t* ml_dpos = nullptr;
   double ml_t = 0.0;
   // cycles run levels >= cl32.l0 (FP32) or cl64.l0 (FP64) as one cluster launch
+  bool single_rhs = true;  // false: a member of a many-mesh handle, whose cycles are all batched
   gmg::ClusterDesc<float> cl32{};
   gmg::ClusterDesc<double> cl64{};
   float* Ainv32 = nullptr;  // coarsest inverse in FP32 for the cluster launch
