@@ -108,22 +108,57 @@ __device__ __forceinline__ T combine_parts(T acc, int warp, int lane) {
   return acc;
 }
 
-// Sum of partial[0 .. count) by one block of 256 threads in a fixed order
-// (strided per-thread sums, then a tree); every thread gets the result.
-// Partials written by other blocks of the same grid are read through L2.
-__device__ double block_final_sum(int count, const double* partial, double* red) {
-  double s = 0.0;
-  for (int i = threadIdx.x; i < count; i += 256) s += __ldcg(partial + i);
+// Sums of NS values per thread over a block of 256 threads in a fixed order
+// (the tree t += t + o, o = 128 .. 1); thread 0 gets them.  The last five
+// levels are one warp's shuffles: a level is then one dependent FP64 addition,
+// without the barrier and the shared-memory round trip.
+template <int NS>
+__device__ __forceinline__ void block_sums(double (&v)[NS], double (*red)[256]) {
+  const int t = threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) red[k][t] = v[k];
   __syncthreads();
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
+#pragma unroll
+  for (int o = 128; o >= 32; o >>= 1) {
+    if (t < o) {
+#pragma unroll
+      for (int k = 0; k < NS; ++k) {
+        v[k] += red[k][t + o];
+        red[k][t] = v[k];
+      }
+    }
+    if (o > 32) __syncthreads();
   }
-  const double v = red[0];
+  if (t < 32) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < NS; ++k) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+  }
+}
+
+// Sums of partial[k * stride + (0 .. count)), k < NS, by one block of 256
+// threads in a fixed order (strided per-thread sums, then the tree); thread 0
+// gets them.  Partials written by other blocks of the same grid are read
+// through L2, four at a time.
+template <int NS>
+__device__ __forceinline__ void block_final_sums(int count, const double* partial, int stride, double (&v)[NS],
+                                                 double (*red)[256]) {
+#pragma unroll
+  for (int k = 0; k < NS; ++k) v[k] = 0.0;
+  for (int i0 = threadIdx.x; i0 < count; i0 += 1024) {
+    double p[NS][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int k = 0; k < NS; ++k) p[k][q] = i0 + 256 * q < count ? __ldcg(partial + k * stride + i0 + 256 * q) : 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int k = 0; k < NS; ++k) v[k] += p[k][q];
+  }
   __syncthreads();
-  return v;
+  block_sums<NS>(v, red);
 }
 
 // True in the one block of the grid that arrives last (after every block has
@@ -169,19 +204,6 @@ __global__ void __launch_bounds__(256, (G == 1 && sizeof(T) == 4) ? 8 : 1) k_gs(
   if (part == 0 && p.active) x[p.row] = (bv - acc) * di;
 }
 
-// Block sums in the fixed order of k_dot_partial (same grid, same per-thread
-// ranges, same tree), so the fused kernels below give the same bits as a
-// separate dot product.
-__device__ __forceinline__ void block_sum_store(double v, double* red, double* out) {
-  red[threadIdx.x] = v;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *out = red[0];
-}
-
 // The start of a device-driven solve (one thread): the initial relative
 // residual, and whether the right-hand side is nonzero and both are finite
 // (the iterations of a solve that must not run are discarded by k_store).
@@ -220,39 +242,52 @@ struct NormEnd {
 // r = b - A x over all slices.  With NORM also ||r||^2 into sc[S_RR]: fixed
 // block sums, added in block order by the last block, which then runs the
 // test named in `end` (a separate one-block sum and a one-thread test cost a
-// launch each: 5 us per iteration of the refinement modes).
+// launch each: 5 us per iteration of the refinement modes).  With NORM a block
+// takes every gridDim-th group of slices: a block's reduction (nine dependent
+// FP64 additions, a fence and an atomic, about 3 us) then falls due once per
+// resident block and not once per 256 rows (1M-vertex torus: 59 -> 32 us).
 template <class T, int G, bool NORM>
-__global__ void __launch_bounds__(256) k_residual(int64_t nslice, const int64_t* __restrict__ ptr,
+__global__ void __launch_bounds__(256, NORM ? 4 : 1) k_residual(int64_t nslice, const int64_t* __restrict__ ptr,
                                                   const int32_t* __restrict__ row0, const int32_t* __restrict__ nrow,
                                                   const int32_t* __restrict__ col, const T* __restrict__ val,
                                                   const T* __restrict__ diag, const T* x, const T* b, T* r,
                                                   NormEnd end) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, part = warp % G;
-  const int64_t s = (int64_t)blockIdx.x * (8 / G) + warp / G;
-  const RowPart p = row_part<G>(s, nslice, ptr, row0, nrow, part, lane);
-  T pv[kPrefetch];
-  int pc[kPrefetch];
-  prefetch_row<T, G>(p, col, val, pv, pc);
-  const T d = (part == 0 && p.active) ? diag[p.row] : T(0);
-  pdl_wait();
-  pdl_trigger();
-  const bool own = part == 0 && p.active;
-  const T bv = own ? b[p.row] : T(0), xv = own ? x[p.row] : T(0);  // issued with the gathers
-  T acc = row_dot<T, G>(p, pv, pc, col, val, x);
-  acc = combine_parts<T, G>(acc, warp, lane);
   double sq = 0.0;
-  if (own) {
-    const T rv = bv - (acc + d * xv);
-    r[p.row] = rv;
-    sq = to_f64(rv) * to_f64(rv);
+  bool first = true;
+  for (int64_t s0 = (int64_t)blockIdx.x * (8 / G); s0 < nslice; s0 += (int64_t)gridDim.x * (8 / G)) {
+    const RowPart p = row_part<G>(s0 + warp / G, nslice, ptr, row0, nrow, part, lane);
+    T pv[kPrefetch];
+    int pc[kPrefetch];
+    prefetch_row<T, G>(p, col, val, pv, pc);
+    const T d = (part == 0 && p.active) ? diag[p.row] : T(0);
+    if (first) {
+      pdl_wait();
+      pdl_trigger();
+      first = false;
+    } else if constexpr (G > 1) {
+      __syncthreads();  // the sums of the group before have been read
+    }
+    const bool own = part == 0 && p.active;
+    const T bv = own ? b[p.row] : T(0), xv = own ? x[p.row] : T(0);  // issued with the gathers
+    T acc = row_dot<T, G>(p, pv, pc, col, val, x);
+    acc = combine_parts<T, G>(acc, warp, lane);
+    if (own) {
+      const T rv = bv - (acc + d * xv);
+      r[p.row] = rv;
+      if constexpr (NORM) sq += to_f64(rv) * to_f64(rv);
+    }
+    if constexpr (!NORM) break;
   }
   if constexpr (NORM) {
-    __shared__ double red[256];
-    block_sum_store(sq, red, end.partial + blockIdx.x);
+    __shared__ double red[1][256];
+    double v[1] = {sq};
+    block_sums<1>(v, red);
+    if (threadIdx.x == 0) end.partial[blockIdx.x] = v[0];
     if (last_block(end.counter)) {
-      const double v = block_final_sum(gridDim.x, end.partial, red);
+      block_final_sums<1>(gridDim.x, end.partial, 0, v, red);
       if (threadIdx.x == 0) {
-        end.sc[S_RR] = v;
+        end.sc[S_RR] = v[0];
         if (end.what == kNormStart) start_check(end.sc, end.hist);
         if (end.what == kNormIter) iter_check(end.sc, end.it, end.hist, end.h);
       }
@@ -260,38 +295,45 @@ __global__ void __launch_bounds__(256) k_residual(int64_t nslice, const int64_t*
   }
 }
 
-// q = A p (FP64) with per-block partials of p.q (fixed-shape reduction).
-__global__ void __launch_bounds__(256) k_spmv_dot(int64_t nslice, const int64_t* __restrict__ ptr,
+// q = A p (FP64) and p.q into *out; blocks take every gridDim-th group of
+// eight slices, as in k_residual.  What bounds it then is the FP64 pipe (a
+// warp's FP64 instruction takes 64 cycles of its sub-partition): eight per
+// slice of a mesh Laplacian are 14 us on the 1M-vertex torus.  47 -> 27 us.
+__global__ void __launch_bounds__(256, 4) k_spmv_dot(int64_t nslice, const int64_t* __restrict__ ptr,
                                                   const int32_t* __restrict__ row0, const int32_t* __restrict__ nrow,
                                                   const int32_t* __restrict__ col, const double* __restrict__ val,
                                                   const double* __restrict__ diag, const double* p,
                                                   double* q, double* __restrict__ partial, int* counter,
                                                   double* out) {
   const int lane = threadIdx.x & 31;
-  const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const RowPart rp = row_part<1>(s, nslice, ptr, row0, nrow, 0, lane);
-  double pv[kPrefetch];
-  int pc[kPrefetch];
-  prefetch_row<double, 1>(rp, col, val, pv, pc);
-  pdl_wait();
-  pdl_trigger();
+  const int64_t step = (int64_t)gridDim.x * 8;
   double pq = 0.0;
-  if (rp.active) {
-    const double acc = row_dot<double, 1>(rp, pv, pc, col, val, p) + diag[rp.row] * p[rp.row];
-    q[rp.row] = acc;
-    pq = p[rp.row] * acc;
+  bool first = true;
+  for (int64_t s = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); s < nslice || first; s += step) {
+    const RowPart rp = row_part<1>(s, nslice, ptr, row0, nrow, 0, lane);
+    double pv[kPrefetch];
+    int pc[kPrefetch];
+    prefetch_row<double, 1>(rp, col, val, pv, pc);
+    const double d = rp.active ? diag[rp.row] : 0.0;
+    if (first) {
+      pdl_wait();
+      pdl_trigger();
+      first = false;
+    }
+    if (rp.active) {
+      const double pr = p[rp.row];
+      const double acc = row_dot<double, 1>(rp, pv, pc, col, val, p) + d * pr;
+      q[rp.row] = acc;
+      pq += pr * acc;
+    }
   }
-  __shared__ double red[256];
-  red[threadIdx.x] = pq;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
+  __shared__ double red[1][256];
+  double v[1] = {pq};
+  block_sums<1>(v, red);
+  if (threadIdx.x == 0) partial[blockIdx.x] = v[0];
   if (last_block(counter)) {
-    const double v = block_final_sum(gridDim.x, partial, red);
-    if (threadIdx.x == 0) *out = v;
+    block_final_sums<1>(gridDim.x, partial, 0, v, red);
+    if (threadIdx.x == 0) *out = v[0];
   }
 }
 
@@ -404,12 +446,12 @@ __global__ void k_add_f2d(int64_t n, const float* e, double* x) {
 // counter and limit: one launch instead of two gathers, two reduction kernels
 // and two copies from the host.  Sums: fixed grid (kRedBlocks x 256), fixed
 // per-thread ranges, fixed tree.
-__global__ void __launch_bounds__(256) k_load(int64_t n, const int32_t* __restrict__ perm,
+__global__ void __launch_bounds__(256, 4) k_load(int64_t n, const int32_t* __restrict__ perm,
                                               const double* __restrict__ b, const double* __restrict__ x,
                                               double* __restrict__ bs, double* __restrict__ xs,
                                               double* __restrict__ partial, int* counter, double* sc, int* it,
                                               double tol, int max_iter) {
-  __shared__ double red[256];
+  __shared__ double red[1][256];
   pdl_wait();
   pdl_trigger();
   double s = 0.0;
@@ -421,11 +463,13 @@ __global__ void __launch_bounds__(256) k_load(int64_t n, const int32_t* __restri
     xs[i] = x[o];
     s += bi * bi;
   }
-  block_sum_store(s, red, partial + blockIdx.x);
+  double v[1] = {s};
+  block_sums<1>(v, red);
+  if (threadIdx.x == 0) partial[blockIdx.x] = v[0];
   if (last_block(counter)) {
-    const double v = block_final_sum(gridDim.x, partial, red);
+    block_final_sums<1>(gridDim.x, partial, 0, v, red);
     if (threadIdx.x == 0) {
-      sc[S_NB2] = v;
+      sc[S_NB2] = v[0];
       sc[S_TOL] = tol;
       it[0] = 0;
       it[1] = max_iter;
@@ -471,14 +515,14 @@ __global__ void __launch_bounds__(256) k_store(int64_t n, const int32_t* __restr
 // With `check` the last block also runs the convergence test of the
 // device-side loop.  Grid: kRedBlocks x 256.
 template <class Z>
-__global__ void __launch_bounds__(256) k_pcg_axpy(int64_t n, double* sc, const double* __restrict__ p,
+__global__ void __launch_bounds__(256, 4) k_pcg_axpy(int64_t n, double* sc, const double* __restrict__ p,
                                                   const double* __restrict__ q, double* __restrict__ x,
                                                   double* __restrict__ r, double* __restrict__ rold,
                                                   float* __restrict__ b32, Z* __restrict__ z0,
                                                   const Z* __restrict__ dinv, int64_t n0,
                                                   double* __restrict__ partial, int* counter, int check, int* it,
                                                   double* hist, cudaGraphConditionalHandle h) {
-  __shared__ double red[256];
+  __shared__ double red[1][256];
   pdl_wait();
   pdl_trigger();
   const double alpha = sc[S_RZ] / sc[S_PQ];
@@ -499,11 +543,13 @@ __global__ void __launch_bounds__(256) k_pcg_axpy(int64_t n, double* sc, const d
     }
     rr += rn * rn;
   }
-  block_sum_store(rr, red, partial + blockIdx.x);
+  double v[1] = {rr};
+  block_sums<1>(v, red);
+  if (threadIdx.x == 0) partial[blockIdx.x] = v[0];
   if (last_block(counter)) {
-    const double v = block_final_sum(gridDim.x, partial, red);
+    block_final_sums<1>(gridDim.x, partial, 0, v, red);
     if (threadIdx.x == 0) {
-      sc[S_RR] = v;
+      sc[S_RR] = v[0];
       if (check) iter_check(sc, it, hist, h);
     }
   }
@@ -514,10 +560,10 @@ __global__ void __launch_bounds__(256) k_pcg_axpy(int64_t n, double* sc, const d
 // last block, which sets beta = num / rz_old and rz = r.z for the next
 // iteration.  Grid: kRedBlocks x 256.
 template <class Z>
-__global__ void __launch_bounds__(256) k_pcg_zdots(int64_t n, const Z* __restrict__ z, const double* __restrict__ r,
+__global__ void __launch_bounds__(256, 4) k_pcg_zdots(int64_t n, const Z* __restrict__ z, const double* __restrict__ r,
                                                    const double* __restrict__ rold, double* __restrict__ partial,
                                                    int* counter, double* sc) {
-  __shared__ double red[256];
+  __shared__ double red[2][256];
   pdl_wait();
   pdl_trigger();
   double num = 0.0, rz = 0.0;
@@ -527,17 +573,19 @@ __global__ void __launch_bounds__(256) k_pcg_zdots(int64_t n, const Z* __restric
     num += zi * (ri - rold[i]);
     rz += ri * zi;
   }
-  block_sum_store(num, red, partial + blockIdx.x);
-  __syncthreads();
-  block_sum_store(rz, red, partial + gridDim.x + blockIdx.x);
+  double v[2] = {num, rz};
+  block_sums<2>(v, red);
+  if (threadIdx.x == 0) {
+    partial[blockIdx.x] = v[0];
+    partial[gridDim.x + blockIdx.x] = v[1];
+  }
   if (last_block(counter)) {
-    const double a = block_final_sum(gridDim.x, partial, red);
-    const double rzn = block_final_sum(gridDim.x, partial + gridDim.x, red);
+    block_final_sums<2>(gridDim.x, partial, gridDim.x, v, red);
     if (threadIdx.x == 0) {
-      sc[S_NUM] = a;
-      sc[S_BETA] = a / sc[S_RZ];
-      sc[S_RZN] = rzn;
-      sc[S_RZ] = rzn;
+      sc[S_NUM] = v[0];
+      sc[S_BETA] = v[0] / sc[S_RZ];
+      sc[S_RZN] = v[1];
+      sc[S_RZ] = v[1];
     }
   }
 }
@@ -545,10 +593,10 @@ __global__ void __launch_bounds__(256) k_pcg_zdots(int64_t n, const Z* __restric
 // The start of CG, z = MGI(0, r) given: p = z and r.z into sc[S_RZ] (partials,
 // finished by the last block).  Grid: kRedBlocks x 256.
 template <class Z>
-__global__ void __launch_bounds__(256) k_pcg_first(int64_t n, const Z* __restrict__ z, const double* __restrict__ r,
+__global__ void __launch_bounds__(256, 4) k_pcg_first(int64_t n, const Z* __restrict__ z, const double* __restrict__ r,
                                                    double* __restrict__ p, double* __restrict__ partial,
                                                    int* counter, double* sc) {
-  __shared__ double red[256];
+  __shared__ double red[1][256];
   pdl_wait();
   pdl_trigger();
   double rz = 0.0;
@@ -558,10 +606,12 @@ __global__ void __launch_bounds__(256) k_pcg_first(int64_t n, const Z* __restric
     p[i] = zi;
     rz += r[i] * zi;
   }
-  block_sum_store(rz, red, partial + blockIdx.x);
+  double v[1] = {rz};
+  block_sums<1>(v, red);
+  if (threadIdx.x == 0) partial[blockIdx.x] = v[0];
   if (last_block(counter)) {
-    const double v = block_final_sum(gridDim.x, partial, red);
-    if (threadIdx.x == 0) sc[S_RZ] = v;
+    block_final_sums<1>(gridDim.x, partial, 0, v, red);
+    if (threadIdx.x == 0) sc[S_RZ] = v[0];
   }
 }
 
@@ -617,7 +667,8 @@ gmg_status launch_gs_colour(Level& L, int colour, const T* b, T* x, cudaStream_t
 template <class T, bool NORM>
 static gmg_status launch_residual_n(Level& L, const T* x, const T* b, T* r, const NormEnd& end, cudaStream_t s) {
   const int G = L.rlanes;
-  const int64_t grid = (L.A.nslice + (8 / G) - 1) / (8 / G);
+  int64_t grid = (L.A.nslice + (8 / G) - 1) / (8 / G);
+  if (NORM) grid = std::min<int64_t>(grid, kRedBlocks);  // one reduction per resident block
   const Ell& A = L.A;
   switch (G) {
     case 1: return launch(k_residual<T, 1, NORM>, grid, 256, s, A.nslice, A.ptr, A.row0, A.nrow, A.col, Vec<T>::v(A), Vec<T>::diag(L), x, b, r, end);
@@ -766,11 +817,6 @@ gmg_status launch_f2d(int64_t n, const float* a, double* b, cudaStream_t s) {
 // (kNorm*) with the loop condition h.
 static gmg_status outer_residual(gmg_ctx* c, int what, cudaStream_t s, cudaGraphConditionalHandle h = 0) {
   Level& L = c->L[0];
-  const int64_t blocks = (L.A.nslice + (8 / L.rlanes) - 1) / (8 / L.rlanes);
-  if (blocks > c->red_cap) {
-    set_error("outer residual: more blocks than reduction partials");
-    return GMG_ERR_TOO_LARGE;
-  }
   const NormEnd end{c->red, c->red_cnt + 4, c->scal, c->dloop, c->dhist, h, what};
   return launch_residual_n<double, true>(L, c->xs, c->bs, c->rs, end, s);
 }
@@ -810,11 +856,7 @@ gmg_status iteration_body(gmg_ctx* c, int mode, int seg, cudaStream_t s, cudaGra
   }
   const bool f64 = mode == GMG_FP64_PCG;
   if (seg == 0) {
-    const int64_t nb = (L.A.nslice * 32 + 255) / 256;
-    if (nb > c->red_cap) {
-      set_error("PCG: more blocks than reduction partials");
-      return GMG_ERR_TOO_LARGE;
-    }
+    const int64_t nb = std::min<int64_t>((L.A.nslice + 7) / 8, kRedBlocks);  // one reduction per resident block
     GMG_TRY(launch(k_spmv_dot, nb, 256, s, L.A.nslice, L.A.ptr, L.A.row0, L.A.nrow, L.A.col, L.A.v64, L.diag64,
                    (const double*)c->ps, c->qs, c->red, c->red_cnt, c->scal + S_PQ));
     if (f64)
