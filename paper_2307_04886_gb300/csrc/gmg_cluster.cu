@@ -54,9 +54,12 @@
 
 #include <algorithm>
 #include <atomic>
+#include <condition_variable>
 #include <cstdlib>
 #include <cstring>
 #include <exception>
+#include <functional>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <system_error>
@@ -418,7 +421,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
   // end(bytes), called by every thread when its messages are on their way,
   // sets the halo bytes that the phase brings.
   int ph = 0;
-    const bool sends_token = warp == kClWarps - 1 && lane < npart;
+  const bool sends_token = warp == kClWarps - 1 && lane < npart;
   uint32_t tok_a = 0, tok_m = 0;
   if (sends_token) {
     tok_a = cl_map(sm0 + (uint32_t)D.o_tok + 4u * (uint32_t)cta, (unsigned)partners[lane]);
@@ -964,55 +967,100 @@ void push_lists(const std::vector<int32_t>& owner, const std::vector<int32_t>& l
   }
 }
 
-// Runs f(0) .. f(n - 1) on as many threads as the work (in table entries) is
-// worth: a thread costs about 30 us to start, which some 20,000 entries take.
-// What a call throws is thrown again here, after every thread has ended.
-template <class F>
-void run_parts(int n, int64_t work, F f) {
-  const int hw = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-  const int m = (int)std::min<int64_t>({(int64_t)n, (int64_t)hw, 1 + work / 20000});
-  std::atomic<int> next{0};
-  std::exception_ptr err;
-  std::mutex lock;
-  auto work_on = [&] {
-    try {
-      for (int i = next++; i < n; i = next++) f(i);
-    } catch (...) {
-      std::lock_guard<std::mutex> g(lock);
-      err = std::current_exception();
-    }
-  };
-  std::vector<std::thread> th;
-  th.reserve(m);
-  for (int i = 1; i < m; ++i) {
-    try {
-      th.emplace_back(work_on);
-    } catch (const std::system_error&) {
-      break;  // no more threads: the others do the rest
+// Host threads that build one precision's tables, started once for all the
+// stages (starting a thread takes about 30 us: five stages that each started
+// up to 15 spent 2 ms of 3.5 on it).
+class Team {
+ public:
+  explicit Team(int workers) {
+    th_.reserve(workers);
+    for (int i = 0; i < workers; ++i) {
+      try {
+        th_.emplace_back([this] { serve(); });
+      } catch (const std::system_error&) {
+        break;  // no more threads: the others do the rest
+      }
     }
   }
-  work_on();
-  for (auto& x : th) x.join();
-  if (err) std::rethrow_exception(err);
-}
+  ~Team() {
+    {
+      std::lock_guard<std::mutex> g(lock_);
+      stop_ = true;
+    }
+    wake_.notify_all();
+    for (auto& t : th_) t.join();
+  }
+  // Runs f(0) .. f(n - 1) on the team and the calling thread.  What a call
+  // throws is thrown again here, after every call has ended.
+  void run(int n, const std::function<void(int)>& f) {
+    {
+      std::lock_guard<std::mutex> g(lock_);
+      f_ = &f;
+      n_ = n;
+      next_ = 0;
+      err_ = nullptr;
+      ++stage_;
+    }
+    wake_.notify_all();
+    work(f, n);
+    std::unique_lock<std::mutex> g(lock_);
+    f_ = nullptr;  // a thread that wakes later finds nothing to do
+    done_.wait(g, [this] { return busy_ == 0; });
+    if (err_) std::rethrow_exception(err_);
+  }
+
+ private:
+  void work(const std::function<void(int)>& f, int n) {
+    try {
+      for (int i = next_++; i < n; i = next_++) f(i);
+    } catch (...) {
+      std::lock_guard<std::mutex> g(lock_);
+      err_ = std::current_exception();
+    }
+  }
+  void serve() {
+    std::unique_lock<std::mutex> g(lock_);
+    for (unsigned seen = 0;;) {
+      wake_.wait(g, [&] { return stop_ || stage_ != seen; });
+      if (stop_) return;
+      seen = stage_;
+      if (!f_) continue;
+      const std::function<void(int)>* f = f_;
+      const int n = n_;
+      ++busy_;
+      g.unlock();
+      work(*f, n);
+      g.lock();
+      if (--busy_ == 0) done_.notify_all();
+    }
+  }
+  std::vector<std::thread> th_;
+  std::mutex lock_;
+  std::condition_variable wake_, done_;
+  const std::function<void(int)>* f_ = nullptr;
+  int n_ = 0, busy_ = 0;
+  unsigned stage_ = 0;
+  bool stop_ = false;
+  std::atomic<int> next_{0};
+  std::exception_ptr err_;
+};
 
 // The tables of levels l0 .. lambda over ncta CTAs (host); false when a CTA
 // would hold too many rows.  The CTAs' parts are independent given the owners
 // and local indices of the rows, and so are the levels' halo lists: they are
 // built side by side.
-bool build_tables(gmg_ctx* c, int l0, int ncta, int per_unit, const std::vector<std::vector<int64_t>>& hrp,
+bool build_tables(Team& team, const gmg_ctx* c, int l0, int ncta, int per_unit, const std::vector<std::vector<int64_t>>& hrp,
                   const std::vector<std::vector<int32_t>>& hcol, const std::vector<std::vector<int32_t>>& perm,
                   const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P, std::vector<Tab>& tab) {
   const int lam = c->nlev - 1, nl = lam - l0;
   tab.assign(nl + 1, Tab());
-  int64_t entries = 0, nmax = 0;
-  for (int t = 0; t < nl; ++t) entries += c->L[l0 + t].nnz;
+  int64_t nmax = 0;
   // transposed prolongation from level t + 1's rows (fine rows ascending)
   std::vector<std::vector<int64_t>> tptr(nl);
   std::vector<std::vector<int32_t>> tcol(nl);
   std::vector<std::vector<double>> tw(nl);
   for (int t = 0; t <= nl; ++t) nmax = std::max(nmax, c->L[l0 + t].n);
-  run_parts(2 * nl + 1, entries, [&](int q) {
+  team.run(2 * nl + 1, [&](int q) {
     if (q <= nl) {
       const int t = q;
       const Level& L = c->L[l0 + t];
@@ -1062,7 +1110,7 @@ bool build_tables(gmg_ctx* c, int l0, int ncta, int per_unit, const std::vector<
                                : lanes_per_row((double)tab[t + 1].n / ncta,
                                                (double)tptr[t].back() / (double)tab[t + 1].n);
   std::atomic<bool> fits{true};
-  run_parts(ncta, 2 * entries, [&](int a) {
+  team.run(ncta, [&](int a) {
     std::vector<int32_t> loc, stamp;
     loc.reserve(nmax);
     stamp.reserve(nmax);
@@ -1198,7 +1246,7 @@ bool build_tables(gmg_ctx* c, int l0, int ncta, int per_unit, const std::vector<
     }
   });
   if (!fits) return false;
-  run_parts(2 * nl + 1, entries / 4, [&](int q) {
+  team.run(2 * nl + 1, [&](int q) {
     Tab& T = tab[q / 2];
     push_lists(T.owner, T.local, T.part, q % 2 != 0);
   });
@@ -1289,12 +1337,9 @@ bool check_level(const std::vector<Tab>& tab, int per_unit, int t) {
   return true;
 }
 
-bool check_tables(const std::vector<Tab>& tab, int per_unit) {
-  int64_t entries = 0;
-  for (const Tab& T : tab)
-    for (const Part& p : T.part) entries += (int64_t)p.ecol.size();
+bool check_tables(Team& team, const std::vector<Tab>& tab, int per_unit) {
   std::atomic<bool> ok{true};
-  run_parts((int)tab.size(), entries / 4, [&](int t) {
+  team.run((int)tab.size(), [&](int t) {
     if (!check_level(tab, per_unit, t)) ok = false;
   });
   return ok;
@@ -1454,7 +1499,7 @@ int32_t first_store(const Part& p, int i) {
 
 // Lays the tables of `tab` out as D says and uploads them.
 template <class T>
-gmg_status upload_tables(gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>& D) {
+gmg_status upload_tables(Team& team, gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>& D) {
   constexpr size_t pu = sizeof(T) == 4 ? 2 : 1;  // entries per unit
   const int nl = (int)tab.size() - 1, ncta = D.ncta;
   Blob B;
@@ -1499,7 +1544,6 @@ gmg_status upload_tables(gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>
   };
   std::vector<Off> off(nl + 1);
   size_t o_l2g = 0;
-  int64_t entries = 0;
   for (int t = 0; t <= nl; ++t) {
     ClusterLevel<T>& L = D.lv[t];
     const size_t no = (size_t)ncta * L.n_own_max;
@@ -1509,7 +1553,6 @@ gmg_status upload_tables(gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>
     const int64_t ent = L.streamed ? 0 : (int64_t)tab[t].ent * pu;
     L.n_ent = ent;
     L.nvsrc = ncta * ent;
-    entries += c->L[D.l0 + t].nnz;
     off[t].vi = B.add(&L.vimg, (size_t)ncta * L.val_bytes);
     off[t].ds = B.add(&L.dsrc, no);
     off[t].vs = B.add(&L.vsrc, (size_t)L.nvsrc);
@@ -1521,7 +1564,7 @@ gmg_status upload_tables(gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>
   }
   B.h.resize(B.size);
   // each CTA's part of every array
-  run_parts(ncta, entries, [&](int q) {
+  team.run(ncta, [&](int q) {
     for (int t = 0; t <= nl; ++t) {
       const Tab& A = tab[t];
       const ClusterLevel<T>& L = D.lv[t];
@@ -1614,19 +1657,25 @@ gmg_status upload_tables(gmg_ctx* c, const std::vector<Tab>& tab, ClusterDesc<T>
   return B.upload(c->arena);
 }
 
+// The host tables of one precision's cluster (plan.l0 stays -1: none).
 template <class T>
-gmg_status build_one(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
-                     const std::vector<std::vector<int32_t>>& hcol, const std::vector<std::vector<int32_t>>& perm,
-                     const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P) {
-  ClusterDesc<T>& D = Src<T>::desc(c);
-  D = ClusterDesc<T>{};
-  D.l0 = -1;
+struct Plan {
+  std::unique_ptr<Team> team;
+  std::vector<Tab> tab;
+  ClusterDesc<T> D;
+  bool checked = true;
+};
+
+template <class T>
+void plan_one(const gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
+              const std::vector<std::vector<int32_t>>& hcol, const std::vector<std::vector<int32_t>>& perm,
+              const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P, Plan<T>& plan) {
   const int lam = c->nlev - 1;
   auto env = [](const char* name) {
     const char* e = std::getenv(name);
     return e && e[0] == '1';
   };
-  if (lam < 1 || env("GMG_NO_TAIL")) return GMG_OK;
+  if (lam < 1 || env("GMG_NO_TAIL")) return;
   const bool small_only = env("GMG_NO_CLUSTER_LEVEL");
   std::vector<int> sizes = {16, 8};
   if (const char* e = std::getenv("GMG_TAIL_CTAS")) sizes = {std::atoi(e)};
@@ -1649,8 +1698,15 @@ gmg_status build_one(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
         stage = std::max(stage, 2 * e / std::max(1, L.ncolor));
       }
       if (skip || least + std::min(ent, stage) > kSmemLimit) continue;
-      std::vector<Tab> tab;
-      if (!build_tables(c, l0, ncta, pu, hrp, hcol, perm, iperm, P, tab)) continue;
+      std::vector<Tab>& tab = plan.tab;
+      if (!plan.team) {  // a thread for some 20,000 entries, four in all where that is less
+        int64_t entries = 0;
+        for (int l = l0; l < lam; ++l) entries += c->L[l].nnz;
+        const int hw = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+        plan.team.reset(new Team((int)std::min<int64_t>(hw, std::max<int64_t>(4, entries / 20000)) - 1));
+      }
+      Team& team = *plan.team;
+      if (!build_tables(team, c, l0, ncta, pu, hrp, hcol, perm, iperm, P, tab)) continue;
       // where the ranks are not local (random order: 11-13 halo stores per
       // row on a kNN cloud) a phase would store nearly every row into every CTA
       bool local = true;
@@ -1669,20 +1725,30 @@ gmg_status build_one(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
       E.nu_post = c->opt.nu_post;
       E.post_forward = c->opt.post_forward;
       if (!lay_out(tab, E.nu_pre, E.nu_post, E)) continue;
-      if (!check_tables(tab, pu)) {
-        set_error("internal: cluster tables failed their host check");
-        return GMG_ERR_INVALID_ARG;
+      if (!check_tables(team, tab, pu)) {
+        plan.checked = false;
+        return;
       }
       if (!cluster_fits(E)) break;  // this cluster size cannot be scheduled: try the next
-      E.ainv = Src<T>::ainv(c);
-      E.err = c->dstatus + 3;
-      GMG_CK(cudaMemset(E.err, 0, sizeof(int)));
-      GMG_TRY(upload_tables(c, tab, E));
       for (int t = 0; t < E.nlev; ++t) E.wide[t] = tab[t].wide;
-      D = E;
-      return GMG_OK;
+      plan.D = E;
+      return;
     }
   }
+}
+
+template <class T>
+gmg_status finish_one(gmg_ctx* c, Plan<T>& plan) {
+  if (!plan.checked) {
+    set_error("internal: cluster tables failed their host check");
+    return GMG_ERR_INVALID_ARG;
+  }
+  if (plan.D.l0 < 0) return GMG_OK;
+  plan.D.ainv = Src<T>::ainv(c);
+  plan.D.err = c->dstatus + 3;
+  GMG_CK(cudaMemset(plan.D.err, 0, sizeof(int)));
+  GMG_TRY(upload_tables(*plan.team, c, plan.tab, plan.D));
+  Src<T>::desc(c) = plan.D;
   return GMG_OK;
 }
 
@@ -1718,16 +1784,59 @@ gmg_status refresh_one(gmg_ctx* c, cudaStream_t s) {
 
 }  // namespace
 
-gmg_status build_cluster(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
-                         const std::vector<std::vector<int32_t>>& hcol, const std::vector<std::vector<int32_t>>& perm,
-                         const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P) {
-  c->cl32.l0 = c->cl64.l0 = -1;
-  if (!c->single_rhs) return GMG_OK;
-  GMG_TRY(build_one<float>(c, hrp, hcol, perm, iperm, P));
+// The tables being built on host threads, one for each precision.  What a
+// thread throws is thrown again by finish_cluster; the destructor waits for
+// the threads, so the job ends before what they read does.
+struct ClusterJob {
+  Plan<float> p32;
+  Plan<double> p64;
+  std::thread th[2];
+  std::exception_ptr err[2];
+  template <class F>
+  void run(int k, int device, F f) {
+    auto body = [this, k, device, f] {
+      try {
+        cudaSetDevice(device);
+        f();
+      } catch (...) {
+        err[k] = std::current_exception();
+      }
+    };
+    try {
+      th[k] = std::thread(body);
+    } catch (const std::system_error&) {
+      body();  // no more threads: here and now
+    }
+  }
+  void wait() {
+    for (auto& t : th)
+      if (t.joinable()) t.join();
+  }
+  ~ClusterJob() { wait(); }
+};
+
+std::shared_ptr<ClusterJob> start_cluster(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
+                                          const std::vector<std::vector<int32_t>>& hcol,
+                                          const std::vector<std::vector<int32_t>>& perm,
+                                          const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P) {
+  auto job = std::make_shared<ClusterJob>();
+  ClusterJob& j = *job;
+  c->cl32 = ClusterDesc<float>{};
+  c->cl64 = ClusterDesc<double>{};
+  if (!c->single_rhs) return job;
   // FP64 cycles in a solve: the modes that run them
   if (c->opt.precision == GMG_FP64 || c->opt.precision == GMG_FP64_PCG)
-    GMG_TRY(build_one<double>(c, hrp, hcol, perm, iperm, P));
-  return GMG_OK;
+    j.run(1, c->device, [&, c, P] { plan_one<double>(c, hrp, hcol, perm, iperm, P, j.p64); });
+  j.run(0, c->device, [&, c, P] { plan_one<float>(c, hrp, hcol, perm, iperm, P, j.p32); });
+  return job;
+}
+
+gmg_status finish_cluster(gmg_ctx* c, ClusterJob& job) {
+  job.wait();
+  for (auto& e : job.err)
+    if (e) std::rethrow_exception(e);
+  GMG_TRY(finish_one<float>(c, job.p32));
+  return finish_one<double>(c, job.p64);
 }
 
 gmg_status refresh_cluster_values(gmg_ctx* c, cudaStream_t s) {

@@ -6,6 +6,7 @@
 #include <chrono>
 #include <cstdint>
 #include <cstdlib>
+#include <memory>
 #include <string>
 #include <utility>
 #include <vector>
@@ -357,11 +358,16 @@ gmg_status join_inverse(gmg_ctx* c, cudaStream_t s, bool check);
 // Reads the pivot check of a joined inverse once (GMG_ERR_CHOLESKY on failure).
 gmg_status inverse_status(gmg_ctx* c, cudaStream_t s);
 // The cluster form of the coarse levels (gmg_cluster.cu): tables from the
-// levels' patterns and numberings (host), values after a numeric set-up, the
-// launch x <- MGI(x, b, l0), and the state of its bounded waits.
-gmg_status build_cluster(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
-                         const std::vector<std::vector<int32_t>>& hcol, const std::vector<std::vector<int32_t>>& perm,
-                         const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P);
+// levels' patterns and numberings (built on host threads between start and
+// finish, which uploads them; the arguments outlive the job), values after a
+// numeric set-up, the launch x <- MGI(x, b, l0), and the state of its bounded
+// waits.
+struct ClusterJob;
+std::shared_ptr<ClusterJob> start_cluster(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
+                                          const std::vector<std::vector<int32_t>>& hcol,
+                                          const std::vector<std::vector<int32_t>>& perm,
+                                          const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P);
+gmg_status finish_cluster(gmg_ctx* c, ClusterJob& job);
 gmg_status refresh_cluster_values(gmg_ctx* c, cudaStream_t s);
 template <class T>
 gmg_status launch_cluster(gmg_ctx* c, T* x, const T* b, bool c0_first, cudaStream_t s);

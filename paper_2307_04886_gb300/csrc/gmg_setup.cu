@@ -1888,6 +1888,9 @@ gmg_status setup_impl(gmg_ctx* c, const gmg_csr* A, int nP, const gmg_prolong* P
   for (int l = 0; l < c->nlev; ++l)
     GMG_TRY(build_level_structure(c, l, hrp[l].data(), hcol[l].data(), coloring ? coloring[l] : nullptr, *jobs[l],
                                   perm[l], iperm[l]));
+  // the cluster tables, which need the levels' numberings only, are built on
+  // host threads while the transfers are laid out and the vectors allocated
+  const std::shared_ptr<ClusterJob> cluster = start_cluster(c, hrp, hcol, perm, iperm, P);
   lap(6, "gmg_setup: transfer layouts");
   for (int l = 0; l + 1 < c->nlev; ++l)
     GMG_TRY(build_transfer_structure(c, l, P[l], perm[l], iperm[l], perm[l + 1], iperm[l + 1]));
@@ -1924,7 +1927,7 @@ gmg_status setup_impl(gmg_ctx* c, const gmg_csr* A, int nP, const gmg_prolong* P
   GMG_TRY(a.alloc(&c->dhist, (size_t)c->opt.max_iter + 2));
   GMG_CK(cudaMallocHost((void**)&c->h_scal, 128 * sizeof(double)));
   lap(3, "gmg_setup: cluster tables");
-  GMG_TRY(build_cluster(c, hrp, hcol, perm, iperm, P));
+  GMG_TRY(finish_cluster(c, *cluster));
   for (Level& L : c->L) std::vector<int64_t>().swap(L.h_ptr);
   lap(4, "gmg_setup: numeric set-up");
   const gmg_status st = numeric_setup(c, s, false);
