@@ -164,13 +164,12 @@ def gs_kernel_name(split, t="float"):
     return f"k_gs<{t}, {split}>"
 
 
-def level_breakdown(dims, lanes, levels, cycles, s=4, paths=None):
-    """Per smoothed level of the timed cycles: Gauss-Seidel launches, average
-    launch time and algorithmic GB/s, the transfer (residual, restriction,
-    prolongation) time, and the cluster tail (levels it covers, time).  A
-    cluster level (paths[l] == 1) runs its sweeps and transfers in two cluster
-    launches: its time per Gauss-Seidel phase includes the transfers."""
-    out, tail = [], None
+def level_breakdown(dims, lanes, levels, cycles, s=4):
+    """Per smoothed level with launches of its own, over the timed cycles:
+    Gauss-Seidel launches, average launch time and algorithmic GB/s, the transfer
+    (residual, restriction, prolongation) time; and the cluster launch of the
+    coarser levels (levels it covers, time)."""
+    out, cluster = [], None
     cyc = max(cycles, 1)
     for l, (gs_ms, gs_n, tr_ms, whole_ms) in enumerate(levels):
         if l >= len(dims) - 1:
@@ -178,14 +177,14 @@ def level_breakdown(dims, lanes, levels, cycles, s=4, paths=None):
         if gs_n > 0:
             us = 1e3 * gs_ms / gs_n
             b = gs_level_launch_bytes(dims, l, s)
-            kern = "k_level_cluster" if paths and paths[l] == 1 else gs_kernel_name(lanes[l])
-            out.append({"level": l, "rows": dims[l][0], "colours": dims[l][2], "kernel": kern,
+            out.append({"level": l, "rows": dims[l][0], "colours": dims[l][2], "kernel": gs_kernel_name(lanes[l]),
                         "gs_launches_per_cycle": gs_n / cyc, "gs_us_per_launch": us,
                         "gs_bytes_per_launch": b, "gs_gbs": b / (us * 1e-6) / 1e9,
                         "gs_us_per_cycle": 1e3 * gs_ms / cyc, "transfer_us_per_cycle": 1e3 * tr_ms / cyc})
-        elif whole_ms > 0 and tail is None:
-            tail = {"kernel": "k_tail_cycle", "levels": list(range(l, len(dims))), "us_per_cycle": 1e3 * whole_ms / cyc}
-    return out, tail
+        elif whole_ms > 0 and cluster is None:
+            cluster = {"kernel": "k_cluster_cycle", "levels": list(range(l, len(dims))),
+                       "us_per_cycle": 1e3 * whole_ms / cyc}
+    return out, cluster
 
 
 def dominant_gs(per_level):
@@ -211,9 +210,6 @@ def ncu_traffic(workload, per_level, levels, kernel):
     try:
         with open(os.path.join(ROOT, "profiles", "ncu_traffic.json")) as f:
             j = json.load(f)[workload]
-        if kernel == "k_level_cluster":  # the two launches of a V-cycle, per Gauss-Seidel phase like the bytes
-            r = next(r for r in per_level if r["level"] in levels)
-            return float(j["cluster_level_bytes_per_cycle"]) / r["gs_launches_per_cycle"]
         if not kernel.startswith("k_gs<"):
             return None
         d = j["gs_bytes_per_launch_by_level"]
@@ -476,12 +472,12 @@ def other_workloads(g, names, steps):
                 pr = sv.profile_read()
                 lv = sv.profile_levels()
                 sv.profile(False)
-                per_level, tail = level_breakdown(sv.dims, lanes, lv, int(pr[3]), paths=sv.paths)
+                per_level, cluster = level_breakdown(sv.dims, lanes, lv, int(pr[3]))
                 res[name] = {"rows": s.n, "levels": [d[0] for d in sv.dims], "nnz": [d[1] for d in sv.dims],
                              "colours": [d[2] for d in sv.dims], "fp32_pcg_ms": ms, "iterations": out["r"][1],
                              "vcycle_us_fp32": 1e3 * pr[2] / max(pr[3], 1),
                              "vcycle_gbs_fp32": algorithmic_bytes(sv.dims, s.Ps, 4) / (pr[2] / max(pr[3], 1) * 1e-3) / 1e9,
-                             "per_level": per_level, "tail": tail}
+                             "per_level": per_level, "cluster": cluster}
                 sv.close()
         except Exception as e:  # reported, not fatal: the headline stands on its own
             res[name] = {"error": f"{type(e).__name__}: {e}"}
@@ -699,7 +695,7 @@ def main():
     peak, peak_kind = load_peaks()
     smooth_ms, gs_launches, cyc_ms, cycles = pr
     cycles = int(cycles)
-    per_level, tail = level_breakdown(dims, lanes, lv, cycles, paths=solver.paths)
+    per_level, cluster = level_breakdown(dims, lanes, lv, cycles)
     kname, k_us, k_bytes, k_us_cyc, k_levels = dominant_gs(per_level)
     achieved = k_bytes / (k_us * 1e-6) / 1e9
     vc_us32 = 1e3 * cyc_ms / max(cycles, 1)
@@ -765,8 +761,8 @@ def main():
             "workload": WORKLOAD_DESC, "levels": [d[0] for d in dims], "nnz": [d[1] for d in dims],
             "colours": [d[2] for d in dims], "warps_per_row": lanes,
             "level_paths": solver.paths,
-            "level_paths_legend": "FP32 cycle per level: 0 one launch per colour, 1 cluster level (two cluster "
-                                  "launches), 2 cluster tail, 3 coarsest direct solve",
+            "level_paths_legend": "FP32 cycle per level: 0 one launch per colour; 1, 2 in the cluster launch, one "
+                                  "thread or several lanes per row; 3 coarsest direct solve",
             "precision": "FP64 conjugate gradients preconditioned by one FP32 V-cycle (nu=2/2, multicolour GS) "
                          "per iteration; FP64 residual, dots and explicit coarsest inverse; the iterations run in a device-side "
                          "graph loop (conditional WHILE node)",
@@ -793,7 +789,7 @@ def main():
             "vcycle_us_fp32": vc_us32, "vcycle_gbs_fp32": vc_gbs32,
             "vcycle_bytes_fp32": vc_bytes32, "vcycle_us_fp64": vc_us64,
             "vcycle_gbs_fp64": vc_gbs64, "vcycle_bytes_fp64": vc_bytes64,
-            "per_level_fp32": per_level, "tail_fp32": tail, "per_level_fp64": per_level64,
+            "per_level_fp32": per_level, "cluster_fp32": cluster, "per_level_fp64": per_level64,
             "wall_ms_timed_region": wall,
             "parallelism": f"replicas x{ws}" if ws > 1 else "single GPU",
             "workloads": extra,
