@@ -962,8 +962,10 @@ __global__ void k_many_gate(int K, const int* __restrict__ state, const cudaGrap
 // After an iteration: every mesh that ran gets its worst column's relative
 // residual and one more iteration, and is done once that is <= tol (a
 // non-finite residual ends the whole loop).  The loop continues while a mesh
-// is not done and the iteration limit is not reached.  One block.
-__global__ void k_many_check(int K, int nrhs, int* state, const double* __restrict__ nb, double* rel,
+// is not done and the iteration limit is not reached.  All NR columns of the
+// block are tested: the graph serves every call of its width, and the columns
+// that a call does not use have norm 0.  One block.
+__global__ void k_many_check(int K, int NR, int* state, const double* __restrict__ nb, double* rel,
                              const double* tol, double* const* rr, cudaGraphConditionalHandle hw) {
   __shared__ int open, bad;
   if (threadIdx.x == 0) {
@@ -976,7 +978,7 @@ __global__ void k_many_check(int K, int nrhs, int* state, const double* __restri
     if (st[0]) continue;
     double w = 0.0;
     bool fin = true;
-    for (int q = 0; q < nrhs; ++q) {
+    for (int q = 0; q < NR; ++q) {
       const double b = nb[k * kMaxRhs + q];
       const double r = b > 0.0 ? sqrt(rr[k][q]) / b : 0.0;
       if (!isfinite(r)) fin = false;
@@ -1028,8 +1030,9 @@ static gmg_status many_graph(gmg_many_ctx* m, cudaGraphExec_t* out, uint64_t* ke
 
 // The device-side loop: WHILE { gate -> IF_k { iteration of mesh k } for all k -> check }.
 template <int NR>
-static gmg_status many_loop(gmg_many_ctx* m, int slot, int nrhs) {
+static gmg_status many_loop(gmg_many_ctx* m, int slot) {
   const int K = (int)m->h.size();
+  int width = NR;
   cudaGraph_t g = nullptr;
   GMG_CK(cudaGraphCreate(&g, 0));
   cudaError_t e = cudaSuccess;
@@ -1081,7 +1084,7 @@ static gmg_status many_loop(gmg_many_ctx* m, int slot, int nrhs) {
   }
   if (e == cudaSuccess && st == GMG_OK) {
     cudaKernelNodeParams kp = {};
-    void* args[] = {(void*)&K, (void*)&nrhs, (void*)&m->d_state, (void*)&m->d_nb, (void*)&m->d_rel,
+    void* args[] = {(void*)&K, (void*)&width, (void*)&m->d_state, (void*)&m->d_nb, (void*)&m->d_rel,
                     (void*)&m->d_tol, (void*)&m->d_rr, (void*)&hw};
     kp.func = (void*)k_many_check;
     kp.gridDim = dim3(1);
@@ -1186,7 +1189,7 @@ static gmg_status many_solve(gmg_many_ctx* m, int nrhs, const double* const* B, 
     for (int attempt = 0; attempt < 2 && !m->loop[slot]; ++attempt) {
       g_pdl_suspended = attempt == 1;  // plain stream order if the driver refuses programmatic edges here
       m->loop_refused[slot] = false;
-      const gmg_status sl = many_loop<NR>(m, slot, nrhs);
+      const gmg_status sl = many_loop<NR>(m, slot);
       g_pdl_suspended = false;
       GMG_TRY(sl);
     }
