@@ -426,14 +426,14 @@ __global__ void __launch_bounds__(256) k_add_f2d_m(int64_t m, const float* e, do
 // After an iteration of the batched solve (one warp): the worst column's
 // relative residual into hist[k] (a non-finite column's value as it is), and
 // whether the loop goes on.  it: iterations done, limit, columns; nb: column
-// norms of B (0: a zero column).
+// norms of B, finite (0: a zero column).
 __global__ void k_batched_check(int* it, double* hist, const double* rr, const double* nb, const double* tol,
                                 cudaGraphConditionalHandle h) {
   pdl_wait();
   pdl_trigger();
   const int lane = threadIdx.x;
   const double b = lane < it[2] ? nb[lane] : 0.0;
-  const double r = b > 0.0 ? sqrt(rr[lane]) / b : 0.0;
+  const double r = b == 0.0 ? 0.0 : sqrt(rr[lane]) / b;
   const unsigned bad = __ballot_sync(0xffffffffu, !isfinite(r));
   double w = r;
   for (int o = 16; o > 0; o >>= 1) w = fmax(w, __shfl_xor_sync(0xffffffffu, w, o));
@@ -673,7 +673,8 @@ static gmg_status solve_m(gmg_ctx* c, int nrhs, const double* B, double* X, doub
   auto worst = [&]() {
     double w = 0.0;
     for (int q = 0; q < nrhs; ++q) {
-      const double r = nb[q] > 0 ? std::sqrt(c->h_scal[8 + q]) / nb[q] : 0.0;
+      // a norm that is not finite: so is the quotient (0 only where B's column is zero)
+      const double r = nb[q] == 0.0 ? 0.0 : std::sqrt(c->h_scal[8 + q]) / nb[q];
       if (!std::isfinite(r)) return r;
       w = std::max(w, r);
     }
@@ -980,7 +981,7 @@ __global__ void k_many_check(int K, int NR, int* state, const double* __restrict
     bool fin = true;
     for (int q = 0; q < NR; ++q) {
       const double b = nb[k * kMaxRhs + q];
-      const double r = b > 0.0 ? sqrt(rr[k][q]) / b : 0.0;
+      const double r = b == 0.0 ? 0.0 : sqrt(rr[k][q]) / b;
       if (!isfinite(r)) fin = false;
       w = fmax(w, r);
     }
@@ -1163,7 +1164,7 @@ static gmg_status many_solve(gmg_many_ctx* m, int nrhs, const double* const* B, 
       double w = 0.0;
       for (int q = 0; q < nrhs; ++q) {
         const double b = nb[(size_t)k * kMaxRhs + q];
-        const double r = b > 0 ? std::sqrt(m->h[k]->h_scal[8 + q]) / b : 0.0;
+        const double r = b == 0.0 ? 0.0 : std::sqrt(m->h[k]->h_scal[8 + q]) / b;
         w = std::isfinite(r) ? std::max(w, r) : r;
         if (!std::isfinite(r)) break;
       }
