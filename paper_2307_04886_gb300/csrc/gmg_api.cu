@@ -106,7 +106,7 @@ static void drop_graphs(gmg_ctx* c) {
       if (g) cudaGraphExecDestroy(g);
       g = nullptr;
     }
-    c->loop_refused[m] = false;
+    c->loop_refused[m][0] = c->loop_refused[m][1] = false;
   }
 }
 
@@ -136,7 +136,7 @@ static cudaError_t capture_into(gmg_ctx* c, cudaGraph_t g, std::vector<cudaGraph
 // launch and one synchronisation then serve a solve.  The kernels keep their
 // programmatic launch edges if the CUDA driver instantiates them around and
 // inside a conditional body, else all is captured again in plain stream order;
-// if neither instantiates, the mode keeps the host loop.
+// if neither instantiates, the host loop serves what this form would.
 static gmg_status build_loop(gmg_ctx* c, int mode, bool whole) {
   if (!c->g_stream) GMG_CK(cudaStreamCreateWithFlags(&c->g_stream, cudaStreamNonBlocking));
   cudaGraphExec_t& exec = c->loops[mode][whole];
@@ -203,7 +203,7 @@ static gmg_status build_loop(gmg_ctx* c, int mode, bool whole) {
       exec = nullptr;
     }
   }
-  if (!exec) c->loop_refused[mode] = true;
+  if (!exec) c->loop_refused[mode][whole] = true;
   if (const char* e = std::getenv("GMG_VERBOSE"))
     if (e[0] == '1')
       std::fprintf(stderr, "gmg: device-side loop for mode %d: %s\n", mode,
@@ -213,14 +213,19 @@ static gmg_status build_loop(gmg_ctx* c, int mode, bool whole) {
 
 // Whether a solve in `mode` runs device-driven: graphs on, no per-cycle timing
 // (event nodes are not allowed in a conditional body), GMG_NO_DEVICE_LOOP
-// unset, an iteration to do, and the graph instantiated.
+// unset, an iteration to do, and the graph instantiated.  GMG_NO_RESTART_LOOP=1
+// leaves out the form that continues after a start on the stream (tests: the
+// host loop then goes on from a restart, as where that graph is refused).
 static gmg_status device_loop_ready(gmg_ctx* c, int mode, bool whole, bool* ok) {
   static const bool off = [] {
     const char* e = std::getenv("GMG_NO_DEVICE_LOOP");
     return e && e[0] == '1';
   }();
   *ok = false;
-  if (off || !c->opt.use_graphs || c->prof || c->loop_refused[mode] || c->opt.max_iter <= 0) return GMG_OK;
+  if (off || !c->opt.use_graphs || c->prof || c->loop_refused[mode][whole] || c->opt.max_iter <= 0) return GMG_OK;
+  if (!whole)
+    if (const char* e = std::getenv("GMG_NO_RESTART_LOOP"))
+      if (e[0] == '1') return GMG_OK;
   if (!c->loops[mode][whole]) GMG_TRY(build_loop(c, mode, whole));
   *ok = c->loops[mode][whole] != nullptr;
   return GMG_OK;
@@ -260,7 +265,7 @@ struct SolveRun {
   int k = 0;
   double rel = 0.0;
   gmg_status st = GMG_ERR_NOT_CONVERGED;
-  bool rewrite = false;      // on_device: xs changed after it was stored
+  bool rewrite = false;      // on_device: xs changes after it was stored
   bool wait_failed = false;  // on_device: a bounded wait ran out
 
   void record(int kk, double v) {
@@ -343,10 +348,14 @@ struct SolveRun {
         st = GMG_OK;
         return GMG_OK;
       }
+      if (!is_pcg(mode) || k >= c->opt.max_iter) break;
       bool again = false;
-      if (is_pcg(mode) && k < c->opt.max_iter) GMG_TRY(device_loop_ready(c, mode, false, &again));
-      if (!again) break;
+      GMG_TRY(device_loop_ready(c, mode, false, &again));
       GMG_TRY(pcg_start(c, mode, s));  // restart from the current iterate
+      if (!again) {  // no graph for what follows a restart
+        rewrite = true;
+        return host_steps(nb);
+      }
       whole = false;
     }
     set_error("gmg_solve: max_iter reached");
@@ -363,6 +372,11 @@ struct SolveRun {
     if (!go) return GMG_OK;
     if (!is_pcg(mode)) GMG_TRY(join_inverse(c, s, false));
     if (is_pcg(mode)) GMG_TRY(pcg_start(c, mode, s));
+    return host_steps(nb);
+  }
+
+  // The iterations from k on (CG: after a start or restart).
+  gmg_status host_steps(double nb) {
     bool fresh = true;  // CG: no step since the (re)start
     while (k < c->opt.max_iter) {
       if (is_pcg(mode) && !fresh) GMG_TRY(run_cycle_body(c, mode, 1, s));
@@ -546,7 +560,7 @@ gmg_status gmg_solve(gmg_handle h, const double* b, double* x, double tol, int m
     info->rel_res = run.rel;
   }
   GMG_TRY(inverse_status(c, s));  // the pivot check of an inverse this solve joined
-  if (!dev || run.wait_failed) GMG_TRY(cluster_status(c, s));
+  if (!dev || run.rewrite || run.wait_failed) GMG_TRY(cluster_status(c, s));
   return run.st;
 }
 

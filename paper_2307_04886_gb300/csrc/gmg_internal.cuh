@@ -318,7 +318,7 @@ struct gmg_ctx {
   cudaGraphExec_t loops[4][2] = {};
   uint64_t loop_once[4][2] = {};     // kernel nodes outside the loop
   uint64_t loop_kernels[4] = {};     // kernel nodes of one loop iteration
-  bool loop_refused[4] = {};         // instantiation failed: the host loop serves the mode
+  bool loop_refused[4][2] = {};      // instantiation failed: the host loop serves what this graph would
   // the same for the batched solve, by block width NR = 1, 2, 4, 8, 16
   cudaGraphExec_t mloops[5] = {};
   uint64_t mloop_kernels[5] = {};
