@@ -59,8 +59,12 @@ typedef enum {
 enum {
   GMG_FP64 = 0,        /* plain Alg. 1: FP64 V-cycles, x <- MGI(x, b, 1)       */
   GMG_FP32_REFINE = 1, /* FP64 iterative refinement: r = b - A x (FP64),
-                          e = MGI(0, r, 1) in FP32 (coarsest solve FP64),
-                          x += e; identical to GMG_FP64 in exact arithmetic   */
+                          e = MGI(0, r, 1) in FP32, x += e; identical to
+                          GMG_FP64 in exact arithmetic.  FP32 cycles apply the
+                          coarsest inverse in FP64, but in FP32 (an FP32 copy,
+                          FP32 sums) inside a cluster launch (gmg_level_path)
+                          whose last smoothed level is small (some 6,000 rows)
+                          and not the only one                                */
   GMG_FP32_PCG = 2,    /* FP64 conjugate gradients preconditioned by one FP32
                           V-cycle per iteration (flexible Polak-Ribiere beta)  */
   GMG_FP64_PCG = 3     /* the same conjugate gradients preconditioned by one

@@ -64,6 +64,7 @@
 #include <string>
 #include <system_error>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "gmg_cycle.cuh"
@@ -285,8 +286,10 @@ __device__ __forceinline__ void l2_prefetch(const void* p, int64_t bytes, int ti
 
 // x <- MGI(x, b, l0) of Alg. 2 for the levels of D.  With c0_first the rows
 // of colour 0 of level l0 have already had their first update from x = 0.
-// All CTAs run the same sequence of phases.
-template <class T>
+// All CTAs run the same sequence of phases.  A: type of the coarsest solve's
+// coefficients and sums (a kernel of its own for each: with both in one the
+// registers of the phases ran out, 6 us a cycle).
+template <class T, class A>
 __global__ void __launch_bounds__(kClThreads, 1)
     k_cluster_cycle(const __grid_constant__ ClusterDesc<T> D, T* xg, const T* bg, int c0_first) {
   extern __shared__ __align__(16) char smem[];
@@ -302,6 +305,9 @@ __global__ void __launch_bounds__(kClThreads, 1)
   const uint32_t mimg = sm0 + (uint32_t)D.o_mbar, mst = mimg + 8u * (kClMaxLevels + 1);
   const uint32_t mph = mst + 8u * kClStages, mbc = mph + 16u;  // two phase barriers, the coarsest right-hand side's
   const int NL = D.nlev;  // smoothed levels; lv[NL] is the coarsest
+  const A* ainv;
+  if constexpr (std::is_same<A, T>::value) ainv = D.ainv;
+  else ainv = D.ainv64;
   // after a wait that gave up, in this launch or an earlier one, nothing is worth waiting for
   int polls = *reinterpret_cast<volatile int*>(D.err) ? 1 : kWaitPolls;
   if (tid == 0) {
@@ -383,9 +389,10 @@ __global__ void __launch_bounds__(kClThreads, 1)
   for (int k = 0; k < kX; ++k) g[k] = tid + k * kClThreads < n0loc ? l2g[tid + k * kClThreads] : 0;
   mbar_wait(mimg + 8u * NL, 0u, D.err, polls);
 #pragma unroll 1
-  for (int i = warp; i < reinterpret_cast<const int*>(sm + D.lv[NL].o_img)[0]; i += kClWarps)
-    l2_prefetch(D.ainv + (int64_t)reinterpret_cast<const int*>(sm + D.lv[NL].o_img + D.lv[NL].i_cr)[i] * D.nc,
-                (int64_t)sizeof(T) * D.nc, lane, 32);
+  for (int i = warp; i < reinterpret_cast<const int*>(sm + D.lv[NL].o_img)[0]; i += kClWarps) {
+    const int64_t row = reinterpret_cast<const int*>(sm + D.lv[NL].o_img + D.lv[NL].i_cr)[i];
+    l2_prefetch(ainv + row * D.nc, (int64_t)sizeof(A) * D.nc, lane, 32);
+  }
   pdl_wait();  // x and b were written by the previous kernels
   pdl_trigger();
   {
@@ -531,7 +538,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
     if (h == NL) {
       // coarsest: x_c = A^-1 b_c, a warp per kC own rows at a time, the first
       // rows' coefficients loaded before the wait (they come from L2, so many have
-      // to be in flight)
+      // to be in flight); sums in the coefficients' type
       {
         const ClusterLevel<T>& L = D.lv[NL];
         char* img = sm + L.o_img;
@@ -539,42 +546,55 @@ __global__ void __launch_bounds__(kClThreads, 1)
         const int* gid = reinterpret_cast<const int*>(img + L.i_cr);
         const int bytes = *reinterpret_cast<const int*>(img + L.i_ex);
         const uint32_t a_xd = sm0 + (uint32_t)(L.o_img + L.i_xd), a_x = sm0 + (uint32_t)L.o_x;
-        constexpr int kC = sizeof(T) == 4 ? 4 : 1, kA = 24;
+        constexpr bool kWiden = sizeof(A) > sizeof(T);
+        // rows at a time and coefficients of each that a lane holds: as many as
+        // the registers take without spills (columns past 32 kA are loaded as
+        // they are added)
+        constexpr int kC = sizeof(A) == 4 ? 4 : 1, kA = 24;
+        const uint32_t a_rhs = kWiden ? sm0 + (uint32_t)D.o_bd : a_bc;
         const int n = D.nc;
-        T a[kC][kA];
+        A a[kC][kA];
         auto coefs = [&](int i) {
 #pragma unroll
           for (int c = 0; c < kC; ++c) {
-            const T* ar = D.ainv + (int64_t)gid[i + c < nown ? i + c : i] * n;
+            const A* ar = ainv + (int64_t)gid[i + c < nown ? i + c : i] * n;
 #pragma unroll
-            for (int q = 0; q < kA; ++q) a[c][q] = lane + 32 * q < n ? ar[lane + 32 * q] : T(0);
+            for (int q = 0; q < kA; ++q) a[c][q] = lane + 32 * q < n ? ar[lane + 32 * q] : A(0);
           }
         };
         int i = warp * kC;
         if (i < nown) coefs(i);
         begin();
         mbar_wait(mbc, 0u, D.err, polls);
+        if constexpr (kWiden) {  // the right-hand side in FP64, once for all rows
+          for (int j = tid; j < n; j += kClThreads) {
+            T bv;
+            lds1(a_bc + (uint32_t)sizeof(T) * (uint32_t)j, bv);
+            sts(a_rhs + 8u * (uint32_t)j, to_f64(bv));
+          }
+          __syncthreads();
+        }
 #pragma unroll 1
         while (i < nown) {
-          T acc[kC];
+          A acc[kC];
 #pragma unroll
           for (int c = 0; c < kC; ++c) acc[c] = 0;
 #pragma unroll
           for (int q = 0; q < kA; ++q) {
-            T bv = 0;
-            if (lane + 32 * q < n) lds1(a_bc + (uint32_t)sizeof(T) * (uint32_t)(lane + 32 * q), bv);
+            A bv = 0;
+            if (lane + 32 * q < n) lds1(a_rhs + (uint32_t)sizeof(A) * (uint32_t)(lane + 32 * q), bv);
 #pragma unroll
             for (int c = 0; c < kC; ++c) acc[c] += a[c][q] * bv;
           }
           if (n > 32 * kA)
 #pragma unroll 1
             for (int c = 0; c < kC; ++c) {
-              const T* ar = D.ainv + (int64_t)gid[i + c < nown ? i + c : i] * n;
-              T t = 0;
+              const A* ar = ainv + (int64_t)gid[i + c < nown ? i + c : i] * n;
+              A t = 0;
 #pragma unroll 4
               for (int q = lane + 32 * kA; q < n; q += 32) {
-                T bv;
-                lds1(a_bc + (uint32_t)sizeof(T) * (uint32_t)q, bv);
+                A bv;
+                lds1(a_rhs + (uint32_t)sizeof(A) * (uint32_t)q, bv);
                 t += ar[q] * bv;
               }
               acc[c] += t;
@@ -586,7 +606,11 @@ __global__ void __launch_bounds__(kClThreads, 1)
           for (int c = 0; c < kC; ++c) {
 #pragma unroll 1
             for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-            if (lane == c && cur + c < nown) sts(a_x + (uint32_t)sizeof(T) * (uint32_t)(cur + c), acc[c]);
+            if (lane == c && cur + c < nown) {
+              const uint32_t xc = a_x + (uint32_t)sizeof(T) * (uint32_t)(cur + c);
+              if constexpr (kWiden) sts(xc, f32_rn(acc[c]));
+              else sts(xc, acc[c]);
+            }
           }
         }
         __syncthreads();
@@ -872,19 +896,25 @@ cudaLaunchConfig_t cluster_config(const ClusterDesc<T>& D, cudaLaunchAttribute* 
   return cfg;
 }
 
+// The kernel that a cluster runs.
+template <class T>
+auto cluster_kernel(const ClusterDesc<T>& D) {
+  return D.coarse64 ? k_cluster_cycle<T, double> : k_cluster_cycle<T, T>;
+}
+
 // Whether the device can run such a cluster (sets the kernel's attributes).
 template <class T>
 bool cluster_fits(const ClusterDesc<T>& D) {
-  if (cudaFuncSetAttribute(k_cluster_cycle<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-      cudaFuncSetAttribute(k_cluster_cycle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) !=
-          cudaSuccess) {  // the limit every handle's layout stays within
+  auto* k = cluster_kernel(D);
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess) {  // the limit every handle's layout stays within
     cudaGetLastError();
     return false;
   }
   cudaLaunchAttribute at[2];
   cudaLaunchConfig_t cfg = cluster_config(D, at, nullptr);
   int nclusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&nclusters, k_cluster_cycle<T>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&nclusters, k, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -1425,6 +1455,8 @@ bool lay_out(const std::vector<Tab>& tab, int nu_pre, int nu_post, ClusterDesc<T
     }
     D.o_bc = (int)std::min<int64_t>(cur, INT32_MAX);
     cur = al16(cur + (int64_t)sizeof(T) * tab[nl].n);
+    D.o_bd = (int)std::min<int64_t>(cur, INT32_MAX);
+    if (D.coarse64 && sizeof(T) == 4) cur = al16(cur + 8 * tab[nl].n);
     D.o_buf = (int)std::min<int64_t>(cur, INT32_MAX);
     D.nsteps = nsteps;
     const bool all = std::all_of(streamed.begin(), streamed.end(), [](char v) { return v != 0; });
@@ -1666,6 +1698,25 @@ struct Plan {
   bool checked = true;
 };
 
+// Whether the coarsest solve of FP32 cycles takes the FP32 copy of the inverse
+// and FP32 sums: hierarchies of two or more smoothed levels the last of which
+// is small (vectors of all its rows and a CTA's share of its entries within
+// one CTA's shared memory: some 6,000 rows).  Elsewhere, on two-level
+// hierarchies above all, it takes the FP64 inverse with FP64 sums, as the
+// launch-per-phase form does: with one smoothed level the coarsest solve is
+// the whole coarse correction, and on a nearly singular system (condition
+// number of the coarsest operator above 2^24) the FP32 inverse made solves
+// stall (a 642-vertex sphere, (S + 1e-7 M) x = M y to 1e-7: 12 steps for 6).
+// The price is the narrow FP64 pipe: 402 rows take 4.5 us more a cycle
+// (2,562-vertex sphere, FP32-PCG: 252 -> 278 us).
+inline bool coarsest_in_fp32(const gmg_ctx* c) {
+  const int lam = c->nlev - 1;
+  if (lam < 2) return false;
+  const Level& L = c->L[lam - 1];
+  const int64_t bytes = 24 * L.n + L.A.entries * 8 / 16 * 11 / 10 + 8 * c->L[lam].n;
+  return bytes <= kSmemLimit;
+}
+
 template <class T>
 void plan_one(const gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
               const std::vector<std::vector<int32_t>>& hcol, const std::vector<std::vector<int32_t>>& perm,
@@ -1724,6 +1775,7 @@ void plan_one(const gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
       E.nu_pre = c->opt.nu_pre;
       E.nu_post = c->opt.nu_post;
       E.post_forward = c->opt.post_forward;
+      E.coarse64 = sizeof(T) == 8 || !coarsest_in_fp32(c);
       if (!lay_out(tab, E.nu_pre, E.nu_post, E)) continue;
       if (!check_tables(team, tab, pu)) {
         plan.checked = false;
@@ -1745,6 +1797,7 @@ gmg_status finish_one(gmg_ctx* c, Plan<T>& plan) {
   }
   if (plan.D.l0 < 0) return GMG_OK;
   plan.D.ainv = Src<T>::ainv(c);
+  plan.D.ainv64 = c->Ainv;
   plan.D.err = c->dstatus + 3;
   GMG_CK(cudaMemset(plan.D.err, 0, sizeof(int)));
   GMG_TRY(upload_tables(*plan.team, c, plan.tab, plan.D));
@@ -1850,7 +1903,7 @@ gmg_status launch_cluster(gmg_ctx* c, T* x, const T* b, bool c0_first, cudaStrea
   cudaLaunchAttribute at[2];
   cudaLaunchConfig_t cfg = cluster_config(D, at, s);
   cfg.numAttrs = use_pdl() ? 2 : 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_cluster_cycle<T>, D, x, b, c0_first ? 1 : 0);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, cluster_kernel(D), D, x, b, c0_first ? 1 : 0);
   if (e != cudaSuccess) {
     set_error(std::string("cluster launch: ") + cudaGetErrorString(e));
     return GMG_ERR_CUDA;

@@ -13,7 +13,8 @@
 // atomics, a fixed summation order); it also clears the coarse iterate (the
 // recursive call of Alg. 2 starts from zero).  The prolongation reads three
 // packed (index, weight) slots per fine row.  The coarsest level applies the
-// explicit FP64 inverse of its operator as a warp-per-row GEMV.
+// explicit FP64 inverse of its operator as a warp-per-row GEMV (the cluster
+// launch, gmg_cluster.cu, has its own coarsest solve).
 //
 // Launches use programmatic dependent launch: a kernel may start while its
 // predecessor drains; it loads only setup-time data (matrix values, column

@@ -257,10 +257,12 @@ struct ClusterDesc {
   int l0 = -1;  // first level (-1: no cluster)
   int ncta = 0, nlev = 0, nc = 0;
   int nu_pre = 0, nu_post = 0, post_forward = 0;
+  bool coarse64 = false;  // FP32 cycles: coarsest solve with the FP64 inverse and FP64 sums
   int nstage = 0, nsteps = 0, stage_bytes = 0;
-  int o_mbar = 0, o_tok = 0, o_r[2] = {0, 0}, o_bc = 0, o_buf = 0, i_steps = 0, i_partners = 0, smem = 0;
+  int o_mbar = 0, o_tok = 0, o_r[2] = {0, 0}, o_bc = 0, o_bd = 0, o_buf = 0, i_steps = 0, i_partners = 0, smem = 0;
   int* err = nullptr;  // set when a bounded wait for an entry block gave up
   const T* ainv = nullptr;
+  const double* ainv64 = nullptr;
   const int32_t* l2g = nullptr;  // level l0: global rows of each CTA's own and halo rows
   const uint4* s_ent = nullptr;  // streamed entry units
   const int32_t* s_src = nullptr;
