@@ -443,15 +443,22 @@ gmg_status gmg_pivot_reciprocal(int64_t n, const double *d, double *out, void *s
 gmg_status gmg_convert(int64_t n, int dir, const void *in, void *out, void *stream);
 
 /* Self-test of the bounded device-side wait (no counterpart in the paper).
- * The cluster kernel waits for its streamed matrix entries on an
- * mbarrier with a limit of polls, after which they set an error word that
- * gmg_solve reports as GMG_ERR_TIMEOUT, instead of hanging.  This runs that
- * wait, in one warp, on an mbarrier that nothing arrives on: *timed_out
+ * The cluster kernel waits for its tables, its streamed matrix entries and
+ * the other CTAs' values on mbarriers with a limit of polls, after which it
+ * sets an error word that gmg_solve reports as GMG_ERR_TIMEOUT, waits no more
+ * and ends, instead of hanging.  This runs that wait, in one warp, on an mbarrier that nothing arrives on: *timed_out
  * receives 1 when the wait gave up (the expected outcome), *ms (may be NULL)
  * its device time.  polls <= 0 uses the limit of the solve kernels.  The
  * kernel returns normally, so the context stays usable.  Errors: INVALID_ARG
  * (null timed_out), OOM, CUDA. */
 gmg_status gmg_wait_selftest(int polls, int *timed_out, double *ms, void *stream);
+
+/* Sets the limit of polls after which a wait of this handle's cluster
+ * launches gives up (no counterpart in the paper): < 0 the default (about one
+ * second), 0 gives up at once, which takes a solve through the path of a lost
+ * copy without losing one.  Call between solves; it drops captured graphs
+ * (they are re-captured on the next solve).  Errors: INVALID_ARG. */
+gmg_status gmg_wait_limit(gmg_handle h, int polls);
 
 /* ---- allocation-free residual (no counterpart in the paper) ----
  * For callers that cannot allocate device memory (code running inside

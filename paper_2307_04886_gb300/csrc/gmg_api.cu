@@ -564,6 +564,13 @@ gmg_status gmg_solve(gmg_handle h, const double* b, double* x, double tol, int m
   return run.st;
 }
 
+gmg_status gmg_wait_limit(gmg_handle h, int polls) {
+  GMG_TRY(check_handle(h));
+  set_wait_polls(h, polls);
+  drop_graphs(h);  // they hold the limit they were captured with
+  return GMG_OK;
+}
+
 gmg_status gmg_profile(gmg_handle h, int enable) {
   GMG_TRY(check_handle(h));
   if ((enable != 0) == h->prof) return GMG_OK;

@@ -43,6 +43,24 @@
 // before the one that writes it.  Prolongated values of the colour that the
 // post-smoothing updates first are not sent: nobody reads them.
 //
+// Waits that give up.  Every wait on an mbarrier is bounded, and what follows
+// one that gave up stays in range and ends:
+//  * the tables are waited for before anything is read from them; a CTA that
+//    misses one copies them all by plain loads;
+//  * a warp that misses a block of entries leaves its rows from then on, and
+//    the thread that issues the blocks issues no more;
+//  * a lost message leaves an old value in a halo, nothing else; the thread
+//    that arms the phase barriers arms none whose last phase it missed, and the
+//    messages of a whole cycle stay within a barrier's byte count, so that a
+//    CTA that waits no more may run ahead;
+//  * every CTA reaches both cluster barriers, since its waits end; before the
+//    second it waits, bounded, for its own copies in flight, and after it a CTA
+//    that missed something stays a while for messages on their way to it.
+// No CTA leaves the phases early: a way out of them, or a function call, cost
+// 4 to 7 % of every solve (the compiler then takes the phase loops for
+// divergent).  The error word makes later launches wait no more, and the
+// solve that reads it report GMG_ERR_TIMEOUT.
+//
 // Entries stay in shared memory where they fit; the entries of the largest
 // levels stream from L2 by TMA bulk copies, one phase's block per stage,
 // issued up to three phases ahead.
@@ -136,7 +154,7 @@ __device__ __forceinline__ bool mbar_try(uint32_t m, unsigned parity) {
   return done != 0;
 }
 // Waits for the phase of m with the given parity to complete; gives up after
-// `polls` polls (sets *err, and polls to 1 for the waits that follow) so that
+// `polls` polls (sets *err, and polls to 0: the thread waits no more) so that
 // a lost copy or message cannot hang the GPU.  A failing poll suspends the
 // warp for about 3.8 us on GB300 (measured with gmg_wait_selftest), so the
 // limit gives up after about one second; a poll does not advance while the
@@ -147,7 +165,7 @@ __device__ __forceinline__ void mbar_wait(uint32_t m, unsigned parity, int* err,
   for (int it = 0; it < polls; ++it)
     if (mbar_try(m, parity)) return;
   atomicOr(err, 1);
-  polls = 1;
+  polls = 0;
 }
 
 // Shared-memory accesses by 32-bit address, kept in program order with the
@@ -282,6 +300,18 @@ __device__ __forceinline__ void l2_prefetch(const void* p, int64_t bytes, int ti
     asm volatile("prefetch.global.L2 [%0];" ::"l"(c + o));
 }
 
+// Stays 0.1 ms for messages that may be on their way to a CTA that missed some.
+__device__ __forceinline__ void linger() {
+  unsigned long long t0, t1;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+#pragma unroll 1
+  for (int it = 0; it < 1024; ++it) {
+    __nanosleep(500);
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+    if (t1 - t0 > 100000) break;
+  }
+}
+
 }  // namespace
 
 // x <- MGI(x, b, l0) of Alg. 2 for the levels of D.  With c0_first the rows
@@ -308,8 +338,8 @@ __global__ void __launch_bounds__(kClThreads, 1)
   const A* ainv;
   if constexpr (std::is_same<A, T>::value) ainv = D.ainv;
   else ainv = D.ainv64;
-  // after a wait that gave up, in this launch or an earlier one, nothing is worth waiting for
-  int polls = *reinterpret_cast<volatile int*>(D.err) ? 1 : kWaitPolls;
+  // after a wait that gave up in an earlier launch nothing is worth waiting for
+  int polls = *reinterpret_cast<volatile int*>(D.err) ? 0 : D.polls;
   if (tid == 0) {
 #pragma unroll 1
     for (int q = 0; q <= NL; ++q) mbar_init(mimg + 8u * q, 1);
@@ -348,7 +378,21 @@ __global__ void __launch_bounds__(kClThreads, 1)
 #pragma unroll 1
     for (int i = tid; i < D.lv[t].n_loc_max; i += kClThreads) x[i] = T(0);
   }
-  mbar_wait(mimg, 0u, D.err, polls);
+#pragma unroll 1
+  for (int q = 0; q <= NL; ++q) mbar_wait(mimg + 8u * q, 0u, D.err, polls);
+  if (__syncthreads_or(polls == 0)) {  // by plain loads then: what follows indexes with them
+#pragma unroll 1
+    for (int t = 0; t <= NL; ++t) {
+      const ClusterLevel<T>& L = D.lv[t];
+      const int* img = reinterpret_cast<const int*>(L.img + (int64_t)cta * L.img_bytes);
+      const int* val = reinterpret_cast<const int*>(L.vimg + (int64_t)cta * L.val_bytes);
+#pragma unroll 1
+      for (int i = tid; i < L.img_bytes / 4; i += kClThreads) reinterpret_cast<int*>(sm + L.o_img)[i] = img[i];
+#pragma unroll 1
+      for (int i = tid; i < L.val_bytes / 4; i += kClThreads) reinterpret_cast<int*>(sm + L.o_val)[i] = val[i];
+    }
+    __syncthreads();
+  }
   // stream step j's entry block into stage j % nstage (level l0's table
   // starts with the phase of colour 0, skipped with c0_first)
   const int skip = c0_first && D.lv[0].streamed ? 1 : 0;
@@ -357,8 +401,10 @@ __global__ void __launch_bounds__(kClThreads, 1)
   int j = 0, jst = 0;     // next stream step to use, its stage
   unsigned jpar = 0;      // and that stage's parity
   int ji = 0, jist = 0;   // next step to issue, its stage
+  int issued = 0;         // steps issued (the issuing thread's)
   auto issue = [&]() {
-    if (ji < S && tid == kClThreads - 32) {
+    if (ji < S && tid == kClThreads - 32 && polls > 0) {
+      issued = ji + 1;
       const uint2 st = steps[ji];
       const uint32_t m = mst + 8u * (uint32_t)jist;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the stage's earlier reads come first
@@ -387,7 +433,6 @@ __global__ void __launch_bounds__(kClThreads, 1)
   int g[kX];
 #pragma unroll
   for (int k = 0; k < kX; ++k) g[k] = tid + k * kClThreads < n0loc ? l2g[tid + k * kClThreads] : 0;
-  mbar_wait(mimg + 8u * NL, 0u, D.err, polls);
 #pragma unroll 1
   for (int i = warp; i < reinterpret_cast<const int*>(sm + D.lv[NL].o_img)[0]; i += kClWarps) {
     const int64_t row = reinterpret_cast<const int*>(sm + D.lv[NL].o_img + D.lv[NL].i_cr)[i];
@@ -441,7 +486,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
     cl_send_if(sends_token, tok_a, tok_m + 8u * (uint32_t)(ph & 1), 0.f);
   };
   auto end = [&](int bytes) {
-    if (tid == 0) mbar_expect(mcur(), (unsigned)(bytes + 4 * npart));
+    if (tid == 0 && polls > 0) mbar_expect(mcur(), (unsigned)(bytes + 4 * npart));
     ++ph;
   };
 
@@ -464,17 +509,19 @@ __global__ void __launch_bounds__(kClThreads, 1)
     int k = q0 % C;
     uint4 cr = lds4(a_cr + 16u * (uint32_t)(descending ? C - 1 - k : k)), d = make_uint4(0, 0, 0, 0);
     if (warp < (int)cr.y) d = lds4(a_sl + 16u * cr.x);
+    bool landed = true;  // the warp has missed no block of entries
 #pragma unroll 1
     for (int q = q0;;) {
       if (streamed) {
         a_ent = sm0 + (uint32_t)(D.o_buf + jst * D.stage_bytes) + 16u * (uint32_t)lane;
         mbar_wait(mst + 8u * (uint32_t)jst, jpar, D.err, polls);
+        landed = __all_sync(0xffffffffu, polls > 0);
       }
       uint4 ncr = cr, nd = d;
       bool waited = false;
 #pragma unroll 1
       for (int si = warp;;) {
-        const bool any = si < (int)cr.y;
+        const bool any = si < (int)cr.y && landed;
         const int row0 = (int)(d.x & 0xFFFFu), row = row0 + ri, np = (int)(d.w & 1023u);
         const uint32_t ea = a_ent + 16u * d.z, a_row = a_bd + 2u * (uint32_t)sizeof(T) * (uint32_t)row;
         uint4 u[4];
@@ -730,7 +777,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
               par ^= 1;
             }
           }
-          const int se = cr[k + nk - 1].x + cr[k + nk - 1].y;
+          const int se = __all_sync(0xffffffffu, polls > 0) ? cr[k + nk - 1].x + cr[k + nk - 1].y : 0;
 #pragma unroll 1
           for (int s = cr[k].x + warp, q = 0; s < se; s += kClWarps) {
 #pragma unroll 1
@@ -786,7 +833,6 @@ __global__ void __launch_bounds__(kClThreads, 1)
       };
       int s = warp;
       if (s < nrs) start(s);
-      mbar_wait(mimg + 8u * (t + 1), 0u, D.err, polls);
       char* nimg = sm + N.o_img;
       const bool first_upd = D.nu_pre > 0 && t + 1 < NL;
       const int nc0 = first_upd ? reinterpret_cast<const int*>(nimg)[4] : 0;
@@ -846,8 +892,18 @@ __global__ void __launch_bounds__(kClThreads, 1)
 #pragma unroll 1
     for (int i = tid; i < n0own; i += kClThreads) xg[l2g[i]] = x[i];
   }
+  // the copies in flight land first: tables, the last block issued into every stage
+  if ((tid == 0 || tid == kClThreads - 32) && polls == 0) {
+    int again = kWaitPolls;
+#pragma unroll 1
+    for (int q = 0; q <= NL; ++q) mbar_wait(mimg + 8u * q, 0u, D.err, again);
+#pragma unroll 1
+    for (int q = issued > NS ? issued - NS : 0; q < issued; ++q)
+      mbar_wait(mst + 8u * (uint32_t)(q % NS), (unsigned)(q / NS) & 1u, D.err, again);
+  }
   cl_arrive();  // no CTA's shared memory goes before every message has landed
   cl_wait();
+  if (polls == 0) linger();
 }
 
 // Element e of a job is the level's value in slot src[e] >= 0, 0 for -1, or
@@ -1767,6 +1823,19 @@ void plan_one(const gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
         local = local && (!tab[t].wide || stores <= 3 * tab[t].n);
       }
       if (!local) continue;
+      // a CTA that waits no more may send all of a cycle's messages before a
+      // partner has taken the first: they have to stay within the 2^20 - 1
+      // bytes that a barrier counts (each halo row once a sweep and once or
+      // twice besides, the residual's halo once, a token of 4 bytes a phase
+      // from each of 15 partners)
+      double bytes = 0;
+      for (const Tab& t : tab) {
+        size_t halo = 0, rhalo = 0;
+        for (const Part& p : t.part) halo = std::max(halo, p.halo.size()), rhalo = std::max(rhalo, p.rhalo.size());
+        const double nu = (double)c->opt.nu_pre + c->opt.nu_post;
+        bytes += (nu + 2) * (double)(sizeof(T) * halo) + (double)(sizeof(T) * rhalo) + 60 * (nu * t.ncolor + 4);
+      }
+      if (bytes >= 1048575.0) continue;
       ClusterDesc<T> E{};
       E.l0 = l0;
       E.ncta = ncta;
@@ -1799,6 +1868,7 @@ gmg_status finish_one(gmg_ctx* c, Plan<T>& plan) {
   plan.D.ainv = Src<T>::ainv(c);
   plan.D.ainv64 = c->Ainv;
   plan.D.err = c->dstatus + 3;
+  plan.D.polls = kWaitPolls;
   GMG_CK(cudaMemset(plan.D.err, 0, sizeof(int)));
   GMG_TRY(upload_tables(*plan.team, c, plan.tab, plan.D));
   Src<T>::desc(c) = plan.D;
@@ -1914,6 +1984,9 @@ gmg_status launch_cluster(gmg_ctx* c, T* x, const T* b, bool c0_first, cudaStrea
 template gmg_status launch_cluster<float>(gmg_ctx*, float*, const float*, bool, cudaStream_t);
 template gmg_status launch_cluster<double>(gmg_ctx*, double*, const double*, bool, cudaStream_t);
 
+// The polls after which the waits of this handle's cluster launches give up.
+void set_wait_polls(gmg_ctx* c, int polls) { c->cl32.polls = c->cl64.polls = polls < 0 ? kWaitPolls : polls; }
+
 // Self-test of the bounded wait: one warp waits on an mbarrier that nothing
 // arrives on, so every poll fails and the wait gives up; elapsed device time
 // in *ns.
@@ -1929,8 +2002,8 @@ __global__ void k_wait_selftest(int polls, int* err, unsigned long long* ns) {
   if (threadIdx.x == 0) *ns = t1 - t0;
 }
 
-// GMG_ERR_TIMEOUT once if a cluster launch gave up waiting for an entry block
-// (its results are then not to be trusted); clears the flag.
+// GMG_ERR_TIMEOUT once if a wait of a cluster launch gave up (its results are
+// then not to be trusted); clears the flag.
 gmg_status cluster_status(gmg_ctx* c, cudaStream_t s) {
   int* err = c->cl32.l0 >= 0 ? c->cl32.err : c->cl64.l0 >= 0 ? c->cl64.err : nullptr;
   if (!err) return GMG_OK;
@@ -1939,7 +2012,7 @@ gmg_status cluster_status(gmg_ctx* c, cudaStream_t s) {
   GMG_CK(cudaStreamSynchronize(s));
   if (h) {
     GMG_CK(cudaMemsetAsync(err, 0, sizeof(int), s));
-    set_error("cluster launch: a wait for streamed matrix entries timed out");
+    set_error("cluster launch: a wait for tables, matrix entries or another CTA's values timed out");
     return GMG_ERR_TIMEOUT;
   }
   return GMG_OK;

@@ -260,7 +260,8 @@ struct ClusterDesc {
   bool coarse64 = false;  // FP32 cycles: coarsest solve with the FP64 inverse and FP64 sums
   int nstage = 0, nsteps = 0, stage_bytes = 0;
   int o_mbar = 0, o_tok = 0, o_r[2] = {0, 0}, o_bc = 0, o_bd = 0, o_buf = 0, i_steps = 0, i_partners = 0, smem = 0;
-  int* err = nullptr;  // set when a bounded wait for an entry block gave up
+  int* err = nullptr;  // set when a bounded wait gave up (for a table, an entry block or a message)
+  int polls = 0;       // limit of each wait
   const T* ainv = nullptr;
   const double* ainv64 = nullptr;
   const int32_t* l2g = nullptr;  // level l0: global rows of each CTA's own and halo rows
@@ -374,4 +375,5 @@ gmg_status refresh_cluster_values(gmg_ctx* c, cudaStream_t s);
 template <class T>
 gmg_status launch_cluster(gmg_ctx* c, T* x, const T* b, bool c0_first, cudaStream_t s);
 gmg_status cluster_status(gmg_ctx* c, cudaStream_t s);
+void set_wait_polls(gmg_ctx* c, int polls);
 }  // namespace gmg

@@ -1,0 +1,48 @@
+"""Solves whose cluster launches' waits give up (a limit of no polls: the path
+of a copy that does not come, without losing one): GMG_ERR_TIMEOUT, nothing
+read or written that should not be, and the bits of an undisturbed handle once
+the limit is back."""
+import numpy as np
+import pytest
+
+import gmg_inputs as gi
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gmg(cuda):
+    import paper_2307_04886_gb300 as g
+
+    g.load_library()
+    return g
+
+
+SYSTEMS = {
+    "one_launch": lambda: gi.icosphere_system(4),
+    "streamed": lambda: gi.workloads.bilaplacian_system(256, 120),
+    "below_a_colour_launch": lambda: gi.torus_system(320, 150, 1e-4, 3),
+}
+
+
+@pytest.mark.parametrize("name", sorted(SYSTEMS))
+@pytest.mark.parametrize("host_loop", [False, True])
+@pytest.mark.parametrize("precision", [0, 1, 2, 3])
+def test_a_wait_that_gives_up_is_reported(gmg, name, precision, host_loop):
+    import torch
+
+    s = SYSTEMS[name]()
+    b = torch.tensor(s.b, device="cuda")
+    g = gmg.Solver(s.A, s.Ps, precision=precision, max_iter=60)
+    assert any(p in (1, 2) for p in g.paths)
+    g.profile(host_loop)
+    x, it, rr, _, st = g.solve(b, tol=1e-9)
+    lib = gmg.load_library()
+    for _ in range(2):
+        assert lib.gmg_wait_limit(g.handle, 0) == gmg.GMG_OK
+        assert g.solve(b, tol=1e-9, raise_on_fail=False)[4] == gmg.GMG_ERR_TIMEOUT
+        assert lib.gmg_wait_limit(g.handle, -1) == gmg.GMG_OK
+        y, it2, rr2, _, st2 = g.solve(b, tol=1e-9)
+        assert st2 == gmg.GMG_OK and it2 == it and rr2 == rr
+        assert np.array_equal(y.cpu().numpy(), x.cpu().numpy())
+    g.close()
