@@ -414,7 +414,9 @@ gmg_status gmg_restrict(gmg_handle h, int l, int fp32, const double *r, double *
 gmg_status gmg_prolong_add(gmg_handle h, int l, int fp32, const double *u, double *x, void *stream);
 /* x = A_lambda^-1 b on the coarsest level (FP64 factor in both modes). */
 gmg_status gmg_coarse_solve(gmg_handle h, int fp32, const double *b, double *x, void *stream);
-/* One V-cycle x <- MGI(x, b, 1) of Alg. 2 on the finest level. */
+/* One V-cycle x <- MGI(x, b, 1) of Alg. 2 on the finest level.  The call does
+ * not synchronise; should a bounded wait of its cluster launch give up
+ * (GMG_ERR_TIMEOUT in a solve), x is NaN in every entry. */
 gmg_status gmg_vcycle(gmg_handle h, int fp32, const double *b, double *x, void *stream);
 /* One FP32 V-cycle X <- MGI(X, B, 1) of Alg. 2 applied to nrhs columns at
  * once, with the kernels gmg_solve_batched and gmg_solve_many run (each matrix

@@ -1869,7 +1869,6 @@ gmg_status finish_one(gmg_ctx* c, Plan<T>& plan) {
   plan.D.ainv64 = c->Ainv;
   plan.D.err = c->dstatus + 3;
   plan.D.polls = kWaitPolls;
-  GMG_CK(cudaMemset(plan.D.err, 0, sizeof(int)));
   GMG_TRY(upload_tables(*plan.team, c, plan.tab, plan.D));
   Src<T>::desc(c) = plan.D;
   return GMG_OK;

@@ -407,6 +407,16 @@ __global__ void k_gather(int64_t n, const int32_t* __restrict__ perm, const doub
   pdl_trigger();
   GRID_LOOP(i, n) dst[i] = src[perm[i]];
 }
+// The end of a single V-cycle: dst[perm] = src, or NaN everywhere if a bounded
+// wait of its cluster launch gave up (the call does not synchronise, so that it
+// cannot return the status).
+__global__ void k_scatter_cycle(int64_t n, const int32_t* __restrict__ perm, const double* src, double* dst,
+                                const int* wait_failed) {
+  pdl_wait();
+  pdl_trigger();
+  const bool failed = *wait_failed != 0;
+  GRID_LOOP(i, n) dst[perm[i]] = failed ? __longlong_as_double(0x7FF8000000000000LL) : src[i];
+}
 __global__ void k_scatter_vec(int64_t n, const int32_t* __restrict__ perm, const double* src, double* dst) {
   pdl_wait();
   pdl_trigger();
@@ -445,13 +455,13 @@ __global__ void k_add_f2d(int64_t n, const float* e, double* x) {
 // The vectors of a solve in the level's numbering, bs = b[perm] and
 // xs = x[perm], ||b||^2 into sc[S_NB2], and the solve's tolerance, iteration
 // counter and limit: one launch instead of two gathers, two reduction kernels
-// and two copies from the host.  Sums: fixed grid (kRedBlocks x 256), fixed
+// and two copies from the host; the bounded waits' error word is cleared.  Sums: fixed grid (kRedBlocks x 256), fixed
 // per-thread ranges, fixed tree.
 __global__ void __launch_bounds__(256, 4) k_load(int64_t n, const int32_t* __restrict__ perm,
                                               const double* __restrict__ b, const double* __restrict__ x,
                                               double* __restrict__ bs, double* __restrict__ xs,
                                               double* __restrict__ partial, int* counter, double* sc, int* it,
-                                              double tol, int max_iter) {
+                                              double tol, int max_iter, int* wait_failed) {
   __shared__ double red[1][256];
   pdl_wait();
   pdl_trigger();
@@ -474,6 +484,7 @@ __global__ void __launch_bounds__(256, 4) k_load(int64_t n, const int32_t* __res
       sc[S_TOL] = tol;
       it[0] = 0;
       it[1] = max_iter;
+      *wait_failed = 0;  // what an earlier call on the handle left there is not this solve's
     }
   }
 }
@@ -802,6 +813,10 @@ template gmg_status vcycle<float>(gmg_ctx*, int, cudaStream_t, bool, float*, con
 gmg_status launch_gather(int64_t n, const int32_t* perm, const double* src, double* dst, cudaStream_t s) {
   return launch(k_gather, blocks_for(n), 256, s, n, perm, src, dst);
 }
+gmg_status launch_scatter_cycle(gmg_ctx* c, const double* src, double* dst, cudaStream_t s) {
+  Level& L = c->L[0];
+  return launch(k_scatter_cycle, blocks_for(L.n), 256, s, L.n, L.perm, src, dst, (const int*)(c->dstatus + 3));
+}
 gmg_status launch_scatter(int64_t n, const int32_t* perm, const double* src, double* dst, cudaStream_t s) {
   return launch(k_scatter_vec, blocks_for(n), 256, s, n, perm, src, dst);
 }
@@ -913,7 +928,7 @@ gmg_status outer_residual_norm(gmg_ctx* c, bool start, cudaStream_t s) {
 gmg_status load_system(gmg_ctx* c, const double* b, const double* x, double tol, cudaStream_t s) {
   Level& L = c->L[0];
   return launch(k_load, kRedBlocks, 256, s, L.n, L.perm, b, x, c->bs, c->xs, c->red, c->red_cnt + 5, c->scal, c->dloop,
-                tol, c->opt.max_iter);
+                tol, c->opt.max_iter, c->dstatus + 3);
 }
 
 gmg_status store_solution(gmg_ctx* c, double* x, cudaStream_t s) {

@@ -79,6 +79,7 @@ enum { REP_NB2 = 0, REP_RR = 1, REP_OK = 2, REP_ITERS = 3, REP_REL = 4, REP_PIVO
 // loop's condition `h` (captured into the body of a WHILE node).
 gmg_status loop_body(gmg_ctx* c, int mode, cudaGraphConditionalHandle h, cudaStream_t s);
 gmg_status launch_gather(int64_t n, const int32_t* perm, const double* src, double* dst, cudaStream_t s);
+gmg_status launch_scatter_cycle(gmg_ctx* c, const double* src, double* dst, cudaStream_t s);
 gmg_status launch_scatter(int64_t n, const int32_t* perm, const double* src, double* dst, cudaStream_t s);
 
 }  // namespace gmg

@@ -1827,6 +1827,7 @@ gmg_status setup_impl(gmg_ctx* c, const gmg_csr* A, int nP, const gmg_prolong* P
   c->nlev = nP + 1;
   c->L.resize(c->nlev);
   GMG_TRY(a.alloc(&c->dstatus, 4));
+  GMG_CK(cudaMemset(c->dstatus, 0, 4 * sizeof(int)));
   // level 0 CSR (caller numbering)
   Level& L0 = c->L[0];
   L0.n = A->n;
