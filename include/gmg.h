@@ -174,7 +174,8 @@ gmg_status gmg_colour(int64_t n, const int64_t *rowptr, const int32_t *col, int3
  * gmg_solve_batched, gmg_vcycle, gmg_vcycle_batched, gmg_coarse_solve, or
  * another refresh) makes its own stream wait for it (a CG solve only right
  * before its first coarsest solve, so the first cycle's descent overlaps
- * it) and reports a non-positive pivot of it as CHOLESKY.
+ * it, unless one cluster launch is the whole cycle: gmg_level_path 1 or 2 on
+ * level 0) and reports a non-positive pivot of it as CHOLESKY.
  * Errors: NOT_SPD, NONFINITE (this call); CHOLESKY (the next such call). */
 gmg_status gmg_set_values(gmg_handle h, const double *val, int mem, void *stream);
 

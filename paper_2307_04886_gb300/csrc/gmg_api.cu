@@ -548,7 +548,10 @@ gmg_status gmg_solve(gmg_handle h, const double* b, double* x, double tol, int m
   SolveRun run{c, s, mode, tol, info};
   // a CG start joins a pending coarsest inverse right before its first coarse
   // solve (its down-leg overlaps the inverse), so it runs on the stream, not
-  // in a graph; the other modes join before their first iteration
+  // in a graph; the other modes join before their first iteration, and so does
+  // CG where one cluster launch is the whole cycle: there is no down-leg to
+  // overlap, and the whole solve is one graph
+  if (is_pcg(mode) && (mode == GMG_FP32_PCG ? c->cl32.l0 : c->cl64.l0) == 0) GMG_TRY(join_inverse(c, s, false));
   bool dev = false;
   const bool whole = !(is_pcg(mode) && c->inv_pending);
   GMG_TRY(device_loop_ready(c, mode, whole, &dev));
