@@ -392,7 +392,9 @@ gmg_status gmg_level_info(gmg_handle h, int l, int64_t *n, int64_t *nnz, int *nc
  * warp per row), 2 with each row's sum split over up to eight lanes; 3 = the
  * coarsest level (direct solve).  The FP64 cycle runs its coarse levels the
  * same way on handles whose options ask for FP64 cycles, and with one launch
- * per colour on the others.  Errors: INVALID_ARG. */
+ * per colour on the others.  On the former the FP32 cycle's tables are built
+ * by the first call of this function or of gmg_vcycle with fp32 (outside a
+ * stream capture; inside one it runs path 0).  Errors: INVALID_ARG, OOM, CUDA. */
 gmg_status gmg_level_path(gmg_handle h, int l, int *path);
 /* Copies level l's Galerkin operator A_l (CSR, caller numbering, rowptr n+1,
  * col/val nnz) and its colouring (n) into host buffers; any may be NULL. */

@@ -254,11 +254,9 @@ class Solver:
             n, nnz, nc = ctypes.c_int64(), ctypes.c_int64(), ctypes.c_int()
             lib.gmg_level_info(h, l, ctypes.byref(n), ctypes.byref(nnz), ctypes.byref(nc))
             self.dims.append((n.value, nnz.value, nc.value))
-        self.paths = []  # per level, how the FP32 cycle runs it (gmg_level_path)
-        for l in range(self.nlev):
-            p = ctypes.c_int()
-            lib.gmg_level_path(h, l, ctypes.byref(p))
-            self.paths.append(p.value)
+        self._paths = None
+        if precision in (GMG_FP32_REFINE, GMG_FP32_PCG):
+            self.paths
         fl, dev = ctypes.c_uint32(0), ctypes.c_double(0.0)
         _check(lib.gmg_warnings(h, ctypes.byref(fl), ctypes.byref(dev)), "gmg_warnings")
         self.warnings = fl.value  # GMG_WARN_P_UNITY: some P_l row's weights do not sum to 1 within 1e-12
@@ -278,6 +276,18 @@ class Solver:
     @property
     def handle(self):
         return self._h
+
+    @property
+    def paths(self):
+        """Per level, how the FP32 cycle runs it (gmg_level_path).  With FP64
+        cycles asked once, before close(): it has the FP32 cycle's tables built."""
+        if self._paths is None:
+            paths, p = [], ctypes.c_int()
+            for l in range(self.nlev):
+                _check(self._lib.gmg_level_path(self._h, l, ctypes.byref(p)), "gmg_level_path")
+                paths.append(p.value)
+            self._paths = paths
+        return self._paths
 
     # ---- whole solves ----
     def solve(self, b, x=None, tol: float = 1e-10, history: int = 0, raise_on_fail: bool = True):

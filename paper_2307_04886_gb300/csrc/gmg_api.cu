@@ -756,6 +756,10 @@ gmg_status gmg_level_info(gmg_handle h, int l, int64_t* n, int64_t* nnz, int* nc
 
 gmg_status gmg_level_path(gmg_handle h, int l, int* path) {
   if (!h || !path || l < 0 || l >= h->nlev) return GMG_ERR_INVALID_ARG;
+  if (l < h->nlev - 1 && h->cl32_late) {
+    GMG_TRY(check_handle(h));
+    GMG_TRY(late_cluster(h, nullptr, false));
+  }
   if (l == h->nlev - 1)
     *path = 3;
   else if (h->cl32.l0 >= 0 && l >= h->cl32.l0)
@@ -864,6 +868,7 @@ gmg_status gmg_vcycle(gmg_handle h, int fp32, const double* b, double* x, void* 
   cudaStream_t s = (cudaStream_t)stream;
   GMG_TRY(join_inverse(h, s, true));
   Level& L = h->L[0];
+  if (fp32) GMG_TRY(late_cluster(h, s, true));
   if (fp32 ? h->cl32.l0 >= 0 : h->cl64.l0 >= 0) GMG_CK(cudaMemsetAsync(h->dstatus + 3, 0, sizeof(int), s));
   GMG_TRY(to_level(h, 0, fp32, b, L.b64, L.b32, s));
   GMG_TRY(to_level(h, 0, fp32, x, L.x64, L.x32, s));

@@ -1773,21 +1773,24 @@ inline bool coarsest_in_fp32(const gmg_ctx* c) {
   return bytes <= kSmemLimit;
 }
 
+// Whether level l takes no part in a cluster of ncta CTAs whatever fits.
+inline bool too_large(const gmg_ctx* c, int l, int ncta) {
+  const Level& L = c->L[l];
+  const int64_t parts = std::max(1, L.ncolor) * (int64_t)ncta;
+  return (L.nnz - L.n) / parts > kClPhaseEntries || (c->cl_small && L.n / parts >= kClWide) || L.A.entries > INT32_MAX;
+}
+inline std::vector<int> cluster_sizes(const gmg_ctx* c) {
+  return c->cl_ctas > 0 ? std::vector<int>{c->cl_ctas} : std::vector<int>{16, 8};
+}
+
 template <class T>
 void plan_one(const gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
               const std::vector<std::vector<int32_t>>& hcol, const std::vector<std::vector<int32_t>>& perm,
               const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P, Plan<T>& plan) {
   const int lam = c->nlev - 1;
-  auto env = [](const char* name) {
-    const char* e = std::getenv(name);
-    return e && e[0] == '1';
-  };
-  if (lam < 1 || env("GMG_NO_TAIL")) return;
-  const bool small_only = env("GMG_NO_CLUSTER_LEVEL");
-  std::vector<int> sizes = {16, 8};
-  if (const char* e = std::getenv("GMG_TAIL_CTAS")) sizes = {std::atoi(e)};
-  for (int ncta : sizes) {
-    if (ncta < 1 || ncta > 16) continue;
+  if (lam < 1 || c->cl_off) return;
+  for (int ncta : cluster_sizes(c)) {
+    if (ncta > 16) continue;
     for (int l0 = std::max(0, lam - kClMaxLevels); l0 < lam; ++l0) {
       // a quick lower bound of the shared memory before the tables are built
       constexpr int pu = sizeof(T) == 4 ? 2 : 1;
@@ -1795,9 +1798,7 @@ void plan_one(const gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
       bool skip = false;
       for (int l = l0; l < lam; ++l) {
         const Level& L = c->L[l];
-        const int64_t rows = L.n / (std::max(1, L.ncolor) * ncta);
-        skip = skip || (L.nnz - L.n) / (std::max(1, L.ncolor) * (int64_t)ncta) > kClPhaseEntries ||
-               (small_only && rows >= kClWide) || L.A.entries > INT32_MAX;
+        skip = skip || too_large(c, l, ncta);
         // x, b, 1/a_ii and a_ii of the rows; entries in shared memory, or two stages of a phase
         least += (L.n / ncta) * (int64_t)(4 * sizeof(T)) + (l == l0 ? (int64_t)sizeof(T) * (L.n / ncta) : 0);
         const int64_t e = (L.nnz - L.n) * (16 / pu) / ncta;
@@ -1868,7 +1869,7 @@ gmg_status finish_one(gmg_ctx* c, Plan<T>& plan) {
   plan.D.ainv = Src<T>::ainv(c);
   plan.D.ainv64 = c->Ainv;
   plan.D.err = c->dstatus + 3;
-  plan.D.polls = kWaitPolls;
+  plan.D.polls = c->wait_polls < 0 ? kWaitPolls : c->wait_polls;
   GMG_TRY(upload_tables(*plan.team, c, plan.tab, plan.D));
   Src<T>::desc(c) = plan.D;
   return GMG_OK;
@@ -1906,7 +1907,12 @@ gmg_status refresh_one(gmg_ctx* c, cudaStream_t s) {
 
 }  // namespace
 
-// The tables being built on host threads, one for each precision.  What a
+// Whether the handle's solves run FP64 cycles.
+static bool fp64_cycles(const gmg_ctx* c) {
+  return c->opt.precision == GMG_FP64 || c->opt.precision == GMG_FP64_PCG;
+}
+
+// The tables being built on host threads, of either precision.  What a
 // thread throws is thrown again by finish_cluster; the destructor waits for
 // the threads, so the job ends before what they read does.
 struct ClusterJob {
@@ -1946,10 +1952,21 @@ std::shared_ptr<ClusterJob> start_cluster(gmg_ctx* c, const std::vector<std::vec
   c->cl32 = ClusterDesc<float>{};
   c->cl64 = ClusterDesc<double>{};
   if (!c->single_rhs) return job;
-  // FP64 cycles in a solve: the modes that run them
-  if (c->opt.precision == GMG_FP64 || c->opt.precision == GMG_FP64_PCG)
+  auto env = [](const char* name) {
+    const char* e = std::getenv(name);
+    return e && e[0] == '1';
+  };
+  c->cl_off = env("GMG_NO_TAIL");
+  c->cl_small = env("GMG_NO_CLUSTER_LEVEL");
+  if (const char* e = std::getenv("GMG_TAIL_CTAS")) {
+    c->cl_ctas = std::atoi(e);
+    c->cl_off = c->cl_off || c->cl_ctas < 1;
+  }
+  c->cl32_late = fp64_cycles(c);
+  if (c->cl32_late)
     j.run(1, c->device, [&, c, P] { plan_one<double>(c, hrp, hcol, perm, iperm, P, j.p64); });
-  j.run(0, c->device, [&, c, P] { plan_one<float>(c, hrp, hcol, perm, iperm, P, j.p32); });
+  else
+    j.run(0, c->device, [&, c, P] { plan_one<float>(c, hrp, hcol, perm, iperm, P, j.p32); });
   return job;
 }
 
@@ -1961,8 +1978,57 @@ gmg_status finish_cluster(gmg_ctx* c, ClusterJob& job) {
   return finish_one<double>(c, job.p64);
 }
 
+gmg_status late_cluster(gmg_ctx* c, cudaStream_t s, bool values) try {
+  if (!c->cl32_late && !(values && c->cl32_stale)) return GMG_OK;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  bool capturing = cudaStreamIsCapturing(s, &cs) != cudaSuccess;  // the legacy stream while another one captures
+  if (capturing) cudaGetLastError();
+  capturing = capturing || cs != cudaStreamCaptureStatusNone;
+  if (c->cl32_late) {
+    if (capturing) return GMG_OK;
+    const int lam = c->nlev - 1, most = cluster_sizes(c)[0];
+    int lo = lam;  // the levels that may take part
+    while (lo > 0 && lo > lam - kClMaxLevels && !too_large(c, lo - 1, most)) --lo;
+    std::vector<std::vector<int64_t>> hrp(c->nlev);
+    std::vector<std::vector<int32_t>> hcol(c->nlev), perm(c->nlev), iperm(c->nlev), pidx(c->nlev);
+    std::vector<std::vector<double>> pw(c->nlev);
+    std::vector<gmg_prolong> P(c->nlev);
+    auto get = [](auto& v, const auto* d, int64_t n) {
+      v.resize((size_t)n);
+      return cudaMemcpy(v.data(), d, sizeof(v[0]) * (size_t)n, cudaMemcpyDeviceToHost);
+    };
+    for (int l = lo; l <= lam && lo < lam && !c->cl_off; ++l) {
+      Level& L = c->L[l];
+      GMG_CK(get(hrp[l], L.csr_rowptr, L.n + 1));
+      GMG_CK(get(hcol[l], L.csr_col, L.nnz));
+      GMG_CK(get(perm[l], L.perm, L.n));
+      GMG_CK(get(iperm[l], L.iperm, L.n));
+      if (l == lam) break;
+      GMG_CK(get(L.h_ptr, L.A.ptr, L.A.nslice + 1));
+      GMG_CK(get(pidx[l], L.p_idx_o, 3 * L.n));
+      GMG_CK(get(pw[l], L.p_w_o, 3 * L.n));
+      P[l] = {L.n, L.nc, pidx[l].data(), pw[l].data()};
+    }
+    Plan<float> plan;
+    if (lo < lam) plan_one<float>(c, hrp, hcol, perm, iperm, P.data(), plan);
+    for (Level& L : c->L) std::vector<int64_t>().swap(L.h_ptr);
+    GMG_TRY(finish_one<float>(c, plan));
+    c->cl32_late = false;
+    c->cl32_stale = c->cl32.l0 >= 0;
+  }
+  if (values && c->cl32_stale) {
+    GMG_TRY(refresh_one<float>(c, s));
+    c->cl32_stale = capturing;  // a captured launch has filled nothing yet
+  }
+  return GMG_OK;
+} catch (const std::exception& e) {
+  set_error(std::string("FP32 cluster tables: ") + e.what());
+  return GMG_ERR_OOM;
+}
+
 gmg_status refresh_cluster_values(gmg_ctx* c, cudaStream_t s) {
-  GMG_TRY(refresh_one<float>(c, s));
+  if (fp64_cycles(c)) c->cl32_stale = c->cl32.l0 >= 0;
+  else GMG_TRY(refresh_one<float>(c, s));
   return refresh_one<double>(c, s);
 }
 
@@ -1984,7 +2050,10 @@ template gmg_status launch_cluster<float>(gmg_ctx*, float*, const float*, bool, 
 template gmg_status launch_cluster<double>(gmg_ctx*, double*, const double*, bool, cudaStream_t);
 
 // The polls after which the waits of this handle's cluster launches give up.
-void set_wait_polls(gmg_ctx* c, int polls) { c->cl32.polls = c->cl64.polls = polls < 0 ? kWaitPolls : polls; }
+void set_wait_polls(gmg_ctx* c, int polls) {
+  c->wait_polls = polls;
+  c->cl32.polls = c->cl64.polls = polls < 0 ? kWaitPolls : polls;
+}
 
 // Self-test of the bounded wait: one warp waits on an mbarrier that nothing
 // arrives on, so every poll fails and the wait gives up; elapsed device time

@@ -297,6 +297,12 @@ struct gmg_ctx {
   bool single_rhs = true;  // false: a member of a many-mesh handle, whose cycles are all batched
   gmg::ClusterDesc<float> cl32{};
   gmg::ClusterDesc<double> cl64{};
+  // handles whose solves run FP64 cycles: the FP32 tables are built for the first
+  // FP32 cycle, and filled again for the first one after a refresh
+  bool cl32_late = false, cl32_stale = false;
+  bool cl_off = false, cl_small = false;  // GMG_NO_TAIL, GMG_NO_CLUSTER_LEVEL and
+  int cl_ctas = 0;                        // GMG_TAIL_CTAS at set-up (0: 16, else 8)
+  int wait_polls = -1;                    // limit of the cluster launches' waits (-1: the default)
   float* Ainv32 = nullptr;  // coarsest inverse in FP32 for the cluster launch
   int* dstatus = nullptr;   // device status words
   // outer iteration (finest level, permuted numbering, FP64)
@@ -361,9 +367,9 @@ gmg_status join_inverse(gmg_ctx* c, cudaStream_t s, bool check);
 // Reads the pivot check of a joined inverse once (GMG_ERR_CHOLESKY on failure).
 gmg_status inverse_status(gmg_ctx* c, cudaStream_t s);
 // The cluster form of the coarse levels (gmg_cluster.cu): tables from the
-// levels' patterns and numberings (built on host threads between start and
-// finish, which uploads them; the arguments outlive the job), values after a
-// numeric set-up, the launch x <- MGI(x, b, l0), and the state of its bounded
+// levels' patterns and numberings, for the precision of the handle's cycles
+// (built on host threads between start and finish, which uploads them; the
+// arguments outlive the job), values after a numeric set-up, the launch x <- MGI(x, b, l0), and the state of its bounded
 // waits.
 struct ClusterJob;
 std::shared_ptr<ClusterJob> start_cluster(gmg_ctx* c, const std::vector<std::vector<int64_t>>& hrp,
@@ -371,6 +377,10 @@ std::shared_ptr<ClusterJob> start_cluster(gmg_ctx* c, const std::vector<std::vec
                                           const std::vector<std::vector<int32_t>>& perm,
                                           const std::vector<std::vector<int32_t>>& iperm, const gmg_prolong* P);
 gmg_status finish_cluster(gmg_ctx* c, ClusterJob& job);
+// The FP32 tables of a handle whose solves run FP64 cycles, if they have not
+// been built; with `values` also filled from the level values.  Nothing is
+// built while s is capturing (the cycle then runs as launches per colour).
+gmg_status late_cluster(gmg_ctx* c, cudaStream_t s, bool values);
 gmg_status refresh_cluster_values(gmg_ctx* c, cudaStream_t s);
 template <class T>
 gmg_status launch_cluster(gmg_ctx* c, T* x, const T* b, bool c0_first, cudaStream_t s);
