@@ -49,7 +49,7 @@ typedef enum {
   GMG_ERR_CHOLESKY = 4,       /* coarsest operator not positive definite     */
   GMG_ERR_NOT_CONVERGED = 5,  /* max_iter reached; x holds the last iterate  */
   GMG_ERR_NONFINITE = 6,      /* NaN/Inf in an input or in an iterate        */
-  GMG_ERR_OOM = 7,            /* device allocation failed                    */
+  GMG_ERR_OOM = 7,            /* device allocation, host memory or threads    */
   GMG_ERR_CUDA = 8,           /* a CUDA runtime call failed                  */
   GMG_ERR_TIMEOUT = 9,        /* a bounded device-side wait gave up          */
   GMG_ERR_TOO_LARGE = 10      /* a size exceeds a documented limit           */

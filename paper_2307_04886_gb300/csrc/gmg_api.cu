@@ -5,9 +5,10 @@
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
+#include <exception>
 #include <new>
-#include <vector>
 #include <string>
+#include <vector>
 
 #include "gmg_cycle.cuh"
 
@@ -440,7 +441,13 @@ gmg_status new_handle(gmg_handle* h, const gmg_csr* A, int n_prolong, const gmg_
     delete c;
     return GMG_ERR_INVALID_ARG;
   }
-  gmg_status st = setup_impl(c, A, n_prolong, P, coloring, (cudaStream_t)stream);
+  gmg_status st;
+  try {
+    st = setup_impl(c, A, n_prolong, P, coloring, (cudaStream_t)stream);
+  } catch (const std::exception& e) {  // host memory or threads: no exception leaves a C entry
+    set_error(std::string("gmg_setup: ") + e.what());
+    st = GMG_ERR_OOM;
+  }
   if (st != GMG_OK) {
     std::string keep = g_last_error;
     gmg_destroy(c);
