@@ -25,8 +25,12 @@ struct MCols {
   static constexpr int V = NR < 4 ? NR : 4;
   static constexpr int Q = NR / V;
 };
-constexpr int kMPre = 8;            // entries of a row part whose gathers are in flight together
-constexpr int kMRestrictParts = 4;  // warps per coarse row in the restriction (18-40 terms per row)
+// Entries of a row part whose gathers are in flight together (131,072 rows x 8
+// columns: 4.14 ms a solve, 4.56 with four).
+constexpr int kMPre = 8;
+// Warps per coarse row in the restriction (18-40 terms per row): 4.20, 4.17,
+// 4.14 and 4.21 ms for the same solve with 1, 2, 4 and 8.
+constexpr int kMRestrictParts = 4;
 
 template <int V>
 __device__ __forceinline__ void load_cols(const float* p, float (&o)[V]) {

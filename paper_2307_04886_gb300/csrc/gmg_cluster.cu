@@ -73,6 +73,7 @@
 #include <algorithm>
 #include <atomic>
 #include <condition_variable>
+#include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <exception>
@@ -94,10 +95,14 @@ namespace {
 constexpr int kClThreads = 256;
 constexpr int kClWarps = kClThreads / 32;
 constexpr int kClSlack = 2048;  // shared memory past the last entry unit
-constexpr int kClWide = 64;  // rows per phase and CTA from which a level keeps one thread per row
-// Entries per phase and CTA up to which a level runs here: above, a phase is
-// bound by the shared-memory gathers of 16 SMs and a grid launch over all SMs
-// is as fast.
+// Rows per phase and CTA from which a level keeps one thread per row, with the
+// sums of the per-colour kernels (32, 64 and 128 measure alike, within 0.5 %, on
+// spheres, tori, the bi-Laplacian and the book: the line is drawn for the bits
+// of the large levels, not for speed).
+constexpr int kClWide = 64;
+// Entries per phase and CTA up to which a level is considered: two stages of
+// more would fill the shared memory (FP32: 96 KB each of 227), and the tables
+// of levels that cannot fit are not built.
 constexpr int64_t kClPhaseEntries = 12288;
 
 __device__ __forceinline__ unsigned cl_rank() {
@@ -594,9 +599,12 @@ __global__ void __launch_bounds__(kClThreads, 1)
         const int bytes = *reinterpret_cast<const int*>(img + L.i_ex);
         const uint32_t a_xd = sm0 + (uint32_t)(L.o_img + L.i_xd), a_x = sm0 + (uint32_t)L.o_x;
         constexpr bool kWiden = sizeof(A) > sizeof(T);
-        // rows at a time and coefficients of each that a lane holds: as many as
-        // the registers take without spills (columns past 32 kA are loaded as
-        // they are added)
+        // rows at a time and coefficients of each that a lane holds (and loads
+        // before the wait): as many as the registers take without spills.
+        // Columns past 32 kA are loaded as they are added, which a wait for L2
+        // each 128 columns makes dear: with kA = 12 the solve on the 250x122
+        // torus (761 columns) took 892 us for 822, the bi-Laplacian 2407 for
+        // 2267; two rows at a time measure as four
         constexpr int kC = sizeof(A) == 4 ? 4 : 1, kA = 24;
         const uint32_t a_rhs = kWiden ? sm0 + (uint32_t)D.o_bd : a_bc;
         const int n = D.nc;
@@ -1872,6 +1880,10 @@ gmg_status finish_one(gmg_ctx* c, Plan<T>& plan) {
   plan.D.polls = c->wait_polls < 0 ? kWaitPolls : c->wait_polls;
   GMG_TRY(upload_tables(*plan.team, c, plan.tab, plan.D));
   Src<T>::desc(c) = plan.D;
+  if (const char* e = std::getenv("GMG_VERBOSE"))
+    if (e[0] == '1')
+      std::fprintf(stderr, "gmg: FP%d cluster: from level %d, %d CTAs, %d stages, %d bytes of shared memory\n",
+                   8 * (int)sizeof(T), plan.D.l0, plan.D.ncta, plan.D.nstage, plan.D.smem);
   return GMG_OK;
 }
 
