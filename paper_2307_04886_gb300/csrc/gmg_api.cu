@@ -876,13 +876,15 @@ gmg_status gmg_vcycle(gmg_handle h, int fp32, const double* b, double* x, void* 
   GMG_TRY(join_inverse(h, s, true));
   Level& L = h->L[0];
   if (fp32) GMG_TRY(late_cluster(h, s, true));
-  if (fp32 ? h->cl32.l0 >= 0 : h->cl64.l0 >= 0) GMG_CK(cudaMemsetAsync(h->dstatus + 3, 0, sizeof(int), s));
+  // the error word is this cycle's only where a cluster launch is part of it
+  const bool cluster = (fp32 ? h->cl32.l0 : h->cl64.l0) >= 0;
+  if (cluster) GMG_CK(cudaMemsetAsync(h->dstatus + 3, 0, sizeof(int), s));
   GMG_TRY(to_level(h, 0, fp32, b, L.b64, L.b32, s));
   GMG_TRY(to_level(h, 0, fp32, x, L.x64, L.x32, s));
   if (fp32) GMG_TRY(vcycle<float>(h, 0, s));
   else GMG_TRY(vcycle<double>(h, 0, s));
   if (fp32) GMG_TRY(launch_f2d(L.n, L.x32, L.x64, s));
-  return launch_scatter_cycle(h, L.x64, x, s);
+  return cluster ? launch_scatter_cycle(h, L.x64, x, s) : launch_scatter(L.n, L.perm, L.x64, x, s);
 }
 
 }  // extern "C"
