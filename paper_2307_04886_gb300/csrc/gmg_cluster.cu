@@ -1991,7 +1991,7 @@ gmg_status finish_cluster(gmg_ctx* c, ClusterJob& job) {
 }
 
 gmg_status late_cluster(gmg_ctx* c, cudaStream_t s, bool values) try {
-  if (!c->cl32_late && !(values && c->cl32_stale)) return GMG_OK;
+  if (!c->cl32_late && !(values && fp64_cycles(c) && c->cl32.l0 >= 0)) return GMG_OK;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   bool capturing = cudaStreamIsCapturing(s, &cs) != cudaSuccess;  // the legacy stream while another one captures
   if (capturing) cudaGetLastError();
@@ -2031,6 +2031,8 @@ gmg_status late_cluster(gmg_ctx* c, cudaStream_t s, bool values) try {
   if (values && c->cl32_stale) {
     GMG_TRY(refresh_one<float>(c, s));
     c->cl32_stale = capturing;  // a captured launch has filled nothing yet
+  } else if (values && capturing && c->cl32.l0 >= 0) {
+    c->cl32_captured = true;  // replayed after refreshes without coming by here
   }
   return GMG_OK;
 } catch (const std::exception& e) {
@@ -2039,7 +2041,7 @@ gmg_status late_cluster(gmg_ctx* c, cudaStream_t s, bool values) try {
 }
 
 gmg_status refresh_cluster_values(gmg_ctx* c, cudaStream_t s) {
-  if (fp64_cycles(c)) c->cl32_stale = c->cl32.l0 >= 0;
+  if (fp64_cycles(c) && !c->cl32_captured) c->cl32_stale = c->cl32.l0 >= 0;
   else GMG_TRY(refresh_one<float>(c, s));
   return refresh_one<double>(c, s);
 }

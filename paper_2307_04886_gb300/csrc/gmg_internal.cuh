@@ -298,8 +298,9 @@ struct gmg_ctx {
   gmg::ClusterDesc<float> cl32{};
   gmg::ClusterDesc<double> cl64{};
   // handles whose solves run FP64 cycles: the FP32 tables are built for the first
-  // FP32 cycle, and filled again for the first one after a refresh
-  bool cl32_late = false, cl32_stale = false;
+  // FP32 cycle, and filled again for the first one after a refresh (by every
+  // refresh once a caller's capture holds an FP32 cycle that reads them as they are)
+  bool cl32_late = false, cl32_stale = false, cl32_captured = false;
   bool cl_off = false, cl_small = false;  // GMG_NO_TAIL, GMG_NO_CLUSTER_LEVEL and
   int cl_ctas = 0;                        // GMG_TAIL_CTAS at set-up (0: 16, else 8)
   int wait_polls = -1;                    // limit of the cluster launches' waits (-1: the default)
