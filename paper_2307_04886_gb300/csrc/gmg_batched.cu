@@ -1327,7 +1327,8 @@ extern "C" gmg_status gmg_setup_many(gmg_many* out, int nmesh, const gmg_csr* A,
   if (ok) {
     std::vector<double*> rr(nmesh);
     for (int k = 0; k < nmesh; ++k) rr[k] = m->h[k]->scal + 8;
-    ok = ck(cudaMemcpy(m->d_rr, rr.data(), sizeof(double*) * (size_t)nmesh, cudaMemcpyHostToDevice));
+    ok = ck(cudaMemcpy(m->d_rr, rr.data(), sizeof(double*) * (size_t)nmesh, cudaMemcpyHostToDevice)) &&
+         uploads_landed() == GMG_OK;
   }
   if (!ok) {
     gmg_destroy_many(m);

@@ -2025,6 +2025,7 @@ gmg_status late_cluster(gmg_ctx* c, cudaStream_t s, bool values) try {
     if (lo < lam) plan_one<float>(c, hrp, hcol, perm, iperm, P.data(), plan);
     for (Level& L : c->L) std::vector<int64_t>().swap(L.h_ptr);
     GMG_TRY(finish_one<float>(c, plan));
+    GMG_TRY(uploads_landed());
     c->cl32_late = false;
     c->cl32_stale = c->cl32.l0 >= 0;
   }

@@ -145,6 +145,15 @@ struct Arena {
   }
 };
 
+// Set-up tables are copied (and cleared) through the legacy stream from pageable
+// memory: such a call may return while the last of it is on its way, and a
+// caller's stream need not wait for that stream.  Called before the first
+// kernel that reads them.
+inline gmg_status uploads_landed() {
+  GMG_CK(cudaStreamSynchronize(cudaStreamLegacy));
+  return GMG_OK;
+}
+
 // A sliced-ELL matrix: rows grouped in slices of 32 consecutive rows; slice s
 // stores width_s columns as [k][lane] (entry (row0_s + lane, k) at
 // ptr[s] + k * 32 + lane), so a warp's loads of one k are contiguous.

@@ -125,6 +125,7 @@ gmg_status gmg_setup_ML(gmg_handle* h, const double* M_diag, const gmg_csr* L, d
     set_error("gmg_setup_ML: upload failed");
     return fail(GMG_ERR_CUDA);
   }
+  if ((st = uploads_landed()) != GMG_OK) return fail(st);
   c->ml_t = t;
   return GMG_OK;
 }

@@ -1556,6 +1556,7 @@ static gmg_status galerkin_symbolic(gmg_ctx* c, int l, cudaStream_t s, std::vect
   GMG_TRY(upload(c->arena, &C.plan_mirror, mir.data(), mir.size()));
   GMG_TRY(upload(c->arena, &C.plan_up, up.data(), up.size()));
   GMG_TRY(upload(c->arena, &C.plan_sptr, sptr.data(), sptr.size()));
+  GMG_TRY(uploads_landed());
   GMG_TRY(c->arena.alloc(&C.plan_sedge, (size_t)sptr.back()));
   GMG_TRY(c->arena.alloc(&C.plan_scoef, (size_t)sptr.back()));
   k_plan_slice<<<grid_for(C.plan_nup, 256), 256, 0, s>>>(C.plan_nup, C.plan_up, C.plan_ptr, C.plan_edge, C.plan_coef,
@@ -1876,6 +1877,7 @@ gmg_status setup_impl(gmg_ctx* c, const gmg_csr* A, int nP, const gmg_prolong* P
   };
   lap(0, "gmg_setup: symbolic Galerkin product");
   start_colouring(0);
+  GMG_TRY(uploads_landed());
   for (int l = 0; l + 1 < c->nlev; ++l) {
     GMG_TRY(galerkin_symbolic(c, l, s, hrp[l + 1], hcol[l + 1]));
     start_colouring(l + 1);
@@ -1930,6 +1932,7 @@ gmg_status setup_impl(gmg_ctx* c, const gmg_csr* A, int nP, const gmg_prolong* P
   lap(3, "gmg_setup: cluster tables");
   GMG_TRY(finish_cluster(c, *cluster));
   for (Level& L : c->L) std::vector<int64_t>().swap(L.h_ptr);
+  GMG_TRY(uploads_landed());
   lap(4, "gmg_setup: numeric set-up");
   const gmg_status st = numeric_setup(c, s, false);
   if (const char* e = std::getenv("GMG_VERBOSE"))
