@@ -552,7 +552,6 @@ static gmg_status ensure_batched(gmg_ctx* c) {
     GMG_TRY(c->arena.alloc(&L.R32, (size_t)L.n * kMaxRhs));
   }
   const int64_t n = c->L[0].n;
-  GMG_TRY(c->arena.alloc(&c->XS, (size_t)n * kMaxRhs));
   GMG_TRY(c->arena.alloc(&c->BS, (size_t)n * kMaxRhs));
   GMG_TRY(c->arena.alloc(&c->RS, (size_t)n * kMaxRhs));
   // per-column partials of the batched residual, and never smaller than the
@@ -562,7 +561,9 @@ static gmg_status ensure_batched(gmg_ctx* c) {
   GMG_TRY(c->arena.alloc(&red2, (size_t)need));
   c->red = red2;
   c->red_cap = need;
-  return GMG_OK;
+  // last: it says that all of them are there (a call that ran out of memory on
+  // the way leaves it null, and the next one starts again)
+  return c->arena.alloc(&c->XS, (size_t)n * kMaxRhs);
 }
 
 // The device-side loop of the batched solve for blocks of NR columns: a graph

@@ -124,6 +124,7 @@ struct Arena {
     ms_alloc += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     ++n_alloc;
     if (e != cudaSuccess) {
+      cudaGetLastError();  // reported here, not by the next launch
       set_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
       return GMG_ERR_OOM;
     }
