@@ -1011,7 +1011,7 @@ static gmg_status build_one(int64_t n, int64_t nnz, const double* X, const int64
     int64_t nlat = 0;
     GMG_CK(cudaMemcpyAsync(&nlat, off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     GMG_CK(cudaStreamSynchronize(s));
-    GMG_TRY(B.get(&later, (size_t)nlat));
+    GMG_TRY(B.get(&later, (size_t)nlat + 1));  // k_mis_chain prefetches the start of an empty list, too
     k_balls<<<G, 128, 0, s>>>(n, len, rp, ci, geo, nlater, blockers, off, later, err, err2);
     GMG_LAUNCHED();
   }
